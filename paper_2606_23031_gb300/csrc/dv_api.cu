@@ -131,7 +131,7 @@ struct BatchState {
     float4* nrm = nullptr;  // per record voxel normal (world), when the call renders normals
     uint32_t* sorted_g = nullptr;
     uint32_t* pval = nullptr;
-    uint8_t* pmask = nullptr;  // per pair: 8x4-pixel blocks of the tile the voxel touches
+    uint16_t* prect = nullptr;  // per pair: the voxel's pixel rectangle within the tile
     uint2* range = nullptr;
     uint32_t* vis_start = nullptr;
     uint32_t* tile_order = nullptr;
@@ -542,7 +542,7 @@ struct StateBuffers1 {
     VoxRec* rec = nullptr;
     float4* nrm = nullptr;
     uint32_t* pval = nullptr;
-    uint8_t* pmask = nullptr;
+    uint16_t* prect = nullptr;
 };
 
 Layout state1_layout(int64_t n_vis, int64_t P, bool normals, StateBuffers1* b) {
@@ -551,7 +551,7 @@ Layout state1_layout(int64_t n_vis, int64_t P, bool normals, StateBuffers1* b) {
     L.add(b ? &b->rec : nullptr, n_vis);
     if (normals) L.add(b ? &b->nrm : nullptr, n_vis);
     L.add(b ? &b->pval : nullptr, P);
-    L.add(b ? &b->pmask : nullptr, P);
+    L.add(b ? &b->prect : nullptr, P);
     return L;
 }
 
@@ -876,7 +876,7 @@ dv_status render_batch(dv_ctx* ctx, const dv_octree* oct, int n_oct, const dv_po
     B.rec = sb1.rec;
     B.nrm = sb1.nrm;
     B.pval = sb1.pval;
-    B.pmask = sb1.pmask;
+    B.prect = sb1.prect;
     bp.sorted_g = B.sorted_g;
     bp.nrm = B.nrm;
     e = cudaMemsetAsync(post.zero, 0, (size_t)post.zero_bytes, s);
@@ -909,7 +909,7 @@ dv_status render_batch(dv_ctx* ctx, const dv_octree* oct, int n_oct, const dv_po
         // the call's own sort flag goes to its status slot (read by dv_state_check, the backward and
         // the serving loop), so a timeout is reported to the call that had it
         if (e == cudaSuccess)
-            e = launch_pair_mask(bp, sorted_tile, B.pval, post.rect_sorted, P, n_vis, B.pmask, B.range,
+            e = launch_pair_rect(bp, sorted_tile, B.pval, post.rect_sorted, P, n_vis, B.prect, B.range,
                                  B.d_sort_err, B.h_status_dev, s);
         if (e == cudaSuccess) B.published = true;
         if (e == cudaSuccess)
@@ -919,7 +919,7 @@ dv_status render_batch(dv_ctx* ctx, const dv_octree* oct, int n_oct, const dv_po
     {
         Prof p(ctx, KP_FWD, s);
         if (e == cudaSuccess)
-            e = launch_composite_fwd(bp, B.rec, B.pval, B.pmask, B.range, B.vis_start, B.tile_order, B.n_seg,
+            e = launch_composite_fwd(bp, B.rec, B.pval, B.prect, B.range, B.vis_start, B.tile_order, B.n_seg,
                                      B.t_final, B.work, &ctx->fork, s);
     }
     ar.release();
@@ -939,7 +939,7 @@ dv_status backward_batch(dv_ctx* ctx, dv_state* st, const float* d_rgb, const fl
     {
         Prof p(ctx, KP_BWD, s);
         if (e == cudaSuccess)
-            e = dv::launch_composite_bwd(B.bp, B.rec, B.pval, B.pmask, B.range, B.vis_start, B.tile_order, B.t_final,
+            e = dv::launch_composite_bwd(B.bp, B.rec, B.pval, B.prect, B.range, B.vis_start, B.tile_order, B.t_final,
                                          d_rgb, d_depth, d_alpha, d_normal, grad, &ctx->fork, s);
     }
     {
@@ -1244,7 +1244,7 @@ dv_status dv_state_weights(dv_ctx* ctx, dv_state* st, const int64_t* offsets, ui
     if (B.n_pix == 0 || B.n_vis == 0) return DV_OK;
     if (!offsets || !voxel || !weight) return fail(ctx, DV_ERR_INVALID_ARG, "NULL buffer");
     DeviceGuard g(ctx->device);
-    cudaError_t e = dv::launch_composite_export(B.bp, B.rec, B.pval, B.pmask, B.range, B.vis_start, B.tile_order,
+    cudaError_t e = dv::launch_composite_export(B.bp, B.rec, B.pval, B.prect, B.range, B.vis_start, B.tile_order,
                                                 offsets, voxel, weight, &ctx->fork, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "weights export");
     return DV_OK;

@@ -61,6 +61,7 @@ struct GradLayout {
 // that 5 or more cover (beyond 8, the remaining actors take the per-thread walk)
 constexpr int NTA_SMALL = 4;
 constexpr int NTA_LARGE = 8;
+constexpr int LANE_GAIN = 2;  // see walk_actor
 
 struct PixBase {
     float C0, C1, C2, D, T;
@@ -491,10 +492,45 @@ __device__ __forceinline__ void warp_reduce_add(const float* acc, float* gp) {
     if (nreal > 0 && v[0] != 0.0f) atomicAdd(gp + idx, v[0]);
 }
 
+// One lane's gradient values of record r, added with 16-byte vector atomics (the rows are 16-byte
+// aligned and padded to a multiple of four floats).
+template <bool NRM>
+__device__ __forceinline__ void lane_add(float* grad_rec, uint32_t r, const float* acc) {
+    constexpr int NV = GradLayout<NRM>::NV;
+    float4* gp = reinterpret_cast<float4*>(grad_rec + (size_t)r * GradLayout<NRM>::STRIDE);
+#pragma unroll
+    for (int c = 0; c < NV; c += 4)
+        atomicAdd(gp + c / 4, make_float4(acc[c], acc[c + 1], c + 2 < NV ? acc[c + 2] : 0.0f, c + 3 < NV ? acc[c + 3] : 0.0f));
+}
+
 // Record of pair q.  Every pair's record is below n_vis unless a sort's bounded wait ran out (the
 // call is then reported as timed out); the clamp keeps the reads and gradient atomics in range.
 __device__ __forceinline__ uint32_t rec_index(const BatchParams& bp, const uint32_t* __restrict__ pval, uint32_t q) {
     return min(__ldg(pval + q), (uint32_t)(bp.n_vis - 1));
+}
+
+// Pixels of the 8x4 block (bx, by) of a tile that a pair's pixel rectangle covers, as lane bits (lane
+// l renders pixel (l & 7, l >> 3) of the block).  rc: the rectangle within the tile, x0 | x1 << 4 |
+// y0 << 8 | y1 << 12.
+__device__ __forceinline__ uint32_t block_pixels(uint32_t rc, int bx, int by) {
+    const int x0 = (int)(rc & 15u) - 8 * bx, x1 = (int)((rc >> 4) & 15u) - 8 * bx;
+    const int y0 = (int)((rc >> 8) & 15u) - 4 * by, y1 = (int)((rc >> 12) & 15u) - 4 * by;
+    const uint32_t xm = (0xffu << max(x0, 0)) & (0xffu >> max(7 - x1, 0));
+    const uint32_t ym = (0xfu << max(y0, 0)) & (0xfu >> max(3 - y1, 0));
+    return (xm & 0xffu) * (((ym & 0xfu) * 0x00204081u) & 0x01010101u);
+}
+
+// Transpose of the 32x32 bit matrix whose row l is lane l's x: afterwards bit j of lane l is bit l of
+// what lane j held.
+__device__ __forceinline__ uint32_t warp_transpose(uint32_t x) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int k = 16; k >= 1; k >>= 1) {
+        const uint32_t m = k == 16 ? 0x0000ffffu : k == 8 ? 0x00ff00ffu : k == 4 ? 0x0f0f0f0fu : k == 2 ? 0x33333333u : 0x55555555u;
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, k);
+        x = (lane & k) ? (x & ~m) | ((y >> k) & m) : (x & m) | ((y << k) & ~m);
+    }
+    return x;
 }
 
 // Per-lane walk of one actor's sub-list (divergent; only for actors beyond the
@@ -502,15 +538,15 @@ __device__ __forceinline__ uint32_t rec_index(const BatchParams& bp, const uint3
 template <bool GRAD, int KS, bool NRM, bool WEX>
 __device__ __noinline__ void walk_actor_lane(Pix<NRM>& ps, const Bwd<NRM>& bw, const BatchParams& bp,
                                              const OctParams* __restrict__ vo, const ActInt& it,
-                                             const uint32_t* __restrict__ pval, const uint8_t* __restrict__ pmask,
-                                             uint32_t wbit, const VoxRec* __restrict__ rec, uint32_t q0, uint32_t q1,
+                                             const uint32_t* __restrict__ pval, const uint16_t* __restrict__ prect,
+                                             int bx, int by, const VoxRec* __restrict__ rec, uint32_t q0, uint32_t q1,
                                              const float* dc, float* grad_rec, ExportSink* ex) {
     const OctParams& P = vo[it.o];
     float d[3];
     rotate(P.A, dc, d);
     const InvDir inv = inv_dir(d);
     for (uint32_t q = q0; q < q1 && !ps.done; ++q) {
-        if (!(__ldg(pmask + q) & wbit)) continue;
+        if (!((block_pixels(__ldg(prect + q), bx, by) >> (threadIdx.x & 31)) & 1u)) continue;
         ps.tests += 1;
         const uint32_t r = rec_index(bp, pval, q);
         const float4* R = rec[r].v;
@@ -568,7 +604,7 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
                                                   : DV_PLAIN_MIN_BLOCKS) k_composite(const __grid_constant__ BatchParams bp,
                                                         const VoxRec* __restrict__ rec,
                                                         const uint32_t* __restrict__ pval,
-                                                        const uint8_t* __restrict__ pmask,
+                                                        const uint16_t* __restrict__ prect,
                                                         const uint2* __restrict__ tile_range,
                                                         const uint32_t* __restrict__ vis_start,
                                                         const uint32_t* __restrict__ tile_order,
@@ -584,13 +620,15 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
     pdl_wait();
     pdl_launch_dependents();
     constexpr bool REPLAY = BWD || WEX;  // phase 3 replays every actor interval the ray reached
-    __shared__ float4 s_rec[2][CT_THREADS][4];
+    constexpr bool ACT = NTA > 0;
+    // with actors, lanes read different records at once: rows of 80 bytes spread them over the banks
+    constexpr int RS = ACT ? 5 : 4;
+    __shared__ float4 s_rec[2][CT_THREADS][RS];
     __shared__ float4 s_nv[NRM ? 2 : 1][NRM ? CT_THREADS : 1];  // voxel normals of the staged records
     __shared__ uint32_t s_r[2][CT_THREADS];
-    __shared__ uint8_t s_m[2][CT_THREADS];
+    __shared__ uint16_t s_m[2][CT_THREADS];         // pixel rectangles of the staged pairs within the tile
     __shared__ uint32_t s_sub[DV_MAX_OCTREES + 1];  // sub-list of octree o: [s_sub[o], s_sub[o+1])
     __shared__ uint32_t s_vs[DV_MAX_OCTREES + 1];   // first record of octree o in this view
-    constexpr bool ACT = NTA > 0;
     // the backward carries the residual form: the actor partials, the states recorded at actor
     // entries and the replays hold (R, T) instead of the prefix colour, depth (and normal)
     constexpr bool RFORM = BWD;
@@ -629,9 +667,9 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
     rg.x = min(rg.x, rg.y);
     // per-pixel set-up first: its loads overlap the tile set-up below
     const int lane = tid & 31, warp = tid >> 5;
-    const uint32_t wbit = 1u << ((half * 2 + (warp >> 1)) * 2 + (warp & 1));  // this warp's 8x4 block
-    const int u = tx * DV_TILE + (warp & 1) * 8 + (lane & 7);
-    const int v = ty * DV_TILE + half * 8 + (warp >> 1) * 4 + (lane >> 3);
+    const int bx = warp & 1, by = half * 2 + (warp >> 1);  // this warp's 8x4 block of the tile
+    const int u = tx * DV_TILE + bx * 8 + (lane & 7);
+    const int v = ty * DV_TILE + by * 4 + (lane >> 3);
     const bool valid = u < W && v < H;
     const int64_t lpix = (int64_t)v * W + u;       // pixel within the view's own images
     const int64_t pix = fp.pix_base + lpix;        // pixel within the call's per-pixel arrays
@@ -778,10 +816,10 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
 
     // Every sub-list (an actor's, then the background's) streams through the shared
     // two-slot ring, CT_THREADS records per batch (cp.async, one batch ahead).  Each warp
-    // visits the records of a batch that touch its 8x4 block (ballot over the pair
-    // masks), 32 at a time: chunk(slot, c0, m) gets the ring slot, the first record of
-    // the 32 and the mask of those to visit, and returns true once the warp has nothing
-    // left to do in this list.  The batch loop, its barriers and its early exit are
+    // visits the records of a batch that touch its 8x4 block, 32 at a time: chunk(slot, c0, pm)
+    // gets the ring slot, the first record of the 32 and, in lane i, the pixels of the block
+    // that record c0 + i may touch, and returns true once the warp has nothing left to do in
+    // this list.  The batch loop, its barriers and its early exit are
     // CTA-uniform.
     auto stream = [&](uint32_t q0, uint32_t q1, auto&& chunk) {
         const uint32_t n_batch = q1 > q0 ? (q1 - q0 + CT_THREADS - 1) / CT_THREADS : 0u;
@@ -795,13 +833,13 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
                 for (int k = 0; k < 4; ++k) cp_async16(&s_rec[0][tid][k], R + k);
                 if (NRM) cp_async16(&s_nv[0][NRM ? tid : 0], bp.nrm + r);
                 s_r[0][tid] = r;
-                s_m[0][tid] = __ldg(pmask + qa);
+                s_m[0][tid] = __ldg(prect + qa);
             }
             cp_async_commit();
             const uint32_t qb = q0 + CT_THREADS + tid;
             if (qb < q1) {
                 r_ahead = rec_index(bp, pval, qb);
-                m_ahead = __ldg(pmask + qb);
+                m_ahead = __ldg(prect + qb);
             }
         }
         bool fin = false;
@@ -815,13 +853,13 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
                     for (int k = 0; k < 4; ++k) cp_async16(&s_rec[slot ^ 1][tid][k], R + k);
                     if (NRM) cp_async16(&s_nv[NRM ? (slot ^ 1) : 0][NRM ? tid : 0], bp.nrm + r_ahead);
                     s_r[slot ^ 1][tid] = r_ahead;
-                    s_m[slot ^ 1][tid] = (uint8_t)m_ahead;
+                    s_m[slot ^ 1][tid] = (uint16_t)m_ahead;
                 }
                 cp_async_commit();
                 const uint32_t qb = q0 + (bi + 2) * CT_THREADS + tid;
                 if (qb < q1) {
                     r_ahead = rec_index(bp, pval, qb);
-                    m_ahead = __ldg(pmask + qb);
+                    m_ahead = __ldg(prect + qb);
                 }
             }
             cp_async_wait_one();  // batch bi has landed (only batch bi+1 may still be in flight)
@@ -829,8 +867,7 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
             const uint32_t cnt = min((uint32_t)CT_THREADS, q1 - q0 - bi * CT_THREADS);
             for (uint32_t c0 = 0; c0 < cnt && !fin; c0 += 32) {
                 const uint32_t jl = c0 + lane;
-                const unsigned m = __ballot_sync(0xffffffffu, jl < cnt && (s_m[slot][jl < cnt ? jl : 0] & wbit));
-                fin = chunk(slot, c0, m);
+                fin = chunk(slot, c0, jl < cnt ? block_pixels(s_m[slot][jl], bx, by) : 0u);
             }
             // every warp is done with this slot before batch bi+2 is copied into it
             if (__syncthreads_or(!fin) == 0) break;
@@ -846,9 +883,15 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
     constexpr int NV = GradLayout<NRM>::NV;
     constexpr int GS = GradLayout<NRM>::STRIDE;
 
-    // Lockstep walk of actor o's sub-list: lanes not yet done composite the segments inside
-    // their interval [a, b] of that actor into pt, with the stop rule (and, with G, the
-    // per-record gradients reduced across the warp).
+    // Walk of actor o's sub-list: lanes not yet done composite the segments inside their interval
+    // [a, b] of that actor into pt, with the stop rule (and, with G, the per-record gradients).
+    // An actor's voxels are a few pixels large or less, so of a warp's 32 pixels few meet a given
+    // record: visited in lockstep, a record costs the whole warp a step.  Instead the 32 records of
+    // a chunk are turned into one list per lane (a bit transpose of the records' pixel masks) and
+    // every lane steps through its own records, in list order, two at a time without gradients.
+    // With gradients a lane adds its own values to the record with 16-byte vector atomics; a chunk
+    // whose longest lane list is above 1 / LANE_GAIN of its records is walked in lockstep, where
+    // the warp sums a record's values first.
     auto walk_actor = [&](Pix<NRM>& pt, int o, float a, float b, auto grad, auto wex) {
         constexpr bool G = decltype(grad)::value;
         constexpr bool X = decltype(wex)::value;
@@ -856,18 +899,24 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
         float d[3];
         rotate(P.A, dc, d);
         const InvDir inv = inv_dir(d);
-        stream(s_sub[o], s_sub[o + 1], [&](int slot, uint32_t c0, unsigned m) -> bool {
-            while (m) {
-                if (__all_sync(0xffffffffu, pt.done)) return true;
-                const uint32_t j = c0 + (uint32_t)(__ffs(m) - 1);
-                m &= m - 1;
-                if constexpr (!G && !X && KS == 1) {
-                    if (m) {
-                        // two records at once (no gradients): both slab tests and optical depths, then the
-                        // two compositing steps in list order with the stop rule -- the arithmetic of two
-                        // single steps, with more independent work per warp on the actor walks
-                        const uint32_t j1 = c0 + (uint32_t)(__ffs(m) - 1);
-                        m &= m - 1;
+        stream(s_sub[o], s_sub[o + 1], [&](int slot, uint32_t c0, uint32_t pm) -> bool {
+            if (__all_sync(0xffffffffu, pt.done)) return true;
+            unsigned m = __ballot_sync(0xffffffffu, pm != 0u);
+            if (!m) return false;
+            uint32_t mine = warp_transpose(pm);
+            if (pt.done) mine = 0u;
+            bool lanes = true;
+            if constexpr (G) lanes = (int)__reduce_max_sync(0xffffffffu, (unsigned)__popc(mine)) * LANE_GAIN <= __popc(m);
+            if (lanes) {
+                while (mine) {
+                    const uint32_t j = c0 + (uint32_t)(__ffs(mine) - 1);
+                    mine &= mine - 1;
+                    if constexpr (!G && !X && KS == 1) {
+                        // two records at once: both slab tests and optical depths, then the two compositing
+                        // steps in list order with the stop rule -- the arithmetic of two single steps
+                        const bool two = mine != 0u;
+                        const uint32_t j1 = two ? c0 + (uint32_t)(__ffs(mine) - 1) : j;
+                        mine &= mine - 1;
                         const float4 g0 = s_rec[slot][j][0], g1 = s_rec[slot][j1][0];
                         float u0, v0, u1, v1;
                         const bool x0 = slab_cube(inv, g0, u0, v0), x1 = slab_cube(inv, g1, u1, v1);
@@ -875,8 +924,7 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
                         v0 = fminf(v0, b);
                         u1 = fmaxf(u1, a);
                         v1 = fminf(v1, b);
-                        const bool live = !pt.done;
-                        const bool h0 = live && x0 && v0 > u0, h1 = live && x1 && v1 > u1;
+                        const bool h0 = x0 && v0 > u0, h1 = two && x1 && v1 > u1;
                         const float s0 = h0 ? u0 : 0.0f, e0 = h0 ? v0 : 0.0f, s1 = h1 ? u1 : 0.0f, e1 = h1 ? v1 : 0.0f;
                         const float4 col0 = s_rec[slot][j][3], col1 = s_rec[slot][j1][3];
                         const float r0[3] = {g0.x, g0.y, g0.z}, r1[3] = {g1.x, g1.y, g1.z};
@@ -899,15 +947,45 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
                                 composite_tau<NRM>(pt, tau, col, nv, t0, t1, bp.eps_stop);
                             }
                         };
-                        pt.tests += live ? 1u : 0u;
+                        pt.tests += 1;
                         if (h0) apply(tau0, col0, staged_nv(slot, j), s0, e0);
-                        pt.tests += (live && !pt.done) ? 1u : 0u;
+                        pt.tests += (two && !pt.done) ? 1u : 0u;
                         if (h1 && !pt.done) apply(tau1, col1, staged_nv(slot, j1), s1, e1);
-                        continue;
+                    } else {
+                        pt.tests += 1;
+                        const float4 g = s_rec[slot][j][0];
+                        float t0, t1;
+                        if (slab_cube(inv, g, t0, t1)) {
+                            t0 = fmaxf(t0, a);
+                            t1 = fminf(t1, b);
+                            if (t1 > t0) {
+                                float acc[NV];
+                                if constexpr (G && RFORM && KS == 1) {
+                                    bwd_single_step<NRM>(pt, bw, bp, g, s_rec[slot][j][1], s_rec[slot][j][2],
+                                                         s_rec[slot][j][3], staged_nv(slot, j), d, t0, t1, true, acc);
+                                } else {
+#pragma unroll
+                                    for (int i = 0; i < NV; ++i) acc[i] = 0.0f;
+                                    const float rel[3] = {g.x, g.y, g.z};
+                                    add_segment<G, true, KS, NRM, X, RFORM>(pt, bw, bp, s_rec[slot][j][1],
+                                                                            s_rec[slot][j][2], s_rec[slot][j][3],
+                                                                            staged_nv(slot, j), rel, d, t0, t1, acc,
+                                                                            s_r[slot][j], &ex);
+                                }
+                                if constexpr (G) lane_add<NRM>(grad_rec, s_r[slot][j], acc);
+                            }
+                        }
                     }
+                    if (pt.done) mine = 0u;
                 }
-                if constexpr (G && RFORM && !X && KS == 1) {
-                    // replay with gradients: inside one actor interval a lane meets a record at most once
+                __syncwarp();
+                return __all_sync(0xffffffffu, pt.done);
+            }
+            if constexpr (G) {
+                while (m) {
+                    if (__all_sync(0xffffffffu, pt.done)) return true;
+                    const uint32_t j = c0 + (uint32_t)(__ffs(m) - 1);
+                    m &= m - 1;
                     const float4 g = s_rec[slot][j][0];
                     const bool live = !pt.done;
                     float t0, t1;
@@ -918,36 +996,20 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
                     pt.tests += live ? 1u : 0u;
                     if (!__any_sync(0xffffffffu, hit)) continue;
                     float acc[NV];
-                    bwd_single_step<NRM>(pt, bw, bp, g, s_rec[slot][j][1], s_rec[slot][j][2], s_rec[slot][j][3],
-                                         staged_nv(slot, j), d, hit ? t0 : 0.0f, hit ? t1 : 0.0f, hit, acc);
-                    warp_reduce_add<NV>(acc, grad_rec + (size_t)s_r[slot][j] * GS);
-                    continue;
-                }
-                float acc[NV];
-                if (G) {
+                    if constexpr (RFORM && KS == 1) {
+                        // inside one actor interval a lane meets a record at most once
+                        bwd_single_step<NRM>(pt, bw, bp, g, s_rec[slot][j][1], s_rec[slot][j][2], s_rec[slot][j][3],
+                                             staged_nv(slot, j), d, hit ? t0 : 0.0f, hit ? t1 : 0.0f, hit, acc);
+                    } else {
 #pragma unroll
-                    for (int i = 0; i < NV; ++i) acc[i] = 0.0f;
-                }
-                bool hit = false;
-                if (!pt.done) {
-                    pt.tests += 1;
-                    const float4 g = s_rec[slot][j][0];
-                    float t0, t1;
-                    if (slab_cube(inv, g, t0, t1)) {
-                        t0 = fmaxf(t0, a);
-                        t1 = fminf(t1, b);
-                        if (t1 > t0) {
-                            const float rel[3] = {g.x, g.y, g.z};
+                        for (int i = 0; i < NV; ++i) acc[i] = 0.0f;
+                        const float rel[3] = {g.x, g.y, g.z};
+                        if (hit)
                             add_segment<G, true, KS, NRM, X, RFORM>(pt, bw, bp, s_rec[slot][j][1], s_rec[slot][j][2],
-                                                             s_rec[slot][j][3], staged_nv(slot, j), rel, d, t0, t1,
-                                                             acc, s_r[slot][j], &ex);
-                            hit = true;
-                        }
+                                                                    s_rec[slot][j][3], staged_nv(slot, j), rel, d, t0,
+                                                                    t1, acc, s_r[slot][j], &ex);
                     }
-                }
-                if (G) {
-                    const unsigned any = __ballot_sync(0xffffffffu, hit);
-                    if (any) warp_reduce_add<NV>(acc, grad_rec + (size_t)s_r[slot][j] * GS);
+                    warp_reduce_add<NV>(acc, grad_rec + (size_t)s_r[slot][j] * GS);
                 }
             }
             return __all_sync(0xffffffffu, pt.done);
@@ -1065,14 +1127,15 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
             const ActInt il = it;
             const float dl[3] = {dc[0], dc[1], dc[2]};
             ExportSink xl = ex;
-            walk_actor_lane<BWD, KS, NRM, WEX>(pl, bl, bp, vo, il, pval, pmask, wbit, rec, s_sub[il.o],
+            walk_actor_lane<BWD, KS, NRM, WEX>(pl, bl, bp, vo, il, pval, prect, bx, by, rec, s_sub[il.o],
                                                s_sub[il.o + 1], dl, grad_rec, &xl);
             ps = pl;
             ex = xl;
         }
     };
 
-    stream(s_sub[0], s_sub[1], [&](int slot, uint32_t c0, unsigned m) -> bool {
+    stream(s_sub[0], s_sub[1], [&](int slot, uint32_t c0, uint32_t pm) -> bool {
+        unsigned m = __ballot_sync(0xffffffffu, pm != 0u);
         // one record of the batch, visited by the whole warp: actor entries, stop rule, gradients
         auto visit = [&](uint32_t j) {
             if constexpr (BWD && NTA == 0 && KS == 1) {
@@ -1456,7 +1519,7 @@ __global__ void __launch_bounds__(256) k_sh_bwd(const __grid_constant__ ShBwdPar
 // a frame -- are dispatched first), forked from and joined back into the call's stream by events, the
 // plain launch on the call's stream.  Without the extra streams they run one after the other.
 template <bool BWD, int KS, bool NRM, bool WEX>
-void composite_launch(const BatchParams& bp, const VoxRec* rec, const uint32_t* pval, const uint8_t* pmask,
+void composite_launch(const BatchParams& bp, const VoxRec* rec, const uint32_t* pval, const uint16_t* prect,
                       const uint2* tile_range, const uint32_t* vis_start, const uint32_t* tile_order,
                       uint32_t* n_seg, float* t_final, const float* g_rgb, const float* g_depth,
                       const float* g_alpha, const float* g_normal, float* grad_rec, unsigned long long* work,
@@ -1472,18 +1535,18 @@ void composite_launch(const BatchParams& bp, const VoxRec* rec, const uint32_t* 
     }
     if (n_large > 0) {
         launch_pdl(k_composite<BWD, KS, NRM, WEX, NTA_LARGE>, dim3(2 * n_large), dim3(CT_THREADS), s_large, bp, rec,
-                   pval, pmask, tile_range, vis_start, tile_order, n_seg, t_final, g_rgb, g_depth, g_alpha, g_normal,
+                   pval, prect, tile_range, vis_start, tile_order, n_seg, t_final, g_rgb, g_depth, g_alpha, g_normal,
                    grad_rec, work, ex_off, ex_vid, ex_w);
         count_launches(1);
     }
     if (n_small > 0) {
         launch_pdl(k_composite<BWD, KS, NRM, WEX, NTA_SMALL>, dim3(2 * n_small), dim3(CT_THREADS), s_small, bp, rec,
-                   pval, pmask, tile_range, vis_start, tile_order + n_large, n_seg, t_final, g_rgb, g_depth, g_alpha,
+                   pval, prect, tile_range, vis_start, tile_order + n_large, n_seg, t_final, g_rgb, g_depth, g_alpha,
                    g_normal, grad_rec, work, ex_off, ex_vid, ex_w);
         count_launches(1);
     }
     if (n_plain > 0) {
-        launch_pdl(k_composite<BWD, KS, NRM, WEX, 0>, dim3(2 * n_plain), dim3(CT_THREADS), s, bp, rec, pval, pmask,
+        launch_pdl(k_composite<BWD, KS, NRM, WEX, 0>, dim3(2 * n_plain), dim3(CT_THREADS), s, bp, rec, pval, prect,
                    tile_range, vis_start, tile_order + n_large + n_small, n_seg, t_final, g_rgb, g_depth, g_alpha,
                    g_normal, grad_rec, work, ex_off, ex_vid, ex_w);
         count_launches(1);
@@ -1499,21 +1562,21 @@ void composite_launch(const BatchParams& bp, const VoxRec* rec, const uint32_t* 
 }
 
 template <bool NRM>
-void composite_fwd_k(const BatchParams& bp, const VoxRec* rec, const uint32_t* pair_val, const uint8_t* pair_mask,
+void composite_fwd_k(const BatchParams& bp, const VoxRec* rec, const uint32_t* pair_val, const uint16_t* pair_rect,
                      const uint2* tile_range, const uint32_t* vis_start, const uint32_t* tile_order, uint32_t* n_seg,
                      float* t_final, unsigned long long* work, const Fork* fk, cudaStream_t s) {
     if (bp.K == 1)
-        composite_launch<false, 1, NRM, false>(bp, rec, pair_val, pair_mask, tile_range, vis_start, tile_order, n_seg,
+        composite_launch<false, 1, NRM, false>(bp, rec, pair_val, pair_rect, tile_range, vis_start, tile_order, n_seg,
                                                t_final, nullptr, nullptr, nullptr, nullptr, nullptr, work, nullptr,
                                                nullptr, nullptr, fk, s);
     else
-        composite_launch<false, 0, NRM, false>(bp, rec, pair_val, pair_mask, tile_range, vis_start, tile_order, n_seg,
+        composite_launch<false, 0, NRM, false>(bp, rec, pair_val, pair_rect, tile_range, vis_start, tile_order, n_seg,
                                                t_final, nullptr, nullptr, nullptr, nullptr, nullptr, work, nullptr,
                                                nullptr, nullptr, fk, s);
 }
 
 template <bool NRM>
-void composite_bwd_k(const BatchParams& bp, const VoxRec* rec, const uint32_t* pair_val, const uint8_t* pair_mask,
+void composite_bwd_k(const BatchParams& bp, const VoxRec* rec, const uint32_t* pair_val, const uint16_t* pair_rect,
                      const uint2* tile_range, const uint32_t* vis_start, const uint32_t* tile_order,
                      const float* t_final, const float* g_rgb, const float* g_depth, const float* g_alpha,
                      const float* g_normal, float* grad_rec, const Fork* fk, cudaStream_t s) {
@@ -1521,11 +1584,11 @@ void composite_bwd_k(const BatchParams& bp, const VoxRec* rec, const uint32_t* p
     // are only read in the backward
     float* tf = const_cast<float*>(t_final);
     if (bp.K == 1)
-        composite_launch<true, 1, NRM, false>(bp, rec, pair_val, pair_mask, tile_range, vis_start, tile_order, nullptr,
+        composite_launch<true, 1, NRM, false>(bp, rec, pair_val, pair_rect, tile_range, vis_start, tile_order, nullptr,
                                               tf, g_rgb, g_depth, g_alpha, g_normal, grad_rec, nullptr, nullptr,
                                               nullptr, nullptr, fk, s);
     else
-        composite_launch<true, 0, NRM, false>(bp, rec, pair_val, pair_mask, tile_range, vis_start, tile_order, nullptr,
+        composite_launch<true, 0, NRM, false>(bp, rec, pair_val, pair_rect, tile_range, vis_start, tile_order, nullptr,
                                               tf, g_rgb, g_depth, g_alpha, g_normal, grad_rec, nullptr, nullptr,
                                               nullptr, nullptr, fk, s);
 }
@@ -1533,45 +1596,45 @@ void composite_bwd_k(const BatchParams& bp, const VoxRec* rec, const uint32_t* p
 }  // namespace
 
 cudaError_t launch_composite_fwd(const BatchParams& bp, const VoxRec* rec, const uint32_t* pair_val,
-                                 const uint8_t* pair_mask, const uint2* tile_range, const uint32_t* vis_start,
+                                 const uint16_t* pair_rect, const uint2* tile_range, const uint32_t* vis_start,
                                  const uint32_t* tile_order, uint32_t* n_seg, float* t_final,
                                  unsigned long long* work, const Fork* fk, cudaStream_t s) {
     if (bp.n_tiles <= 0) return cudaSuccess;
     if (bp.normals)
-        composite_fwd_k<true>(bp, rec, pair_val, pair_mask, tile_range, vis_start, tile_order, n_seg, t_final, work,
+        composite_fwd_k<true>(bp, rec, pair_val, pair_rect, tile_range, vis_start, tile_order, n_seg, t_final, work,
                               fk, s);
     else
-        composite_fwd_k<false>(bp, rec, pair_val, pair_mask, tile_range, vis_start, tile_order, n_seg, t_final, work,
+        composite_fwd_k<false>(bp, rec, pair_val, pair_rect, tile_range, vis_start, tile_order, n_seg, t_final, work,
                                fk, s);
     return cudaGetLastError();
 }
 
 cudaError_t launch_composite_bwd(const BatchParams& bp, const VoxRec* rec, const uint32_t* pair_val,
-                                 const uint8_t* pair_mask, const uint2* tile_range, const uint32_t* vis_start,
+                                 const uint16_t* pair_rect, const uint2* tile_range, const uint32_t* vis_start,
                                  const uint32_t* tile_order, const float* t_final, const float* g_rgb,
                                  const float* g_depth, const float* g_alpha, const float* g_normal, float* grad_rec,
                                  const Fork* fk, cudaStream_t s) {
     if (bp.n_tiles <= 0) return cudaSuccess;
     if (g_normal)
-        composite_bwd_k<true>(bp, rec, pair_val, pair_mask, tile_range, vis_start, tile_order, t_final, g_rgb,
+        composite_bwd_k<true>(bp, rec, pair_val, pair_rect, tile_range, vis_start, tile_order, t_final, g_rgb,
                               g_depth, g_alpha, g_normal, grad_rec, fk, s);
     else
-        composite_bwd_k<false>(bp, rec, pair_val, pair_mask, tile_range, vis_start, tile_order, t_final, g_rgb,
+        composite_bwd_k<false>(bp, rec, pair_val, pair_rect, tile_range, vis_start, tile_order, t_final, g_rgb,
                                g_depth, g_alpha, nullptr, grad_rec, fk, s);
     return cudaGetLastError();
 }
 
 cudaError_t launch_composite_export(const BatchParams& bp, const VoxRec* rec, const uint32_t* pair_val,
-                                    const uint8_t* pair_mask, const uint2* tile_range, const uint32_t* vis_start,
+                                    const uint16_t* pair_rect, const uint2* tile_range, const uint32_t* vis_start,
                                     const uint32_t* tile_order, const int64_t* offsets, uint32_t* voxel, float* weight,
                                     const Fork* fk, cudaStream_t s) {
     if (bp.n_tiles <= 0) return cudaSuccess;
     if (bp.K == 1)
-        composite_launch<false, 1, false, true>(bp, rec, pair_val, pair_mask, tile_range, vis_start, tile_order, nullptr,
+        composite_launch<false, 1, false, true>(bp, rec, pair_val, pair_rect, tile_range, vis_start, tile_order, nullptr,
                                                 nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, offsets,
                                                 voxel, weight, fk, s);
     else
-        composite_launch<false, 0, false, true>(bp, rec, pair_val, pair_mask, tile_range, vis_start, tile_order, nullptr,
+        composite_launch<false, 0, false, true>(bp, rec, pair_val, pair_rect, tile_range, vis_start, tile_order, nullptr,
                                                 nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, offsets,
                                                 voxel, weight, fk, s);
     return cudaGetLastError();

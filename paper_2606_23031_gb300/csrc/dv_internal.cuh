@@ -208,10 +208,10 @@ cudaError_t launch_records_emit(const BatchParams& bp, const uint32_t* sorted_g,
                                 uint32_t* tile_cnt, unsigned long long* lb_status, uint32_t* ticket,
                                 uint32_t* call_err, uint32_t* dev_err, cudaStream_t s);
 int64_t records_emit_blocks(int64_t n_vis);
-// per tile-sorted pair: its 8x4-block mask; per tile with pairs: its [first, end) range of the
+// per tile-sorted pair: its voxel's pixel rectangle within the tile; per tile with pairs: its [first, end) range of the
 // tile-sorted pair list; also copies *sort_err into the call's mapped status word
-cudaError_t launch_pair_mask(const BatchParams& bp, const uint32_t* pair_key, const uint32_t* pair_val,
-                             const uint64_t* rect_sorted, int64_t n_pairs, int64_t n_vis, uint8_t* mask,
+cudaError_t launch_pair_rect(const BatchParams& bp, const uint32_t* pair_key, const uint32_t* pair_val,
+                             const uint64_t* rect_sorted, int64_t n_pairs, int64_t n_vis, uint16_t* pair_rect,
                              uint2* tile_range, const uint64_t* sort_err, uint64_t* status_host, cudaStream_t s);
 // the empty range for every tile without pairs, and the tiles ordered by decreasing list length (log2
 // buckets of tile_cnt) within three groups, in this order: the tiles that 5 or more actor clip boxes
@@ -229,20 +229,20 @@ struct Fork {
 
 // outputs go to the views' buffers (ViewParams); n_seg and t_final per pixel are kept for the backward
 cudaError_t launch_composite_fwd(const BatchParams& bp, const VoxRec* rec, const uint32_t* pair_val,
-                                 const uint8_t* pair_mask, const uint2* tile_range, const uint32_t* vis_start,
+                                 const uint16_t* pair_rect, const uint2* tile_range, const uint32_t* vis_start,
                                  const uint32_t* tile_order, uint32_t* n_seg, float* t_final,
                                  unsigned long long* work, const Fork* fk, cudaStream_t s);
 // with g_normal (the call rendered normals): gradient rows of 16 floats (8 densities, 3 colour, 3 normal, 2 pad),
 // else of 12 (8 densities, 3 colour, 1 pad)
 cudaError_t launch_composite_bwd(const BatchParams& bp, const VoxRec* rec, const uint32_t* pair_val,
-                                 const uint8_t* pair_mask, const uint2* tile_range, const uint32_t* vis_start,
+                                 const uint16_t* pair_rect, const uint2* tile_range, const uint32_t* vis_start,
                                  const uint32_t* tile_order, const float* t_final, const float* g_rgb,
                                  const float* g_depth, const float* g_alpha, const float* g_normal, float* grad_rec,
                                  const Fork* fk, cudaStream_t s);
 // replay of the forward that writes, for pixel p, the (voxel, weight T alpha) of each composited
 // segment into slots [offsets[p], offsets[p+1]) (voxel index within the view's concatenated octrees)
 cudaError_t launch_composite_export(const BatchParams& bp, const VoxRec* rec, const uint32_t* pair_val,
-                                    const uint8_t* pair_mask, const uint2* tile_range, const uint32_t* vis_start,
+                                    const uint16_t* pair_rect, const uint2* tile_range, const uint32_t* vis_start,
                                     const uint32_t* tile_order, const int64_t* offsets, uint32_t* voxel, float* weight,
                                     const Fork* fk, cudaStream_t s);
 cudaError_t launch_sh_bwd(const BatchParams& bp, const uint32_t* sorted_g, int64_t n_vis, const VoxRec* rec,

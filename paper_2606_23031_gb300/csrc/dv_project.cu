@@ -17,7 +17,7 @@
 //          of its voxels, one per tile of each rectangle, at the offsets a
 //          single-pass scan (look-back over earlier blocks) gives, counting the
 //          pairs of every tile and the digits of the tile sort on the way.
-// mask     which 8x4-pixel blocks of its tile each sorted pair touches, and the tile ranges.
+// rect     the part of its tile's pixels each sorted pair's rectangle covers, and the tile ranges.
 // order    the tiles by list length (from the per-tile counts) within their actor-coverage group.
 //
 // Depth-order key.  Leaves of one octree are cells of a binary space partition
@@ -512,9 +512,6 @@ __global__ void __launch_bounds__(256) k_records_emit(
     }
 }
 
-// For every sorted pair: which of the tile's eight 8x4-pixel blocks (bit sy*2+sx for
-// the block at x in [8 sx, 8 sx + 8), y in [4 sy, 4 sy + 4)) the voxel's pixel
-// rectangle touches; a warp rendering a block skips the pairs without its bit.
 __device__ __forceinline__ int view_of_tile(const BatchParams& bp, int t) {
     int lo = 0, hi = bp.n_view - 1;
     while (lo < hi) {
@@ -527,13 +524,14 @@ __device__ __forceinline__ int view_of_tile(const BatchParams& bp, int t) {
     return lo;
 }
 
-// one thread per tile-sorted pair: the 8x4-pixel blocks of its tile the voxel's pixel rectangle
-// touches (bit sy * 2 + sx), and the [first, end) range of every tile that has pairs, from the key
-// boundaries.  Thread 0 also copies the call's sort flag into its mapped host status word (the sorts
-// have all completed when this kernel runs).
+// one thread per tile-sorted pair: the voxel's pixel rectangle clipped to the tile, x0 | x1 << 4 |
+// y0 << 8 | y1 << 12 in tile pixels (the compositing kernels turn it into the pixels of each warp's 8x4
+// block), and the [first, end) range of every tile that has pairs, from the key boundaries.  Thread 0
+// also copies the call's sort flag into its mapped host status word (the sorts have all completed when
+// this kernel runs).
 __global__ void k_pair_mask(const __grid_constant__ BatchParams bp, const uint32_t* __restrict__ pkey,
                             const uint32_t* __restrict__ pval, const uint64_t* __restrict__ rect_sorted,
-                            int64_t n_pairs, int64_t n_vis, uint8_t* __restrict__ mask, uint2* __restrict__ range,
+                            int64_t n_pairs, int64_t n_vis, uint16_t* __restrict__ prect, uint2* __restrict__ range,
                             const uint64_t* __restrict__ sort_err, volatile uint64_t* status_out) {
     pdl_wait();
     pdl_launch_dependents();
@@ -556,13 +554,8 @@ __global__ void k_pair_mask(const __grid_constant__ BatchParams bp, const uint32
     const int x0 = (int)(t % (uint32_t)tiles_x) * DV_TILE, y0 = (int)(t / (uint32_t)tiles_x) * DV_TILE;
     const int u0 = (int)(rc & 0xffff) - x0, u1 = (int)((rc >> 16) & 0xffff) - x0;
     const int v0 = (int)((rc >> 32) & 0xffff) - y0, v1 = (int)(rc >> 48) - y0;
-    uint32_t m = 0;
-#pragma unroll
-    for (int sy = 0; sy < 4; ++sy)
-#pragma unroll
-        for (int sx = 0; sx < 2; ++sx)
-            if (u0 <= 8 * sx + 7 && u1 >= 8 * sx && v0 <= 4 * sy + 3 && v1 >= 4 * sy) m |= 1u << (sy * 2 + sx);
-    mask[p] = (uint8_t)m;
+    auto in_tile = [](int x) { return (uint32_t)min(max(x, 0), DV_TILE - 1); };
+    prect[p] = (uint16_t)(in_tile(u0) | (in_tile(u1) << 4) | (in_tile(v0) << 8) | (in_tile(v1) << 12));
 }
 
 // Heaviest tiles first: counting sort of tiles by floor(log2(list length + 1)),
@@ -590,7 +583,7 @@ __device__ __forceinline__ int tile_bucket(const BatchParams& bp, uint32_t n_pai
 }
 
 // one thread per tile: its bucket (kept in bucket[t]) into the global bucket counts hist[96]; a tile
-// without pairs gets the empty range (the pair-mask kernel wrote the others)
+// without pairs gets the empty range (the pair-rectangle kernel wrote the others)
 __global__ void __launch_bounds__(256) k_tile_count(const __grid_constant__ BatchParams bp,
                                                     const uint32_t* __restrict__ tile_cnt, int n_tiles,
                                                     uint8_t* __restrict__ bucket, uint2* __restrict__ range,
@@ -698,12 +691,12 @@ cudaError_t launch_records_emit(const BatchParams& bp, const uint32_t* sorted_g,
 
 int64_t records_emit_blocks(int64_t n_vis) { return (n_vis + 255) / 256; }
 
-cudaError_t launch_pair_mask(const BatchParams& bp, const uint32_t* pair_key, const uint32_t* pair_val,
-                             const uint64_t* rect_sorted, int64_t n_pairs, int64_t n_vis, uint8_t* mask,
+cudaError_t launch_pair_rect(const BatchParams& bp, const uint32_t* pair_key, const uint32_t* pair_val,
+                             const uint64_t* rect_sorted, int64_t n_pairs, int64_t n_vis, uint16_t* pair_rect,
                              uint2* tile_range, const uint64_t* sort_err, uint64_t* status_host, cudaStream_t s) {
     if (n_pairs <= 0) return launch_publish(sort_err, status_host, 1, nullptr, -1, s);
     launch_pdl(k_pair_mask, dim3(nblk(n_pairs, 256)), dim3(256), s, bp, pair_key, pair_val, rect_sorted, n_pairs,
-               n_vis, mask, tile_range, sort_err, (volatile uint64_t*)status_host);
+               n_vis, pair_rect, tile_range, sort_err, (volatile uint64_t*)status_host);
     count_launches(1);
     return cudaGetLastError();
 }
