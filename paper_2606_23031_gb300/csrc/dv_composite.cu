@@ -12,16 +12,19 @@
 //  * Every sub-list (each actor's, the background's) streams through a two-slot
 //    shared-memory ring (cp.async, one batch ahead); each warp visits, in list
 //    order and in lockstep, the records that touch its 8x4 pixel block.
-//  * Phase 1: for every actor of the tile, every lane composites the segments
-//    inside its own interval of that actor into a partial (C_A, D_A, T_A)
-//    starting from T = 1.
+//  * Phase 1: for every actor of the tile, nearest first, every lane composites
+//    the segments inside its own interval of that actor into a partial
+//    (C_A, D_A, T_A) starting from T = 1, unless the partials of its earlier
+//    intervals already hide it.
 //  * Phase 2: the background sub-list.  A background hit that reaches past the
 //    next actor's entry composites its part in front of the box, then applies
 //    that actor's partial with the running transmittance (C += T C_A,
 //    D += T D_A, T *= T_A), then continues behind the box.  If T T_A < eps_stop
-//    the ray must stop inside the actor: the lane records its state and stops.
-//  * Phase 3: lanes that stop inside an actor replay that actor's sub-list in
-//    lockstep from the recorded state with the exact stop rule.
+//    the ray stops inside the actor: at the partial's last segment (the whole
+//    partial applies) if T times the transmittance before it is not below
+//    eps_stop; else the lane records its state for a replay.
+//  * Phase 3: lanes left to replay walk that actor's sub-list from the recorded
+//    state with the exact stop rule.
 //    Since T only decreases along the ray, applying a whole partial is exact
 //    unless the stop falls inside it, which is exactly when T T_A < eps_stop.
 //  * Per segment: trilinear interpolation of the raw corner densities at K
@@ -36,8 +39,8 @@
 //    the prefix state at its entry; phase 3 then replays every reached actor
 //    interval with gradients from that state.  Gradients of records visited in
 //    lockstep are reduced across the warp before the atomics.
-//  * Tiles with more actors than lockstep slots (4, or 16 where 5 or more boxes
-//    cover the tile) handle the extra actors with a per-lane walk of the actor's
+//  * A ray with more actor intervals than slots (4, or 8 where 5 or more boxes
+//    cover the tile) handles those beyond with a per-lane walk of the actor's
 //    sub-list (correct, but divergent).
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -62,9 +65,11 @@ struct GradLayout {
 constexpr int NTA_SMALL = 4;
 constexpr int NTA_LARGE = 8;
 constexpr int LANE_GAIN = 2;  // see walk_actor
+constexpr uint32_t SEARCH_MIN = 512;  // tile lists above this length find their sub-lists by binary search
 
 struct PixBase {
     float C0, C1, C2, D, T;
+    float Tp;  // transmittance before the last composited segment
     float R;  // residual form of the backward: sum over the composited segments of w (dL/dC . c + dL/dD mid)
     uint32_t n;
     uint32_t tests, boxes;  // work counters: voxel slab tests, actor box tests
@@ -101,7 +106,7 @@ struct ExportSink {
 
 struct ActInt {
     int o;  // octree index (-1: none)
-    int q;  // slot in the tile's actor list
+    int q;  // slot in the lane's interval list (NTA: beyond it)
     float a, b;
 };
 
@@ -266,6 +271,7 @@ __device__ __forceinline__ float composite_step(Pix<NRM>& ps, float tau, float4 
         ps.N1 = fmaf(w, nv.y, ps.N1);
         ps.N2 = fmaf(w, nv.z, ps.N2);
     }
+    ps.Tp = ps.T;
     ps.T = ps.T * e;
     ps.n += 1;
     return w;
@@ -426,7 +432,7 @@ __device__ __forceinline__ ActInt next_interval(const OctParams* __restrict__ vo
                                                 const int16_t* tact, int n_ta, const float* dc, float tau_cur) {
     ActInt r;
     r.o = -1;
-    r.q = -1;
+    r.q = 1 << 16;  // not in the lane's list
     r.a = INFINITY;
     r.b = 0.0f;
     for (int q = 0; q < n_ta; ++q) {
@@ -442,7 +448,6 @@ __device__ __forceinline__ ActInt next_interval(const OctParams* __restrict__ vo
         if (!(b > a) || !(b > tau_cur)) continue;
         if (a < r.a) {
             r.o = tact[q];
-            r.q = q;
             r.a = a;
             r.b = b;
         }
@@ -575,13 +580,15 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_one() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
-// per-lane actor bookkeeping in shared memory, slot q < NTA:
-//   s_iv[q][0/1][lane]  = the lane's owned interval [a, b) of that actor (a > b: none)
-//   s_st[q][0..4][lane] = phase 1: partial (C0, C1, C2, D, T); phase 2 overwrites it with the
-//                         state at the interval's entry (C0, C1, C2, D, T) when it is replayed
-//   s_st[q][5][lane]    = phase 1: partial segment count; phase 2: 0 not reached,
-//                         1 partial applied, 2 stop inside (replay)
-//   s_st[q][6..8][lane] = with normals: the partial normal state N_A, then N at the entry
+// per-lane actor bookkeeping in shared memory: slot k < NTA holds the lane's k-th actor interval along
+// its ray (a ray meets few of the boxes that cover its tile, so the slots bound the intervals of one ray,
+// not the boxes of the tile)
+//   s_iv[k][0/1][lane] = the interval [a, b), s_id[k][lane] its actor (position in the tile's list)
+//   s_st[k][..][lane]  = phase 1: the actor's partial; phase 2 overwrites it with the state at the
+//                        interval's entry when it is replayed.  Rows:
+//     ST_T, ST_N = transmittance and segment count (phase 2: 0 not reached, 1 partial applied, 2 replay);
+//     ST_R = residual sum (backward), else ST_C.. = C0, C1, C2, D, with normals N0, N1, N2 from ST_V;
+//     ST_P = transmittance before the partial's last segment (forward)
 
 #ifndef DV_FWD_MIN_BLOCKS
 #define DV_FWD_MIN_BLOCKS 5  // resident CTAs per SM the forward is compiled for
@@ -598,7 +605,7 @@ __device__ __forceinline__ void cp_async_wait_one() { asm volatile("cp.async.wai
 // NTA: lockstep actor slots (0: the tile is covered by no actor clip box).  Tiles that no box covers
 // (most of a frame) run the variant without the actor machinery: no interval walk, partials or
 // replays, no per-pixel actor state in shared memory, and about half the registers, so about twice
-// the resident warps per SM.  Tiles that many boxes cover get 16 slots, the others 4.
+// the resident warps per SM.  Tiles that 5 or more boxes cover get 8 slots, the others 4.
 template <bool BWD, int KS, bool NRM, bool WEX, int NTA>
 __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_BLOCKS : DV_FWD_MIN_BLOCKS)
                                                   : DV_PLAIN_MIN_BLOCKS) k_composite(const __grid_constant__ BatchParams bp,
@@ -621,6 +628,9 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
     pdl_launch_dependents();
     constexpr bool REPLAY = BWD || WEX;  // phase 3 replays every actor interval the ray reached
     constexpr bool ACT = NTA > 0;
+    // the backward carries the residual form: the actor partials, the states recorded at actor
+    // entries and the replays hold (R, T) instead of the prefix colour, depth (and normal)
+    constexpr bool RFORM = BWD;
     // with actors, lanes read different records at once: rows of 80 bytes spread them over the banks
     constexpr int RS = ACT ? 5 : 4;
     __shared__ float4 s_rec[2][CT_THREADS][RS];
@@ -629,13 +639,14 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
     __shared__ uint16_t s_m[2][CT_THREADS];         // pixel rectangles of the staged pairs within the tile
     __shared__ uint32_t s_sub[DV_MAX_OCTREES + 1];  // sub-list of octree o: [s_sub[o], s_sub[o+1])
     __shared__ uint32_t s_vs[DV_MAX_OCTREES + 1];   // first record of octree o in this view
-    // the backward carries the residual form: the actor partials, the states recorded at actor
-    // entries and the replays hold (R, T) instead of the prefix colour, depth (and normal)
-    constexpr bool RFORM = BWD;
     __shared__ bool s_flag[ACT ? DV_MAX_OCTREES : 1];  // actor o's box covers this tile
-    __shared__ int16_t s_act[ACT ? DV_MAX_OCTREES : 1];
+    __shared__ int16_t s_act[ACT ? DV_MAX_OCTREES : 1];   // the tile's actors in octree order
+    __shared__ int16_t s_near[ACT ? DV_MAX_OCTREES : 1];  // positions in s_act, nearest box centre first
+    constexpr int ST_T = 0, ST_N = 1, ST_R = 2, ST_C = 2, ST_P = 6, ST_V = 7;
+    constexpr int ST_ROWS = RFORM ? 3 : NRM ? 10 : 7;
     __shared__ float s_iv[ACT ? NTA : 1][2][ACT ? CT_THREADS : 1];
-    __shared__ float s_st[ACT ? NTA : 1][NRM ? 9 : 6][ACT ? CT_THREADS : 1];
+    __shared__ uint8_t s_id[ACT ? NTA : 1][ACT ? CT_THREADS : 1];
+    __shared__ float s_st[ACT ? NTA : 1][ST_ROWS][ACT ? CT_THREADS : 1];
     __shared__ int s_nact;
 
     const int tid = threadIdx.x;
@@ -692,6 +703,7 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
     ps.C0 = ps.C1 = ps.C2 = ps.D = 0.0f;
     if constexpr (NRM) ps.N0 = ps.N1 = ps.N2 = 0.0f;
     ps.T = 1.0f;
+    ps.Tp = 1.0f;
     ps.R = 0.0f;
     ps.n = 0;
     ps.tests = 0;
@@ -752,9 +764,26 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
     __syncthreads();
     // the tile's list is grouped by octree (records are in depth-key order, octree above
     // the BSP path), so octree o's sub-list starts at the first entry whose record is at
-    // or after s_vs[o]; entry q finds its octree by a search of s_vs and marks the starts
-    // of the octrees between its predecessor's and its own
-    {
+    // or after s_vs[o].  In a short list every entry finds its octree by a search of s_vs and
+    // marks the starts of the octrees between its predecessor's and its own (two dependent
+    // loads per entry); in a long one every start is a binary search of the list (a few
+    // hundred entries take as long either way).
+    if (rg.y - rg.x > SEARCH_MIN) {
+        for (int o = tid; o <= n_oct; o += CT_THREADS) {
+            const uint32_t first = s_vs[o];
+            uint32_t lo = rg.x, hi = rg.y;
+            while (lo < hi) {
+                const uint32_t mid = lo + ((hi - lo) >> 1);
+                if (o < n_oct && rec_index(bp, pval, mid) < first)
+                    lo = mid + 1;
+                else if (o < n_oct)
+                    hi = mid;
+                else
+                    lo = hi;
+            }
+            s_sub[o] = lo;
+        }
+    } else {
         auto oct_of = [&](uint32_t r) {
             int lo = 0, hi = n_oct - 1;  // largest o with s_vs[o] <= r
             while (lo < hi) {
@@ -792,27 +821,97 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
     __syncthreads();
 
     const int n_ta = ACT ? s_nact : 0;  // 0 at compile time without actors: the actor code folds away
-    const int n_lock = n_ta < NTA ? n_ta : NTA;
 
-    // ---- owned actor intervals of this ray (lockstep slots) ----
-    for (int q = 0; q < n_lock; ++q) {
-        s_iv[q][0][tid] = INFINITY;
-        s_iv[q][1][tid] = -INFINITY;
-        s_st[q][5][tid] = 0.0f;
-    }
-    if (valid && n_ta > 0) {
-        float tau = t_near;
-        for (int guard = 0; guard < n_ta; ++guard) {
-            const ActInt it = next_interval(vo, t_near, t_far, s_act, n_ta, dc, tau);
-            ps.boxes += n_ta;
-            if (it.o < 0) break;
-            if (it.q < NTA) {
-                s_iv[it.q][0][tid] = it.a;
-                s_iv[it.q][1][tid] = it.b;
+    // ---- owned actor intervals of this ray, in order along it, and the actors by distance ----
+    int n_iv = 0;       // intervals in the lane's slots
+    bool more = false;  // there may be others behind the last slot
+    if constexpr (ACT) {
+        if (valid) {
+            // the boxes the ray meets, inserted by entry (equal entries keep octree order)
+            for (int q = 0; q < n_ta && !more; ++q) {
+                const OctParams& P = vo[s_act[q]];
+                float d[3], inv[3], a, b;
+                rotate(P.A, dc, d);
+                inv[0] = 1.0f / d[0];
+                inv[1] = 1.0f / d[1];
+                inv[2] = 1.0f / d[2];
+                if (!slab_box(P.o_loc, inv, P.clip_half, a, b)) continue;
+                a = fmaxf(a, t_near);
+                b = fminf(b, t_far);
+                if (!(b > a) || !(b > t_near)) continue;
+                if (n_iv == NTA) {
+                    more = true;
+                    break;
+                }
+                int k = n_iv++;
+                for (; k > 0 && s_iv[k - 1][0][tid] > a; --k) {
+                    s_iv[k][0][tid] = s_iv[k - 1][0][tid];
+                    s_iv[k][1][tid] = s_iv[k - 1][1][tid];
+                    s_id[k][tid] = s_id[k - 1][tid];
+                }
+                s_iv[k][0][tid] = a;
+                s_iv[k][1][tid] = b;
+                s_id[k][tid] = (uint8_t)q;
             }
-            tau = it.b;
+            ps.boxes += n_ta;
+            float tau = t_near;
+            if (!more) {
+                // the box entered first owns any overlap; a box keeps what lies behind the last one
+                const int n = n_iv;
+                n_iv = 0;
+                for (int k = 0; k < n; ++k) {
+                    const float a = s_iv[k][0][tid], b = s_iv[k][1][tid];
+                    const uint8_t id = s_id[k][tid];
+                    if (!(b > tau)) continue;
+                    s_iv[n_iv][0][tid] = fmaxf(a, tau);
+                    s_iv[n_iv][1][tid] = b;
+                    s_id[n_iv][tid] = id;
+                    ++n_iv;
+                    tau = b;
+                }
+            } else {
+                // more boxes than slots: the first NTA intervals one by one
+                for (n_iv = 0; n_iv < NTA;) {
+                    const ActInt it = next_interval(vo, t_near, t_far, s_act, n_ta, dc, tau);
+                    ps.boxes += n_ta;
+                    if (it.o < 0) break;
+                    int q = 0;
+                    while (s_act[q] != it.o) ++q;
+                    s_iv[n_iv][0][tid] = it.a;
+                    s_iv[n_iv][1][tid] = it.b;
+                    s_id[n_iv][tid] = (uint8_t)q;
+                    ++n_iv;
+                    tau = it.b;
+                }
+                more = n_iv == NTA;
+            }
         }
+        for (int k = 0; k < n_iv; ++k) {
+            s_st[k][ST_T][tid] = 1.0f;
+            s_st[k][ST_N][tid] = 0.0f;
+        }
+        // phase 1 takes the actors nearest box centre first, so that what hides an actor from a ray is
+        // mostly known before the actor's turn
+        for (int q = tid; q < n_ta; q += CT_THREADS) {
+            const float* m = vo[s_act[q]].m;
+            const float dq = fmaf(m[0], m[0], fmaf(m[1], m[1], m[2] * m[2]));
+            int rank = 0;
+            for (int x = 0; x < n_ta; ++x) {
+                const float* mx = vo[s_act[x]].m;
+                const float dx = fmaf(mx[0], mx[0], fmaf(mx[1], mx[1], mx[2] * mx[2]));
+                rank += (dx < dq || (dx == dq && x < q)) ? 1 : 0;
+            }
+            s_near[rank] = (int16_t)q;
+        }
+        __syncthreads();
     }
+    // the lane's slot of the tile's actor q (-1: the ray does not meet it, or beyond the slots)
+    auto slot_of = [&](int q) {
+        int r = -1;
+        for (int k = 0; k < n_iv; ++k)
+            if (s_id[k][tid] == q) r = k;
+        return r;
+    };
 
     // Every sub-list (an actor's, then the background's) streams through the shared
     // two-slot ring, CT_THREADS records per batch (cp.async, one batch ahead).  Each warp
@@ -1016,39 +1115,52 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
         });
     };
 
-    // ---- phase 1: partial composite of every lockstep actor interval ----
-    for (int q = 0; q < n_lock; ++q) {
-        const float a = s_iv[q][0][tid], b = s_iv[q][1][tid];
-        const bool act = valid && b > a;
+    // ---- phase 1: partial composite of the actor intervals ----
+    // Transmittance never rises along a ray, so if the partials of the lane's earlier intervals
+    // already multiply to less than eps_stop the ray stops before this one, and its partial is
+    // not needed (phase 2 multiplies the same factors in the same order, and the background's on
+    // top, so it cannot get past them).
+    for (int i = 0; i < n_ta; ++i) {
+        const int q = s_near[ACT ? i : 0];
+        const int k = slot_of(q);
+        bool act = k >= 0;
+        if (act) {
+            float T = 1.0f;
+            for (int x = 0; x < k; ++x) T *= s_st[x][ST_T][tid];
+            act = !(T < bp.eps_stop);
+        }
         if (__syncthreads_or(act) == 0) continue;
         Pix<NRM> pt;
         pt.C0 = pt.C1 = pt.C2 = pt.D = 0.0f;
         if constexpr (NRM) pt.N0 = pt.N1 = pt.N2 = 0.0f;
         pt.T = 1.0f;
+        pt.Tp = 1.0f;
         pt.R = 0.0f;
         pt.n = 0;
         pt.tests = 0;
         pt.boxes = 0;
         pt.done = !act;
+        const float a = act ? s_iv[k][0][tid] : 0.0f, b = act ? s_iv[k][1][tid] : 0.0f;
         // a lane whose own transmittance already falls below eps_stop will stop inside this
         // actor whatever T it enters with (T <= 1), so its partial may stop there too
-        walk_actor(pt, s_act[q], a, b, std::false_type(), std::false_type());
+        walk_actor(pt, s_act[ACT ? q : 0], a, b, std::false_type(), std::false_type());
         ps.tests += pt.tests;
-        if (act && RFORM) {
-            s_st[q][0][tid] = pt.R;
-            s_st[q][4][tid] = pt.T;
-            s_st[q][5][tid] = __int_as_float((int)pt.n);
-        } else if (act) {
-            s_st[q][0][tid] = pt.C0;
-            s_st[q][1][tid] = pt.C1;
-            s_st[q][2][tid] = pt.C2;
-            s_st[q][3][tid] = pt.D;
-            s_st[q][4][tid] = pt.T;
-            s_st[q][5][tid] = __int_as_float((int)pt.n);
-            if constexpr (NRM) {
-                s_st[q][NRM ? 6 : 0][tid] = pt.N0;
-                s_st[q][NRM ? 7 : 0][tid] = pt.N1;
-                s_st[q][NRM ? 8 : 0][tid] = pt.N2;
+        if (act) {
+            s_st[k][ST_T][tid] = pt.T;
+            s_st[k][ST_N][tid] = __int_as_float((int)pt.n);
+            if constexpr (RFORM) {
+                s_st[k][ST_R][tid] = pt.R;
+            } else {
+                s_st[k][ST_C][tid] = pt.C0;
+                s_st[k][ST_C + 1][tid] = pt.C1;
+                s_st[k][ST_C + 2][tid] = pt.C2;
+                s_st[k][ST_C + 3][tid] = pt.D;
+                s_st[k][ST_P][tid] = pt.Tp;
+                if constexpr (NRM) {
+                    s_st[k][ST_V][tid] = pt.N0;
+                    s_st[k][ST_V + 1][tid] = pt.N1;
+                    s_st[k][ST_V + 2][tid] = pt.N2;
+                }
             }
         }
     }
@@ -1057,21 +1169,37 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
     float tau_cur = t_near;
     ActInt nxt;
     nxt.o = -1;
-    if (valid && n_ta > 0) {
-        nxt = next_interval(vo, t_near, t_far, s_act, n_ta, dc, tau_cur);
-        ps.boxes += n_ta;
-    }
+    nxt.q = -1;
+    nxt.a = nxt.b = 0.0f;
+    // the interval behind the current one: the lane's next slot, then (beyond the slots) a search
+    auto advance = [&]() {
+        if constexpr (ACT) {
+            const int k = nxt.q + 1;
+            if (k < n_iv) {
+                nxt.o = s_act[s_id[k][tid]];
+                nxt.q = k;
+                nxt.a = s_iv[k][0][tid];
+                nxt.b = s_iv[k][1][tid];
+            } else if (more) {
+                nxt = next_interval(vo, t_near, t_far, s_act, n_ta, dc, tau_cur);
+                ps.boxes += n_ta;
+            } else {
+                nxt.o = -1;
+            }
+        }
+    };
+    if (valid) advance();
     // enters actor interval `it`: apply its partial, or stop inside it, or walk it per lane
     auto enter_actor = [&](const ActInt& it) {
         if (RFORM && it.q < NTA) {
             // backward: record the entry state (R, T) for the replay, then apply the partial
-            const int q = it.q;
-            const float pR = s_st[q][0][tid], pT = s_st[q][4][tid];
-            const uint32_t pn = (uint32_t)__float_as_int(s_st[q][5][tid]);
+            const int k = it.q;
+            const float pR = s_st[k][ST_R][tid], pT = s_st[k][ST_T][tid];
+            const uint32_t pn = (uint32_t)__float_as_int(s_st[k][ST_N][tid]);
             const bool stop_inside = ps.T * pT < bp.eps_stop;
-            s_st[q][0][tid] = ps.R;
-            s_st[q][4][tid] = ps.T;
-            s_st[q][5][tid] = stop_inside ? 2.0f : 1.0f;
+            s_st[k][ST_R][tid] = ps.R;
+            s_st[k][ST_T][tid] = ps.T;
+            s_st[k][ST_N][tid] = stop_inside ? 2.0f : 1.0f;
             if (stop_inside) {
                 ps.done = true;
             } else {
@@ -1079,34 +1207,37 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
                 ps.T = ps.T * pT;
                 ps.n += pn;
             }
-        } else if (it.q < NTA) {
-            const int q = it.q;
-            const float pC0 = s_st[q][0][tid], pC1 = s_st[q][1][tid], pC2 = s_st[q][2][tid];
-            const float pD = s_st[q][3][tid], pT = s_st[q][4][tid];
-            const uint32_t pn = (uint32_t)__float_as_int(s_st[q][5][tid]);
+        } else if (!RFORM && it.q < NTA) {
+            const int k = it.q;
+            const float pC0 = s_st[k][ST_C][tid], pC1 = s_st[k][ST_C + 1][tid], pC2 = s_st[k][ST_C + 2][tid];
+            const float pD = s_st[k][ST_C + 3][tid], pT = s_st[k][ST_T][tid], pP = s_st[k][ST_P][tid];
+            const uint32_t pn = (uint32_t)__float_as_int(s_st[k][ST_N][tid]);
             float pN0 = 0.0f, pN1 = 0.0f, pN2 = 0.0f;
-            if (NRM) {
-                pN0 = s_st[q][NRM ? 6 : 0][tid];
-                pN1 = s_st[q][NRM ? 7 : 0][tid];
-                pN2 = s_st[q][NRM ? 8 : 0][tid];
+            if constexpr (NRM) {
+                pN0 = s_st[k][ST_V][tid];
+                pN1 = s_st[k][ST_V + 1][tid];
+                pN2 = s_st[k][ST_V + 2][tid];
             }
+            // The ray stops inside when T T_A falls below eps_stop.  If it had not before the
+            // partial's last segment (by more than rounding), that segment is where it stops and the
+            // whole partial applies; else the interval is replayed from the entry state.
             const bool stop_inside = ps.T * pT < bp.eps_stop;
-            if (REPLAY || stop_inside) {
-                s_st[q][0][tid] = ps.C0;
-                s_st[q][1][tid] = ps.C1;
-                s_st[q][2][tid] = ps.C2;
-                s_st[q][3][tid] = ps.D;
-                s_st[q][4][tid] = ps.T;
+            const bool at_end = ps.T * pP >= bp.eps_stop * 1.00001f && ps.T * pT < bp.eps_stop * 0.99999f;
+            const bool replay = stop_inside && !at_end;
+            if (REPLAY || replay) {
+                s_st[k][ST_C][tid] = ps.C0;
+                s_st[k][ST_C + 1][tid] = ps.C1;
+                s_st[k][ST_C + 2][tid] = ps.C2;
+                s_st[k][ST_C + 3][tid] = ps.D;
+                s_st[k][ST_T][tid] = ps.T;
                 if constexpr (NRM) {
-                    s_st[q][NRM ? 6 : 0][tid] = ps.N0;
-                    s_st[q][NRM ? 7 : 0][tid] = ps.N1;
-                    s_st[q][NRM ? 8 : 0][tid] = ps.N2;
+                    s_st[k][ST_V][tid] = ps.N0;
+                    s_st[k][ST_V + 1][tid] = ps.N1;
+                    s_st[k][ST_V + 2][tid] = ps.N2;
                 }
             }
-            s_st[q][5][tid] = stop_inside ? 2.0f : 1.0f;
-            if (stop_inside) {
-                ps.done = true;
-            } else {
+            s_st[k][ST_N][tid] = replay ? 2.0f : 1.0f;
+            if (!replay) {
                 ps.C0 = fmaf(ps.T, pC0, ps.C0);
                 ps.C1 = fmaf(ps.T, pC1, ps.C1);
                 ps.C2 = fmaf(ps.T, pC2, ps.C2);
@@ -1119,6 +1250,7 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
                 ps.T = ps.T * pT;
                 ps.n += pn;
             }
+            if (stop_inside) ps.done = true;
         } else {
             // the out-of-line walk takes copies: an object whose address reaches a call stays in
             // local memory everywhere, so the hot-path state (ps, bw, dc, nxt, ex) never does
@@ -1209,8 +1341,7 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
                         enter_actor(nxt);
                         tau_cur = nxt.b;
                         cur = fmaxf(cur, nxt.b);
-                        nxt = next_interval(vo, t_near, t_far, s_act, n_ta, dc, tau_cur);
-                        ps.boxes += n_ta;
+                        advance();
                     }
                     if (!ps.done && t_out > cur) {
                         add_segment<BWD, true, KS, NRM, WEX, RFORM>(ps, bw, bp, da, dd, col, nv, rel, db_, cur, t_out, acc,
@@ -1280,40 +1411,42 @@ __global__ void __launch_bounds__(CT_THREADS, NTA ? ((BWD || WEX) ? DV_BWD_MIN_B
     while (nxt.o >= 0 && !ps.done) {
         enter_actor(nxt);
         tau_cur = nxt.b;
-        nxt = next_interval(vo, t_near, t_far, s_act, n_ta, dc, tau_cur);
-        ps.boxes += n_ta;
+        advance();
     }
 
     // ---- phase 3: actor intervals replayed from their entry state ----
-    //   forward: only those where the ray stops; backward: every one reached (gradients)
-    for (int q = 0; q < n_lock; ++q) {
-        const int status = valid ? (int)s_st[q][5][tid] : 0;
+    //   forward: only those where the ray stops before the partial's end; backward: every one
+    //   reached (gradients)
+    for (int q = 0; q < n_ta; ++q) {
+        const int k = slot_of(q);
+        const int status = k >= 0 ? (int)s_st[k][ST_N][tid] : 0;
         const bool act = REPLAY ? status >= 1 : status == 2;
         if (__syncthreads_or(act) == 0) continue;
         Pix<NRM> pt;
-        pt.T = act ? s_st[q][4][tid] : 1.0f;
-        if (RFORM) {
-            pt.R = act ? s_st[q][0][tid] : 0.0f;
-            pt.C0 = pt.C1 = pt.C2 = pt.D = 0.0f;
-            if constexpr (NRM) pt.N0 = pt.N1 = pt.N2 = 0.0f;
-        } else {
-            pt.R = 0.0f;
-            pt.C0 = act ? s_st[q][0][tid] : 0.0f;
-            pt.C1 = act ? s_st[q][1][tid] : 0.0f;
-            pt.C2 = act ? s_st[q][2][tid] : 0.0f;
-            pt.D = act ? s_st[q][3][tid] : 0.0f;
+        pt.T = act ? s_st[k][ST_T][tid] : 1.0f;
+        pt.Tp = 1.0f;
+        pt.R = 0.0f;
+        pt.C0 = pt.C1 = pt.C2 = pt.D = 0.0f;
+        if constexpr (NRM) pt.N0 = pt.N1 = pt.N2 = 0.0f;
+        if constexpr (RFORM) {
+            if (act) pt.R = s_st[k][ST_R][tid];
+        } else if (act) {
+            pt.C0 = s_st[k][ST_C][tid];
+            pt.C1 = s_st[k][ST_C + 1][tid];
+            pt.C2 = s_st[k][ST_C + 2][tid];
+            pt.D = s_st[k][ST_C + 3][tid];
             if constexpr (NRM) {
-                pt.N0 = act ? s_st[q][6][tid] : 0.0f;
-                pt.N1 = act ? s_st[q][7][tid] : 0.0f;
-                pt.N2 = act ? s_st[q][8][tid] : 0.0f;
+                pt.N0 = s_st[k][ST_V][tid];
+                pt.N1 = s_st[k][ST_V + 1][tid];
+                pt.N2 = s_st[k][ST_V + 2][tid];
             }
         }
         pt.n = 0;
         pt.tests = 0;
         pt.boxes = 0;
         pt.done = !act;
-        walk_actor(pt, s_act[q], s_iv[q][0][tid], s_iv[q][1][tid], std::integral_constant<bool, BWD>(),
-                   std::integral_constant<bool, WEX>());
+        walk_actor(pt, s_act[ACT ? q : 0], act ? s_iv[k][0][tid] : 0.0f, act ? s_iv[k][1][tid] : 0.0f,
+                   std::integral_constant<bool, BWD>(), std::integral_constant<bool, WEX>());
         ps.tests += pt.tests;
         if (!REPLAY && act) {
             ps.C0 = pt.C0;
