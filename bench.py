@@ -213,8 +213,10 @@ STAGE_KERNELS = {
     "records": (("k_records_emit",), ("dv_project.cu", "dv_internal.cuh")),
     "sort_pairs": (("k_os_pass<unsigned int",), ("dv_scan_sort.cu", "dv_internal.cuh")),
     "ranges": (("k_pair_mask", "k_tile_count", "k_tile_scatter"), ("dv_project.cu", "dv_internal.cuh")),
-    "composite_fwd": (("k_composite<0",), ("dv_composite.cu", "dv_internal.cuh", "dv_project.cu")),
-    "composite_bwd": (("k_composite<1",), ("dv_composite.cu", "dv_internal.cuh", "dv_project.cu")),
+    "composite_fwd": (("k_composite<0", "k_composite_act<0"),
+                      ("dv_composite.cu", "dv_composite_act.cu", "dv_composite.cuh", "dv_internal.cuh", "dv_project.cu")),
+    "composite_bwd": (("k_composite<1", "k_composite_act<1"),
+                      ("dv_composite.cu", "dv_composite_act.cu", "dv_composite.cuh", "dv_internal.cuh", "dv_project.cu")),
     "sh_bwd": (("k_sh_bwd",), ("dv_composite.cu", "dv_internal.cuh")),
 }
 

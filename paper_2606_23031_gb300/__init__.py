@@ -23,7 +23,7 @@ _ROOT = os.path.dirname(_HERE)
 _CSRC = os.path.join(_HERE, "csrc")
 _INC = os.path.join(_ROOT, "include")
 LIB_PATH = os.path.join(_HERE, "libdv.so")
-SOURCES = ["dv_api.cu", "dv_scan_sort.cu", "dv_project.cu", "dv_composite.cu", "dv_serve.cu", "dv_sky.cu", "dv_features.cu",
+SOURCES = ["dv_api.cu", "dv_scan_sort.cu", "dv_project.cu", "dv_composite.cu", "dv_composite_act.cu", "dv_serve.cu", "dv_sky.cu", "dv_features.cu",
            "dv_init.cu", "dv_measure.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
@@ -44,7 +44,7 @@ def _nvcc():
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile csrc/*.cu for sm_103a (in parallel) and link libdv.so in-tree."""
     srcs = [os.path.join(_CSRC, s) for s in SOURCES]
-    deps = srcs + [os.path.join(_CSRC, "dv_internal.cuh"), os.path.join(_INC, "dv.h")]
+    deps = srcs + [os.path.join(_CSRC, "dv_internal.cuh"), os.path.join(_CSRC, "dv_composite.cuh"), os.path.join(_INC, "dv.h")]
     if not force and os.path.exists(LIB_PATH):
         t = os.path.getmtime(LIB_PATH)
         if all(os.path.getmtime(d) <= t for d in deps):

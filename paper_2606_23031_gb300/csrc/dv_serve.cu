@@ -299,7 +299,10 @@ dv_status dv_serve_wait(dv_server* S, int64_t ticket, double timeout_ms, double*
     auto it = S->live.find(ticket);
     if (it == S->live.end()) return DV_ERR_INVALID_ARG;
     std::shared_ptr<Request> r = it->second;
-    const bool ok = S->cv_done.wait_for(lk, std::chrono::duration<double, std::milli>(timeout_ms),
+    // no time to wait: answered as things stand (a timed wait of zero still gives up the lock and sleeps
+    // for some tens of microseconds, in which a small request can finish)
+    if (!(timeout_ms > 0.0) && !r->done) return DV_ERR_TIMEOUT;
+    const bool ok = r->done || S->cv_done.wait_for(lk, std::chrono::duration<double, std::milli>(timeout_ms),
                                         [&] { return r->done; });
     if (!ok) return DV_ERR_TIMEOUT;
     if (lat_ms) *lat_ms = latency_ms(*r);
