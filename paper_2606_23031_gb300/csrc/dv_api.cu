@@ -679,7 +679,7 @@ dv_status render_batch(dv_ctx* ctx, const dv_octree* oct, int n_oct, const dv_po
     bp.inv_k = 1.0f / (float)opt.K;
     bp.eps_stop = opt.eps_stop;
     bp.normals = normals ? 1 : 0;
-    bp.activation = opt.activation;
+    bp.act_thr = opt.activation == DV_ACT_IDENTITY ? -INFINITY : 1.1f;
     int Lkey = 0;
     for (int i = 0; i < n_oct; ++i) Lkey = std::max(Lkey, (int)oct[i].max_level);
     bp.Lkey = Lkey;

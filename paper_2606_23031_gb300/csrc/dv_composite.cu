@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(CT_THREADS, DV_PLAIN_MIN_BLOCKS) k_composite(c
     }
     const InvDir ib = inv_dir(db_);
     Pix<NRM> ps;
-    init_pix<NRM>(ps, !valid);
+    init_pix<NRM>(ps, valid ? t_far : -1.0f);
     ExportSink ex;
     if constexpr (WEX) init_sink(ex, A, view, pix, valid);
     Bwd<NRM> bw;
@@ -120,24 +120,24 @@ __global__ void __launch_bounds__(CT_THREADS, DV_PLAIN_MIN_BLOCKS) k_composite(c
     constexpr int NV = GradLayout<NRM>::NV;
     constexpr int GS = GradLayout<NRM>::STRIDE;
 
+    uint32_t seen = 0;  // records visited so far; a ray that stops keeps the count as its tests
     // voxel normal of staged record j (zero without normals)
     auto staged_nv = [&](int slot, uint32_t j) {
         return NRM ? s_nv[NRM ? slot : 0][NRM ? j : 0] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     };
     // the lane's segment of a record: entry and exit, true if it has any length
     auto clip = [&](float4 g, float& t_in, float& t_out) {
-        const bool x = slab_cube(ib, g, t_in, t_out);
+        slab_cube(ib, g, t_in, t_out);
         t_in = fmaxf(t_in, t_near);
-        t_out = fminf(t_out, t_far);
-        return x && t_out > t_in;
+        t_out = fminf(t_out, ps.end);
+        return t_out > t_in;
     };
     // one record of the batch, visited by the whole warp
     auto visit = [&](int slot, uint32_t j) {
         const float4 g = s_rec[slot][j][0];
-        const bool live = !ps.done;
         float t_in, t_out;
-        const bool hit = clip(g, t_in, t_out) && live;
-        ps.tests += live ? 1u : 0u;
+        const bool hit = clip(g, t_in, t_out);
+        seen += 1;
         if constexpr (BWD) {
             if (!__any_sync(0xffffffffu, hit)) return;
         }
@@ -159,13 +159,14 @@ __global__ void __launch_bounds__(CT_THREADS, DV_PLAIN_MIN_BLOCKS) k_composite(c
                 add_segment<BWD, true, KS, NRM, WEX, BWD>(ps, bw, bp, s_rec[slot][j][1], s_rec[slot][j][2],
                                                           s_rec[slot][j][3], staged_nv(slot, j), rel, db_, t_in, t_out,
                                                           acc, s_r[slot][j], &ex);
+            if (!BWD && hit && ps.done()) ps.tests = seen;
         }
         if constexpr (BWD) warp_reduce_add<NV>(acc, A.grad_rec + (size_t)s_r[slot][j] * GS);
     };
     // 32 records of the batch, m: those that touch this warp's 8x4 block; true once the warp is done
     auto chunk = [&](int slot, uint32_t c0, unsigned m) -> bool {
         while (m) {
-            if (__all_sync(0xffffffffu, ps.done)) return true;
+            if (__all_sync(0xffffffffu, ps.done())) return true;
             const uint32_t j0 = c0 + (uint32_t)(__ffs(m) - 1);
             m &= m - 1;
             if (BWD || WEX || m == 0) {
@@ -178,22 +179,25 @@ __global__ void __launch_bounds__(CT_THREADS, DV_PLAIN_MIN_BLOCKS) k_composite(c
             // list order with the stop rule -- the same arithmetic as two visits
             const float4 g0 = s_rec[slot][j0][0], g1 = s_rec[slot][j1][0];
             float a0, b0, a1, b1;
-            const bool live = !ps.done;
-            const bool h0 = clip(g0, a0, b0) && live, h1 = clip(g1, a1, b1) && live;
+            const bool h0 = clip(g0, a0, b0), h1 = clip(g1, a1, b1);
             const float4 da0 = s_rec[slot][j0][1], dd0 = s_rec[slot][j0][2], col0 = s_rec[slot][j0][3];
             const float4 da1 = s_rec[slot][j1][1], dd1 = s_rec[slot][j1][2], col1 = s_rec[slot][j1][3];
             const float r0[3] = {g0.x, g0.y, g0.z}, r1[3] = {g1.x, g1.y, g1.z};
-            const float u0 = h0 ? a0 : 0.0f, v0 = h0 ? b0 : 0.0f, u1 = h1 ? a1 : 0.0f, v1 = h1 ? b1 : 0.0f;
-            const float tau0 = seg_tau<false, KS>(da0, dd0, col0.w, r0, db_, u0, v0, bp.K, bp.inv_k, bp.activation,
+            const float tau0 = seg_tau<false, KS>(da0, dd0, col0.w, r0, db_, a0, b0, bp.K, bp.inv_k, bp.act_thr,
                                                   nullptr, nullptr);
-            const float tau1 = seg_tau<false, KS>(da1, dd1, col1.w, r1, db_, u1, v1, bp.K, bp.inv_k, bp.activation,
+            const float tau1 = seg_tau<false, KS>(da1, dd1, col1.w, r1, db_, a1, b1, bp.K, bp.inv_k, bp.act_thr,
                                                   nullptr, nullptr);
-            ps.tests += live ? 1u : 0u;
-            if (h0) composite_tau<NRM>(ps, tau0, col0, staged_nv(slot, j0), u0, v0, bp.eps_stop);
-            ps.tests += (live && !ps.done) ? 1u : 0u;
-            if (h1 && !ps.done) composite_tau<NRM>(ps, tau1, col1, staged_nv(slot, j1), u1, v1, bp.eps_stop);
+            if (h0) {
+                composite_tau<NRM>(ps, tau0, col0, staged_nv(slot, j0), a0, b0, bp.eps_stop);
+                if (ps.done()) ps.tests = seen + 1;
+            }
+            if (h1 && !ps.done()) {
+                composite_tau<NRM>(ps, tau1, col1, staged_nv(slot, j1), a1, b1, bp.eps_stop);
+                if (ps.done()) ps.tests = seen + 2;
+            }
+            seen += 2;
         }
-        return __all_sync(0xffffffffu, ps.done);
+        return __all_sync(0xffffffffu, ps.done());
     };
 
     // The list streams through a two-slot shared-memory ring, CT_THREADS records per batch (cp.async, one
@@ -241,7 +245,7 @@ __global__ void __launch_bounds__(CT_THREADS, DV_PLAIN_MIN_BLOCKS) k_composite(c
     asm volatile("cp.async.wait_all;\n" ::: "memory");  // no copy outlives the list (early exit)
 
     if constexpr (!BWD && !WEX) {
-        if (A.work) add_work(A.work, ps.tests, ps.boxes, ps.n);
+        if (A.work) add_work(A.work, !valid ? 0u : ps.done() ? ps.tests : seen, ps.boxes, ps.n);
         if (valid) store_pix<NRM>(ps, A, fp, lpix, pix);
     }
 }

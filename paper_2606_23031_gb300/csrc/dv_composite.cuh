@@ -47,7 +47,11 @@ struct PixBase {
     float R;  // residual form of the backward: sum over the composited segments of w (dL/dC . c + dL/dD mid)
     uint32_t n;
     uint32_t tests, boxes;  // work counters: voxel slab tests, actor box tests
-    bool done;
+    // the ray is composited up to here; -1 once it has stopped (or for a lane without a pixel), so that
+    // the clip of a segment alone leaves it out
+    float end;
+    __device__ __forceinline__ bool done() const { return end < 0.0f; }
+    __device__ __forceinline__ void stop() { end = -1.0f; }
 };
 template <bool NRM>
 struct Pix : PixBase {};
@@ -92,15 +96,15 @@ __device__ __forceinline__ float explin_low(float x) {
     return ex2_sfu(fmaf(x, 1.3115409462626941f, -1.3051915171390283f));
 }
 
-__device__ __forceinline__ float act_fn(float x, int act) {
-    if (act == DV_ACT_IDENTITY) return x;
-    return x > 1.1f ? x : explin_low(x);
+// thr: 1.1, or -infinity for the identity activation (BatchParams::act_thr)
+__device__ __forceinline__ float act_fn(float x, float thr) { return x > thr ? x : explin_low(x); }
+
+__device__ __forceinline__ float act_grad(float x, float thr) {
+    return x > thr ? 1.0f : explin_low(x) * 0.90909090909090909f;
 }
 
-__device__ __forceinline__ float act_grad(float x, int act) {
-    if (act == DV_ACT_IDENTITY) return 1.0f;
-    return x > 1.1f ? 1.0f : explin_low(x) * 0.90909090909090909f;
-}
+// exp(-x) on the SFU
+__device__ __forceinline__ float exp_neg(float x) { return ex2_sfu(x * -1.4426950408889634f); }
 
 __device__ __forceinline__ void rotate(const float* A, const float* x, float* y) {
 #pragma unroll
@@ -144,8 +148,9 @@ __device__ __forceinline__ InvDir inv_dir(const float* d) {
 // Ray / voxel slab test.  g = (min corner - ray origin, size): along axis k the ray
 // crosses the min plane at g_k / d_k and the max plane at (g_k + size) / d_k; which of
 // the two it enters by follows from the sign of d_k.  The x and y axes go through packed two-lane
-// multiplies and FMAs (the same roundings as scalar ones, half the instructions).
-__device__ __forceinline__ bool slab_cube(const InvDir& v, float4 g, float& t0, float& t1) {
+// multiplies and FMAs (the same roundings as scalar ones, half the instructions).  The ray misses the
+// voxel where t1 <= t0; a caller that clips both ends only compares once, after the clip.
+__device__ __forceinline__ void slab_cube(const InvDir& v, float4 g, float& t0, float& t1) {
     const float2 ww = make_float2(g.w, g.w);
     const float2 ta = __fmul2_rn(make_float2(g.x, g.y), make_float2(v.inv[0], v.inv[1]));
     const float2 en = __ffma2_rn(ww, make_float2(v.in[0], v.in[1]), ta);
@@ -153,7 +158,6 @@ __device__ __forceinline__ bool slab_cube(const InvDir& v, float4 g, float& t0, 
     const float tz = g.z * v.inv[2];
     t0 = max3f(en.x, en.y, fmaf(g.w, v.in[2], tz));
     t1 = min3f(ex.x, ex.y, fmaf(g.w, v.ip[2], tz));
-    return t0 < t1;
 }
 
 
@@ -164,7 +168,7 @@ __device__ __forceinline__ bool slab_cube(const InvDir& v, float4 g, float& t0, 
 // activation's slope times the step and the sample's voxel coordinates, and dtd is not written.
 template <bool GRAD, int KS>
 __device__ __forceinline__ float seg_tau(float4 da, float4 db, float is, const float* rel, const float* d, float t0,
-                                         float t1, int K_rt, float inv_k_rt, int act, float* dtd, float* sxyz) {
+                                         float t1, int K_rt, float inv_k_rt, float thr, float* dtd, float* sxyz) {
     const int K = KS > 0 ? KS : K_rt;
     const float inv_k = KS == 1 ? 1.0f : inv_k_rt;
     const float h = (t1 - t0) * inv_k;
@@ -174,7 +178,7 @@ __device__ __forceinline__ float seg_tau(float4 da, float4 db, float is, const f
         for (int c = 0; c < 8; ++c) dtd[c] = 0.0f;
     }
     for (int k = 0; k < K; ++k) {
-        const float t = fmaf((float)k + 0.5f, h, t0);
+        const float t = KS == 1 ? 0.5f * (t0 + t1) : fmaf((float)k + 0.5f, h, t0);
         // voxel-local coordinates of the sample o + t d: (t d - (min - o)) / size
         const float x = __saturatef(fmaf(t, d[0], -rel[0]) * is);
         const float y = __saturatef(fmaf(t, d[1], -rel[1]) * is);
@@ -187,14 +191,14 @@ __device__ __forceinline__ float seg_tau(float4 da, float4 db, float is, const f
         const float2 pB = __ffma2_rn(make_float2(db.z, db.w), xx, make_float2(db.x, db.y));
         const float2 qq = __ffma2_rn(pB, make_float2(y, y), pA);
         const float rho = fmaf(qq.y, z, qq.x);
-        tau += act_fn(rho, act);
+        tau += act_fn(rho, thr);
         if (GRAD && KS == 1) {
-            sxyz[0] = act_grad(rho, act) * h;
+            sxyz[0] = act_grad(rho, thr) * h;
             sxyz[1] = x;
             sxyz[2] = y;
             sxyz[3] = z;
         } else if (GRAD) {
-            const float s = act_grad(rho, act) * h;
+            const float s = act_grad(rho, thr) * h;
             const float x0 = 1.0f - x, y0 = 1.0f - y, z0 = 1.0f - z;
             dtd[0] = fmaf(s, x0 * y0 * z0, dtd[0]);
             dtd[1] = fmaf(s, x * y0 * z0, dtd[1]);
@@ -212,7 +216,7 @@ __device__ __forceinline__ float seg_tau(float4 da, float4 db, float is, const f
 // Front-to-back compositing of one segment of optical depth tau; returns its weight T alpha.
 template <bool NRM>
 __device__ __forceinline__ float composite_step(Pix<NRM>& ps, float tau, float4 col, float4 nv, float t0, float t1) {
-    const float e = __expf(-tau);  // transmittance of the segment
+    const float e = exp_neg(tau);  // transmittance of the segment
     const float alpha = 1.0f - e;
     const float w = ps.T * alpha;
     const float mid = 0.5f * (t0 + t1);
@@ -235,7 +239,7 @@ template <bool NRM>
 __device__ __forceinline__ void composite_tau(Pix<NRM>& ps, float tau, float4 col, float4 nv, float t0, float t1,
                                               float eps_stop) {
     composite_step<NRM>(ps, tau, col, nv, t0, t1);
-    if (ps.T < eps_stop) ps.done = true;
+    if (ps.T < eps_stop) ps.stop();
 }
 
 // d L / d dens[c] of one segment, added into acc[0..7], from gt = d L / d tau
@@ -272,10 +276,10 @@ __device__ __forceinline__ void add_segment(Pix<NRM>& ps, const Bwd<NRM>& bw, co
                                             float4 col, float4 nv, const float* rel, const float* d, float t0,
                                             float t1, float* acc, uint32_t r = 0, ExportSink* ex = nullptr) {
     float dtd[8], sxyz[4];
-    const float tau = seg_tau<GRAD, KS>(da, db, col.w, rel, d, t0, t1, bp.K, bp.inv_k, bp.activation, dtd, sxyz);
+    const float tau = seg_tau<GRAD, KS>(da, db, col.w, rel, d, t0, t1, bp.K, bp.inv_k, bp.act_thr, dtd, sxyz);
     if constexpr (RF) {
         // (without GRAD: an actor's partial in the backward, R only)
-        const float e = __expf(-tau);
+        const float e = exp_neg(tau);
         const float w = ps.T * (1.0f - e);
         const float mid = 0.5f * (t0 + t1);
         float s = fmaf(bw.g0, col.x, fmaf(bw.g1, col.y, fmaf(bw.g2, col.z, bw.gD * mid)));
@@ -295,7 +299,7 @@ __device__ __forceinline__ void add_segment(Pix<NRM>& ps, const Bwd<NRM>& bw, co
                 acc[13] = fmaf(bw.gN2, w, acc[13]);
             }
         }
-        if (STOP && ps.T < bp.eps_stop) ps.done = true;
+        if (STOP && ps.T < bp.eps_stop) ps.stop();
         return;
     }
     const float w = composite_step<NRM>(ps, tau, col, nv, t0, t1);
@@ -327,7 +331,7 @@ __device__ __forceinline__ void add_segment(Pix<NRM>& ps, const Bwd<NRM>& bw, co
         acc[9] = fmaf(bw.g1, w, acc[9]);
         acc[10] = fmaf(bw.g2, w, acc[10]);
     }
-    if (STOP && ps.T < bp.eps_stop) ps.done = true;
+    if (STOP && ps.T < bp.eps_stop) ps.stop();
 }
 
 // One backward step in residual form with one sample, for a lane that meets the record at most once
@@ -341,8 +345,8 @@ __device__ __forceinline__ void bwd_single_step(Pix<NRM>& ps, const Bwd<NRM>& bw
                                                 float u1, bool hit, float* acc) {
     const float rel[3] = {g.x, g.y, g.z};
     float sxyz[4];
-    const float tau = seg_tau<true, 1>(da, dd, col.w, rel, d, u0, u1, bp.K, bp.inv_k, bp.activation, nullptr, sxyz);
-    const float e = __expf(-tau);
+    const float tau = seg_tau<true, 1>(da, dd, col.w, rel, d, u0, u1, bp.K, bp.inv_k, bp.act_thr, nullptr, sxyz);
+    const float e = exp_neg(tau);
     const float w = ps.T * (1.0f - e);
     const float mid = 0.5f * (u0 + u1);
     float sg = fmaf(bw.g0, col.x, fmaf(bw.g1, col.y, fmaf(bw.g2, col.z, bw.gD * mid)));
@@ -378,7 +382,7 @@ __device__ __forceinline__ void bwd_single_step(Pix<NRM>& ps, const Bwd<NRM>& bw
         acc[NRM ? 12 : 0] = bw.gN1 * w;
         acc[NRM ? 13 : 0] = bw.gN2 * w;
     }
-    if (ps.T < bp.eps_stop) ps.done = true;
+    if (ps.T < bp.eps_stop) ps.stop();
 }
 
 // Sum of acc[0..NV-1] over the warp, transposed.  Each butterfly level (lane distance 16, 8, 4, 2,
@@ -391,11 +395,20 @@ __device__ __forceinline__ void fold_level(float* v, int lane, int& idx, int& nr
     if constexpr (D >= 1) {
         constexpr int H = (N + 1) / 2;
         const bool up = lane & D;
+        float own[H + 1], got[H + 1];
 #pragma unroll
         for (int i = 0; i < H; ++i) {
             const float lo = v[i];
             const float hi = (H + i < N) ? v[H + i] : 0.0f;
-            v[i] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, D);
+            own[i] = up ? hi : lo;
+            got[i] = __shfl_xor_sync(0xffffffffu, up ? lo : hi, D);
+        }
+        own[H] = got[H] = 0.0f;
+#pragma unroll
+        for (int i = 0; i < H; i += 2) {  // packed two-lane additions
+            const float2 s = __fadd2_rn(make_float2(own[i], own[i + 1]), make_float2(got[i], got[i + 1]));
+            v[i] = s.x;
+            if (i + 1 < H) v[i + 1] = s.y;
         }
         idx += up ? H : 0;
         nreal = up ? max(nreal - H, 0) : min(nreal, H);
@@ -475,7 +488,7 @@ __device__ __forceinline__ void pixel_ray(const ViewParams& fp, int u, int v, fl
 }
 
 template <bool NRM>
-__device__ __forceinline__ void init_pix(Pix<NRM>& p, bool done) {
+__device__ __forceinline__ void init_pix(Pix<NRM>& p, float end) {
     p.C0 = p.C1 = p.C2 = p.D = 0.0f;
     if constexpr (NRM) p.N0 = p.N1 = p.N2 = 0.0f;
     p.T = p.Tp = 1.0f;
@@ -483,7 +496,7 @@ __device__ __forceinline__ void init_pix(Pix<NRM>& p, bool done) {
     p.n = 0;
     p.tests = 0;
     p.boxes = 0;
-    p.done = done;
+    p.end = end;
 }
 
 template <bool BWD, bool NRM>

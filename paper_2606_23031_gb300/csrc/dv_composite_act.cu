@@ -138,7 +138,7 @@ __device__ __noinline__ void walk_actor_lane(Pix<NRM>& ps, const Bwd<NRM>& bw, c
     float d[3];
     rotate(P.A, dc, d);
     const InvDir inv = inv_dir(d);
-    for (uint32_t q = q0; q < q1 && !ps.done; ++q) {
+    for (uint32_t q = q0; q < q1 && !ps.done(); ++q) {
         if (!((block_pixels(__ldg(prect + q), bx, by) >> (threadIdx.x & 31)) & 1u)) continue;
         ps.tests += 1;
         const uint32_t r = rec_index(bp, pval, q);
@@ -146,7 +146,7 @@ __device__ __noinline__ void walk_actor_lane(Pix<NRM>& ps, const Bwd<NRM>& bw, c
         const float4 g = __ldg(R);
         float t0, t1;
         const float rel[3] = {g.x, g.y, g.z};
-        if (!slab_cube(inv, g, t0, t1)) continue;
+        slab_cube(inv, g, t0, t1);
         t0 = fmaxf(t0, it.a);
         t1 = fminf(t1, it.b);
         if (!(t1 > t0)) continue;
@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
     rotate(vo[0].A, dc, db_);
     const InvDir ib = inv_dir(db_);
     Pix<NRM> ps;
-    init_pix<NRM>(ps, !valid);
+    init_pix<NRM>(ps, valid ? t_far : -1.0f);
     ExportSink ex;
     if constexpr (WEX)
         init_sink(ex, A, view, pix, valid);
@@ -510,9 +510,9 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
     };
 
     // Walk of actor o's sub-list: lanes not yet done composite the segments inside their interval
-    // [a, b] of that actor into pt, with the stop rule (and, with G, the per-record gradients), two
+    // [a, pt.end] of that actor into pt, with the stop rule (and, with G, the per-record gradients), two
     // records at a time without gradients.
-    auto walk_actor = [&](Pix<NRM>& pt, int o, float a, float b, auto grad, auto wex) {
+    auto walk_actor = [&](Pix<NRM>& pt, int o, float a, auto grad, auto wex) {
         constexpr bool G = decltype(grad)::value;
         constexpr bool X = decltype(wex)::value;
         const OctParams& P = vo[o];
@@ -520,15 +520,15 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
         rotate(P.A, dc, d);
         const InvDir inv = inv_dir(d);
         auto clip = [&](float4 g, float& t0, float& t1) {
-            const bool x = slab_cube(inv, g, t0, t1);
+            slab_cube(inv, g, t0, t1);
             t0 = fmaxf(t0, a);
-            t1 = fminf(t1, b);
-            return x && t1 > t0;
+            t1 = fminf(t1, pt.end);
+            return t1 > t0;
         };
         stream(s_sub[o], s_sub[o + 1], [&](int bf, int n, uint32_t pm) -> bool {
-            if (__all_sync(0xffffffffu, pt.done)) return true;
+            if (__all_sync(0xffffffffu, pt.done())) return true;
             uint32_t mine = warp_transpose(pm);
-            if (pt.done) mine = 0u;
+            if (pt.done()) mine = 0u;
             bool lanes = true;
             if constexpr (G) lanes = by_lanes(mine, n);
             if (lanes) {
@@ -545,16 +545,15 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
                         const float4 g1 = ring.rec[bf][j1][0];
                         float u0, v0, u1, v1;
                         const bool h0 = clip(g0, u0, v0), h1 = clip(g1, u1, v1) && two;
-                        const float s0 = h0 ? u0 : 0.0f, e0 = h0 ? v0 : 0.0f, s1 = h1 ? u1 : 0.0f, e1 = h1 ? v1 : 0.0f;
                         const float4 col0 = ring.rec[bf][j][3], col1 = ring.rec[bf][j1][3];
                         const float r0[3] = {g0.x, g0.y, g0.z}, r1[3] = {g1.x, g1.y, g1.z};
-                        const float tau0 = seg_tau<false, 1>(ring.rec[bf][j][1], ring.rec[bf][j][2], col0.w, r0, d, s0,
-                                                             e0, bp.K, bp.inv_k, bp.activation, nullptr, nullptr);
-                        const float tau1 = seg_tau<false, 1>(ring.rec[bf][j1][1], ring.rec[bf][j1][2], col1.w, r1, d, s1,
-                                                             e1, bp.K, bp.inv_k, bp.activation, nullptr, nullptr);
+                        const float tau0 = seg_tau<false, 1>(ring.rec[bf][j][1], ring.rec[bf][j][2], col0.w, r0, d, u0,
+                                                             v0, bp.K, bp.inv_k, bp.act_thr, nullptr, nullptr);
+                        const float tau1 = seg_tau<false, 1>(ring.rec[bf][j1][1], ring.rec[bf][j1][2], col1.w, r1, d, u1,
+                                                             v1, bp.K, bp.inv_k, bp.act_thr, nullptr, nullptr);
                         auto apply = [&](float tau, float4 col, float4 nv, float t0, float t1) {
                             if constexpr (RFORM) {
-                                const float ee = __expf(-tau);
+                                const float ee = exp_neg(tau);
                                 const float w = pt.T * (1.0f - ee);
                                 const float mid = 0.5f * (t0 + t1);
                                 float sg = fmaf(bw.g0, col.x, fmaf(bw.g1, col.y, fmaf(bw.g2, col.z, bw.gD * mid)));
@@ -562,15 +561,15 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
                                 pt.R = fmaf(w, sg, pt.R);
                                 pt.T = pt.T * ee;
                                 pt.n += 1;
-                                if (pt.T < bp.eps_stop) pt.done = true;
+                                if (pt.T < bp.eps_stop) pt.stop();
                             } else {
                                 composite_tau<NRM>(pt, tau, col, nv, t0, t1, bp.eps_stop);
                             }
                         };
                         pt.tests += 1;
-                        if (h0) apply(tau0, col0, staged_nv(bf, j), s0, e0);
-                        pt.tests += (two && !pt.done) ? 1u : 0u;
-                        if (h1 && !pt.done) apply(tau1, col1, staged_nv(bf, j1), s1, e1);
+                        if (h0) apply(tau0, col0, staged_nv(bf, j), u0, v0);
+                        pt.tests += (two && !pt.done()) ? 1u : 0u;
+                        if (h1 && !pt.done()) apply(tau1, col1, staged_nv(bf, j1), u1, v1);
                     } else {
                         pt.tests += 1;
                         float t0, t1;
@@ -591,17 +590,15 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
                             if constexpr (G) lane_add<NRM>(A.grad_rec, ring.r[bf][j], acc);
                         }
                     }
-                    if (pt.done) mine = 0u;
+                    if (pt.done()) mine = 0u;
                 }
                 __syncwarp();
             } else if constexpr (G) {
                 for (uint32_t j = 0; j < (uint32_t)n; ++j) {
-                    if (__all_sync(0xffffffffu, pt.done)) return true;
+                    if (__all_sync(0xffffffffu, pt.done())) return true;
                     const float4 g = ring.rec[bf][j][0];
-                    const bool live = !pt.done;
                     float t0, t1;
-                    const bool hit = clip(g, t0, t1) && live;
-                    pt.tests += live ? 1u : 0u;
+                    const bool hit = clip(g, t0, t1);
                     if (!__any_sync(0xffffffffu, hit)) continue;
                     float acc[NV];
                     if constexpr (KS == 1) {
@@ -620,7 +617,7 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
                     warp_reduce_add<NV>(acc, A.grad_rec + (size_t)ring.r[bf][j] * GS);
                 }
             }
-            return __all_sync(0xffffffffu, pt.done);
+            return __all_sync(0xffffffffu, pt.done());
         });
     };
 
@@ -641,11 +638,10 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
         }
         if (!__any_sync(0xffffffffu, act)) continue;
         Pix<NRM> pt;
-        init_pix<NRM>(pt, !act);
+        init_pix<NRM>(pt, act ? iv(k, 1) : -1.0f);
         // a lane whose own transmittance already falls below eps_stop will stop inside this
         // actor whatever T it enters with (T <= 1), so its partial may stop there too
-        walk_actor(pt, s_act[q], act ? iv(k, 0) : 0.0f, act ? iv(k, 1) : 0.0f, std::false_type(),
-                   std::false_type());
+        walk_actor(pt, s_act[q], act ? iv(k, 0) : 0.0f, std::false_type(), std::false_type());
         ps.tests += pt.tests;
         if (act) {
             st(k, ST_N) = __int_as_float((int)pt.n);
@@ -768,13 +764,13 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
                     ps.n += pn;
                 }
             }
-            if (stop_inside) ps.done = true;
+            if (stop_inside) ps.stop();
         };
         auto clip = [&](float4 g, float& t_in, float& t_out) {
-            const bool x = slab_cube(ib, g, t_in, t_out);
+            slab_cube(ib, g, t_in, t_out);
             t_in = fmaxf(t_in, t_near);
-            t_out = fminf(t_out, t_far);
-            return x && t_out > t_in;
+            t_out = fminf(t_out, ps.end);
+            return t_out > t_in;
         };
         // one lane's segments of staged record j, entering the actor intervals inside them; with
         // gradients the values are added to acc; true if it composited any
@@ -788,19 +784,19 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
             const float4 da = ring.rec[bf][j][1], dd = ring.rec[bf][j][2], col = ring.rec[bf][j][3];
             const float4 nv = staged_nv(bf, j);
             float cur = fmaxf(t_in, tau_cur);
-            while (nxt.o >= 0 && nxt.a < t_out && !ps.done) {
+            while (nxt.o >= 0 && nxt.a < t_out && !ps.done()) {
                 if (nxt.a > cur) {
                     add_segment<BWD, true, KS, NRM, WEX, RFORM>(ps, bw, bp, da, dd, col, nv, rel, db_, cur, nxt.a, acc,
                                                                 ring.r[bf][j], &ex);
                     some = true;
-                    if (ps.done) break;
+                    if (ps.done()) break;
                 }
                 enter_actor(nxt);
                 tau_cur = nxt.b;
                 cur = fmaxf(cur, nxt.b);
                 advance();
             }
-            if (!ps.done && t_out > cur) {
+            if (!ps.done() && t_out > cur) {
                 add_segment<BWD, true, KS, NRM, WEX, RFORM>(ps, bw, bp, da, dd, col, nv, rel, db_, cur, t_out, acc,
                                                             ring.r[bf][j], &ex);
                 some = true;
@@ -808,9 +804,9 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
             return some;
         };
         stream(s_sub[0], s_sub[1], [&](int bf, int n, uint32_t pm) -> bool {
-            if (__all_sync(0xffffffffu, ps.done)) return true;
+            if (__all_sync(0xffffffffu, ps.done())) return true;
             uint32_t mine = warp_transpose(pm);
-            if (ps.done) mine = 0u;
+            if (ps.done()) mine = 0u;
             bool lanes = true;
             if constexpr (BWD) lanes = by_lanes(mine, n);
             if (lanes) {
@@ -839,7 +835,7 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
                         const bool in0 = clip(g0, a0, b0), in1 = clip(g1, a1, b1) && two;
                         if (nxt.o >= 0 && ((in0 && nxt.a < b0) || (in1 && nxt.a < b1))) {
                             visit(bf, j0, nullptr);
-                            if (two && !ps.done) visit(bf, j1, nullptr);
+                            if (two && !ps.done()) visit(bf, j1, nullptr);
                         } else {
                             a0 = fmaxf(a0, tau_cur);
                             a1 = fmaxf(a1, tau_cur);
@@ -847,37 +843,34 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
                             const float4 da0 = ring.rec[bf][j0][1], dd0 = ring.rec[bf][j0][2], col0 = ring.rec[bf][j0][3];
                             const float4 da1 = ring.rec[bf][j1][1], dd1 = ring.rec[bf][j1][2], col1 = ring.rec[bf][j1][3];
                             const float r0[3] = {g0.x, g0.y, g0.z}, r1[3] = {g1.x, g1.y, g1.z};
-                            const float u0 = h0 ? a0 : 0.0f, v0 = h0 ? b0 : 0.0f, u1 = h1 ? a1 : 0.0f, v1 = h1 ? b1 : 0.0f;
-                            const float tau0 = seg_tau<false, KS>(da0, dd0, col0.w, r0, db_, u0, v0, bp.K, bp.inv_k,
-                                                                  bp.activation, nullptr, nullptr);
-                            const float tau1 = seg_tau<false, KS>(da1, dd1, col1.w, r1, db_, u1, v1, bp.K, bp.inv_k,
-                                                                  bp.activation, nullptr, nullptr);
+                            const float tau0 = seg_tau<false, KS>(da0, dd0, col0.w, r0, db_, a0, b0, bp.K, bp.inv_k,
+                                                                  bp.act_thr, nullptr, nullptr);
+                            const float tau1 = seg_tau<false, KS>(da1, dd1, col1.w, r1, db_, a1, b1, bp.K, bp.inv_k,
+                                                                  bp.act_thr, nullptr, nullptr);
                             ps.tests += 1;
-                            if (h0) composite_tau<NRM>(ps, tau0, col0, staged_nv(bf, j0), u0, v0, bp.eps_stop);
-                            ps.tests += (two && !ps.done) ? 1u : 0u;
-                            if (h1 && !ps.done) composite_tau<NRM>(ps, tau1, col1, staged_nv(bf, j1), u1, v1, bp.eps_stop);
+                            if (h0) composite_tau<NRM>(ps, tau0, col0, staged_nv(bf, j0), a0, b0, bp.eps_stop);
+                            ps.tests += (two && !ps.done()) ? 1u : 0u;
+                            if (h1 && !ps.done()) composite_tau<NRM>(ps, tau1, col1, staged_nv(bf, j1), a1, b1, bp.eps_stop);
                         }
                     }
-                    if (ps.done) mine = 0u;
+                    if (ps.done()) mine = 0u;
                 }
                 __syncwarp();
             } else if constexpr (BWD) {
                 for (uint32_t j = 0; j < (uint32_t)n; ++j) {
-                    if (__all_sync(0xffffffffu, ps.done)) return true;
+                    if (__all_sync(0xffffffffu, ps.done())) return true;
                     float acc[NV];
                     bool some = false;
-                    const bool live = !ps.done;
                     if constexpr (KS == 1) {
                         // a record that no lane's segment carries into the next actor interval is met at most
                         // once by every lane, so it takes the branch-free step; a record some lane crosses an
                         // actor entry in goes through the general path below
                         const float4 g = ring.rec[bf][j][0];
                         float t_in, t_out;
-                        const bool in = clip(g, t_in, t_out) && live;
+                        const bool in = clip(g, t_in, t_out);
                         if (!__any_sync(0xffffffffu, in && nxt.o >= 0 && nxt.a < t_out)) {
                             const float cur = fmaxf(t_in, tau_cur);
                             const bool hit = in && t_out > cur;
-                            ps.tests += live ? 1u : 0u;
                             if (!__any_sync(0xffffffffu, hit)) continue;
                             bwd_single_step<NRM>(ps, bw, bp, g, ring.rec[bf][j][1], ring.rec[bf][j][2],
                                                  ring.rec[bf][j][3], staged_nv(bf, j), db_, hit ? cur : 0.0f,
@@ -888,15 +881,15 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
                     }
 #pragma unroll
                     for (int i = 0; i < NV; ++i) acc[i] = 0.0f;
-                    if (live) some = visit(bf, j, acc);
+                    if (!ps.done()) some = visit(bf, j, acc);
                     // every lane visits record j together: reduce across the warp
                     if (__any_sync(0xffffffffu, some)) warp_reduce_add<NV>(acc, A.grad_rec + (size_t)ring.r[bf][j] * GS);
                 }
             }
-            return __all_sync(0xffffffffu, ps.done);
+            return __all_sync(0xffffffffu, ps.done());
         });
         // actor intervals behind the last background hit
-        while (nxt.o >= 0 && !ps.done) {
+        while (nxt.o >= 0 && !ps.done()) {
             enter_actor(nxt);
             tau_cur = nxt.b;
             advance();
@@ -916,7 +909,7 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
             const bool act = REPLAY ? status >= 1 : status == 2;
             if (!__any_sync(0xffffffffu, act)) continue;
             Pix<NRM> pt;
-            init_pix<NRM>(pt, !act);
+            init_pix<NRM>(pt, act ? iv(k, 1) : -1.0f);
             if (act) {
                 pt.T = st(k, ST_T);
                 if constexpr (RFORM) {
@@ -936,8 +929,8 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
                     }
                 }
             }
-            walk_actor(pt, s_act[q], act ? iv(k, 0) : 0.0f, act ? iv(k, 1) : 0.0f,
-                       std::integral_constant<bool, BWD>(), std::integral_constant<bool, WEX>());
+            walk_actor(pt, s_act[q], act ? iv(k, 0) : 0.0f, std::integral_constant<bool, BWD>(),
+                       std::integral_constant<bool, WEX>());
             ps.tests += pt.tests;
             if (!REPLAY && act) {
                 ps.C0 = pt.C0;

@@ -50,7 +50,7 @@ struct BatchParams {
     int32_t K;
     float inv_k;         // 1 / K
     float eps_stop;
-    int32_t activation;
+    float act_thr;       // densities above it are their own activation: 1.1, or -infinity for the identity
     int32_t Lkey;        // BSP key depth (max level over the octrees)
     int32_t oct_shift;   // 3 * Lkey
     int32_t view_shift;  // oct_shift + bits(n_oct)
