@@ -48,19 +48,24 @@ namespace dv {
 
 namespace {
 
-#ifndef DV_PLAIN_MIN_BLOCKS
-#define DV_PLAIN_MIN_BLOCKS 8  // resident CTAs per SM (64 registers)
-#endif
+// The backward takes a chunk lane by lane where its records cover at most this many of the block's 32 pixels on
+// average (8M-leaf six-camera frame / 1080p frame: 0: 2,830 / 209 us, 8: 2,728 / 210, 12: 2,522 / 214, 16: 2,512 /
+// 215, any: 2,540 / 253).
+constexpr int LANE_PIX = 14;
+// Resident CTAs per SM: the forward without normals fits 56 registers (9 CTAs: 1,481 -> 1,455 us on the 8M-leaf
+// frame); the others need 64.
+constexpr int plain_ctas(bool fwd) { return fwd ? 9 : 8; }
 
 // Tiles that no actor box covers (most of a frame): every ray is background only, so the tile's list
 // is the background's.
 // BWD: replay with gradients.  WEX: replay that writes every composited segment's (voxel, weight) into
 // the pixel's slots of the weights export (no outputs, no gradients).
 template <bool BWD, int KS, bool NRM, bool WEX>
-__global__ void __launch_bounds__(CT_THREADS, DV_PLAIN_MIN_BLOCKS) k_composite(const __grid_constant__ CompositeArgs A) {
+__global__ void __launch_bounds__(CT_THREADS, plain_ctas(!BWD && KS == 1 && !NRM && !WEX))
+    k_composite(const __grid_constant__ CompositeArgs A) {
     pdl_wait();
     pdl_launch_dependents();
-    __shared__ float4 s_rec[2][CT_THREADS][4];
+    __shared__ float4 s_rec[2][CT_THREADS][5];  // rows of 80 bytes: lanes can read different records at once
     __shared__ float4 s_nv[NRM ? 2 : 1][NRM ? CT_THREADS : 1];  // voxel normals of the staged records
     __shared__ uint32_t s_r[2][CT_THREADS];
     __shared__ uint16_t s_m[2][CT_THREADS];  // pixel rectangles of the staged pairs within the tile
@@ -120,7 +125,6 @@ __global__ void __launch_bounds__(CT_THREADS, DV_PLAIN_MIN_BLOCKS) k_composite(c
     constexpr int NV = GradLayout<NRM>::NV;
     constexpr int GS = GradLayout<NRM>::STRIDE;
 
-    uint32_t seen = 0;  // records visited so far; a ray that stops keeps the count as its tests
     // voxel normal of staged record j (zero without normals)
     auto staged_nv = [&](int slot, uint32_t j) {
         return NRM ? s_nv[NRM ? slot : 0][NRM ? j : 0] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -132,21 +136,12 @@ __global__ void __launch_bounds__(CT_THREADS, DV_PLAIN_MIN_BLOCKS) k_composite(c
         t_out = fminf(t_out, ps.end);
         return t_out > t_in;
     };
-    // one record of the batch, visited by the whole warp
-    auto visit = [&](int slot, uint32_t j) {
-        const float4 g = s_rec[slot][j][0];
-        float t_in, t_out;
-        const bool hit = clip(g, t_in, t_out);
-        seen += 1;
-        if constexpr (BWD) {
-            if (!__any_sync(0xffffffffu, hit)) return;
-        }
-        float acc[NV];
+    // composites the lane's segment of staged record j (backward and export), with its gradient values in acc.
+    // A lane meets a record at most once, so with one sample a warp that visits a record together runs the same
+    // arithmetic without branches, a lane that misses (hit false) on the empty segment [0, 0], whose optical
+    // depth, weight and gradient are exactly zero.
+    auto segment = [&](int slot, uint32_t j, float4 g, float t_in, float t_out, bool hit, float* acc) {
         if constexpr (BWD && KS == 1) {
-            // A lane meets a record at most once, so once any lane of the warp hits it every lane runs
-            // the same arithmetic without branches, a lane that misses (or is done) on the empty segment
-            // [0, 0], whose optical depth, weight and gradient are exactly zero; the gradient values
-            // are written, not accumulated, so nothing is cleared
             bwd_single_step<NRM>(ps, bw, bp, g, s_rec[slot][j][1], s_rec[slot][j][2], s_rec[slot][j][3],
                                  staged_nv(slot, j), db_, hit ? t_in : 0.0f, hit ? t_out : 0.0f, hit, acc);
         } else {
@@ -159,43 +154,80 @@ __global__ void __launch_bounds__(CT_THREADS, DV_PLAIN_MIN_BLOCKS) k_composite(c
                 add_segment<BWD, true, KS, NRM, WEX, BWD>(ps, bw, bp, s_rec[slot][j][1], s_rec[slot][j][2],
                                                           s_rec[slot][j][3], staged_nv(slot, j), rel, db_, t_in, t_out,
                                                           acc, s_r[slot][j], &ex);
-            if (!BWD && hit && ps.done()) ps.tests = seen;
         }
-        if constexpr (BWD) warp_reduce_add<NV>(acc, A.grad_rec + (size_t)s_r[slot][j] * GS);
     };
-    // 32 records of the batch, m: those that touch this warp's 8x4 block; true once the warp is done
-    auto chunk = [&](int slot, uint32_t c0, unsigned m) -> bool {
-        while (m) {
-            if (__all_sync(0xffffffffu, ps.done())) return true;
-            const uint32_t j0 = c0 + (uint32_t)(__ffs(m) - 1);
-            m &= m - 1;
-            if (BWD || WEX || m == 0) {
-                visit(slot, j0);
-                continue;
+    // 32 records of the batch, from c0; pm: the pixels of this warp's 8x4 block that the lane's record may touch.
+    // True once the warp is done.  The pixel masks, transposed, are a list of records per lane, and every lane
+    // steps through its own, so a record costs only the pixels it covers a step, not the whole warp (8M-leaf
+    // six-camera frame: 33 records visited per pixel for 10 met; plain forward 1,717 ->
+    // 1,480 us).  The backward does so where the records cover few pixels (at most LANE_PIX on average, the
+    // longest lane list at most 1 / LANE_GAIN of the records), each lane adding its own gradient values with
+    // vector atomics; elsewhere the warp visits the records together and sums their values first.
+    auto chunk = [&](int slot, uint32_t c0, uint32_t pm) -> bool {
+        unsigned m = __ballot_sync(0xffffffffu, pm != 0u);
+        if (!m) return false;
+        if (__all_sync(0xffffffffu, ps.done())) return true;
+        const int n = __popc(m);
+        bool lanes = true;
+        if constexpr (BWD) lanes = (int)__reduce_add_sync(0xffffffffu, (unsigned)__popc(pm)) <= n * LANE_PIX;
+        uint32_t mine = 0;
+        if (lanes) {
+            mine = warp_transpose(pm);
+            if (ps.done()) mine = 0u;
+            if constexpr (BWD) lanes = (int)__reduce_max_sync(0xffffffffu, (unsigned)__popc(mine)) * LANE_GAIN <= n;
+        }
+        if (lanes) {
+            if constexpr (!BWD && !WEX) ps.tests += (uint32_t)__popc(mine);
+            while (mine) {
+                const uint32_t j0 = c0 + (uint32_t)(__ffs(mine) - 1);
+                mine &= mine - 1;
+                if constexpr (!BWD && !WEX) {
+                    // forward, two records at once: both slab tests, both optical depths, then compositing in
+                    // list order with the stop rule
+                    const bool two = mine != 0u;
+                    const uint32_t j1 = two ? c0 + (uint32_t)(__ffs(mine) - 1) : j0;
+                    mine &= mine - 1;
+                    const float4 g0 = s_rec[slot][j0][0], g1 = s_rec[slot][j1][0];
+                    float a0, b0, a1, b1;
+                    const bool h0 = clip(g0, a0, b0), h1 = clip(g1, a1, b1) && two;
+                    const float4 da0 = s_rec[slot][j0][1], dd0 = s_rec[slot][j0][2], col0 = s_rec[slot][j0][3];
+                    const float4 da1 = s_rec[slot][j1][1], dd1 = s_rec[slot][j1][2], col1 = s_rec[slot][j1][3];
+                    const float r0[3] = {g0.x, g0.y, g0.z}, r1[3] = {g1.x, g1.y, g1.z};
+                    const float tau0 = seg_tau<false, KS>(da0, dd0, col0.w, r0, db_, a0, b0, bp.K, bp.inv_k, bp.act_thr,
+                                                          nullptr, nullptr);
+                    const float tau1 = seg_tau<false, KS>(da1, dd1, col1.w, r1, db_, a1, b1, bp.K, bp.inv_k, bp.act_thr,
+                                                          nullptr, nullptr);
+                    if (h0) composite_tau<NRM>(ps, tau0, col0, staged_nv(slot, j0), a0, b0, bp.eps_stop);
+                    if (h1 && !ps.done()) composite_tau<NRM>(ps, tau1, col1, staged_nv(slot, j1), a1, b1, bp.eps_stop);
+                    if (ps.done()) {
+                        ps.tests -= (uint32_t)__popc(mine);
+                        mine = 0u;
+                    }
+                } else {
+                    const float4 g = s_rec[slot][j0][0];
+                    float t_in, t_out;
+                    if (clip(g, t_in, t_out)) {
+                        float acc[NV];
+                        segment(slot, j0, g, t_in, t_out, true, acc);
+                        if constexpr (BWD) lane_add<NRM>(A.grad_rec, s_r[slot][j0], acc);
+                    }
+                    if (ps.done()) mine = 0u;
+                }
             }
-            const uint32_t j1 = c0 + (uint32_t)(__ffs(m) - 1);
-            m &= m - 1;
-            // forward, two records at once: both slab tests, both optical depths, then compositing in
-            // list order with the stop rule -- the same arithmetic as two visits
-            const float4 g0 = s_rec[slot][j0][0], g1 = s_rec[slot][j1][0];
-            float a0, b0, a1, b1;
-            const bool h0 = clip(g0, a0, b0), h1 = clip(g1, a1, b1);
-            const float4 da0 = s_rec[slot][j0][1], dd0 = s_rec[slot][j0][2], col0 = s_rec[slot][j0][3];
-            const float4 da1 = s_rec[slot][j1][1], dd1 = s_rec[slot][j1][2], col1 = s_rec[slot][j1][3];
-            const float r0[3] = {g0.x, g0.y, g0.z}, r1[3] = {g1.x, g1.y, g1.z};
-            const float tau0 = seg_tau<false, KS>(da0, dd0, col0.w, r0, db_, a0, b0, bp.K, bp.inv_k, bp.act_thr,
-                                                  nullptr, nullptr);
-            const float tau1 = seg_tau<false, KS>(da1, dd1, col1.w, r1, db_, a1, b1, bp.K, bp.inv_k, bp.act_thr,
-                                                  nullptr, nullptr);
-            if (h0) {
-                composite_tau<NRM>(ps, tau0, col0, staged_nv(slot, j0), a0, b0, bp.eps_stop);
-                if (ps.done()) ps.tests = seen + 1;
+            __syncwarp();
+        } else if constexpr (BWD) {
+            while (m) {
+                if (__all_sync(0xffffffffu, ps.done())) return true;
+                const uint32_t j = c0 + (uint32_t)(__ffs(m) - 1);
+                m &= m - 1;
+                const float4 g = s_rec[slot][j][0];
+                float t_in, t_out;
+                const bool hit = clip(g, t_in, t_out);
+                if (!__any_sync(0xffffffffu, hit)) continue;
+                float acc[NV];
+                segment(slot, j, g, t_in, t_out, hit, acc);
+                warp_reduce_add<NV>(acc, A.grad_rec + (size_t)s_r[slot][j] * GS);
             }
-            if (h1 && !ps.done()) {
-                composite_tau<NRM>(ps, tau1, col1, staged_nv(slot, j1), a1, b1, bp.eps_stop);
-                if (ps.done()) ps.tests = seen + 2;
-            }
-            seen += 2;
         }
         return __all_sync(0xffffffffu, ps.done());
     };
@@ -237,7 +269,7 @@ __global__ void __launch_bounds__(CT_THREADS, DV_PLAIN_MIN_BLOCKS) k_composite(c
         const uint32_t cnt = min((uint32_t)CT_THREADS, q_end - rg.x - bi * CT_THREADS);
         for (uint32_t c0 = 0; c0 < cnt && !fin; c0 += 32) {
             const uint32_t jl = c0 + lane;
-            fin = chunk(slot, c0, __ballot_sync(0xffffffffu, jl < cnt && block_pixels(s_m[slot][jl], bx, by) != 0u));
+            fin = chunk(slot, c0, jl < cnt ? block_pixels(s_m[slot][jl], bx, by) : 0u);
         }
         // every warp is done with this slot before batch bi+2 is copied into it
         if (__syncthreads_or(!fin) == 0) break;
@@ -245,7 +277,7 @@ __global__ void __launch_bounds__(CT_THREADS, DV_PLAIN_MIN_BLOCKS) k_composite(c
     asm volatile("cp.async.wait_all;\n" ::: "memory");  // no copy outlives the list (early exit)
 
     if constexpr (!BWD && !WEX) {
-        if (A.work) add_work(A.work, !valid ? 0u : ps.done() ? ps.tests : seen, ps.boxes, ps.n);
+        if (A.work) add_work(A.work, ps.tests, ps.boxes, ps.n);
         if (valid) store_pix<NRM>(ps, A, fp, lpix, pix);
     }
 }

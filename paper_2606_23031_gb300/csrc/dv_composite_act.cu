@@ -31,10 +31,6 @@ namespace {
 // more cover (a ray with more than 8 intervals takes the per-lane walk for those beyond)
 constexpr int NTA_SMALL = 4;
 constexpr int NTA_LARGE = 8;
-// With gradients a lane adds its own values to a record (three 16-byte vector atomics); a group whose
-// longest lane list is above 1 / LANE_GAIN of its records is walked in lockstep instead, where the warp
-// sums a record's values first.
-constexpr int LANE_GAIN = 2;
 // Tile lists above this length find their sub-lists by binary search (a dozen dependent loads) instead
 // of looking at every entry (two dependent loads per 128 entries)
 constexpr uint32_t SEARCH_MIN = 512;
@@ -100,30 +96,6 @@ __device__ __forceinline__ void atomic_grad(float* grad_rec, uint32_t r, const f
 #pragma unroll
     for (int c = 0; c < GradLayout<NRM>::NV; ++c)
         if (acc[c] != 0.0f) atomicAdd(gp + c, acc[c]);
-}
-
-// One lane's gradient values of record r, added with 16-byte vector atomics (the rows are 16-byte
-// aligned and padded to a multiple of four floats).
-template <bool NRM>
-__device__ __forceinline__ void lane_add(float* grad_rec, uint32_t r, const float* acc) {
-    constexpr int NV = GradLayout<NRM>::NV;
-    float4* gp = reinterpret_cast<float4*>(grad_rec + (size_t)r * GradLayout<NRM>::STRIDE);
-#pragma unroll
-    for (int c = 0; c < NV; c += 4)
-        atomicAdd(gp + c / 4, make_float4(acc[c], acc[c + 1], c + 2 < NV ? acc[c + 2] : 0.0f, c + 3 < NV ? acc[c + 3] : 0.0f));
-}
-
-// Transpose of the 32x32 bit matrix whose row l is lane l's x: afterwards bit j of lane l is bit l of
-// what lane j held.
-__device__ __forceinline__ uint32_t warp_transpose(uint32_t x) {
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int k = 16; k >= 1; k >>= 1) {
-        const uint32_t m = k == 16 ? 0x0000ffffu : k == 8 ? 0x00ff00ffu : k == 4 ? 0x0f0f0f0fu : k == 2 ? 0x33333333u : 0x55555555u;
-        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, k);
-        x = (lane & k) ? (x & ~m) | ((y >> k) & m) : (x & m) | ((y << k) & ~m);
-    }
-    return x;
 }
 
 // Per-lane walk of one actor's sub-list (divergent; only for a ray's intervals beyond
