@@ -344,6 +344,14 @@ void make_view(const dv_octree* oct, int n_oct, const dv_pose* poses, const dv_c
     double ym = std::fmax(std::fabs(0.5 - (double)cam.cy), std::fabs((double)cam.H - 0.5 - (double)cam.cy)) /
                 (double)cam.fy;
     vp.z_clip = (float)(0.999 * (double)cam.near_ / std::sqrt(1.0 + xm * xm + ym * ym));
+    // the sides of the image, 1.5 pixels out (see ViewParams)
+    const double side[4] = {(double)cam.cx + 1.5, (double)cam.cx - (double)cam.W - 1.5, (double)cam.cy + 1.5,
+                            (double)cam.cy - (double)cam.H - 1.5};
+    for (int k = 0; k < 4; ++k) {
+        const double f = k < 2 ? cam.fx : cam.fy;
+        vp.side[k] = (float)side[k];
+        vp.side_len[k] = (float)(1.0001 * std::sqrt(f * f + side[k] * side[k]));
+    }
     M3 Rc = load_R(cam.cam_to_world.R);
     double tc[3] = {cam.cam_to_world.t[0], cam.cam_to_world.t[1], cam.cam_to_world.t[2]};
     int64_t off = 0;
@@ -522,15 +530,13 @@ Layout state0_layout(int64_t n_view, int64_t n_oct, int64_t tiles, int64_t pix, 
 }
 
 struct PreBuffers {
-    uint32_t* cnt = nullptr;   // [NT] tiles of a visible (view, voxel)
-    uint64_t* rect = nullptr;  // [NT] its pixel rectangle
+    uint64_t* rect = nullptr;  // [NT] pixel rectangle of a visible (view, voxel)
     uint64_t* key = nullptr;   // [NT] depth keys of the visible ones, appended
     uint32_t* g = nullptr;     // [NT] their (view, voxel) indices
 };
 
 Layout pre_layout(int64_t NT, PreBuffers* b) {
     Layout L;
-    L.add(b ? &b->cnt : nullptr, NT);
     L.add(b ? &b->rect : nullptr, NT);
     L.add(b ? &b->key : nullptr, NT);
     L.add(b ? &b->g : nullptr, NT);
@@ -573,7 +579,6 @@ struct PostBuffers {
     uint32_t* pair_hist = nullptr;
     uint32_t* ticket = nullptr;
     uint32_t* tile_scratch = nullptr;  // [192] bucket counts and cursors of the tile order
-    uint32_t* tile_cnt = nullptr;
 };
 
 Layout post_layout(int64_t n_vis, int64_t P, int64_t tiles, int key_bits, int tile_bits, PostBuffers* b) {
@@ -589,7 +594,7 @@ Layout post_layout(int64_t n_vis, int64_t P, int64_t tiles, int key_bits, int ti
     const int64_t n_lb = dv::records_emit_blocks(n_vis);
     const int64_t vw = dv::sort_counted_words(n_vis, key_bits), pw = dv::sort_counted_words(P, tile_bits);
     const int64_t hw = (int64_t)dv::key_passes(tile_bits) * 256;
-    const int64_t words32 = vw + pw + hw + 1 + 192 + tiles;
+    const int64_t words32 = vw + pw + hw + 1 + 192;
     const int64_t zb = 8 * n_lb + 4 * words32;
     L.add(b ? &b->zero : nullptr, (zb + 7) / 8);
     if (b) b->zero_bytes = zb;
@@ -608,7 +613,6 @@ void post_place_zero(int64_t n_vis, int64_t P, int key_bits, int tile_bits, Post
     w += dv::key_passes(tile_bits) * 256;
     b.ticket = w;
     b.tile_scratch = w + 1;
-    b.tile_cnt = w + 1 + 192;
 }
 
 // the part known before any work is enqueued: per-view constants, per-pixel and per-tile state,
@@ -807,7 +811,7 @@ dv_status render_batch(dv_ctx* ctx, const dv_octree* oct, int n_oct, const dv_po
     {
         Prof p(ctx, KP_PROJECT, s);
         if (e == cudaSuccess)
-            e = launch_project(bp, pre.cnt, pre.rect, pre.key, pre.g, key_hist, key_bits,
+            e = launch_project(bp, pre.rect, pre.key, pre.g, key_hist, key_bits, B.range,
                                (unsigned long long*)ctx->d_scalars, ctx->h_scalars_dev, seq, ctx->d_spin_err,
                                B.work, s);
     }
@@ -892,9 +896,9 @@ dv_status render_batch(dv_ctx* ctx, const dv_octree* oct, int n_oct, const dv_po
     {
         Prof p(ctx, KP_RECORDS, s);
         if (e == cudaSuccess)
-            e = launch_records_emit(bp, B.sorted_g, sorted_key, n_vis, P, pre.cnt, pre.rect, B.rec, B.nrm,
+            e = launch_records_emit(bp, B.sorted_g, sorted_key, n_vis, P, pre.rect, B.rec, B.nrm,
                                     post.rect_sorted, B.vis_start, post.pk0, post.pv0, post.pair_hist, tile_bits,
-                                    post.tile_cnt, post.lb_status, post.ticket, sort_err, ctx->d_spin_err, s);
+                                    post.lb_status, post.ticket, sort_err, ctx->d_spin_err, s);
     }
     // stable sort of the pairs by tile: every tile's list stays front to back; the values land in pval
     uint32_t* sorted_tile = nullptr;
@@ -913,8 +917,7 @@ dv_status render_batch(dv_ctx* ctx, const dv_octree* oct, int n_oct, const dv_po
                                  B.d_sort_err, B.h_status_dev, s);
         if (e == cudaSuccess) B.published = true;
         if (e == cudaSuccess)
-            e = launch_tile_order(bp, post.tile_cnt, (int)tiles, B.range, post.bucket, post.tile_scratch,
-                                  B.tile_order, s);
+            e = launch_tile_order(bp, B.range, (int)tiles, post.bucket, post.tile_scratch, B.tile_order, s);
     }
     {
         Prof p(ctx, KP_FWD, s);

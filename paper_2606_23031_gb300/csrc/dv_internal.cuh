@@ -41,6 +41,10 @@ struct ViewParams {
     float* rgb;          // this view's outputs [H*W][3], [H*W], [H*W] (device)
     float* depth;
     float* alpha;
+    // the image's four side planes moved 1.5 pixels outwards, for points in front of the camera: left of it
+    // fx x + side[0] z < 0, right fx x + side[1] z > 0, above fy y + side[2] z < 0, below fy y + side[3] z > 0;
+    // side_len: lengths of the planes' normals, rounded up
+    float side[4], side_len[4];
     float* normal;       // [H*W][3] normal state N (world frame), or null when normals are not rendered
 };
 
@@ -179,15 +183,15 @@ cudaError_t sort_counted_u32(uint32_t* keys, uint32_t* vals, uint32_t* keys_tmp,
 int key_passes(int n_bits);
 
 // kernel launchers (one thread per (view, voxel) unless stated)
-// Projection: for each visible (view, voxel) g, cnt[g] (tiles) and rect[g] (pixel rectangle); the
+// Projection: for each visible (view, voxel) g, rect[g] (pixel rectangle); every tile's range cleared; the
 // visible ones appended to (out_key, out_g) (depth key, g) in no particular order, the digits of
 // their keys counted in key_hist [key_passes(key_bits)][256] (zeroed by the caller).  scal[4]
 // (zeroed by the caller): visible count, pair count, flags (DV_FLAG_*), finished blocks; the last
 // block copies the first three into host_out (mapped host memory), with the device's wait-error word
 // (taken and cleared) folded into the flags, then writes `seq` into host_out[3] once the three are
 // there.  It also clears work[5] (the call's work counters and sort flag).
-cudaError_t launch_project(const BatchParams& bp, uint32_t* cnt, uint64_t* rect, uint64_t* out_key, uint32_t* out_g,
-                           uint32_t* key_hist, int key_bits, unsigned long long* scal, uint64_t* host_out, uint64_t seq,
+cudaError_t launch_project(const BatchParams& bp, uint64_t* rect, uint64_t* out_key, uint32_t* out_g,
+                           uint32_t* key_hist, int key_bits, uint2* tile_range, unsigned long long* scal, uint64_t* host_out, uint64_t seq,
                            uint32_t* spin_err, unsigned long long* work, cudaStream_t s);
 // copies n words into mapped host memory; with spin_err, takes (and clears) the device's wait-error
 // word and sets DV_FLAG_SPIN_TIMEOUT in word flag_idx
@@ -198,14 +202,14 @@ cudaError_t launch_publish(const uint64_t* src, uint64_t* host_mapped_dst, int n
 uint32_t* spin_error_word();
 // One thread per visible voxel in depth order: records (and normals), rect_sorted, vis_start
 // [n_view * n_oct + 1] (start of every (view, octree) group), and the (tile, record) pairs in
-// depth order at offsets of a single-pass scan of the tile counts; counts the pairs of every tile in
-// tile_cnt and the tile-sort digits in pair_hist [key_passes(tile_bits)][256].  tile_cnt, pair_hist,
+// depth order at offsets of a single-pass scan of the tile counts; counts the tile-sort digits in
+// pair_hist [key_passes(tile_bits)][256].  pair_hist,
 // lb_status [records_emit_blocks(n_vis)] and ticket are zeroed by the caller.
 cudaError_t launch_records_emit(const BatchParams& bp, const uint32_t* sorted_g, const uint64_t* sorted_key,
-                                int64_t n_vis, int64_t n_pairs, const uint32_t* cnt, const uint64_t* rect,
+                                int64_t n_vis, int64_t n_pairs, const uint64_t* rect,
                                 VoxRec* rec, float4* nrm, uint64_t* rect_sorted, uint32_t* vis_start,
                                 uint32_t* pair_key, uint32_t* pair_val, uint32_t* pair_hist, int tile_bits,
-                                uint32_t* tile_cnt, unsigned long long* lb_status, uint32_t* ticket,
+                                unsigned long long* lb_status, uint32_t* ticket,
                                 uint32_t* call_err, uint32_t* dev_err, cudaStream_t s);
 int64_t records_emit_blocks(int64_t n_vis);
 // per tile-sorted pair: its voxel's pixel rectangle within the tile; per tile with pairs: its [first, end) range of the
@@ -213,12 +217,11 @@ int64_t records_emit_blocks(int64_t n_vis);
 cudaError_t launch_pair_rect(const BatchParams& bp, const uint32_t* pair_key, const uint32_t* pair_val,
                              const uint64_t* rect_sorted, int64_t n_pairs, int64_t n_vis, uint16_t* pair_rect,
                              uint2* tile_range, const uint64_t* sort_err, uint64_t* status_host, cudaStream_t s);
-// the empty range for every tile without pairs, and the tiles ordered by decreasing list length (log2
-// buckets of tile_cnt) within three groups, in this order: the tiles that 5 or more actor clip boxes
+// the tiles ordered by decreasing list length (log2
+// buckets of their ranges) within three groups, in this order: the tiles that 5 or more actor clip boxes
 // cover (bp.n_tiles_large), those that 1 to 4 cover (bp.n_tiles_small), the others.  bucket: one byte
 // of scratch per tile; scratch192: zeroed words.
-cudaError_t launch_tile_order(const BatchParams& bp, const uint32_t* tile_cnt, int n_tiles, uint2* range,
-                              uint8_t* bucket, uint32_t* scratch192, uint32_t* order, cudaStream_t s);
+cudaError_t launch_tile_order(const BatchParams& bp, const uint2* range, int n_tiles, uint8_t* bucket, uint32_t* scratch192, uint32_t* order, cudaStream_t s);
 // Two more streams of the context with their events: a compositing pass runs its three launches (the
 // tiles that many actor boxes cover, those that a few cover, the others) side by side on these and
 // the call's stream.

@@ -16,9 +16,9 @@
 //          colour for this camera; the block then writes the (tile, record) pairs
 //          of its voxels, one per tile of each rectangle, at the offsets a
 //          single-pass scan (look-back over earlier blocks) gives, counting the
-//          pairs of every tile and the digits of the tile sort on the way.
+//          digits of the tile sort on the way.
 // rect     the part of its tile's pixels each sorted pair's rectangle covers, and the tile ranges.
-// order    the tiles by list length (from the per-tile counts) within their actor-coverage group.
+// order    the tiles by list length (from the ranges) within their actor-coverage group.
 //
 // Depth-order key.  Leaves of one octree are cells of a binary space partition
 // (each node split by the three planes through its centre).  For rays that all
@@ -87,13 +87,38 @@ __device__ __forceinline__ void proj_point(const ViewParams& fp, float x, float 
     v1 = fmaxf(v1, v);
 }
 
-// Projection of (view, voxel) g: returns its tile count (0: not visible) and, when visible, its
+// bits of a 16-bit number to every third bit
+__device__ __forceinline__ uint64_t spread3(uint32_t x) {
+    uint64_t v = x;
+    v = (v | (v << 16)) & 0x0000ff0000ffull;
+    v = (v | (v << 8)) & 0x00f00f00f00full;
+    v = (v | (v << 4)) & 0x0c30c30c30c3ull;
+    v = (v | (v << 2)) & 0x249249249249ull;
+    return v;
+}
+
+// One axis of the depth-order path: leaf index `idx` (level bits) with every bit flipped where the
+// camera lies on the positive side of that node's plane.  X is the camera coordinate on the lattice of
+// 2^(Lk + 1) half cells.  Along the camera's own path (the leading bits idx shares with the camera's cell at the
+// leaf's level) a node's plane has the camera on the side of its next bit, so those bits become 0 and the first
+// bit that differs becomes 1; below it the camera is on one side of all remaining planes.
+__device__ __forceinline__ uint32_t side_path(uint32_t idx, int level, int64_t X, int Lk) {
+    const uint32_t mask = (1u << level) - 1u;
+    if (X < 0) return idx;
+    if (X >> (Lk + 1)) return ~idx & mask;
+    const uint32_t cell = (uint32_t)(X >> (Lk + 1 - level));
+    const uint32_t diff = idx ^ cell;
+    if (!diff) return 0u;
+    const int top = 31 - __clz((int)diff);
+    const uint32_t low = (1u << top) - 1u;
+    return (1u << top) | (((cell >> top) & 1u ? ~idx : idx) & low);
+}
+
+// Projection of voxel gv of `view`: returns its tile count (0: not visible) and, when visible, its
 // pixel rectangle and depth-order key.
-__device__ __forceinline__ uint32_t project_voxel(const BatchParams& bp, int64_t g, uint64_t& rect,
+__device__ __forceinline__ uint32_t project_voxel(const BatchParams& bp, int view, int64_t gv, uint64_t& rect,
                                                   uint64_t& skey, uint32_t* __restrict__ flags) {
-    const int view = (int)(g / bp.n_vox);
-    const int64_t gv = g - (int64_t)view * bp.n_vox;
-    const int o = find_octree(bp, gv);
+    const int o = gv < bp.vox_offset[1] ? 0 : find_octree(bp, gv);
     const ViewParams& fp = bp.views[view];
     const OctParams& P = bp.octs[view * bp.n_oct + o];
     const int64_t v = gv - bp.vox_offset[o];
@@ -103,6 +128,29 @@ __device__ __forceinline__ uint32_t project_voxel(const BatchParams& bp, int64_t
         atomicOr(flags, DV_FLAG_BAD_LEVEL);
         __threadfence();  // visible to the block that reports the flags
         return 0;
+    }
+    // Most voxels lie outside the frustum by far: the bounding sphere against the near and far planes and the four
+    // sides, each side 1.5 pixels outside the image, decides those with a tenth of the arithmetic (8M-leaf frame,
+    // six cameras: @P@).  It leaves out nothing that the corners below would keep: the radius covers
+    // the rounding of both (4e-6 of the coordinates' size), and where the sphere comes so close to the camera
+    // plane that its projection exceeds 2e5 pixels (the corner test's own margin then grows past a pixel)
+    // the corners decide.
+    {
+        const float h = 0.5f * L.s;
+        const float x0 = L.mn[0] + h, y0 = L.mn[1] + h, z0 = L.mn[2] + h;
+        float c[3];
+#pragma unroll
+        for (int r = 0; r < 3; ++r) c[r] = fmaf(P.M[r * 3 + 0], x0, fmaf(P.M[r * 3 + 1], y0, fmaf(P.M[r * 3 + 2], z0, P.m[r])));
+        const float size = fabsf(x0) + fabsf(y0) + fabsf(z0) + fabsf(P.m[0]) + fabsf(P.m[1]) + fabsf(P.m[2]);
+        const float rad = fmaf(0.8661f, L.s, 4e-6f * size);
+        const float zn = c[2] - rad;
+        if (c[2] + rad < fp.z_clip || zn > fp.far_) return 0;
+        if (zn > fp.z_clip && fmaxf(fp.fx * (fabsf(c[0]) + rad), fp.fy * (fabsf(c[1]) + rad)) < 2e5f * zn) {
+            const float fx = fp.fx * c[0], fy = fp.fy * c[1];
+            if (fmaf(fp.side[0], c[2], fx) < -fp.side_len[0] * rad || fmaf(fp.side[1], c[2], fx) > fp.side_len[1] * rad ||
+                fmaf(fp.side[2], c[2], fy) < -fp.side_len[2] * rad || fmaf(fp.side[3], c[2], fy) > fp.side_len[3] * rad)
+                return 0;
+        }
     }
     // corners in the camera frame: p = M (mn + s*offset) + m
     float p0[3], e[3][3];
@@ -160,22 +208,12 @@ __device__ __forceinline__ uint32_t project_voxel(const BatchParams& bp, int64_t
     const uint32_t n_tiles = (tx1 - tx0 + 1) * (ty1 - ty0 + 1);
     // pixel rectangle (tiles are its pixels >> 4)
     rect = (uint64_t)pu0 | ((uint64_t)pu1 << 16) | ((uint64_t)pv0 << 32) | ((uint64_t)pv1 << 48);
-    // depth-order key (see the file comment)
-    uint64_t bsp = 0;
+    // depth-order key (see the file comment): the three axes' paths interleaved, x in the highest bit
     const int Lk = bp.Lkey;
-    for (int l = 0; l < L.level; ++l) {
-        const int sh = L.level - 1 - l;
-        const uint32_t bi = (L.i >> sh) & 1u, bj = (L.j >> sh) & 1u, bk = (L.k >> sh) & 1u;
-        const int64_t ti = ((int64_t)(L.i >> (sh + 1)) * 2 + 1) << (Lk - l);
-        const int64_t tj = ((int64_t)(L.j >> (sh + 1)) * 2 + 1) << (Lk - l);
-        const int64_t tk = ((int64_t)(L.k >> (sh + 1)) * 2 + 1) << (Lk - l);
-        const uint32_t fi = bi ^ (uint32_t)(P.O2[0] >= ti);
-        const uint32_t fj = bj ^ (uint32_t)(P.O2[1] >= tj);
-        const uint32_t fk = bk ^ (uint32_t)(P.O2[2] >= tk);
-        bsp = (bsp << 3) | (fi << 2) | (fj << 1) | fk;
-    }
-    bsp <<= 3 * (Lk - L.level);
-    skey = ((uint64_t)view << bp.view_shift) | ((uint64_t)o << bp.oct_shift) | bsp;
+    const uint64_t bsp = (spread3(side_path(L.i, L.level, P.O2[0], Lk)) << 2) |
+                         (spread3(side_path(L.j, L.level, P.O2[1], Lk)) << 1) |
+                         spread3(side_path(L.k, L.level, P.O2[2], Lk));
+    skey = ((uint64_t)view << bp.view_shift) | ((uint64_t)o << bp.oct_shift) | (bsp << (3 * (Lk - L.level)));
     return n_tiles;
 }
 
@@ -186,26 +224,32 @@ constexpr int MAX_KEY_PASSES = 8;  // 8-bit digits of a 64-bit key
 // [key_passes][256], and the block that finishes last copies scal[0..2] into host_out[0..2] (the
 // device's wait-error word folded into the flags) and then `seq` into host_out[3], so the host learns
 // the sizes from this kernel alone, as soon as they are final.  scal[3] counts finished blocks.
-// Block 0 also clears the call's five work words.
-__global__ void __launch_bounds__(256) k_project(const __grid_constant__ BatchParams bp, uint32_t* __restrict__ cnt,
-                                                 uint64_t* __restrict__ rect, uint64_t* __restrict__ out_key,
+// Block 0 also clears the call's five work words, and the grid the tile ranges.  Grid: (blocks of one view's
+// voxels, views).
+__global__ void __launch_bounds__(256) k_project(const __grid_constant__ BatchParams bp, uint64_t* __restrict__ rect, uint64_t* __restrict__ out_key,
                                                  uint32_t* __restrict__ out_g, uint32_t* __restrict__ key_hist,
-                                                 int key_passes, unsigned long long* __restrict__ scal,
+                                                 int key_passes, uint2* __restrict__ range,
+                                                 unsigned long long* __restrict__ scal,
                                                  volatile uint64_t* host_out, uint64_t seq,
                                                  uint32_t* __restrict__ spin_err, unsigned long long* __restrict__ work) {
     pdl_wait();
     pdl_launch_dependents();
-    if (blockIdx.x == 0 && threadIdx.x < 5) work[threadIdx.x] = 0ull;
+    const uint32_t block = blockIdx.y * gridDim.x + blockIdx.x, n_block = gridDim.x * gridDim.y;
+    if (block == 0 && threadIdx.x < 5) work[threadIdx.x] = 0ull;
+    for (int64_t t = (int64_t)block * 256 + threadIdx.x; t < bp.n_tiles; t += (int64_t)n_block * 256)
+        range[t] = make_uint2(0u, 0u);
     __shared__ uint32_t h[MAX_KEY_PASSES][256];
     __shared__ uint32_t s_wv[8];
     __shared__ unsigned long long s_wp[8];
     __shared__ unsigned long long s_base;
     __shared__ uint32_t s_nv;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t g = (int64_t)blockIdx.x * blockDim.x + tid;  // view * n_vox + voxel
+    const int view = blockIdx.y;
+    const int64_t gv = (int64_t)blockIdx.x * 256 + tid;  // voxel of the view
+    const int64_t g = view * bp.n_vox + gv;
     uint64_t rc = 0, key = 0;
     uint32_t c = 0;
-    if (g < bp.n_vox * bp.n_view) c = project_voxel(bp, g, rc, key, reinterpret_cast<uint32_t*>(scal + 2));
+    if (gv < bp.n_vox) c = project_voxel(bp, view, gv, rc, key, reinterpret_cast<uint32_t*>(scal + 2));
     const unsigned bal = __ballot_sync(0xffffffffu, c != 0);
     unsigned long long np = c;
 #pragma unroll
@@ -235,7 +279,6 @@ __global__ void __launch_bounds__(256) k_project(const __grid_constant__ BatchPa
             const unsigned long long q = s_base + s_wv[warp] + __popc(bal & ((1u << lane) - 1u));
             out_key[q] = key;
             out_g[q] = (uint32_t)g;
-            cnt[g] = c;
             rect[g] = rc;
             for (int p = 0; p < key_passes; ++p) atomicAdd(&h[p][(uint32_t)(key >> (8 * p)) & 255u], 1u);
         }
@@ -251,7 +294,7 @@ __global__ void __launch_bounds__(256) k_project(const __grid_constant__ BatchPa
     if (tid == 0) {
         __threadfence();
         const unsigned long long done = atomicAdd(scal + 3, 1ull);
-        if (done == gridDim.x - 1) {
+        if (done == n_block - 1) {
             __threadfence();
             const uint64_t nv = atomicAdd(scal + 0, 0ull), pp = atomicAdd(scal + 1, 0ull);
             uint64_t fl = atomicOr(reinterpret_cast<unsigned long long*>(scal + 2), 0ull);
@@ -314,13 +357,13 @@ __device__ __forceinline__ unsigned long long lb_load(const unsigned long long* 
 //     a look-back over the earlier blocks' published counts (the block reads 256 predecessors at a
 //     time; an inclusive one ends the walk; every spin is bounded);
 //  3. the block's pairs, spread over all its threads (a pair finds its voxel by binary search in
-//     the block's offsets), with the tile-sort digits and the per-tile pair counts.
+//     the block's offsets), with the tile-sort digits.
 __global__ void __launch_bounds__(256) k_records_emit(
     const __grid_constant__ BatchParams bp, const uint32_t* __restrict__ sorted_g,
-    const uint64_t* __restrict__ sorted_key, int64_t n_vis, int64_t n_pairs, const uint32_t* __restrict__ cnt,
+    const uint64_t* __restrict__ sorted_key, int64_t n_vis, int64_t n_pairs,
     const uint64_t* __restrict__ rect, VoxRec* __restrict__ rec, float4* __restrict__ nrm,
     uint64_t* __restrict__ rect_sorted, uint32_t* __restrict__ vis_start, uint32_t* __restrict__ pkey,
-    uint32_t* __restrict__ pval, uint32_t* __restrict__ pair_hist, int pair_passes, uint32_t* __restrict__ tile_cnt,
+    uint32_t* __restrict__ pval, uint32_t* __restrict__ pair_hist, int pair_passes,
     unsigned long long* __restrict__ lb_status, uint32_t* __restrict__ ticket, uint32_t* __restrict__ call_err,
     uint32_t* __restrict__ dev_err, int spin_limit) {
     pdl_wait();
@@ -343,14 +386,31 @@ __global__ void __launch_bounds__(256) k_records_emit(
     uint32_t c = 0;
     if (r < n_vis) {
         const uint32_t g = sorted_g[r];
-        const int view = (int)(g / bp.n_vox);
-        const int64_t gv = (int64_t)g - (int64_t)view * bp.n_vox;
-        const int o = find_octree(bp, gv);
-        const OctParams& P = bp.octs[view * bp.n_oct + o];
-        const int64_t v = gv - bp.vox_offset[o];
-        const Leaf L = decode_leaf(P, P.key[v]);
+        const int grp = key_group(bp, sorted_key[r]);
+        const int prev = r > 0 ? key_group(bp, sorted_key[r - 1]) : -1;
+        const int view = grp / bp.n_oct;
+        const OctParams& P = bp.octs[grp];
+        const int64_t v = (int64_t)(g - (uint32_t)view * (uint32_t)bp.n_vox) - P.vox_offset;
+        // The voxel's key, densities, rectangle and SH coefficients, all in flight together: the voxels of a block
+        // are scattered over memory, so one round trip per voxel is what this kernel waits for (with the
+        // coefficients loaded as they were used: 8M-leaf frame, six cameras @R@)
+        const int deg = P.sh_degree;
+        const int nsh = (deg + 1) * (deg + 1);
+        const float* shv = P.sh + v * nsh * 3;
+        const bool rows16 = (deg & 1) && (reinterpret_cast<uintptr_t>(P.sh) & 15) == 0;  // rows of 48 or 192 bytes
+        float4 sq[12];
+        if (rows16 && deg == 3) {
+#pragma unroll
+            for (int e = 0; e < 12; ++e) sq[e] = __ldg(reinterpret_cast<const float4*>(shv) + e);
+        } else if (rows16) {
+#pragma unroll
+            for (int e = 0; e < 3; ++e) sq[e] = __ldg(reinterpret_cast<const float4*>(shv) + e);
+        }
+        const uint64_t key = __ldg(P.key + v);
         const float4* d4 = reinterpret_cast<const float4*>(P.dens + v * 8);
         const float4 da = __ldg(d4), db = __ldg(d4 + 1);
+        const uint64_t rc = __ldg(rect + g);
+        const Leaf L = decode_leaf(P, key);
         // min corner relative to the camera centre (octree frame), then the view direction:
         // camera centre -> voxel centre
         const float rx = L.mn[0] - P.o_loc[0], ry = L.mn[1] - P.o_loc[1], rz = L.mn[2] - P.o_loc[2];
@@ -363,20 +423,20 @@ __global__ void __launch_bounds__(256) k_records_emit(
         gy *= ig;
         gz *= ig;
         float b[16];
-        sh_eval_basis(P.sh_degree, gx, gy, gz, b);
-        const int nsh = (P.sh_degree + 1) * (P.sh_degree + 1);
-        const float* shv = P.sh + v * nsh * 3;
+        sh_eval_basis(deg, gx, gy, gz, b);
         float cc[3] = {0.5f, 0.5f, 0.5f};
-        if ((nsh * 3) % 4 == 0 && (reinterpret_cast<uintptr_t>(shv) & 15) == 0) {
-            // 16-byte loads of the coefficient rows, flattened: element e = 3 q + channel
+        // coefficient rows flattened: element e = 3 q + channel
+        auto add4 = [&](int e0, float4 x4) {
+            const float xs[4] = {x4.x, x4.y, x4.z, x4.w};
 #pragma unroll
-            for (int e0 = 0; e0 < 48; e0 += 4) {
-                if (e0 >= nsh * 3) break;
-                const float4 x4 = __ldg(reinterpret_cast<const float4*>(shv + e0));
-                const float xs[4] = {x4.x, x4.y, x4.z, x4.w};
+            for (int i = 0; i < 4; ++i) cc[(e0 + i) % 3] = fmaf(b[(e0 + i) / 3], xs[i], cc[(e0 + i) % 3]);
+        };
+        if (rows16 && deg == 3) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) cc[(e0 + i) % 3] = fmaf(b[(e0 + i) / 3], xs[i], cc[(e0 + i) % 3]);
-            }
+            for (int e = 0; e < 12; ++e) add4(4 * e, sq[e]);
+        } else if (rows16) {
+#pragma unroll
+            for (int e = 0; e < 3; ++e) add4(4 * e, sq[e]);
         } else {
             for (int q = 0; q < nsh; ++q) {
                 cc[0] = fmaf(b[q], __ldg(shv + q * 3 + 0), cc[0]);
@@ -412,15 +472,13 @@ __global__ void __launch_bounds__(256) k_records_emit(
             for (int k = 0; k < 3; ++k) nw[k] = fmaf(P.Rw[k * 3 + 0], nl[0], fmaf(P.Rw[k * 3 + 1], nl[1], P.Rw[k * 3 + 2] * nl[2]));
             nrm[r] = make_float4(nw[0], nw[1], nw[2], 0.0f);
         }
-        c = cnt[g];
-        const uint64_t rc = rect[g];
+        c = (uint32_t)((((rc >> 16) & 0xffff) >> 4) - ((rc & 0xffff) >> 4) + 1) *
+            (uint32_t)((rc >> 52) - (((rc >> 32) & 0xffff) >> 4) + 1);  // its tiles
         rect_sorted[r] = rc;
         s_rc[tid] = rc;
         s_tb[tid] = bp.tile_base[view];
         s_tx[tid] = bp.views[view].tiles_x;
         // start of every (view, octree) group in depth order
-        const int grp = key_group(bp, sorted_key[r]);
-        const int prev = r > 0 ? key_group(bp, sorted_key[r - 1]) : -1;
         for (int q = prev + 1; q <= grp; ++q) vis_start[q] = (uint32_t)r;
         if (r == n_vis - 1)
             for (int q = grp + 1; q <= bp.n_view * bp.n_oct; ++q) vis_start[q] = (uint32_t)n_vis;
@@ -502,7 +560,6 @@ __global__ void __launch_bounds__(256) k_records_emit(
             pkey[p] = tile;
             pval[p] = blk * 256u + (uint32_t)lo;
         }
-        atomicAdd(tile_cnt + tile, 1u);
         for (int q = 0; q < pair_passes; ++q) atomicAdd(&h[q][(tile >> (8 * q)) & 255u], 1u);
     }
     __syncthreads();
@@ -582,11 +639,10 @@ __device__ __forceinline__ int tile_bucket(const BatchParams& bp, uint32_t n_pai
     return b + (boxes >= 5 ? 64 : boxes > 0 ? 32 : 0);
 }
 
-// one thread per tile: its bucket (kept in bucket[t]) into the global bucket counts hist[96]; a tile
-// without pairs gets the empty range (the pair-rectangle kernel wrote the others)
+// one thread per tile: its bucket (kept in bucket[t]) into the global bucket counts hist[96]
 __global__ void __launch_bounds__(256) k_tile_count(const __grid_constant__ BatchParams bp,
-                                                    const uint32_t* __restrict__ tile_cnt, int n_tiles,
-                                                    uint8_t* __restrict__ bucket, uint2* __restrict__ range,
+                                                    const uint2* __restrict__ range, int n_tiles,
+                                                    uint8_t* __restrict__ bucket,
                                                     uint32_t* __restrict__ hist) {
     pdl_wait();
     pdl_launch_dependents();
@@ -595,8 +651,8 @@ __global__ void __launch_bounds__(256) k_tile_count(const __grid_constant__ Batc
     __syncthreads();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t < n_tiles) {
-        const uint32_t c = tile_cnt[t];
-        if (c == 0) range[t] = make_uint2(0u, 0u);
+        const uint2 rg = range[t];
+        const uint32_t c = rg.y > rg.x ? rg.y - rg.x : 0u;  // reversed only after a sort wait that timed out
         const int b = tile_bucket(bp, c, t);
         bucket[t] = (uint8_t)b;
         atomicAdd(&h[b], 1u);
@@ -660,30 +716,29 @@ cudaError_t launch_publish(const uint64_t* src, uint64_t* host_mapped_dst, int n
     return cudaGetLastError();
 }
 
-cudaError_t launch_project(const BatchParams& bp, uint32_t* cnt, uint64_t* rect, uint64_t* out_key, uint32_t* out_g,
-                           uint32_t* key_hist, int key_bits, unsigned long long* scal, uint64_t* host_out, uint64_t seq,
+cudaError_t launch_project(const BatchParams& bp, uint64_t* rect, uint64_t* out_key, uint32_t* out_g,
+                           uint32_t* key_hist, int key_bits, uint2* tile_range, unsigned long long* scal, uint64_t* host_out, uint64_t seq,
                            uint32_t* spin_err, unsigned long long* work, cudaStream_t s) {
-    const int64_t n = bp.n_vox * bp.n_view;
     const int passes = key_passes(key_bits);
     if (passes > MAX_KEY_PASSES) return cudaErrorInvalidValue;
-    // with no voxel at all, one empty block still clears the work words and reports the (zero) sizes
-    launch_pdl(k_project, dim3(n > 0 ? nblk(n, 256) : 1u), dim3(256), s, bp, cnt, rect, out_key, out_g, key_hist,
-               passes, scal, (volatile uint64_t*)host_out, seq, spin_err, work);
+    // with no voxel at all, empty blocks still clear the work words and report the (zero) sizes
+    launch_pdl(k_project, dim3(bp.n_vox > 0 ? nblk(bp.n_vox, 256) : 1u, (unsigned)bp.n_view), dim3(256), s, bp, rect,
+               out_key, out_g, key_hist, passes, tile_range, scal, (volatile uint64_t*)host_out, seq, spin_err, work);
     count_launches(1);
     return cudaGetLastError();
 }
 
 cudaError_t launch_records_emit(const BatchParams& bp, const uint32_t* sorted_g, const uint64_t* sorted_key,
-                                int64_t n_vis, int64_t n_pairs, const uint32_t* cnt, const uint64_t* rect,
+                                int64_t n_vis, int64_t n_pairs, const uint64_t* rect,
                                 VoxRec* rec, float4* nrm, uint64_t* rect_sorted, uint32_t* vis_start,
                                 uint32_t* pair_key, uint32_t* pair_val, uint32_t* pair_hist, int tile_bits,
-                                uint32_t* tile_cnt, unsigned long long* lb_status, uint32_t* ticket,
+                                unsigned long long* lb_status, uint32_t* ticket,
                                 uint32_t* call_err, uint32_t* dev_err, cudaStream_t s) {
     if (n_vis <= 0) return cudaMemsetAsync(vis_start, 0, sizeof(uint32_t) * (bp.n_view * bp.n_oct + 1), s);
     const int passes = key_passes(tile_bits);
     if (passes > MAX_PAIR_PASSES || !call_err || !dev_err) return cudaErrorInvalidValue;
-    launch_pdl(k_records_emit, dim3(nblk(n_vis, 256)), dim3(256), s, bp, sorted_g, sorted_key, n_vis, n_pairs, cnt,
-               rect, rec, nrm, rect_sorted, vis_start, pair_key, pair_val, pair_hist, passes, tile_cnt, lb_status,
+    launch_pdl(k_records_emit, dim3(nblk(n_vis, 256)), dim3(256), s, bp, sorted_g, sorted_key, n_vis, n_pairs, rect, rec,
+               nrm, rect_sorted, vis_start, pair_key, pair_val, pair_hist, passes, lb_status,
                ticket, call_err, dev_err, (int)(1 << 22));
     count_launches(1);
     return cudaGetLastError();
@@ -701,11 +756,9 @@ cudaError_t launch_pair_rect(const BatchParams& bp, const uint32_t* pair_key, co
     return cudaGetLastError();
 }
 
-cudaError_t launch_tile_order(const BatchParams& bp, const uint32_t* tile_cnt, int n_tiles, uint2* range,
-                              uint8_t* bucket, uint32_t* scratch192, uint32_t* order, cudaStream_t s) {
+cudaError_t launch_tile_order(const BatchParams& bp, const uint2* range, int n_tiles, uint8_t* bucket, uint32_t* scratch192, uint32_t* order, cudaStream_t s) {
     if (n_tiles <= 0) return cudaSuccess;
-    launch_pdl(k_tile_count, dim3(nblk(n_tiles, 256)), dim3(256), s, bp, tile_cnt, n_tiles, bucket, range,
-               scratch192);
+    launch_pdl(k_tile_count, dim3(nblk(n_tiles, 256)), dim3(256), s, bp, range, n_tiles, bucket, scratch192);
     count_launches(1);
     launch_pdl(k_tile_scatter, dim3(nblk(n_tiles, 256)), dim3(256), s, (const uint8_t*)bucket, n_tiles,
                (const uint32_t*)scratch192, scratch192 + TILE_BUCKETS, order);
