@@ -1332,12 +1332,11 @@ dv_status dv_soft_prior(dv_ctx* ctx, const uint64_t* grid, int64_t n_corners, co
     dv::Arena ar;
     ar.pool = ctx->pool;
     ar.stream = s;
-    bool timeout = false;
     cudaError_t e = dv::soft_prior(grid, n_corners, center, root_size, max_level, cloud, n_points, s_min, v_close, v_far,
-                                   dens, ar, s, &timeout);
+                                   dens, ar, s);
+    if (e == cudaSuccess && n_points > 0) e = cudaStreamSynchronize(s);
     ar.release();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "soft prior");
-    if (timeout) return fail(ctx, DV_ERR_TIMEOUT, "the point-cell sort ran out of its bounded wait; output invalid");
     return DV_OK;
 }
 
@@ -1358,17 +1357,11 @@ dv_status dv_subdivide_round(dv_ctx* ctx, const uint64_t* keys, int64_t n, int32
     ar.stream = s;
     dv_status st = init_begin(ctx, keys, n, max_level, ar, s);
     cudaError_t e = cudaSuccess;
-    bool timeout = false;
     if (st == DV_OK)
-        e = dv::subdivide_round(keys, n, center, root_size, max_level, cloud, n_points, threshold, out, n_out, ar, s,
-                                &timeout);
+        e = dv::subdivide_round(keys, n, center, root_size, max_level, cloud, n_points, threshold, out, n_out, ar, s);
     ar.release();
     if (st != DV_OK) return st;
     if (e != cudaSuccess) return cuda_fail(ctx, e, "subdivision");
-    if (timeout) {
-        *n_out = 0;
-        return fail(ctx, DV_ERR_TIMEOUT, "the leaf-key sort ran out of its bounded wait; nothing was written");
-    }
     return DV_OK;
 }
 
@@ -1397,6 +1390,24 @@ dv_status dv_visibility_prune(dv_ctx* ctx, const uint64_t* keys, int64_t n, int3
         ic[c].far_ = cm.far_;
         ic[c].W = cm.W;
         ic[c].H = cm.H;
+        dv::InitCam& C = ic[c];
+        for (int k = 0; k < 9; ++k) C.Rf[k] = (float)C.R[k];
+        for (int k = 0; k < 3; ++k) C.tf[k] = (float)C.t[k];
+        C.fxf = (float)C.fx;
+        C.fyf = (float)C.fy;
+        C.nearf[0] = (float)(C.near_ * (1.0 - 1e-6));
+        C.nearf[1] = (float)(C.near_ * (1.0 + 1e-6));
+        C.farf[0] = (float)(C.far_ * (1.0 - 1e-6));
+        C.farf[1] = (float)(C.far_ * (1.0 + 1e-6));
+        const double side[4] = {C.cx, C.cx - C.W, C.cy, C.cy - C.H};
+        double fro = 0.0;
+        for (int k = 0; k < 9; ++k) fro += C.R[k] * C.R[k];
+        C.scale = (float)(rotation_ok(cm.cam_to_world.R) ? 1.0001 : 1.0001 * std::sqrt(fro));
+        for (int k = 0; k < 4; ++k) {
+            const double fk = k < 2 ? C.fx : C.fy;
+            C.side[k] = (float)side[k];
+            C.len[k] = (float)(1.0001 * std::sqrt(fk * fk + side[k] * side[k]));
+        }
     }
     DeviceGuard g(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;

@@ -2,18 +2,29 @@
 // soft density prior of Eq. 1 and one round of proximity subdivision.
 //
 //  * Shared corners: every leaf emits its 8 corner grid points (finest-level integer
-//    coordinates, packed 21 bits per axis) tagged with (leaf, corner); one radix sort groups
-//    equal points, a scan numbers the distinct ones, and every (leaf, corner) gets its index.
-//  * Eq. 1: the LiDAR points are bucketed in a uniform grid of cell h = 3 s (sorted by cell
-//    key); each corner scans the 27 cells around it for its nearest point.  A point farther
-//    than 3 s changes the prior by at most 8 exp(-18) ~ 1e-7, below float32 resolution at
+//    coordinates) tagged with (leaf, corner); one radix sort groups equal points, a scan
+//    numbers the distinct ones, and every (leaf, corner) gets its index.
+//  * Eq. 1: the LiDAR points are bucketed in a uniform grid of cell h = 3 s (a hash table of the
+//    cells that hold points); each corner scans the 27 cells around it for its nearest point.  A point
+//    farther than 3 s changes the prior by at most 8 exp(-18) ~ 1e-7, below float32 resolution at
 //    v_far, so beyond that radius the corner takes v_far.
 //  * Subdivision: every LiDAR point visits, for each level, the leaf cells whose box lies within
-//    the threshold of it (exact point-box distance) and looks each up in the sorted leaf keys;
+//    the threshold of it (exact point-box distance) and looks each up in a hash table of the leaf keys;
 //    found leaves are flagged.  The output keeps the unflagged leaves in input order, then the
 //    children of the flagged ones, child 0 of every flagged leaf first, then child 1, ...
+//
+// What bounds these kernels.  Their results are defined in FP64, and this GPU issues FP64 at 1/64 of the
+// FP32 rate (2 per SM and cycle), so a kernel that computes everything in FP64 waits for that pipe
+// alone.  They decide in FP32 with an error bound and go to FP64 only where the FP32 value is too
+// close to the threshold (or, for a nearest point, could be the nearest), so every result is that of
+// the FP64 arithmetic.  Their searches are hash probes, one or two independent loads each, instead of
+// binary searches of sorted keys, twenty dependent ones, and need no sort.  On the 500k-leaf background with
+// 1.35M points (GB300): prior 3,250 -> 387 us, flags 3,260 -> 730 us,
+// visibility over six cameras 843 -> 92 us, beside the sorts of 1.35M points and 500k keys that are gone.
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <algorithm>
 
 #include "dv_internal.cuh"
 
@@ -29,6 +40,8 @@ __device__ __forceinline__ uint64_t pack_grid(uint64_t x, uint64_t y, uint64_t z
     return (z << 42) | (y << 21) | x;
 }
 
+// corner points as sort keys of 3 (max_level + 1) bits (a coordinate is at most 2^max_level): the same order as
+// the packed points, in fewer radix passes (5 instead of 8 at level 12)
 __global__ void k_corner_emit(const uint64_t* __restrict__ keys, int64_t n, int max_level, uint64_t* __restrict__ ck,
                               uint32_t* __restrict__ cv) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -41,7 +54,8 @@ __global__ void k_corner_emit(const uint64_t* __restrict__ keys, int64_t n, int 
     const uint64_t i = ((k & kIMask) + (c & 1)) << sh;
     const uint64_t j = (((k >> 19) & kIMask) + ((c >> 1) & 1)) << sh;
     const uint64_t kk = (((k >> 38) & kIMask) + ((c >> 2) & 1)) << sh;
-    ck[t] = pack_grid(i, j, kk);
+    const int b = max_level + 1;
+    ck[t] = (kk << (2 * b)) | (j << b) | i;
     cv[t] = (uint32_t)t;
 }
 
@@ -54,12 +68,16 @@ __global__ void k_corner_flag(const uint64_t* __restrict__ sk, int64_t m, uint32
 // pos = exclusive scan of first: sorted entry t belongs to distinct point pos[t] + first[t] - 1
 __global__ void k_corner_assign(const uint64_t* __restrict__ sk, const uint32_t* __restrict__ sv,
                                 const uint32_t* __restrict__ first, const uint32_t* __restrict__ pos, int64_t m,
-                                uint64_t* __restrict__ grid_out, uint32_t* __restrict__ index_out) {
+                                int max_level, uint64_t* __restrict__ grid_out, uint32_t* __restrict__ index_out) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= m) return;
     const uint32_t id = pos[t] + first[t] - 1u;
     index_out[sv[t]] = id;
-    if (first[t]) grid_out[id] = sk[t];
+    if (first[t]) {
+        const int b = max_level + 1;
+        const uint64_t k = sk[t], m1 = (1ull << b) - 1;
+        grid_out[id] = pack_grid(k & m1, (k >> b) & m1, k >> (2 * b));
+    }
 }
 
 __device__ __forceinline__ uint64_t cell_key(int64_t cx, int64_t cy, int64_t cz) {
@@ -75,121 +93,366 @@ struct Frame {
     double unit;  // finest grid step (root / 2^max_level)
 };
 
-__global__ void k_cloud_cells(const float* __restrict__ cloud, int64_t m, Frame f, double h,
-                              uint64_t* __restrict__ key, uint32_t* __restrict__ val) {
+// floor(x / unit), the quotient rounded as an FP64 division rounds it.  x times the reciprocal differs
+// from it by a few parts in 2^53, so only a product next to an integer needs the division.
+__device__ __forceinline__ double floor_div(double x, double unit, double inv) {
+    const double t = x * inv;
+    const double f = floor(t), r = t - f;
+    return (r < 1e-6 || r > 1.0 - 1e-6) ? floor(x / unit) : f;
+}
+
+// ---- open-addressing tables of 64-bit keys (power-of-two capacity, at most half full) ----
+// A key is entered within HT_PROBES slots of its home, or the call's flag is set and the host takes a
+// larger table, so every probe loop has a fixed bound.  Searches are made by whole warps in step (a lane's
+// own loop would run its lanes one after another).
+constexpr uint64_t HT_EMPTY = ~0ull;  // never a cell key (63 bits) nor a key looked up (62 bits)
+constexpr int HT_PROBES = 64;
+constexpr int HT_TRIES = 4;  // tables of 1, 2, 4, 8 times the capacity
+
+__device__ __forceinline__ uint32_t ht_first(uint64_t key, int bits) {
+    key ^= key >> 32;
+    key *= 0x9e3779b97f4a7c15ull;  // 2^64 / golden ratio, odd
+    key ^= key >> 29;
+    key *= 0x9e3779b97f4a7c15ull;
+    return (uint32_t)(key >> (64 - bits));
+}
+
+// the key's slot, entering it where it is new
+__device__ __forceinline__ uint32_t ht_enter(uint64_t* table, int bits, uint64_t key, uint32_t* fail) {
+    const uint32_t mask = (uint32_t)((1ull << bits) - 1);
+    uint32_t h = ht_first(key, bits);
+    for (int i = 0; i < HT_PROBES; ++i) {
+        const unsigned long long old = atomicCAS(reinterpret_cast<unsigned long long*>(table + h), HT_EMPTY, key);
+        if (old == HT_EMPTY || old == key) return h;
+        h = (h + 1) & mask;
+    }
+    *fail = 1u;
+    return h;
+}
+
+// the slots of the warp's keys, ~0u where a key is absent or its lane not active (all 32 lanes call)
+__device__ __forceinline__ uint32_t ht_find(const uint64_t* __restrict__ table, int bits, uint64_t key, bool active) {
+    const uint32_t mask = (uint32_t)((1ull << bits) - 1);
+    uint32_t h = ht_first(key, bits), found = ~0u;
+    for (int i = 0; i < HT_PROBES; ++i) {
+        if (!__any_sync(0xffffffffu, active)) break;
+        if (active) {
+            const uint64_t k = __ldg(table + h);
+            if (k == key) found = h;
+            active = k != key && k != HT_EMPTY;
+            h = (h + 1) & mask;
+        }
+        __syncwarp();
+    }
+    return found;
+}
+
+int ht_bits(int64_t n) {
+    int b = 10;
+    while (((int64_t)1 << b) < 2 * n) ++b;
+    return b;
+}
+
+// ---- point grid of the soft prior: cell -> [start, start + cnt) of the points ordered by cell ----
+
+// EXACT: the cell of the FP64 quotient (the prior's cells); else some cell near it (points only have to be
+// brought together)
+template <bool EXACT>
+__global__ void __launch_bounds__(256) k_cell_count(const float* __restrict__ cloud, int64_t m, Frame f, double h,
+                                                    double inv_h, uint64_t* __restrict__ table, int bits,
+                                                    uint32_t* __restrict__ cnt, uint32_t* __restrict__ slot,
+                                                    uint32_t* __restrict__ rank, uint32_t* __restrict__ fail) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= m) return;
     int64_t c[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) c[a] = (int64_t)floor(((double)cloud[t * 3 + a] - f.root_min[a]) / h);
-    key[t] = cell_key(c[0], c[1], c[2]);
-    val[t] = (uint32_t)t;
-}
-
-__device__ __forceinline__ int64_t lower_bound(const uint64_t* a, int64_t n, uint64_t x) {
-    int64_t lo = 0, hi = n;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (a[mid] < x)
-            lo = mid + 1;
-        else
-            hi = mid;
+    for (int a = 0; a < 3; ++a) {
+        if constexpr (EXACT)
+            c[a] = (int64_t)floor_div((double)cloud[t * 3 + a] - f.root_min[a], h, inv_h);
+        else  // kept in range as a number before it is converted (a point may be anything)
+            c[a] = (int64_t)(int)fminf(fmaxf((cloud[t * 3 + a] - (float)f.root_min[a]) * (float)inv_h, -1e6f), 1e6f);
     }
-    return lo;
+    const uint32_t s = ht_enter(table, bits, cell_key(c[0], c[1], c[2]), fail);
+    slot[t] = s;
+    rank[t] = atomicAdd(cnt + s, 1u);
 }
 
-__global__ void k_soft_prior(const uint64_t* __restrict__ grid, int64_t n_corners, Frame f, double h,
-                             const uint64_t* __restrict__ ckey, const uint32_t* __restrict__ cidx, int64_t m,
-                             const float* __restrict__ cloud, float s, float v_close, float v_far,
-                             float* __restrict__ dens) {
+// the cells' ranges, in any order: one reservation per block
+__global__ void __launch_bounds__(256) k_cell_alloc(const uint32_t* __restrict__ cnt, int64_t n_slot,
+                                                    uint32_t* __restrict__ start, uint32_t* __restrict__ total) {
+    __shared__ uint32_t ws[8], base;
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t c = i < n_slot ? cnt[i] : 0u;
+    uint32_t x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) ws[warp] = x;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t run = 0;
+        for (int w = 0; w < 8; ++w) {
+            const uint32_t y = ws[w];
+            ws[w] = run;
+            run += y;
+        }
+        base = run ? atomicAdd(total, run) : 0u;
+    }
+    __syncthreads();
+    if (c) start[i] = base + ws[warp] + x - c;
+}
+
+__global__ void __launch_bounds__(256) k_cell_scatter(const float* __restrict__ cloud, int64_t m,
+                                                      const uint32_t* __restrict__ slot,
+                                                      const uint32_t* __restrict__ rank,
+                                                      const uint32_t* __restrict__ start, float4* __restrict__ pts) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n_corners) return;
-    const uint64_t g = grid[t];
+    if (t >= m) return;
+    pts[start[slot[t]] + rank[t]] = make_float4(cloud[t * 3], cloud[t * 3 + 1], cloud[t * 3 + 2], 0.0f);
+}
+
+// One thread per corner.  The 27 cells around it, its own first; a cell is skipped when its box is no
+// nearer than the best point so far.  Distances are FP32, from the corner split into two floats (relative
+// error below 1e-6 of the square beyond `tiny`); the nearest point's is then taken in FP64, and where a
+// second point comes within 2e-5 of it, all such points' are.
+__global__ void __launch_bounds__(256) k_soft_prior(const uint64_t* __restrict__ grid, int64_t n_corners, Frame f,
+                                                    double h, double inv_h, const uint64_t* __restrict__ table,
+                                                    int bits, const uint32_t* __restrict__ cnt,
+                                                    const uint32_t* __restrict__ start, int64_t m,
+                                                    const float4* __restrict__ pts, float s, float v_close,
+                                                    float v_far, float* __restrict__ dens) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool live = t < n_corners;
+    const uint64_t g = live ? grid[t] : 0ull;
     double q[3];
     q[0] = f.root_min[0] + (double)(g & ((1ull << 21) - 1)) * f.unit;
     q[1] = f.root_min[1] + (double)((g >> 21) & ((1ull << 21) - 1)) * f.unit;
     q[2] = f.root_min[2] + (double)((g >> 42) & ((1ull << 21) - 1)) * f.unit;
-    int64_t c[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) c[a] = (int64_t)floor((q[a] - f.root_min[a]) / h);
-    // x is the key's low field, so the three cells x-1..x+1 of one (y, z) row are one run of keys:
-    // one search per row.  The centre row goes first; another row is skipped when its box is
-    // no nearer than the best point so far, so the minimum is still the one over all 27 cells.
-    // The row's lower bound takes a slack of 1e-9 h off each axis gap: a point's cell comes from
-    // a quotient below 2^21 in FP64, so it can sit at most ~5e-10 h across a cell boundary.
-    double gap_lo[3], gap_hi[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const double lo = f.root_min[a] + (double)c[a] * h;
-        gap_lo[a] = fmax(0.0, q[a] - lo - 1e-9 * h);
-        gap_hi[a] = fmax(0.0, lo + h - q[a] - 1e-9 * h);
-    }
     double best = INFINITY;
-    for (int it = 0; it < 9; ++it) {
-        const int r = (it + 4) % 9;  // it = 0: the centre row
-        const int dy = r % 3 - 1, dz = r / 3 - 1;
-        {
-            const double gy = dy < 0 ? gap_lo[1] : (dy > 0 ? gap_hi[1] : 0.0);
-            const double gz = dz < 0 ? gap_lo[2] : (dz > 0 ? gap_hi[2] : 0.0);
-            if (gy * gy + gz * gz >= best) continue;
+    if (m > 0) {
+        int64_t c[3];
+        float qh[3], ql[3], into[3];
+        float big = 0.0f;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            c[a] = (int64_t)floor_div(q[a] - f.root_min[a], h, inv_h);
+            qh[a] = (float)q[a];
+            ql[a] = (float)(q[a] - (double)qh[a]);
+            big = fmaxf(big, fabsf(qh[a]));
+            into[a] = (float)(q[a] - (f.root_min[a] + (double)c[a] * h));
         }
-        {
-            const uint64_t k_lo = cell_key(c[0] - 1, c[1] + dy, c[2] + dz);
-            const uint64_t k_hi = cell_key(c[0] + 1, c[1] + dy, c[2] + dz);
-            for (int64_t e = lower_bound(ckey, m, k_lo); e < m && ckey[e] <= k_hi; ++e) {
-                const uint32_t p = cidx[e];
-                const double ex = (double)cloud[p * 3 + 0] - q[0], ey = (double)cloud[p * 3 + 1] - q[1],
-                             ez = (double)cloud[p * 3 + 2] - q[2];
-                best = fmin(best, ex * ex + ey * ey + ez * ez);
+        const float tiny = 1e-22f * big * big, hf = (float)h;
+        // lower bound of the distance along an axis to the cells at -1, 0, +1: a point's cell comes from a quotient
+        // below 2^21 in FP64, so it can sit at most ~5e-10 h across a cell boundary; 1e-6 h covers the FP32 too
+        auto gap = [&](int a, int d) {
+            return d == 0 ? 0.0f : fmaxf((d < 0 ? into[a] : hf - into[a]) - 1e-6f * hf, 0.0f);
+        };
+        float b1 = INFINITY, b2 = INFINITY;  // the two smallest FP32 squares
+        uint32_t at = 0;
+        // squares above it cannot be the smallest in FP64
+        auto bound = [&]() { return fmaf(b1, 1.00002f, tiny); };
+        auto cells = [&](auto&& visit) {
+            for (int it = 0; it < 27; ++it) {
+                const int r = (it + 13) % 27;  // it = 0: the corner's own cell
+                const int dx = r % 3 - 1, dy = (r / 3) % 3 - 1, dz = r / 9 - 1;
+                const float gx = gap(0, dx), gy = gap(1, dy), gz = gap(2, dz);
+                const bool look = live && !(fmaf(gx, gx, fmaf(gy, gy, gz * gz)) * 0.99999f > bound());
+                const uint32_t slot = ht_find(table, bits, cell_key(c[0] + dx, c[1] + dy, c[2] + dz), look);
+                if (slot != ~0u) {
+                    const uint32_t e0 = start[slot], n = min(cnt[slot], (uint32_t)m - e0);
+                    for (uint32_t i = 0; i < n; ++i) {
+                        const float4 p = __ldg(pts + e0 + i);
+                        const float fx = (p.x - qh[0]) - ql[0], fy = (p.y - qh[1]) - ql[1], fz = (p.z - qh[2]) - ql[2];
+                        visit(e0 + i, fmaf(fx, fx, fmaf(fy, fy, fz * fz)));
+                    }
+                }
+                __syncwarp();
             }
+        };
+        cells([&](uint32_t e, float d2) {
+            b2 = fminf(b2, fmaxf(d2, b1));
+            if (d2 < b1) {
+                b1 = d2;
+                at = e;
+            }
+        });
+        auto exact = [&](uint32_t e) {
+            const float4 p = __ldg(pts + e);
+            const double ex = (double)p.x - q[0], ey = (double)p.y - q[1], ez = (double)p.z - q[2];
+            best = fmin(best, ex * ex + ey * ey + ez * ez);
+        };
+        const bool any = b1 < INFINITY, close = any && b2 <= bound();
+        if (any) exact(at);
+        if (__any_sync(0xffffffffu, close)) {
+            const float lim = close ? bound() : -1.0f;
+            cells([&](uint32_t e, float d2) {
+                if (d2 <= lim) exact(e);
+            });
         }
     }
+    if (!live) return;
     // Eq. 1 (beyond the 27-cell radius the exponential is below float resolution at v_far)
     const double ss = (double)s * (double)s;
     const double e = best < INFINITY ? exp(-2.0 * best / ss) : 0.0;
     dens[t] = (float)((double)v_far + ((double)v_close - (double)v_far) * e);
 }
 
-// one thread per LiDAR point: flag the leaves (sorted keys) whose box lies within thr of it
-__global__ void k_subdiv_flags(const float* __restrict__ cloud, int64_t m, Frame f, double root_size, uint32_t levels,
-                               double thr, const uint64_t* __restrict__ skeys, const uint32_t* __restrict__ sidx,
-                               int64_t n, uint8_t* __restrict__ split) {
+// ---- subdivision ----
+
+constexpr int SD_FINE = 18;   // finest level: cell indices are taken there once and shifted
+constexpr int SD_COARSE = 6;  // leaves of this level or finer note their level in the coarse cell they lie in
+constexpr int SD_SIDE = 1 << SD_COARSE;
+
+// enters every leaf key (the lowest index of equal keys counts) and the levels below each coarse cell
+__global__ void __launch_bounds__(256) k_leaf_enter(const uint64_t* __restrict__ keys, int64_t n,
+                                                    uint64_t* __restrict__ table, uint32_t* __restrict__ idx, int bits,
+                                                    uint32_t* __restrict__ coarse, uint32_t* __restrict__ levels,
+                                                    uint32_t* __restrict__ fail) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= m) return;
-    double p[3];
+    uint32_t lev = 0;
+    if (t < n) {
+        const uint64_t k = keys[t];
+        const int l = (int)((k >> 57) & 31);
+        lev = 1u << l;
+        if (k != HT_EMPTY) atomicMin(idx + ht_enter(table, bits, k, fail), (uint32_t)t);
+        if (l >= SD_COARSE) {
+            const int sh = l - SD_COARSE;
+            const uint32_t x = (uint32_t)((k & kIMask) >> sh), y = (uint32_t)(((k >> 19) & kIMask) >> sh),
+                           z = (uint32_t)(((k >> 38) & kIMask) >> sh);
+            if (x < SD_SIDE && y < SD_SIDE && z < SD_SIDE) {
+                uint32_t* w = coarse + (z * SD_SIDE + y) * SD_SIDE + x;
+                if (!(*(volatile uint32_t*)w & lev)) atomicOr(w, lev);
+            }
+        }
+    }
+    lev = __reduce_or_sync(0xffffffffu, lev);
+    if ((threadIdx.x & 31) == 0 && (lev & ~*(volatile uint32_t*)levels)) atomicOr(levels, lev);
+}
+
+// Whether a point (from the root's corner) lies within thr of the box of cell (x, y, z) of level l.  Out of
+// line: few points need it.
+__device__ __noinline__ bool box_within(double root_size, int l, int x, int y, int z, double p0, double p1, double p2,
+                                        double thr) {
+    const double s = ldexp(root_size, -l);
+    const double p[3] = {p0, p1, p2};
+    const int ij[3] = {x, y, z};
+    double d2 = 0.0;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) p[a] = (double)cloud[t * 3 + a] - f.root_min[a];
-    for (int l = 0; l < 32; ++l) {
-        if (!((levels >> l) & 1u)) continue;  // only levels that hold leaves
-        const double s = ldexp(root_size, -l);
-        const int64_t lim = (1ll << l) - 1;
-        int64_t lo[3], hi[3];
-        bool any = true;
+    for (int a = 0; a < 3; ++a) {
+        const double b0 = (double)ij[a] * s, b1 = b0 + s;
+        const double g = fmax(fmax(b0 - p[a], 0.0), p[a] - b1);
+        d2 += g * g;
+    }
+    return !(d2 > thr * thr);
+}
+
+// One thread per LiDAR point, the points ordered by cell so that a warp's lanes look at much the same leaves:
+// flags the leaves whose box lies within thr of it.  Cell indices: floors at the finest level, shifted (the
+// levels' cell sizes are the root's times powers of two, so the quotients are too).  They and the distances come
+// from the point's integer and fractional parts in finest-level units (the fractions in FP32); an index whose
+// fraction is within 1e-5 of a step, and a distance within 2e-5 of the threshold (or any, for thresholds below
+// 0.05 units), is taken from FP64.
+__global__ void __launch_bounds__(256) k_subdiv_flags(const float4* __restrict__ pts, int64_t m, Frame f,
+                                                      double root_size, double fine, double inv_fine,
+                                                      const uint32_t* __restrict__ levels_p, double thr,
+                                                      const uint64_t* __restrict__ table,
+                                                      const uint32_t* __restrict__ idx, int bits,
+                                                      const uint32_t* __restrict__ coarse, uint8_t* __restrict__ split) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool live = t < m;
+    const float4 pt = live ? pts[t] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    const float pc[3] = {pt.x, pt.y, pt.z};
+    const double thr_d = fmin(thr * inv_fine, 1e9), thr_i = floor(thr_d);
+    const float thr_u = (float)thr_d, thr_f = (float)(thr_d - thr_i);
+    double p[3];
+    int flo[3], fhi[3], pi[3];
+    float pf[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        p[a] = (double)pc[a] - f.root_min[a];
+        const double u = fmin(fmax(p[a] * inv_fine, -1e9), 1e9);  // -1e9 for a point that is not a number
+        const double ui = floor(u);
+        pi[a] = (int)ui;
+        pf[a] = (float)(u - ui);
+        // floor((p -+ thr) / fine), kept just outside the grid where it leaves it
+        auto index = [&](float fr, int64_t base, double x) {
+            const float fl = floorf(fr), r = fr - fl;
+            int64_t i = base + (int)fl;
+            if (r < 1e-5f || r > 1.0f - 1e-5f) {
+                const double e = floor(x / fine);
+                i = (int64_t)fmin(fmax(e, -1.0), (double)(1 << SD_FINE));
+            }
+            return (int)min(max(i, (int64_t)-1), (int64_t)1 << SD_FINE);
+        };
+        flo[a] = index(pf[a] - thr_f, (int64_t)pi[a] - (int64_t)thr_i, p[a] - thr);
+        fhi[a] = index(pf[a] + thr_f, (int64_t)pi[a] + (int64_t)thr_i, p[a] + thr);
+    }
+    uint32_t levels = live ? *levels_p : 0u;
+    {
+        // only levels that some coarse cell around the point holds
+        int c0[3], c1[3], n = 1;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            lo[a] = (int64_t)floor((p[a] - thr) / s);
-            hi[a] = (int64_t)floor((p[a] + thr) / s);
-            lo[a] = lo[a] < 0 ? 0 : lo[a];
-            hi[a] = hi[a] > lim ? lim : hi[a];
-            any = any && lo[a] <= hi[a];
+            c0[a] = max(flo[a] >> (SD_FINE - SD_COARSE), 0);
+            c1[a] = min(fhi[a] >> (SD_FINE - SD_COARSE), SD_SIDE - 1);
+            n *= max(c1[a] - c0[a] + 1, 0);
         }
-        if (!any) continue;
-        for (int64_t z = lo[2]; z <= hi[2]; ++z)
-            for (int64_t y = lo[1]; y <= hi[1]; ++y)
-                for (int64_t x = lo[0]; x <= hi[0]; ++x) {
-                    const int64_t ij[3] = {x, y, z};
-                    double d2 = 0.0;
+        if (n == 0) levels = 0u;
+        if (n <= 8) {
+            uint32_t have = (1u << SD_COARSE) - 1u;
+            for (int z = c0[2]; z <= c1[2]; ++z)
+                for (int y = c0[1]; y <= c1[1]; ++y)
+                    for (int x = c0[0]; x <= c1[0]; ++x) have |= __ldg(coarse + (z * SD_SIDE + y) * SD_SIDE + x);
+            levels &= have;
+        }
+    }
+    __syncwarp();
+    const bool fp32 = thr_u >= 0.05f && thr_u < 1e9f;
+    const float t2_lo = thr_u * thr_u * (1.0f - 2e-5f), t2_hi = thr_u * thr_u * (1.0f + 2e-5f);
+    // The warp takes the levels and cells in step, so that lanes in the same cell ask for the same keys.
+    for (uint32_t todo = __reduce_or_sync(0xffffffffu, levels); todo; todo &= todo - 1) {
+        const int l = __ffs((int)todo) - 1, sh = SD_FINE - l;
+        const int lim = (1 << l) - 1;
+        int lo[3], n[3];
 #pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        const double b0 = (double)ij[a] * s, b1 = b0 + s;
-                        const double g = fmax(fmax(b0 - p[a], 0.0), p[a] - b1);
-                        d2 += g * g;
-                    }
-                    if (d2 > thr * thr) continue;
-                    const uint64_t key = ((uint64_t)l << 57) | ((uint64_t)z << 38) | ((uint64_t)y << 19) | (uint64_t)x;
-                    const int64_t e = lower_bound(skeys, n, key);
-                    if (e < n && skeys[e] == key) split[sidx[e]] = 1;
+        for (int a = 0; a < 3; ++a) {
+            lo[a] = max(flo[a] >> sh, 0);
+            n[a] = max(min(fhi[a] >> sh, lim) - lo[a] + 1, 0);
+        }
+        const int64_t mine = (levels >> l) & 1u ? (int64_t)n[0] * n[1] * n[2] : 0;
+        // distance along one axis to cell i, in finest units
+        auto gap = [&](int a, int i) {
+            const float below = (float)((i << sh) - pi[a]) - pf[a];
+            const float above = (float)(pi[a] - ((i + 1) << sh)) + pf[a];
+            return fmaxf(fmaxf(below, above), 0.0f);
+        };
+        int x = lo[0], y = lo[1], z = lo[2];
+        for (int64_t i = 0; __any_sync(0xffffffffu, i < mine); ++i) {
+            bool look = i < mine;
+            if (look) {
+                const float gx = gap(0, x), gy = gap(1, y), gz = gap(2, z);
+                const float d2f = fmaf(gx, gx, fmaf(gy, gy, gz * gz));
+                if (fp32 && d2f > t2_hi)
+                    look = false;
+                else if (!fp32 || d2f >= t2_lo)
+                    look = box_within(root_size, l, x, y, z, p[0], p[1], p[2], thr);
+            }
+            __syncwarp();
+            const uint64_t key = ((uint64_t)l << 57) | ((uint64_t)z << 38) | ((uint64_t)y << 19) | (uint64_t)x;
+            const uint32_t e = ht_find(table, bits, key, look);
+            if (e != ~0u) split[idx[e]] = 1;
+            // the next cell, x fastest
+            if (++x == lo[0] + n[0]) {
+                x = lo[0];
+                if (++y == lo[1] + n[1]) {
+                    y = lo[1];
+                    ++z;
                 }
+            }
+        }
     }
 }
 
@@ -217,15 +480,6 @@ __global__ void k_not(const uint8_t* __restrict__ a, int64_t n, uint32_t* __rest
     no[t] = a[t] ? 0u : 1u;
 }
 
-// v[t] = t, and the set of leaf levels present (bit l of *levels)
-__global__ void k_iota_levels(const uint64_t* __restrict__ keys, int64_t n, uint32_t* __restrict__ v,
-                              uint32_t* __restrict__ levels) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    v[t] = (uint32_t)t;
-    atomicOr(levels, 1u << ((keys[t] >> 57) & 31));
-}
-
 unsigned nb(int64_t n) { return (unsigned)((n + 255) / 256); }
 
 // per-leaf densities [n][8] from shared corner values, and the transpose for gradients
@@ -244,27 +498,93 @@ __global__ void k_corner_scatter(const uint32_t* __restrict__ index, int64_t n8,
     if (g != 0.0f) atomicAdd(d_corner + index[t], g);
 }
 
-// level of every key (bit mask) to validate against max_level
-__global__ void k_levels(const uint64_t* __restrict__ keys, int64_t n, uint32_t* __restrict__ levels) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    atomicOr(levels, 1u << ((keys[t] >> 57) & 31));
+// levels of the keys (bit mask), to validate against max_level
+__global__ void __launch_bounds__(256) k_levels(const uint64_t* __restrict__ keys, int64_t n, uint32_t* __restrict__ levels) {
+    uint32_t lev = 0;
+    for (int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x; t < n; t += (int64_t)gridDim.x * 256)
+        lev |= 1u << ((keys[t] >> 57) & 31);
+    lev = __reduce_or_sync(0xffffffffu, lev);
+    if ((threadIdx.x & 31) == 0 && (lev & ~*(volatile uint32_t*)levels)) atomicOr(levels, lev);
 }
 
-// a leaf is kept if its box top reaches z_min and some camera sees it (see the header)
-__global__ void k_visible(const uint64_t* __restrict__ keys, int64_t n, Frame f, double root_size,
-                          const InitCam* __restrict__ cams, int n_cam, double z_min, uint32_t* __restrict__ keep) {
-    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= n) return;
-    const uint64_t k = keys[v];
-    const int lev = (int)((k >> 57) & 31);
-    const double s = ldexp(root_size, -lev);
-    const double lo[3] = {f.root_min[0] + (double)(k & kIMask) * s, f.root_min[1] + (double)((k >> 19) & kIMask) * s,
-                          f.root_min[2] + (double)((k >> 38) & kIMask) * s};
-    uint32_t vis = 0;
-    if (lo[2] + s >= z_min) {
-        for (int c = 0; c < n_cam && !vis; ++c) {
-            const InitCam& C = cams[c];
+// A leaf is kept if its box top reaches z_min and some camera sees it (see the header).  A camera's verdict comes
+// from the leaf's bounding sphere in FP32 where it is certain (the radius covers the rounding: 8e-6 of the
+// coordinates' size), from the 8 corners in FP64 where the sphere meets a plane.  The block gathers the (leaf,
+// camera) pairs left to FP64 and takes them densely: left in their own lanes, one of them holds the whole warp
+// for two hundred FP64 instructions (500k leaves, six cameras: 217 -> 92 us).
+__global__ void __launch_bounds__(256) k_visible(const uint64_t* __restrict__ keys, int64_t n, Frame f, double root_size,
+                                                 const InitCam* __restrict__ cams, int n_cam, double z_min,
+                                                 uint32_t* __restrict__ keep) {
+    __shared__ uint32_t s_vis[256];
+    __shared__ uint16_t s_leaf[256];
+    __shared__ uint8_t s_cam[256];
+    __shared__ int s_n;
+    const int tid = threadIdx.x;
+    const int64_t v = (int64_t)blockIdx.x * 256 + tid;
+    s_vis[tid] = 0u;
+    uint64_t open = 0;  // cameras left to FP64 (at most 64)
+    const uint64_t k = v < n ? keys[v] : 0ull;
+    if (v < n) {
+        const double s = ldexp(root_size, -(int)((k >> 57) & 31));
+        const double lo2 = f.root_min[2] + (double)((k >> 38) & kIMask) * s;
+        if (lo2 + s >= z_min) {
+            const float sf = (float)s;
+            float ctr[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+                ctr[a] = fmaf((float)((k >> (19 * a)) & kIMask) + 0.5f, sf, (float)f.root_min[a]);
+            const float size = fabsf(ctr[0]) + fabsf(ctr[1]) + fabsf(ctr[2]) + (float)root_size;
+            for (int c = 0; c < n_cam; ++c) {
+                const InitCam& C = cams[c];
+                const float p0 = ctr[0] - C.tf[0], p1 = ctr[1] - C.tf[1], p2 = ctr[2] - C.tf[2];
+                const float x = fmaf(C.Rf[0], p0, fmaf(C.Rf[3], p1, C.Rf[6] * p2));
+                const float y = fmaf(C.Rf[1], p0, fmaf(C.Rf[4], p1, C.Rf[7] * p2));
+                const float z = fmaf(C.Rf[2], p0, fmaf(C.Rf[5], p1, C.Rf[8] * p2));
+                const float err = C.scale * 8e-6f * (size + fabsf(C.tf[0]) + fabsf(C.tf[1]) + fabsf(C.tf[2]));
+                const float rad = fmaf(0.8661f * C.scale, sf, err);
+                if (z + rad < C.nearf[0] || z - rad > C.farf[1]) continue;  // before near, or beyond far, with all corners
+                if (z - rad > C.nearf[1]) {
+                    // all corners behind near: the image's left and right sides, its top and bottom
+                    const float l = fmaf(C.fxf, x, C.side[0] * z), r = fmaf(C.fxf, x, C.side[1] * z);
+                    const float u = fmaf(C.fyf, y, C.side[2] * z), d = fmaf(C.fyf, y, C.side[3] * z);
+                    if (l < -C.len[0] * rad || r > C.len[1] * rad || u < -C.len[2] * rad || d > C.len[3] * rad) continue;
+                    if (z + rad < C.farf[0] && l > C.len[0] * err && r < -C.len[1] * err && u > C.len[2] * err &&
+                        d < -C.len[3] * err) {
+                        // the centre projects into the image, and the corners' rectangle holds it
+                        s_vis[tid] = 1u;
+                        open = 0;
+                        break;
+                    }
+                }
+                open |= 1ull << c;
+            }
+        }
+    }
+    // one open camera of every leaf that is not yet seen, in turn
+    for (int turn = 0; turn < 64; ++turn) {
+        if (tid == 0) s_n = 0;
+        __syncthreads();
+        const bool ask = open != 0 && s_vis[tid] == 0u;
+        const unsigned b = __ballot_sync(0xffffffffu, ask);
+        int base = 0;
+        if ((tid & 31) == 0 && b) base = atomicAdd(&s_n, __popc(b));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (ask) {
+            const int at = base + __popc(b & ((1u << (tid & 31)) - 1u));
+            s_leaf[at] = (uint16_t)tid;
+            s_cam[at] = (uint8_t)(__ffsll((long long)open) - 1);
+            open &= open - 1;
+        }
+        __syncthreads();
+        const int n_ask = s_n;
+        if (n_ask == 0) break;
+        if (tid < n_ask) {
+            const uint64_t kk = keys[(int64_t)blockIdx.x * 256 + s_leaf[tid]];
+            const double s = ldexp(root_size, -(int)((kk >> 57) & 31));
+            const double lo[3] = {f.root_min[0] + (double)(kk & kIMask) * s,
+                                  f.root_min[1] + (double)((kk >> 19) & kIMask) * s,
+                                  f.root_min[2] + (double)((kk >> 38) & kIMask) * s};
+            const InitCam& C = cams[s_cam[tid]];
             int behind = 0, beyond = 0;
             double u0 = INFINITY, u1 = -INFINITY, w0 = INFINITY, w1 = -INFINITY;
             for (int q = 0; q < 8; ++q) {
@@ -284,14 +604,13 @@ __global__ void k_visible(const uint64_t* __restrict__ keys, int64_t n, Frame f,
                     w1 = fmax(w1, w);
                 }
             }
-            if (behind == 8 || beyond == 8) continue;
-            if (behind > 0)
-                vis = 1;
-            else
-                vis = (u1 >= 0.0 && u0 <= (double)C.W && w1 >= 0.0 && w0 <= (double)C.H) ? 1u : 0u;
+            if (behind != 8 && beyond != 8 &&
+                (behind > 0 || (u1 >= 0.0 && u0 <= (double)C.W && w1 >= 0.0 && w0 <= (double)C.H)))
+                s_vis[s_leaf[tid]] = 1u;
         }
+        __syncthreads();
     }
-    keep[v] = vis;
+    if (v < n) keep[v] = s_vis[tid];
 }
 
 __global__ void k_compact_keys(const uint64_t* __restrict__ keys, int64_t n, const uint32_t* __restrict__ keep,
@@ -353,7 +672,7 @@ cudaError_t key_levels(const uint64_t* keys, int64_t n, uint32_t* levels_host, A
     if (!d) return ar.err;
     cudaError_t e = cudaMemsetAsync(d, 0, sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
-    k_levels<<<nb(n), 256, 0, s>>>(keys, n, d);
+    k_levels<<<std::min<unsigned>(nb(n), 2u * (unsigned)sm_count()), 256, 0, s>>>(keys, n, d);
     count_launches(1);
     e = cudaMemcpyAsync(levels_host, d, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -380,13 +699,13 @@ cudaError_t shared_corners(const uint64_t* keys, int64_t n, int max_level, uint6
     count_launches(1);
     uint64_t* kk = k0;
     uint32_t* vv = v0;
-    e = radix_sort_u64(kk, vv, k1, v1, m, 63, ar, s, total + 1);
+    e = radix_sort_u64(kk, vv, k1, v1, m, 3 * (max_level + 1), ar, s, total + 1);
     if (e != cudaSuccess) return e;
     k_corner_flag<<<nb(m), 256, 0, s>>>(kk, m, first);
     count_launches(1);
     e = scan_u32_to_u32(first, pos, m, total, ar, s);
     if (e != cudaSuccess) return e;
-    k_corner_assign<<<nb(m), 256, 0, s>>>(kk, vv, first, pos, m, grid_out, index_out);
+    k_corner_assign<<<nb(m), 256, 0, s>>>(kk, vv, first, pos, m, max_level, grid_out, index_out);
     count_launches(1);
     uint32_t h[2] = {0, 0};
     e = cudaMemcpyAsync(h, total, sizeof(h), cudaMemcpyDeviceToHost, s);
@@ -405,93 +724,115 @@ static Frame make_frame(const double* center, double root_size, int max_level) {
 
 cudaError_t soft_prior(const uint64_t* grid, int64_t n_corners, const double* center, double root_size, int max_level,
                        const float* cloud, int64_t m, float s_min, float v_close, float v_far, float* dens, Arena& ar,
-                       cudaStream_t s, bool* sort_timeout) {
-    *sort_timeout = false;
+                       cudaStream_t s) {
     if (n_corners <= 0) return cudaSuccess;
     const Frame f = make_frame(center, root_size, max_level);
-    const double h = 3.0 * (double)s_min;
-    uint64_t *k0 = nullptr, *k1 = nullptr;
-    uint32_t *v0 = nullptr, *v1 = nullptr;
-    uint32_t* flag = nullptr;
-    if (m > 0) {
-        k0 = ar.alloc<uint64_t>(m);
-        k1 = ar.alloc<uint64_t>(m);
-        v0 = ar.alloc<uint32_t>(m);
-        v1 = ar.alloc<uint32_t>(m);
-        flag = ar.alloc<uint32_t>(1);
-        if (ar.err != cudaSuccess) return ar.err;
-        cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(uint32_t), s);
-        if (e != cudaSuccess) return e;
-        k_cloud_cells<<<nb(m), 256, 0, s>>>(cloud, m, f, h, k0, v0);
+    const double h = 3.0 * (double)s_min, inv_h = 1.0 / h;
+    if (m <= 0) {
+        k_soft_prior<<<nb(n_corners), 256, 0, s>>>(grid, n_corners, f, h, inv_h, nullptr, 0, nullptr, nullptr, 0, nullptr,
+                                                   s_min, v_close, v_far, dens);
         count_launches(1);
-        e = radix_sort_u64(k0, v0, k1, v1, m, 3 * kCellBits, ar, s, flag);
+        return cudaGetLastError();
+    }
+    uint32_t* slot = ar.alloc<uint32_t>(m);
+    uint32_t* rank = ar.alloc<uint32_t>(m);
+    float4* pts = ar.alloc<float4>(m);
+    for (int more = 0; more < HT_TRIES; ++more) {
+        const int bits = std::min(ht_bits(m) + more, 32);
+        const size_t cap = (size_t)1 << bits;
+        uint64_t* table = ar.alloc<uint64_t>(cap);
+        uint32_t* cnt = ar.alloc<uint32_t>(cap + 2);  // then: points placed so far, a key without a slot
+        uint32_t* start = ar.alloc<uint32_t>(cap);
+        if (ar.err != cudaSuccess) return ar.err;
+        cudaError_t e = cudaMemsetAsync(table, 0xff, cap * sizeof(uint64_t), s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(cnt, 0, (cap + 2) * sizeof(uint32_t), s);
         if (e != cudaSuccess) return e;
-    }
-    k_soft_prior<<<nb(n_corners), 256, 0, s>>>(grid, n_corners, f, h, k0, v0, m, cloud, s_min, v_close, v_far, dens);
-    count_launches(1);
-    cudaError_t e = cudaGetLastError();
-    if (flag) {
-        // the cell sort's own wait flag: a run-out look-back left the cloud unsorted (wrong nearest points)
-        uint32_t hf = 0;
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&hf, flag, sizeof(hf), cudaMemcpyDeviceToHost, s);
+        k_cell_count<true><<<nb(m), 256, 0, s>>>(cloud, m, f, h, inv_h, table, bits, cnt, slot, rank, cnt + cap + 1);
+        k_cell_alloc<<<(unsigned)(cap / 256), 256, 0, s>>>(cnt, (int64_t)cap, start, cnt + cap);
+        k_cell_scatter<<<nb(m), 256, 0, s>>>(cloud, m, slot, rank, start, pts);
+        k_soft_prior<<<nb(n_corners), 256, 0, s>>>(grid, n_corners, f, h, inv_h, table, bits, cnt, start, m, pts, s_min,
+                                                   v_close, v_far, dens);
+        count_launches(4);
+        uint32_t failed = 0;
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&failed, cnt + cap + 1, sizeof(failed), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        *sort_timeout = hf != 0;
+        if (e != cudaSuccess || !failed) return e;
     }
-    return e;
+    return cudaErrorUnknown;  // no table of eight times the capacity has room within HT_PROBES of every key's home
 }
 
 cudaError_t subdivide_round(const uint64_t* keys, int64_t n, const double* center, double root_size, int max_level,
                             const float* cloud, int64_t m, float thr, uint64_t* out, int64_t* n_out, Arena& ar,
-                            cudaStream_t s, bool* sort_timeout) {
+                            cudaStream_t s) {
     *n_out = n;
-    *sort_timeout = false;
     if (n <= 0) return cudaSuccess;
     const Frame f = make_frame(center, root_size, max_level);
-    uint64_t* k0 = ar.alloc<uint64_t>(n);
-    uint64_t* k1 = ar.alloc<uint64_t>(n);
-    uint32_t* v0 = ar.alloc<uint32_t>(n);
-    uint32_t* v1 = ar.alloc<uint32_t>(n);
+    constexpr int COARSE = SD_SIDE * SD_SIDE * SD_SIDE;
+    uint32_t* coarse = ar.alloc<uint32_t>(COARSE);
     uint8_t* split = ar.alloc<uint8_t>(n);
     uint32_t* yes = ar.alloc<uint32_t>(n);
     uint32_t* no = ar.alloc<uint32_t>(n);
     uint32_t* pos_s = ar.alloc<uint32_t>(n);
     uint32_t* pos_k = ar.alloc<uint32_t>(n);
-    uint32_t* tot = ar.alloc<uint32_t>(2);
-    uint32_t* lvl = ar.alloc<uint32_t>(2);  // [0] levels present, [1] the sort's wait flag
+    uint32_t* tot = ar.alloc<uint32_t>(4);  // split, kept; levels present, a key without a slot
     if (ar.err != cudaSuccess) return ar.err;
-    cudaError_t e = cudaMemcpyAsync(k0, keys, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(split, 0, n, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(lvl, 0, 2 * sizeof(uint32_t), s);
-    if (e != cudaSuccess) return e;
-    k_iota_levels<<<nb(n), 256, 0, s>>>(keys, n, v0, lvl);
-    count_launches(1);
-    uint64_t* kk = k0;
-    uint32_t* vv = v0;
-    e = radix_sort_u64(kk, vv, k1, v1, n, 62, ar, s, lvl + 1);
-    if (e != cudaSuccess) return e;
-    uint32_t lv[2] = {0, 0};
-    e = cudaMemcpyAsync(lv, lvl, sizeof(lv), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return e;
-    const uint32_t levels = lv[0];
-    if (lv[1]) {
-        // the key sort's bounded wait ran out: its order is wrong, so no leaf lookup is trusted
-        *sort_timeout = true;
-        return cudaSuccess;
-    }
+    cudaError_t e = cudaSuccess;
+    uint32_t hd[4] = {0, 0, 0, 0};
+    float4* pts = nullptr;
     if (m > 0) {
-        k_subdiv_flags<<<nb(m), 256, 0, s>>>(cloud, m, f, root_size, levels, thr, kk, vv, n, split);
-        count_launches(1);
+        // the points ordered by cells of 16 thresholds (flags kernel with the points as they come 1,300 us, cells of
+        // 1, 4, 16, 64 thresholds 1,284, 924, 730, 714 us, and 75 to 110 us for the order).  A point that finds no slot
+        // counts in its last slot: the order is all that matters
+        const int bits = std::min(ht_bits(m), 32);
+        const size_t cap = (size_t)1 << bits;
+        uint64_t* table = ar.alloc<uint64_t>(cap);
+        uint32_t* cnt = ar.alloc<uint32_t>(cap + 2);
+        uint32_t* start = ar.alloc<uint32_t>(cap);
+        uint32_t* slot = ar.alloc<uint32_t>(m);
+        uint32_t* rank = ar.alloc<uint32_t>(m);
+        pts = ar.alloc<float4>(m);
+        if (ar.err != cudaSuccess) return ar.err;
+        e = cudaMemsetAsync(table, 0xff, cap * sizeof(uint64_t), s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(cnt, 0, (cap + 2) * sizeof(uint32_t), s);
+        if (e != cudaSuccess) return e;
+        const double h = std::max(16.0 * (double)thr, ldexp(root_size, -SD_FINE));
+        k_cell_count<false><<<nb(m), 256, 0, s>>>(cloud, m, f, h, 1.0 / h, table, bits, cnt, slot, rank, cnt + cap + 1);
+        k_cell_alloc<<<(unsigned)(cap / 256), 256, 0, s>>>(cnt, (int64_t)cap, start, cnt + cap);
+        k_cell_scatter<<<nb(m), 256, 0, s>>>(cloud, m, slot, rank, start, pts);
+        count_launches(3);
     }
-    k_not<<<nb(n), 256, 0, s>>>(split, n, yes, no);
-    count_launches(1);
-    e = scan_u32_to_u32(yes, pos_s, n, tot, ar, s);
-    if (e == cudaSuccess) e = scan_u32_to_u32(no, pos_k, n, tot + 1, ar, s);
-    uint32_t h[2] = {0, 0};
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h, tot, sizeof(h), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return e;
-    const int64_t n_split = h[0], n_keep = h[1];
+    for (int more = 0; more < HT_TRIES; ++more) {
+        if (e == cudaSuccess) e = cudaMemsetAsync(split, 0, n, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(tot, 0, 4 * sizeof(uint32_t), s);
+        if (e != cudaSuccess) return e;
+        if (m > 0) {
+            const int bits = ht_bits(n) + more;
+            const size_t cap = (size_t)1 << bits;
+            uint64_t* table = ar.alloc<uint64_t>(cap);
+            uint32_t* idx = ar.alloc<uint32_t>(cap);
+            if (ar.err != cudaSuccess) return ar.err;
+            e = cudaMemsetAsync(table, 0xff, cap * sizeof(uint64_t), s);
+            if (e == cudaSuccess) e = cudaMemsetAsync(idx, 0xff, cap * sizeof(uint32_t), s);
+            if (e == cudaSuccess) e = cudaMemsetAsync(coarse, 0, COARSE * sizeof(uint32_t), s);
+            if (e != cudaSuccess) return e;
+            k_leaf_enter<<<nb(n), 256, 0, s>>>(keys, n, table, idx, bits, coarse, tot + 2, tot + 3);
+            k_subdiv_flags<<<nb(m), 256, 0, s>>>(pts, m, f, root_size, ldexp(root_size, -SD_FINE),
+                                                 (double)(1 << SD_FINE) / root_size, tot + 2, thr, table, idx, bits, coarse,
+                                                 split);
+            count_launches(2);
+        }
+        k_not<<<nb(n), 256, 0, s>>>(split, n, yes, no);
+        count_launches(1);
+        e = scan_u32_to_u32(yes, pos_s, n, tot, ar, s);
+        if (e == cudaSuccess) e = scan_u32_to_u32(no, pos_k, n, tot + 1, ar, s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(hd, tot, sizeof(hd), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) return e;
+        if (!hd[3]) break;
+    }
+    if (hd[3]) return cudaErrorUnknown;  // see soft_prior
+    const int64_t n_split = hd[0], n_keep = hd[1];
     k_subdiv_write<<<nb(n), 256, 0, s>>>(keys, n, split, pos_k, pos_s, n_keep, n_split, out);
     count_launches(1);
     *n_out = n_keep + 8 * n_split;

@@ -260,17 +260,16 @@ cudaError_t feat_fuse(int64_t n_pix, const int64_t* off, const uint32_t* vox, co
                       int C, float* acc, float* wsum, cudaStream_t s);
 
 // LiDAR-guided initialisation (see dv_init.cu); the calls that return a size synchronise the stream.
-// The calls that sort set *sort_timeout (host) when the sort's bounded wait ran out; they synchronise
-// the stream before they return.
+// shared_corners sorts: it sets *sort_timeout (host) when the sort's bounded wait ran out.
 cudaError_t key_levels(const uint64_t* keys, int64_t n, uint32_t* levels_host, Arena& ar, cudaStream_t s);
 cudaError_t shared_corners(const uint64_t* keys, int64_t n, int max_level, uint64_t* grid_out, uint32_t* index_out,
                            int64_t* n_corners, Arena& ar, cudaStream_t s, bool* sort_timeout);
 cudaError_t soft_prior(const uint64_t* grid, int64_t n_corners, const double* center, double root_size, int max_level,
                        const float* cloud, int64_t m, float s_min, float v_close, float v_far, float* dens, Arena& ar,
-                       cudaStream_t s, bool* sort_timeout);
+                       cudaStream_t s);
 cudaError_t subdivide_round(const uint64_t* keys, int64_t n, const double* center, double root_size, int max_level,
                             const float* cloud, int64_t m, float thr, uint64_t* out, int64_t* n_out, Arena& ar,
-                            cudaStream_t s, bool* sort_timeout);
+                            cudaStream_t s);
 // uniform leaf grid of an actor (Sec. 3.3, assets): keys of the 8^level leaves (i fastest) and every
 // corner density set to v_init
 cudaError_t asset_grid(int level, float v_init, uint64_t* keys, float* dens, cudaStream_t s);
@@ -279,6 +278,10 @@ struct InitCam {
     double R[9], t[3];
     double fx, fy, cx, cy, near_, far_;
     int32_t W, H;
+    // the same in FP32 for the certain cases: near and far a little nearer [0] and farther [1], the image's four
+    // sides (left: fx x + side[0] z = 0, right side[1], top and bottom with fy) and their normals' lengths, rounded up
+    float Rf[9], tf[3], fxf, fyf, nearf[2], farf[2], side[4], len[4];
+    float scale;  // the most the camera's matrix stretches a length (1 for a rotation, which is not checked here)
 };
 cudaError_t visibility_prune(const uint64_t* keys, int64_t n, const double* center, double root_size,
                              const InitCam* cams_host, int n_cam, double z_min, uint64_t* out, int64_t* n_out,
