@@ -100,18 +100,24 @@ __device__ __forceinline__ void pdl_launch_dependents() {
 }
 
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t s, Args... args) {
+inline cudaError_t launch_pdl_smem(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                   Args... args) {
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t s, Args... args) {
+    return launch_pdl_smem(kernel, grid, block, 0, s, args...);
 }
 void count_launches(long long n);
 }
@@ -170,8 +176,8 @@ cudaError_t debug_sort_timeout(int spin_limit, uint32_t* call_flag, uint32_t* de
 // counters and look-back status.  keys/vals and keys_tmp/vals_tmp are the ping-pong buffers (the
 // input is overwritten); the last pass writes vals_out and keys_out, or, with keys_out null, the
 // ping-pong buffer it does not read, returned in keys_out.  call_err (device word, not null) is set
-// to 1 if a bounded look-back wait runs out (the result is then not sorted).  Counts of 2^30 keys
-// or more take reduce-then-scan passes (which count their own digits) and copy to the outputs.
+// to 1 if a bounded look-back wait runs out (the result is then not sorted).  Large sorts count their
+// digits themselves, pass by pass, and nothing of theirs waits.
 int64_t sort_counted_words(int64_t n, int n_bits);
 cudaError_t sort_counted_u64(uint64_t* keys, uint32_t* vals, uint64_t* keys_tmp, uint32_t* vals_tmp,
                              uint64_t*& keys_out, uint32_t* vals_out, int64_t n, int n_bits, const uint32_t* hist,

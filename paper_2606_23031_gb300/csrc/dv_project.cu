@@ -114,44 +114,48 @@ __device__ __forceinline__ uint32_t side_path(uint32_t idx, int level, int64_t X
     return (1u << top) | (((cell >> top) & 1u ? ~idx : idx) & low);
 }
 
-// Projection of voxel gv of `view`: returns its tile count (0: not visible) and, when visible, its
-// pixel rectangle and depth-order key.
-__device__ __forceinline__ uint32_t project_voxel(const BatchParams& bp, int view, int64_t gv, uint64_t& rect,
-                                                  uint64_t& skey, uint32_t* __restrict__ flags) {
+// Whether voxel gv of `view` may be visible.  Most voxels lie outside the frustum by far: the bounding sphere
+// against the near and far planes and the four sides, each side 1.5 pixels outside the image, decides those with a
+// tenth of the arithmetic of the corners.  It leaves out nothing that the corners (project_voxel) would keep: the
+// radius covers the rounding of both (4e-6 of the coordinates' size), and where the sphere comes so close to the
+// camera plane that its projection exceeds 2e5 pixels (the corner test's own margin then grows past a pixel) the
+// corners decide.
+__device__ __forceinline__ bool maybe_visible(const BatchParams& bp, int view, int64_t gv, uint32_t* __restrict__ flags) {
     const int o = gv < bp.vox_offset[1] ? 0 : find_octree(bp, gv);
     const ViewParams& fp = bp.views[view];
     const OctParams& P = bp.octs[view * bp.n_oct + o];
-    const int64_t v = gv - bp.vox_offset[o];
-    const uint64_t key = P.key[v];
-    const Leaf L = decode_leaf(P, key);
+    const Leaf L = decode_leaf(P, P.key[gv - bp.vox_offset[o]]);
     if (L.level > P.max_level || L.i >> L.level || L.j >> L.level || L.k >> L.level) {
         atomicOr(flags, DV_FLAG_BAD_LEVEL);
         __threadfence();  // visible to the block that reports the flags
-        return 0;
+        return false;
     }
-    // Most voxels lie outside the frustum by far: the bounding sphere against the near and far planes and the four
-    // sides, each side 1.5 pixels outside the image, decides those with a tenth of the arithmetic (8M-leaf frame,
-    // six cameras: @P@).  It leaves out nothing that the corners below would keep: the radius covers
-    // the rounding of both (4e-6 of the coordinates' size), and where the sphere comes so close to the camera
-    // plane that its projection exceeds 2e5 pixels (the corner test's own margin then grows past a pixel)
-    // the corners decide.
-    {
-        const float h = 0.5f * L.s;
-        const float x0 = L.mn[0] + h, y0 = L.mn[1] + h, z0 = L.mn[2] + h;
-        float c[3];
+    const float h = 0.5f * L.s;
+    const float x0 = L.mn[0] + h, y0 = L.mn[1] + h, z0 = L.mn[2] + h;
+    float c[3];
 #pragma unroll
-        for (int r = 0; r < 3; ++r) c[r] = fmaf(P.M[r * 3 + 0], x0, fmaf(P.M[r * 3 + 1], y0, fmaf(P.M[r * 3 + 2], z0, P.m[r])));
-        const float size = fabsf(x0) + fabsf(y0) + fabsf(z0) + fabsf(P.m[0]) + fabsf(P.m[1]) + fabsf(P.m[2]);
-        const float rad = fmaf(0.8661f, L.s, 4e-6f * size);
-        const float zn = c[2] - rad;
-        if (c[2] + rad < fp.z_clip || zn > fp.far_) return 0;
-        if (zn > fp.z_clip && fmaxf(fp.fx * (fabsf(c[0]) + rad), fp.fy * (fabsf(c[1]) + rad)) < 2e5f * zn) {
-            const float fx = fp.fx * c[0], fy = fp.fy * c[1];
-            if (fmaf(fp.side[0], c[2], fx) < -fp.side_len[0] * rad || fmaf(fp.side[1], c[2], fx) > fp.side_len[1] * rad ||
-                fmaf(fp.side[2], c[2], fy) < -fp.side_len[2] * rad || fmaf(fp.side[3], c[2], fy) > fp.side_len[3] * rad)
-                return 0;
-        }
+    for (int r = 0; r < 3; ++r) c[r] = fmaf(P.M[r * 3 + 0], x0, fmaf(P.M[r * 3 + 1], y0, fmaf(P.M[r * 3 + 2], z0, P.m[r])));
+    const float size = fabsf(x0) + fabsf(y0) + fabsf(z0) + fabsf(P.m[0]) + fabsf(P.m[1]) + fabsf(P.m[2]);
+    const float rad = fmaf(0.8661f, L.s, 4e-6f * size);
+    const float zn = c[2] - rad;
+    if (c[2] + rad < fp.z_clip || zn > fp.far_) return false;
+    if (zn > fp.z_clip && fmaxf(fp.fx * (fabsf(c[0]) + rad), fp.fy * (fabsf(c[1]) + rad)) < 2e5f * zn) {
+        const float fx = fp.fx * c[0], fy = fp.fy * c[1];
+        if (fmaf(fp.side[0], c[2], fx) < -fp.side_len[0] * rad || fmaf(fp.side[1], c[2], fx) > fp.side_len[1] * rad ||
+            fmaf(fp.side[2], c[2], fy) < -fp.side_len[2] * rad || fmaf(fp.side[3], c[2], fy) > fp.side_len[3] * rad)
+            return false;
     }
+    return true;
+}
+
+// Projection of voxel gv of `view`: returns its tile count (0: not visible) and, when visible, its
+// pixel rectangle and depth-order key.
+__device__ __forceinline__ uint32_t project_voxel(const BatchParams& bp, int view, int64_t gv, uint64_t& rect,
+                                                  uint64_t& skey) {
+    const int o = gv < bp.vox_offset[1] ? 0 : find_octree(bp, gv);
+    const ViewParams& fp = bp.views[view];
+    const OctParams& P = bp.octs[view * bp.n_oct + o];
+    const Leaf L = decode_leaf(P, P.key[gv - bp.vox_offset[o]]);
     // corners in the camera frame: p = M (mn + s*offset) + m
     float p0[3], e[3][3];
 #pragma unroll
@@ -219,17 +223,22 @@ __device__ __forceinline__ uint32_t project_voxel(const BatchParams& bp, int vie
 
 constexpr int MAX_KEY_PASSES = 8;  // 8-bit digits of a 64-bit key
 
-// One thread per (view, voxel).  A block reserves one run of the sort input for its visible voxels
-// (scal[0] counts them, scal[1] their pairs), adds the digits of their keys to key_hist
+// A block takes `rounds` times 256 voxels of one view.  Its threads test them all (maybe_visible), the voxels left
+// gather in a queue in shared memory, and the block projects those, 256 at a time: left in place they would take
+// the corner arithmetic and the depth key to nearly every warp, at an eighth of its lanes (8M-leaf frame, six
+// cameras: 1,166 -> 672 us; the 500k-leaf frame's step is as long either way).  Per 256 the block reserves one run of the sort input for the visible ones
+// (scal[0] counts them, scal[1] their pairs); it adds the digits of their keys to key_hist
 // [key_passes][256], and the block that finishes last copies scal[0..2] into host_out[0..2] (the
 // device's wait-error word folded into the flags) and then `seq` into host_out[3], so the host learns
 // the sizes from this kernel alone, as soon as they are final.  scal[3] counts finished blocks.
 // Block 0 also clears the call's five work words, and the grid the tile ranges.  Grid: (blocks of one view's
 // voxels, views).
-__global__ void __launch_bounds__(256) k_project(const __grid_constant__ BatchParams bp, uint64_t* __restrict__ rect, uint64_t* __restrict__ out_key,
-                                                 uint32_t* __restrict__ out_g, uint32_t* __restrict__ key_hist,
-                                                 int key_passes, uint2* __restrict__ range,
-                                                 unsigned long long* __restrict__ scal,
+constexpr int PROJ_ROUNDS = 4;
+
+__global__ void __launch_bounds__(256) k_project(const __grid_constant__ BatchParams bp, uint64_t* __restrict__ rect,
+                                                 uint64_t* __restrict__ out_key, uint32_t* __restrict__ out_g,
+                                                 uint32_t* __restrict__ key_hist, int key_passes, int rounds,
+                                                 uint2* __restrict__ range, unsigned long long* __restrict__ scal,
                                                  volatile uint64_t* host_out, uint64_t seq,
                                                  uint32_t* __restrict__ spin_err, unsigned long long* __restrict__ work) {
     pdl_wait();
@@ -239,50 +248,69 @@ __global__ void __launch_bounds__(256) k_project(const __grid_constant__ BatchPa
     for (int64_t t = (int64_t)block * 256 + threadIdx.x; t < bp.n_tiles; t += (int64_t)n_block * 256)
         range[t] = make_uint2(0u, 0u);
     __shared__ uint32_t h[MAX_KEY_PASSES][256];
+    __shared__ uint16_t s_queue[PROJ_ROUNDS * 256];  // voxels of the block left to project
     __shared__ uint32_t s_wv[8];
     __shared__ unsigned long long s_wp[8];
     __shared__ unsigned long long s_base;
-    __shared__ uint32_t s_nv;
+    __shared__ uint32_t s_nq;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int view = blockIdx.y;
-    const int64_t gv = (int64_t)blockIdx.x * 256 + tid;  // voxel of the view
-    const int64_t g = view * bp.n_vox + gv;
-    uint64_t rc = 0, key = 0;
-    uint32_t c = 0;
-    if (gv < bp.n_vox) c = project_voxel(bp, view, gv, rc, key, reinterpret_cast<uint32_t*>(scal + 2));
-    const unsigned bal = __ballot_sync(0xffffffffu, c != 0);
-    unsigned long long np = c;
+    const int64_t gv0 = (int64_t)blockIdx.x * 256 * rounds;  // the block's first voxel of the view
+    if (tid == 0) s_nq = 0;
+    __syncthreads();
+    for (int r = 0; r < rounds; ++r) {
+        const int64_t gv = gv0 + r * 256 + tid;
+        const bool in = gv < bp.n_vox && maybe_visible(bp, view, gv, reinterpret_cast<uint32_t*>(scal + 2));
+        const unsigned bal = __ballot_sync(0xffffffffu, in);
+        uint32_t at = 0;
+        if (lane == 0 && bal) at = atomicAdd(&s_nq, (uint32_t)__popc(bal));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (in) s_queue[at + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(r * 256 + tid);
+    }
+    __syncthreads();
+    const uint32_t nq = s_nq;
+    if (nq) {
+        for (int i = tid; i < key_passes * 256; i += 256) (&h[0][0])[i] = 0u;
+        for (uint32_t q0 = 0; q0 < nq; q0 += 256) {
+            uint64_t rc = 0, key = 0;
+            uint32_t c = 0;
+            int64_t gv = 0;
+            if (q0 + tid < nq) {
+                gv = gv0 + s_queue[q0 + tid];
+                c = project_voxel(bp, view, gv, rc, key);
+            }
+            const unsigned bal = __ballot_sync(0xffffffffu, c != 0);
+            unsigned long long np = c;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) np += __shfl_down_sync(0xffffffffu, np, off);
-    if (lane == 0) {
-        s_wv[warp] = __popc(bal);
-        s_wp[warp] = np;
-    }
-    for (int i = tid; i < key_passes * 256; i += 256) (&h[0][0])[i] = 0u;
-    __syncthreads();
-    if (tid == 0) {
-        uint32_t nv = 0;
-        unsigned long long pp = 0;
-        for (int w = 0; w < 8; ++w) {
-            const uint32_t x = s_wv[w];
-            s_wv[w] = nv;  // exclusive offsets of the warps
-            nv += x;
-            pp += s_wp[w];
+            for (int off = 16; off > 0; off >>= 1) np += __shfl_down_sync(0xffffffffu, np, off);
+            if (lane == 0) {
+                s_wv[warp] = __popc(bal);
+                s_wp[warp] = np;
+            }
+            __syncthreads();
+            if (tid == 0) {
+                uint32_t nv = 0;
+                unsigned long long pp = 0;
+                for (int w = 0; w < 8; ++w) {
+                    const uint32_t x = s_wv[w];
+                    s_wv[w] = nv;  // exclusive offsets of the warps
+                    nv += x;
+                    pp += s_wp[w];
+                }
+                s_base = nv ? atomicAdd(scal + 0, (unsigned long long)nv) : 0ull;
+                if (pp) atomicAdd(scal + 1, pp);
+            }
+            __syncthreads();
+            if (c) {
+                const unsigned long long q = s_base + s_wv[warp] + __popc(bal & ((1u << lane) - 1u));
+                const int64_t g = view * bp.n_vox + gv;
+                out_key[q] = key;
+                out_g[q] = (uint32_t)g;
+                rect[g] = rc;
+                for (int p = 0; p < key_passes; ++p) atomicAdd(&h[p][(uint32_t)(key >> (8 * p)) & 255u], 1u);
+            }
+            __syncthreads();
         }
-        s_nv = nv;
-        s_base = nv ? atomicAdd(scal + 0, (unsigned long long)nv) : 0ull;
-        if (pp) atomicAdd(scal + 1, pp);
-    }
-    __syncthreads();
-    if (s_nv) {
-        if (c) {
-            const unsigned long long q = s_base + s_wv[warp] + __popc(bal & ((1u << lane) - 1u));
-            out_key[q] = key;
-            out_g[q] = (uint32_t)g;
-            rect[g] = rc;
-            for (int p = 0; p < key_passes; ++p) atomicAdd(&h[p][(uint32_t)(key >> (8 * p)) & 255u], 1u);
-        }
-        __syncthreads();
         for (int i = tid; i < key_passes * 256; i += 256) {
             const uint32_t x = (&h[0][0])[i];
             if (x) atomicAdd(key_hist + i, x);
@@ -393,7 +421,7 @@ __global__ void __launch_bounds__(256) k_records_emit(
         const int64_t v = (int64_t)(g - (uint32_t)view * (uint32_t)bp.n_vox) - P.vox_offset;
         // The voxel's key, densities, rectangle and SH coefficients, all in flight together: the voxels of a block
         // are scattered over memory, so one round trip per voxel is what this kernel waits for (with the
-        // coefficients loaded as they were used: 8M-leaf frame, six cameras @R@)
+        // coefficients loaded as they were used: 8M-leaf frame, six cameras 1,365 us, this way 966 us)
         const int deg = P.sh_degree;
         const int nsh = (deg + 1) * (deg + 1);
         const float* shv = P.sh + v * nsh * 3;
@@ -722,8 +750,11 @@ cudaError_t launch_project(const BatchParams& bp, uint64_t* rect, uint64_t* out_
     const int passes = key_passes(key_bits);
     if (passes > MAX_KEY_PASSES) return cudaErrorInvalidValue;
     // with no voxel at all, empty blocks still clear the work words and report the (zero) sizes
-    launch_pdl(k_project, dim3(bp.n_vox > 0 ? nblk(bp.n_vox, 256) : 1u, (unsigned)bp.n_view), dim3(256), s, bp, rect,
-               out_key, out_g, key_hist, passes, tile_range, scal, (volatile uint64_t*)host_out, seq, spin_err, work);
+    // fewer blocks than one or two per SM would leave the chip idle below this
+    const int rounds = bp.n_vox * bp.n_view >= 100000 ? PROJ_ROUNDS : 1;
+    launch_pdl(k_project, dim3(bp.n_vox > 0 ? nblk(bp.n_vox, 256 * rounds) : 1u, (unsigned)bp.n_view), dim3(256), s, bp,
+               rect, out_key, out_g, key_hist, passes, rounds, tile_range, scal, (volatile uint64_t*)host_out, seq,
+               spin_err, work);
     count_launches(1);
     return cudaGetLastError();
 }

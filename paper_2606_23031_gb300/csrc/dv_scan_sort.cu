@@ -4,18 +4,18 @@
 // then per-block scans seeded with their offsets.  Inside a block the scan is
 // a warp shuffle scan over per-thread sums.
 //
-// The radix sort processes 8 bits per pass.  A pass is (1) a per-block digit
-// histogram, (2) an exclusive scan of the digit-major histogram table, (3) a
-// stable scatter.  Stability inside a block comes from warp-level ranking:
+// The radix sort processes 8 bits per pass.  Small sorts take one-sweep passes (one kernel each, the
+// digit counts of all passes known beforehand), large ones count, scan and scatter per pass.
+// Stability inside a block comes from warp-level ranking:
 // __match_any_sync groups the lanes holding the same digit, popc of the lower
 // lanes of that group gives the lane's rank, and per-warp digit counts in
-// shared memory order the warps; rounds inside a block keep a running count
-// per digit.  Every pass is therefore stable, so an LSD sequence of passes
+// shared memory order the warps.  Every pass is therefore stable, so an LSD sequence of passes
 // sorts by the full key and keeps equal keys in input order.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include <atomic>
+#include <utility>
 
 #include "dv_internal.cuh"
 
@@ -94,9 +94,9 @@ __global__ void k_scan_top(Tout* __restrict__ bsum, int64_t nb, Tout* __restrict
     if (threadIdx.x == 0 && total) *total = carry_s;
 }
 
+// (in and out may be the same array: a thread reads its entries before it writes them)
 template <typename Tin, typename Tout>
-__global__ void k_scan_down(const Tin* __restrict__ in, int64_t n, const Tout* __restrict__ bsum,
-                            Tout* __restrict__ out) {
+__global__ void k_scan_down(const Tin* in, int64_t n, const Tout* __restrict__ bsum, Tout* out) {
     pdl_wait();
     pdl_launch_dependents();
     const int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
@@ -141,112 +141,8 @@ cudaError_t scan_impl(const Tin* in, Tout* out, int64_t n, Tout* total_dev, Aren
 // ---------------------------------------------------------------------------
 
 constexpr int RS_THREADS = 256;
-constexpr int RS_MAX_ROUNDS = 16;  // keys per thread per pass, chosen per sort (see radix_impl)
 constexpr int RS_WARPS = RS_THREADS / 32;
 constexpr int RS_RADIX = 256;
-
-template <typename K>
-__global__ void __launch_bounds__(RS_THREADS) k_radix_hist(const K* __restrict__ keys, int64_t n, int shift,
-                                                            uint32_t mask, uint32_t* __restrict__ hist,
-                                                            int64_t nblocks, int rounds) {
-    pdl_wait();
-    pdl_launch_dependents();
-    __shared__ uint32_t h[RS_RADIX];
-    h[threadIdx.x] = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * RS_THREADS * rounds;
-#pragma unroll 4
-    for (int r = 0; r < rounds; ++r) {
-        int64_t i = base + (int64_t)r * RS_THREADS + threadIdx.x;
-        if (i < n) atomicAdd(&h[(uint32_t)(keys[i] >> shift) & mask], 1u);
-    }
-    __syncthreads();
-    hist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
-}
-
-template <typename K>
-__global__ void __launch_bounds__(RS_THREADS) k_radix_scatter(const K* __restrict__ keys,
-                                                               const uint32_t* __restrict__ vals, int64_t n,
-                                                               int shift, uint32_t mask,
-                                                               const uint32_t* __restrict__ offs, int64_t nblocks,
-                                                               K* __restrict__ okeys, uint32_t* __restrict__ ovals,
-                                                               int rounds) {
-    pdl_wait();
-    pdl_launch_dependents();
-    __shared__ uint32_t run[RS_RADIX];       // next free slot per digit (global index)
-    __shared__ uint32_t wcnt[RS_WARPS][RS_RADIX];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    run[threadIdx.x] = offs[(int64_t)threadIdx.x * nblocks + blockIdx.x];
-    for (int w = 0; w < RS_WARPS; ++w) wcnt[w][threadIdx.x] = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * RS_THREADS * rounds;
-    const unsigned lt = (1u << lane) - 1u;
-    for (int r = 0; r < rounds; ++r) {
-        int64_t i = base + (int64_t)r * RS_THREADS + threadIdx.x;
-        bool ok = i < n;
-        K key = ok ? keys[i] : K(0);
-        uint32_t val = ok ? vals[i] : 0u;
-        uint32_t d = ok ? ((uint32_t)(key >> shift) & mask) : 0xffffffffu;
-        unsigned peers = __match_any_sync(0xffffffffu, d);
-        int rank = __popc(peers & lt);
-        bool leader = rank == 0;
-        if (ok && leader) wcnt[warp][d] = __popc(peers);
-        __syncthreads();
-        if (ok) {
-            uint32_t before = 0;
-            for (int w = 0; w < warp; ++w) before += wcnt[w][d];
-            uint32_t pos = run[d] + before + (uint32_t)rank;
-            okeys[pos] = key;
-            ovals[pos] = val;
-        }
-        __syncthreads();
-        uint32_t add = 0;
-#pragma unroll
-        for (int w = 0; w < RS_WARPS; ++w) {
-            add += wcnt[w][threadIdx.x];
-            wcnt[w][threadIdx.x] = 0;
-        }
-        run[threadIdx.x] += add;
-        __syncthreads();
-    }
-}
-
-template <typename K>
-cudaError_t radix_impl(K*& keys, uint32_t*& vals, K* keys_alt, uint32_t* vals_alt, int64_t n, int n_bits, Arena& ar,
-                       cudaStream_t s) {
-    if (n <= 1 || n_bits <= 0) return cudaSuccess;
-    // keys per block: as many as possible while still giving every SM two blocks
-    int rounds = RS_MAX_ROUNDS;
-    while (rounds > 1 && (n + (int64_t)RS_THREADS * rounds - 1) / ((int64_t)RS_THREADS * rounds) < 304) rounds >>= 1;
-    const int64_t tile = (int64_t)RS_THREADS * rounds;
-    int64_t nblocks = (n + tile - 1) / tile;
-    uint32_t* hist = ar.alloc<uint32_t>((size_t)(nblocks * RS_RADIX));
-    uint32_t* offs = ar.alloc<uint32_t>((size_t)(nblocks * RS_RADIX));
-    if (!hist || !offs) return ar.err;
-    K* src_k = keys;
-    uint32_t* src_v = vals;
-    K* dst_k = keys_alt;
-    uint32_t* dst_v = vals_alt;
-    for (int shift = 0; shift < n_bits; shift += 8) {
-        int bits = n_bits - shift < 8 ? n_bits - shift : 8;
-        uint32_t mask = (1u << bits) - 1u;
-        launch_pdl(k_radix_hist<K>, dim3((unsigned)nblocks), dim3(RS_THREADS), s, src_k, n, shift, mask, hist, nblocks, rounds);
-        count_launches(1);
-        cudaError_t e = scan_impl<uint32_t, uint32_t>(hist, offs, nblocks * RS_RADIX, nullptr, ar, s);
-        if (e != cudaSuccess) return e;
-        launch_pdl(k_radix_scatter<K>, dim3((unsigned)nblocks), dim3(RS_THREADS), s, src_k, src_v, n, shift, mask, offs, nblocks, dst_k, dst_v, rounds);
-        count_launches(1);
-        K* tk = src_k;
-        src_k = dst_k;
-        dst_k = tk;
-        uint32_t* tv = src_v;
-        src_v = dst_v;
-        dst_v = tv;
-    }
-    keys = src_k;
-    vals = src_v;
-    return cudaGetLastError();
-}
 
 // ---------------------------------------------------------------------------
 // one-sweep radix sort: one kernel per 8-bit pass
@@ -420,6 +316,161 @@ __global__ void __launch_bounds__(OS_THREADS) k_os_pass(const K* __restrict__ ke
     }
 }
 
+// ---------------------------------------------------------------------------
+// large sorts: a pass is the tiles' digit counts, a scan of them and a scatter
+//
+// At millions of keys some three hundred tiles are in flight, and a one-sweep tile walks back over most of them
+// before it meets an inclusive prefix.  Counting the tiles first costs one more read of the keys and no tile
+// waits for another: the 8M-leaf six-camera step (6M depth keys in 7 passes, 10M pairs in 2) 8.29 -> 8.05 ms, the
+// 32M-leaf 4K render (7.6M and 20M) 7.76 -> 7.48 ms, an initialisation round (4M corners in 5) 2.48 -> 2.35 ms.
+// (Ballots of the digit's bits instead of the match instruction: 8.19, 7.68 and 2.43 ms.)
+// A warp ranks its own 512 consecutive keys without block barriers (a counter per warp and digit in shared
+// memory); the tile is put in digit order in shared memory and leaves it in runs of consecutive addresses.
+// ---------------------------------------------------------------------------
+constexpr int OL_ITEMS = 16;
+constexpr int OL_TILE = OS_THREADS * OL_ITEMS;
+
+// per-warp digit counts of a tile's keys; with `place`, each key's rank among its warp's keys of the digit
+template <typename K>
+__device__ __forceinline__ void rank_warp(const K* key, int64_t first, int64_t n, int shift, uint32_t mask,
+                                          uint32_t* mine, uint32_t* place) {
+    const unsigned lt = (1u << (threadIdx.x & 31)) - 1u;
+#pragma unroll
+    for (int i = 0; i < OL_ITEMS; ++i) {
+        const bool ok = first + 32 * i < n;
+        const uint32_t d = ok ? (uint32_t)(key[i] >> shift) & mask : 0xffffffffu;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        const uint32_t before = ok ? mine[d] : 0u;
+        __syncwarp();
+        if (ok && (peers & lt) == 0u) mine[d] = before + __popc(peers);
+        __syncwarp();
+        if (place) place[i] = before + __popc(peers & lt);
+    }
+}
+
+// hist[digit][tile]
+template <typename K>
+__global__ void __launch_bounds__(OS_THREADS) k_ol_count(const K* __restrict__ keys, int64_t n, int shift, uint32_t mask,
+                                                         uint32_t* __restrict__ hist) {
+    pdl_wait();
+    pdl_launch_dependents();
+    __shared__ uint32_t cnt[RS_WARPS][RS_RADIX];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+#pragma unroll
+    for (int w = 0; w < RS_WARPS; ++w) cnt[w][tid] = 0u;
+    const int64_t first = (int64_t)blockIdx.x * OL_TILE + warp * (32 * OL_ITEMS) + lane;
+    K key[OL_ITEMS];
+#pragma unroll
+    for (int i = 0; i < OL_ITEMS; ++i) key[i] = first + 32 * i < n ? keys[first + 32 * i] : K(0);
+    __syncthreads();
+    rank_warp<K>(key, first, n, shift, mask, cnt[warp], nullptr);
+    __syncthreads();
+    uint32_t c = 0;
+#pragma unroll
+    for (int w = 0; w < RS_WARPS; ++w) c += cnt[w][tid];
+    hist[(size_t)tid * gridDim.x + blockIdx.x] = c;
+}
+
+template <typename K>
+struct LargeSmem {
+    uint32_t cnt[RS_WARPS][RS_RADIX];  // keys of the digit in the warp so far, then before the warp
+    uint32_t off[RS_RADIX];            // first place of the digit in the tile
+    uint32_t base[RS_RADIX];           // global place of the tile's first key of the digit, less off
+    uint32_t total;
+    K key[OL_TILE];
+    uint32_t val[OL_TILE];
+};
+
+// offs[digit][tile]: global place of the tile's first key of the digit
+template <typename K>
+__global__ void __launch_bounds__(OS_THREADS, 2) k_ol_scatter(const K* __restrict__ keys,
+                                                              const uint32_t* __restrict__ vals, int64_t n, int shift,
+                                                              uint32_t mask, const uint32_t* __restrict__ offs,
+                                                              K* __restrict__ okeys, uint32_t* __restrict__ ovals) {
+    pdl_wait();
+    pdl_launch_dependents();
+    extern __shared__ __align__(16) unsigned char ol_raw[];
+    LargeSmem<K>& S = *reinterpret_cast<LargeSmem<K>*>(ol_raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+#pragma unroll
+    for (int w = 0; w < RS_WARPS; ++w) S.cnt[w][tid] = 0u;
+    const int64_t first = (int64_t)blockIdx.x * OL_TILE + warp * (32 * OL_ITEMS) + lane;
+    K key[OL_ITEMS];
+    uint32_t val[OL_ITEMS], place[OL_ITEMS];
+#pragma unroll
+    for (int i = 0; i < OL_ITEMS; ++i) {
+        const int64_t q = first + 32 * i;
+        key[i] = q < n ? keys[q] : K(0);
+        val[i] = q < n ? vals[q] : 0u;
+    }
+    const uint32_t goff = offs[(size_t)tid * gridDim.x + blockIdx.x];
+    __syncthreads();
+    rank_warp<K>(key, first, n, shift, mask, S.cnt[warp], place);
+    __syncthreads();
+    // thread tid owns digit tid: the warps' counts before each warp, the digit's place in the tile
+    uint32_t count = 0;
+#pragma unroll
+    for (int w = 0; w < RS_WARPS; ++w) {
+        const uint32_t c = S.cnt[w][tid];
+        S.cnt[w][tid] = count;
+        count += c;
+    }
+    const uint32_t off = block_excl_scan<uint32_t>(count, &S.total);
+    S.off[tid] = off;
+    S.base[tid] = goff - off;  // modulo 2^32: the sum with a place in the tile is below n
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < OL_ITEMS; ++i) {
+        if (first + 32 * i < n) {
+            const uint32_t d = (uint32_t)(key[i] >> shift) & mask;
+            const uint32_t at = S.off[d] + S.cnt[warp][d] + place[i];
+            S.key[at] = key[i];
+            S.val[at] = val[i];
+        }
+    }
+    __syncthreads();
+    const int64_t left = n - (int64_t)blockIdx.x * OL_TILE;
+    const int m = left < OL_TILE ? (int)left : OL_TILE;
+    for (int j = tid; j < m; j += OS_THREADS) {
+        const K k = S.key[j];
+        const uint32_t pos = S.base[(uint32_t)(k >> shift) & mask] + (uint32_t)j;
+        okeys[pos] = k;
+        ovals[pos] = S.val[j];
+    }
+}
+
+// 32-bit words of a large sort's scratch: the counts (scanned in place) and the scan's block sums
+int64_t ol_words(int64_t n) {
+    const int64_t n_tiles = (n + OL_TILE - 1) / OL_TILE, m = n_tiles * RS_RADIX;
+    return m + (m + SCAN_TILE - 1) / SCAN_TILE;
+}
+
+template <typename K>
+cudaError_t large_pass(const K* keys, const uint32_t* vals, int64_t n, int shift, uint32_t mask, uint32_t* words,
+                       K* okeys, uint32_t* ovals, cudaStream_t s) {
+    const unsigned n_tiles = (unsigned)((n + OL_TILE - 1) / OL_TILE);
+    const int64_t m = (int64_t)n_tiles * RS_RADIX, nb = (m + SCAN_TILE - 1) / SCAN_TILE;
+    uint32_t* bsum = words + m;
+    const size_t smem = sizeof(LargeSmem<K>);
+    cudaError_t e = cudaFuncSetAttribute(k_ol_scatter<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    launch_pdl(k_ol_count<K>, dim3(n_tiles), dim3(OS_THREADS), s, keys, n, shift, mask, words);
+    launch_pdl(k_scan_reduce<uint32_t, uint32_t>, dim3((unsigned)nb), dim3(SCAN_THREADS), s, (const uint32_t*)words, m, bsum);
+    launch_pdl(k_scan_top<uint32_t>, dim3(1), dim3(SCAN_THREADS), s, bsum, nb, (uint32_t*)nullptr);
+    launch_pdl(k_scan_down<uint32_t, uint32_t>, dim3((unsigned)nb), dim3(SCAN_THREADS), s, (const uint32_t*)words, m,
+               (const uint32_t*)bsum, words);
+    e = launch_pdl_smem(k_ol_scatter<K>, dim3(n_tiles), dim3(OS_THREADS), smem, s, keys, vals, n, shift, mask,
+                        (const uint32_t*)words, okeys, ovals);
+    count_launches(5);
+    return e;
+}
+
+// Keys from which a sort takes the counted passes: 16 per thread of one 256-thread block per SM (622k keys; with
+// the line at 4 the 298k keys and 354k pairs of a 480x270 view take 574 instead of 514 us, five launches a pass
+// being too many for them).
+constexpr int OL_FROM = 16;
+bool large_sort(int64_t n, int n_sm) { return n > (int64_t)OL_FROM * OS_THREADS * n_sm; }
+
 template <typename K, int ROUNDS>
 cudaError_t onesweep_impl(K*& keys, uint32_t*& vals, K* keys_alt, uint32_t* vals_alt, int64_t n, int n_bits,
                           uint32_t* call_err, int n_sm, Arena& ar, cudaStream_t s) {
@@ -473,6 +524,18 @@ template <typename K>
 cudaError_t onesweep(K*& keys, uint32_t*& vals, K* keys_alt, uint32_t* vals_alt, int64_t n, int n_bits,
                      uint32_t* call_err, Arena& ar, cudaStream_t s) {
     const int n_sm = sm_count();
+    if (large_sort(n, n_sm)) {
+        uint32_t* words = ar.alloc<uint32_t>((size_t)ol_words(n));
+        if (!words) return ar.err;
+        for (int shift = 0; shift < n_bits; shift += 8) {
+            const int bits = n_bits - shift < 8 ? n_bits - shift : 8;
+            const cudaError_t e = large_pass<K>(keys, vals, n, shift, (1u << bits) - 1u, words, keys_alt, vals_alt, s);
+            if (e != cudaSuccess) return e;
+            std::swap(keys, keys_alt);
+            std::swap(vals, vals_alt);
+        }
+        return cudaGetLastError();
+    }
     switch (onesweep_rounds(n, n_sm)) {
     case 1: return onesweep_impl<K, 1>(keys, vals, keys_alt, vals_alt, n, n_bits, call_err, n_sm, ar, s);
     case 2: return onesweep_impl<K, 2>(keys, vals, keys_alt, vals_alt, n, n_bits, call_err, n_sm, ar, s);
@@ -504,10 +567,15 @@ cudaError_t counted_passes(K* keys, uint32_t* vals, K* keys_tmp, uint32_t* vals_
         }
         const int shift = 8 * p;
         const int bits = n_bits - shift < 8 ? n_bits - shift : 8;
-        launch_pdl(k_os_pass<K, ROUNDS>, dim3((unsigned)n_tiles), dim3(OS_THREADS), s, (const K*)sk,
-                   (const uint32_t*)sv, n, shift, (1u << bits) - 1u, hist + p * RS_RADIX,
-                   status + (size_t)p * n_tiles * RS_RADIX, counters + p, call_err, dk, dvv, OS_SPIN_LIMIT);
-        count_launches(1);
+        if constexpr (ROUNDS == OL_ITEMS) {
+            const cudaError_t e = large_pass<K>(sk, sv, n, shift, (1u << bits) - 1u, words, dk, dvv, s);
+            if (e != cudaSuccess) return e;
+        } else {
+            launch_pdl(k_os_pass<K, ROUNDS>, dim3((unsigned)n_tiles), dim3(OS_THREADS), s, (const K*)sk,
+                       (const uint32_t*)sv, n, shift, (1u << bits) - 1u, hist + p * RS_RADIX,
+                       status + (size_t)p * n_tiles * RS_RADIX, counters + p, call_err, dk, dvv, OS_SPIN_LIMIT);
+            count_launches(1);
+        }
         sk = dk;
         sv = dvv;
     }
@@ -526,18 +594,8 @@ cudaError_t sort_counted(K* keys, uint32_t* vals, K* keys_tmp, uint32_t* vals_tm
         if (e == cudaSuccess) e = cudaMemcpyAsync(vals_out, vals, sizeof(uint32_t) * (size_t)n, cudaMemcpyDeviceToDevice, s);
         return e;
     }
-    if (n >= (int64_t)OS_VAL || (n_bits + 7) / 8 > OS_MAX_PASSES) {
-        // counts beyond the 30-bit status words: reduce-then-scan passes, then a copy to the outputs
-        K* kk = keys;
-        uint32_t* vv = vals;
-        cudaError_t e = radix_impl<K>(kk, vv, keys_tmp, vals_tmp, n, n_bits, ar, s);
-        if (e != cudaSuccess) return e;
-        if (!keys_out) keys_out = kk;
-        if (keys_out != kk) e = cudaMemcpyAsync(keys_out, kk, sizeof(K) * (size_t)n, cudaMemcpyDeviceToDevice, s);
-        if (e == cudaSuccess && vals_out != vv)
-            e = cudaMemcpyAsync(vals_out, vv, sizeof(uint32_t) * (size_t)n, cudaMemcpyDeviceToDevice, s);
-        return e;
-    }
+    if (large_sort(n, sm_count()))
+        return counted_passes<K, OL_ITEMS>(keys, vals, keys_tmp, vals_tmp, &keys_out, vals_out, n, n_bits, hist, words, call_err, s);
     switch (onesweep_rounds(n, sm_count())) {
     case 1: return counted_passes<K, 1>(keys, vals, keys_tmp, vals_tmp, &keys_out, vals_out, n, n_bits, hist, words, call_err, s);
     case 2: return counted_passes<K, 2>(keys, vals, keys_tmp, vals_tmp, &keys_out, vals_out, n, n_bits, hist, words, call_err, s);
@@ -549,6 +607,7 @@ cudaError_t sort_counted(K* keys, uint32_t* vals, K* keys_tmp, uint32_t* vals_tm
 }  // namespace
 
 int64_t sort_counted_words(int64_t n, int n_bits) {
+    if (large_sort(n, sm_count())) return ol_words(n);
     const int passes = (n_bits + 7) / 8;
     const int64_t per_tile = (int64_t)OS_THREADS * onesweep_rounds(n, sm_count());
     const int64_t n_tiles = (n + per_tile - 1) / per_tile;
@@ -634,13 +693,10 @@ cudaError_t scan_u32_to_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32
     return scan_impl<uint32_t, uint32_t>(in, out, n, total_dev, ar, s);
 }
 
-// one-sweep passes while the counts fit the 30-bit status words, reduce-then-scan passes beyond
 cudaError_t radix_sort_u64(uint64_t*& keys, uint32_t*& vals, uint64_t* keys_alt, uint32_t* vals_alt, int64_t n,
                            int n_bits, Arena& ar, cudaStream_t s, uint32_t* call_err) {
     if (n <= 1 || n_bits <= 0) return cudaSuccess;
-    if (n < (int64_t)OS_VAL && (n_bits + 7) / 8 <= OS_MAX_PASSES)
-        return onesweep<uint64_t>(keys, vals, keys_alt, vals_alt, n, n_bits, call_err, ar, s);
-    return radix_impl<uint64_t>(keys, vals, keys_alt, vals_alt, n, n_bits, ar, s);
+    return onesweep<uint64_t>(keys, vals, keys_alt, vals_alt, n, n_bits, call_err, ar, s);
 }
 
 }  // namespace dv
