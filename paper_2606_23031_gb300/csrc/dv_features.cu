@@ -6,14 +6,14 @@
 // and weights w = T alpha in slots [off[p], off[p+1]).  Then
 //   render:  F[p][c]  = sum_slots w * feat[voxel][c]
 //   fuse:    acc[v][c] += sum over the slots of voxel v of w * F2d[p][c],  wsum[v] += w
-// Render: one warp per pixel.  When C is a multiple of 4 whose quads divide the warp (C = 4, 8,
-// ..., 64, 128) a lane owns a 16-byte quad of channels and the warp covers 32 / (C / 4) slots at
-// once; other C take one lane per channel, 32 channels per pass over the slots.
+// Render: a group of lanes per pixel, a lane per 16-byte quad of channels (or per channel).
 // Fusion: adding every slot into its voxel's row with its own atomics is bound by the L2's
 // atomic rate (one add per slot and channel), so the slots of a chunk of consecutive pixels are
 // grouped by voxel in shared memory and each voxel's sum over the chunk is added once.
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <algorithm>
 
 #include "dv_internal.cuh"
 
@@ -21,59 +21,96 @@ namespace dv {
 
 namespace {
 
-constexpr int FT_WARPS = 8;  // pixels per 256-thread block
+// ---- render ----
+// A row of U units (16-byte quads where the rows allow, else floats; at most 32 a pass) takes a group of U lanes, and
+// every group of a warp takes a pixel of its own, so no sums are brought together.  A group reads U slots of
+// its pixel at once, a chunk ahead, into shared memory and loads the feature rows of four slots before it uses
+// them.  (A warp per pixel with its slots loaded as they came was a chain of dependent loads, and the groups' sums
+// cost as much again as their slots: 64 channels on a 1080p frame 755 us, this way 572 us; 40 channels on
+// a quarter of it, then a lane per channel, 333 us, now 119 us.)
+constexpr int FT_WARPS = 8;
+constexpr int FT_PIX = 8;  // pixels per warp, or one per group where the groups are more
 
-// Scalar path (any C): one lane per channel, 32 channels per pass over the slots.
+__device__ __forceinline__ void ft_fma(float4& a, float w, float4 f) {
+    a.x = fmaf(w, f.x, a.x);
+    a.y = fmaf(w, f.y, a.y);
+    a.z = fmaf(w, f.z, a.z);
+    a.w = fmaf(w, f.w, a.w);
+}
+__device__ __forceinline__ void ft_fma(float& a, float w, float f) { a = fmaf(w, f, a); }
+__device__ __forceinline__ void ft_zero(float4& a) { a = make_float4(0.f, 0.f, 0.f, 0.f); }
+__device__ __forceinline__ void ft_zero(float& a) { a = 0.0f; }
+
+// T: float4 or float; U: units of a row; rounds: pixels per group; grid.y: passes of 32 units
+template <typename T>
 __global__ void __launch_bounds__(FT_WARPS * 32) k_feat_render(int64_t n_pix, const int64_t* __restrict__ off,
                                                                const uint32_t* __restrict__ vox,
                                                                const float* __restrict__ wgt,
-                                                               const float* __restrict__ feat, int C,
-                                                               float* __restrict__ out) {
-    const int lane = threadIdx.x & 31;
-    const int64_t p = (int64_t)blockIdx.x * FT_WARPS + (threadIdx.x >> 5);
-    if (p >= n_pix) return;
-    const int64_t e0 = off[p], e1 = off[p + 1];
-    for (int c0 = 0; c0 < C; c0 += 32) {
-        const int c = c0 + lane;
-        float acc = 0.0f;
-        for (int64_t e = e0; e < e1; ++e) {
-            const float w = __ldg(wgt + e);
-            const uint32_t v = __ldg(vox + e);
-            if (c < C) acc = fmaf(w, __ldg(feat + (size_t)v * C + c), acc);
+                                                               const T* __restrict__ feat, int U, int rounds,
+                                                               T* __restrict__ out) {
+    constexpr int STEPS = 4;
+    __shared__ uint2 s_slot[FT_WARPS][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int u0 = blockIdx.y * 32, G = min(U - u0, 32);
+    const int S = 32 / G, g = lane / G, j = lane - g * G;
+    const int64_t p0 = ((int64_t)blockIdx.x * FT_WARPS + warp) * S * rounds;
+    if (p0 >= n_pix) return;
+    uint2* mine = &s_slot[warp][g < S ? g * G : 0];
+    const T* col = feat + u0 + j;
+    // the group's pixels p0 + g, p0 + g + S, ...: slot range of the next one, read a pixel ahead
+    int64_t na = 0;
+    int nn = 0;
+    auto range = [&](int r) {
+        const int64_t p = p0 + (int64_t)r * S + g;
+        nn = 0;
+        if (r < rounds && g < S && p < n_pix) {
+            na = off[p];
+            nn = (int)(off[p + 1] - na);
         }
-        if (c < C) out[(size_t)p * C + c] = acc;
+    };
+    range(0);
+    for (int r = 0; r < rounds; ++r) {
+        const int64_t p = p0 + (int64_t)r * S + g;
+        const uint32_t* pv = vox + na;
+        const float* pw = wgt + na;
+        const int n = nn;
+        range(r + 1);
+        const int most = __reduce_max_sync(0xffffffffu, n);
+        T acc;
+        ft_zero(acc);
+        uint32_t v = 0;
+        float w = 0.0f;
+        if (j < n) {
+            v = __ldg(pv + j);
+            w = __ldg(pw + j);
+        }
+        for (int c = 0; c < most; c += G) {
+            __syncwarp();
+            if (g < S) mine[j] = make_uint2(v, __float_as_uint(w));
+            __syncwarp();
+            if (c + G + j < n) {  // the next chunk
+                v = __ldg(pv + c + G + j);
+                w = __ldg(pw + c + G + j);
+            }
+            const int m = n - c, all = min(G, most - c);  // slots of the group's pixel, and of any group's
+            for (int k0 = 0; k0 < all; k0 += STEPS) {
+                uint2 x[STEPS];
+                T f[STEPS];
+#pragma unroll
+                for (int k = 0; k < STEPS; ++k) {
+                    const int i = k0 + k;
+                    if (i < m && i < G) {
+                        x[k] = mine[i];
+                        f[k] = __ldg(col + (size_t)x[k].x * U);
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < STEPS; ++k)
+                    if (k0 + k < m && k0 + k < G) ft_fma(acc, __uint_as_float(x[k].y), f[k]);
+            }
+        }
+        if (g < S && p < n_pix) out[(size_t)p * U + u0 + j] = acc;
     }
-}
-
-// Vector path (C = 4 Q with Q dividing 32): a lane owns one 16-byte quad of channels and the warp
-// walks S = 32 / Q slots at a time, lane group g taking slots e0 + g, e0 + g + S, ...; the S
-// partial sums of a quad are then added across the groups with shuffles.
-__global__ void __launch_bounds__(FT_WARPS * 32) k_feat_render4(int64_t n_pix, const int64_t* __restrict__ off,
-                                                                const uint32_t* __restrict__ vox,
-                                                                const float* __restrict__ wgt,
-                                                                const float4* __restrict__ feat, int Q,
-                                                                float4* __restrict__ out) {
-    const int lane = threadIdx.x & 31;
-    const int64_t p = (int64_t)blockIdx.x * FT_WARPS + (threadIdx.x >> 5);
-    if (p >= n_pix) return;
-    const int S = 32 / Q, q = lane % Q, g = lane / Q;
-    const int64_t e0 = off[p], e1 = off[p + 1];
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int64_t e = e0 + g; e < e1; e += S) {
-        const float w = __ldg(wgt + e);
-        const float4 f = __ldg(feat + (size_t)__ldg(vox + e) * Q + q);
-        acc.x = fmaf(w, f.x, acc.x);
-        acc.y = fmaf(w, f.y, acc.y);
-        acc.z = fmaf(w, f.z, acc.z);
-        acc.w = fmaf(w, f.w, acc.w);
-    }
-    for (int d = Q; d < 32; d <<= 1) {
-        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, d);
-        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, d);
-        acc.z += __shfl_xor_sync(0xffffffffu, acc.z, d);
-        acc.w += __shfl_xor_sync(0xffffffffu, acc.w, d);
-    }
-    if (g == 0) out[(size_t)p * Q + q] = acc;
 }
 
 // ---- fusion by pixel chunks ----
@@ -86,10 +123,11 @@ __global__ void __launch_bounds__(FT_WARPS * 32) k_feat_render4(int64_t n_pix, c
 //  * The slots, FL_PIECE at a time, get a row from an open-addressing table keyed by the voxel
 //    index (compare-and-swap inserts, FL_ROWS rows); a voxel that finds no row within FL_PROBES
 //    probes goes to the overflow row, whose slots are added to the global sums one by one.
-//  * A counting sort by row groups the piece's slots and lists the rows that hold any; warp w takes
-//    listed rows w, w + 8, ...: its four 8-lane groups walk every fourth slot of the row, a lane
-//    holding two 4-channel quads of the sums in registers, and the groups' sums are added by
-//    shuffles before one atomic add per quad.
+//  * A counting sort by row groups the piece's slots and lists the rows that hold any; every half-warp
+//    takes rows of its own, a lane holding one 4-channel quad of the sum in a register until one
+//    atomic add per quad.  A row of a 128-pixel run holds some 16 slots, so what a row costs
+//    besides them counts: with a warp per row, its sums in four groups brought together by 18 shuffles, 64
+//    channels on a 1080p frame took 1,110 us, this way 758 us.
 constexpr int FL_PIX = 128;     // pixels per chunk
 constexpr int FL_SW = 64;       // channels per slice (16 quads)
 constexpr int FL_ROWS = 1023;   // voxel rows; row FL_ROWS holds the overflow slots
@@ -110,9 +148,8 @@ struct FuseSmem {
     uint32_t n_occ;
     uint32_t wtot[FL_THREADS / 32];   // scan: warp totals (slots, then rows)
     uint32_t wocc[FL_THREADS / 32];
-    float sw[FL_PIECE];               // grouped by row: the slot's weight,
-    uint16_t order[FL_PIECE];         //   its index in the piece,
-    uint8_t spl[FL_PIECE];            //   and its pixel within the chunk
+    uint2 slot[FL_PIECE];             // grouped by row: the slot's weight; its pixel within the chunk | its index in
+                                      //   the piece << 16
 };
 
 __device__ __forceinline__ uint32_t fl_hash(uint32_t v) { return ((v * 2654435761u) >> 16) % FL_ROWS; }
@@ -124,13 +161,6 @@ __device__ __forceinline__ void fl_cp_async16(void* smem, const void* gmem) {
 }
 __device__ __forceinline__ void fl_cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void fl_cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-
-__device__ __forceinline__ void fl_add4(float4& a, float w, float4 f) {
-    a.x = fmaf(w, f.x, a.x);
-    a.y = fmaf(w, f.y, a.y);
-    a.z = fmaf(w, f.z, a.z);
-    a.w = fmaf(w, f.w, a.w);
-}
 
 // adds quad a (channels c .. c + 3, those below C) into row v of the global sums
 template <bool VEC>
@@ -156,7 +186,7 @@ __global__ void __launch_bounds__(FL_THREADS, 3) k_fuse_local(int64_t n_pix, con
     extern __shared__ __align__(16) unsigned char fl_raw[];
     FuseSmem& S = *reinterpret_cast<FuseSmem*>(fl_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int q0 = 2 * (lane & 7), g = lane >> 3;  // first of the lane's two channel quads, 8-lane group
+    const int q = lane & 15, half = lane >> 4;  // the lane's channel quad, its half of the warp
     for (int i = tid; i < FL_ROWS; i += FL_THREADS) S.key[i] = FL_EMPTY;
     const int64_t n_chunks = (n_pix + FL_PIX - 1) / FL_PIX;
     const int n_slices = (C + FL_SW - 1) / FL_SW;
@@ -279,60 +309,39 @@ __global__ void __launch_bounds__(FL_THREADS, 3) k_fuse_local(int64_t n_pix, con
                 if (k < ns) {
                     const uint32_t row = r_[j] & 0xffffu;
                     const uint32_t pos = S.start[row] + atomicAdd(&S.cnt[row], 1u);
-                    S.sw[pos] = w_[j];
-                    S.order[pos] = (uint16_t)k;
-                    S.spl[pos] = (uint8_t)(r_[j] >> 16);
+                    S.slot[pos] = make_uint2(__float_as_uint(w_[j]), (r_[j] >> 16) | ((uint32_t)k << 16));
                 }
             }
             if (VEC && e0 == S.off[0]) fl_cp_async_wait_all();  // the feature slice has landed
             __syncthreads();
-            // per row with slots: the warp's four 8-lane groups take every fourth slot, a lane holding
-            // two 4-channel quads (q0, q0 + 1) of the sums in registers
+            // a half-warp per row with slots, a lane per 4-channel quad: no sums to bring together
             const uint32_t n_occ = S.n_occ;
-            for (uint32_t oi = warp; oi < n_occ; oi += FL_THREADS / 32) {
+            for (uint32_t oi = 2 * warp + half; oi < n_occ; oi += FL_THREADS / 16) {
                 const uint32_t r = S.occ[oi];
                 const uint32_t s0 = S.start[r], s1 = S.start[r + 1];
                 if (r < FL_ROWS) {
-                    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+                    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
                     float ws = 0.0f;
-#pragma unroll 2
-                    for (uint32_t i = s0 + g; i < s1; i += 4) {
-                        const float wv = S.sw[i];
-                        const float4* fr = S.f[S.spl[i]];
-                        fl_add4(a, wv, fr[q0]);
-                        fl_add4(b, wv, fr[q0 + 1]);
+#pragma unroll 4
+                    for (uint32_t i = s0; i < s1; ++i) {
+                        const uint2 x = S.slot[i];
+                        const float wv = __uint_as_float(x.x);
+                        ft_fma(a, wv, S.f[x.y & 0xffffu][q]);
                         ws += wv;
                     }
-#pragma unroll
-                    for (int d = 8; d < 32; d <<= 1) {
-                        a.x += __shfl_xor_sync(0xffffffffu, a.x, d);
-                        a.y += __shfl_xor_sync(0xffffffffu, a.y, d);
-                        a.z += __shfl_xor_sync(0xffffffffu, a.z, d);
-                        a.w += __shfl_xor_sync(0xffffffffu, a.w, d);
-                        b.x += __shfl_xor_sync(0xffffffffu, b.x, d);
-                        b.y += __shfl_xor_sync(0xffffffffu, b.y, d);
-                        b.z += __shfl_xor_sync(0xffffffffu, b.z, d);
-                        b.w += __shfl_xor_sync(0xffffffffu, b.w, d);
-                        ws += __shfl_xor_sync(0xffffffffu, ws, d);
-                    }
                     const uint32_t v = S.key[r];
-                    if (g == 0) {
-                        fl_flush4<VEC>(acc, v, C, c0 + 4 * q0, a);
-                        fl_flush4<VEC>(acc, v, C, c0 + 4 * q0 + 4, b);
-                    }
-                    if (lane == 0 && wsum && c0 == 0 && ws != 0.0f) atomicAdd(wsum + v, ws);
+                    fl_flush4<VEC>(acc, v, C, c0 + 4 * q, a);
+                    if (q == 0 && wsum && c0 == 0 && ws != 0.0f) atomicAdd(wsum + v, ws);
                 } else {
                     // overflow row: every slot added on its own
-                    for (uint32_t i = s0 + g; i < s1; i += 4) {
-                        const float wv = S.sw[i];
-                        const uint32_t v = __ldg(vox + e0 + S.order[i]);
-                        const float4* fr = S.f[S.spl[i]];
-                        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-                        fl_add4(a, wv, fr[q0]);
-                        fl_add4(b, wv, fr[q0 + 1]);
-                        fl_flush4<VEC>(acc, v, C, c0 + 4 * q0, a);
-                        fl_flush4<VEC>(acc, v, C, c0 + 4 * q0 + 4, b);
-                        if (q0 == 0 && wsum && c0 == 0 && wv != 0.0f) atomicAdd(wsum + v, wv);
+                    for (uint32_t i = s0; i < s1; ++i) {
+                        const uint2 x = S.slot[i];
+                        const float wv = __uint_as_float(x.x);
+                        const uint32_t v = __ldg(vox + e0 + (x.y >> 16));
+                        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+                        ft_fma(a, wv, S.f[x.y & 0xffffu][q]);
+                        fl_flush4<VEC>(acc, v, C, c0 + 4 * q, a);
+                        if (q == 0 && wsum && c0 == 0 && wv != 0.0f) atomicAdd(wsum + v, wv);
                     }
                 }
             }
@@ -343,23 +352,23 @@ __global__ void __launch_bounds__(FL_THREADS, 3) k_fuse_local(int64_t n_pix, con
     }
 }
 
-// the 16-byte render path needs C = 4 Q with Q a divisor of 32 and 16-byte aligned rows
-bool quad_path(int C, const void* a, const void* b) {
-    if (C % 4 != 0 || C / 4 > 32 || 32 % (C / 4) != 0) return false;
-    return ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15) == 0;
-}
-
 }  // namespace
 
 cudaError_t launch_feat_render(int64_t n_pix, const int64_t* off, const uint32_t* vox, const float* wgt,
                                const float* feat, int C, float* out, cudaStream_t s) {
     if (n_pix <= 0 || C <= 0) return cudaSuccess;
-    const unsigned grid = (unsigned)((n_pix + FT_WARPS - 1) / FT_WARPS);
-    if (quad_path(C, feat, out))
-        k_feat_render4<<<grid, FT_WARPS * 32, 0, s>>>(n_pix, off, vox, wgt, reinterpret_cast<const float4*>(feat),
-                                                      C / 4, reinterpret_cast<float4*>(out));
+    // 16-byte units need rows of a multiple of 16 bytes on 16-byte boundaries
+    const bool quads = C % 4 == 0 && ((reinterpret_cast<uintptr_t>(feat) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
+    const int U = quads ? C / 4 : C;
+    const int S = 32 / std::min(U, 32), rounds = std::max(1, FT_PIX / S);
+    // a last pass of fewer units has more groups, so its blocks cover more pixels than the grid's x asks for
+    const int64_t per_block = (int64_t)FT_WARPS * S * rounds;
+    const dim3 grid((unsigned)((n_pix + per_block - 1) / per_block), (unsigned)((U + 31) / 32));
+    if (quads)
+        k_feat_render<float4><<<grid, FT_WARPS * 32, 0, s>>>(n_pix, off, vox, wgt, reinterpret_cast<const float4*>(feat), U, rounds,
+                                                             reinterpret_cast<float4*>(out));
     else
-        k_feat_render<<<grid, FT_WARPS * 32, 0, s>>>(n_pix, off, vox, wgt, feat, C, out);
+        k_feat_render<float><<<grid, FT_WARPS * 32, 0, s>>>(n_pix, off, vox, wgt, feat, U, rounds, out);
     count_launches(1);
     return cudaGetLastError();
 }
