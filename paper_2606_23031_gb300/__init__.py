@@ -636,8 +636,16 @@ def _autograd_fn():
             n = ctx_.n
             st = ctx_.state
             dev = next(g.device for g in (g_rgb, g_depth, g_alpha, g_normal) if g is not None)
-            d_dens = [T.zeros(s[0], device=dev, dtype=T.float32) for s in ctx_.shapes]
-            d_sh = [T.zeros(s[1], device=dev, dtype=T.float32) for s in ctx_.shapes]
+            shapes = [s[0] for s in ctx_.shapes] + [s[1] for s in ctx_.shapes]
+            if n == 1:
+                grads = [T.zeros(s, device=dev, dtype=T.float32) for s in shapes]
+            else:
+                # one zeroed buffer for all gradients, each starting on a 16-byte boundary: a tensor of its own for each
+                # is a launch and some 20 us of host time for each (with one octree the views cost as much)
+                sizes = [(s.numel() + 3) // 4 * 4 for s in shapes]
+                flat = T.zeros(sum(sizes), device=dev, dtype=T.float32)
+                grads = [b[:s.numel()].view(s) for b, s in zip(flat.split(sizes), shapes)]
+            d_dens, d_sh = grads[:n], grads[n:]
             c = lambda t: None if t is None else t.contiguous()
             dv_render_backward(st, c(g_rgb), c(g_depth), c(g_alpha), d_dens, d_sh,
                                d_normal=c(g_normal) if ctx_.normals else None)
