@@ -122,12 +122,12 @@ const char* dv_last_error(const dv_ctx* ctx);
 /* Library version string. */
 const char* dv_version(void);
 /*
- * Bounded waits.  The one-sweep radix sort's look-back is the library's only
- * wait on other thread blocks (it waits only on tiles that started earlier, so
- * it ends); each spin is bounded, and a bound that runs out marks two words:
- *  - the call's own flag.  Calls that sort and synchronise anyway (feature
- *    fusion, the initialisation calls) read it before they return and fail
- *    with DV_ERR_TIMEOUT.  A render publishes it, after its last sort, into a
+ * Bounded waits.  The look-backs of the one-sweep radix sort and of the records
+ * kernel are the library's only waits on other thread blocks (they wait only on
+ * blocks that started earlier, so they end); each spin is bounded, and a bound
+ * that runs out marks two words:
+ *  - the call's own flag.  dv_shared_corners, which sorts and synchronises
+ *    anyway, reads it before it returns and fails with DV_ERR_TIMEOUT.  A render publishes it, after its last sort, into a
  *    host word of its saved state: dv_state_check reports it, the backward of
  *    that state refuses to run once it is known, and the serving loop fails
  *    the batch's requests.
@@ -411,7 +411,7 @@ dv_status dv_state_stats(const dv_state* state, int32_t view, int64_t* n_visible
 
 /* Work done by the forward compositing of a saved state, over all its views
  * (`view` must be -1, or 0 for a single-view state): voxel slab tests (pixel x
- * list entry examined), actor clip-box tests, and composited segments.
+ * list entry whose pixel rectangle covers it), actor clip-box tests, and composited segments.
  * Synchronises the state's stream.  These are the algorithmic units behind the
  * compositing roofline. */
 dv_status dv_state_work(const dv_state* state, int32_t view, uint64_t* tests, uint64_t* box_tests,

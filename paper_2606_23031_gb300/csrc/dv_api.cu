@@ -1282,16 +1282,17 @@ dv_status dv_features_fuse(dv_ctx* ctx, int64_t n_pix, const int64_t* offsets, c
 // ---- LiDAR-guided initialisation (Sec. 3.3) ----
 
 static dv_status init_begin(dv_ctx* ctx, const uint64_t* keys, int64_t n, int32_t max_level, dv::Arena& ar,
-                            cudaStream_t s) {
+                            cudaStream_t s, bool* outside = nullptr) {
     if (!ctx) return DV_ERR_INVALID_ARG;
     ctx->err.clear();
     if (n < 0 || (n > 0 && !keys)) return fail(ctx, DV_ERR_INVALID_ARG, "bad key array");
     if (n > ((int64_t)1 << 28)) return fail(ctx, DV_ERR_CAPACITY, "more than 2^28 leaves");
     if (max_level < 0 || max_level > 18) return fail(ctx, DV_ERR_INVALID_ARG, "max_level out of range (0..18)");
-    uint32_t lv = 0;
-    cudaError_t e = dv::key_levels(keys, n, &lv, ar, s);
+    uint32_t lv[2] = {0, 0};
+    cudaError_t e = dv::key_levels(keys, n, lv, ar, s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "key levels");
-    if (lv >> (max_level + 1)) return fail(ctx, DV_ERR_INVALID_ARG, "a leaf level above max_level");
+    if (lv[0] >> (max_level + 1)) return fail(ctx, DV_ERR_INVALID_ARG, "a leaf level above max_level");
+    if (outside) *outside = lv[1] != 0;
     return DV_OK;
 }
 
@@ -1306,10 +1307,11 @@ dv_status dv_shared_corners(dv_ctx* ctx, const uint64_t* keys, int64_t n, int32_
     dv::Arena ar;
     ar.pool = ctx ? ctx->pool : nullptr;
     ar.stream = s;
-    dv_status st = init_begin(ctx, keys, n, max_level, ar, s);
+    bool outside = false;
+    dv_status st = init_begin(ctx, keys, n, max_level, ar, s, &outside);
     cudaError_t e = cudaSuccess;
     bool timeout = false;
-    if (st == DV_OK) e = dv::shared_corners(keys, n, max_level, grid, index, n_corners, ar, s, &timeout);
+    if (st == DV_OK) e = dv::shared_corners(keys, n, max_level, outside, grid, index, n_corners, ar, s, &timeout);
     ar.release();
     if (st != DV_OK) return st;
     if (e != cudaSuccess) return cuda_fail(ctx, e, "shared corners");

@@ -1,47 +1,42 @@
 // Front-to-back compositing over each ray's voxel segments (forward) and its
-// replay with gradients (backward), plus the SH-colour backward.
+// replay with gradients (backward), plus the SH-colour backward (Sec. 3.4, Alg. 1).
 //
-// Each CTA renders half of a 16x16 tile (16x8 pixels, 4 warps of 8x4 pixels),
-// one thread per pixel, tiles taken heaviest first (Sec. 3.4, Alg. 1):
 //  * The tile's pair list is grouped by octree and, inside an octree, sorted
 //    front to back for every ray of the camera (depth-order key, see
 //    dv_project.cu).
-//  * Each pixel splits its ray into background and actor intervals with the
-//    actor clip boxes (slab test in each actor's frame, reached through the
-//    inverse pose; the box entered first owns any overlap).
-//  * Every sub-list (each actor's, the background's) streams through a two-slot
-//    shared-memory ring (cp.async, one batch ahead); each warp visits, in list
-//    order and in lockstep, the records that touch its 8x4 pixel block.
-//  * Phase 1: for every actor of the tile, nearest first, every lane composites
-//    the segments inside its own interval of that actor into a partial
-//    (C_A, D_A, T_A) starting from T = 1, unless the partials of its earlier
-//    intervals already hide it.
-//  * Phase 2: the background sub-list.  A background hit that reaches past the
-//    next actor's entry composites its part in front of the box, then applies
-//    that actor's partial with the running transmittance (C += T C_A,
-//    D += T D_A, T *= T_A), then continues behind the box.  If T T_A < eps_stop
-//    the ray stops inside the actor: at the partial's last segment (the whole
-//    partial applies) if T times the transmittance before it is not below
-//    eps_stop; else the lane records its state for a replay.
-//  * Phase 3: lanes left to replay walk that actor's sub-list from the recorded
-//    state with the exact stop rule.
+//  * Tiles that no actor clip box covers are composited here: each CTA renders
+//    half of a 16x16 tile (16x8 pixels, 4 warps of 8x4 pixels), one thread per
+//    pixel, tiles taken heaviest first; the list streams through a two-slot
+//    shared-memory ring (cp.async, one batch ahead).
+//  * In the other tiles each pixel splits its ray into background and actor
+//    intervals with the actor clip boxes (slab test in each actor's frame,
+//    reached through the inverse pose; the box entered first owns any
+//    overlap).  dv_composite_act.cu has them, in three phases:
+//     1. every interval's segments into a partial (C_A, D_A, T_A) starting from
+//        T = 1, nearest first, unless the partials of the ray's earlier intervals
+//        already hide it.
+//     2. the background sub-list.  A background hit that reaches past the next
+//        actor's entry composites its part in front of the box, then applies
+//        that actor's partial with the running transmittance (C += T C_A,
+//        D += T D_A, T *= T_A), then continues behind the box.  If T T_A < eps_stop
+//        the ray stops inside the actor: at the partial's last segment (the whole
+//        partial applies) if T times the transmittance before it is not below
+//        eps_stop; else the state is recorded for a replay.
+//     3. replays walk that actor's sub-list from the recorded state with the
+//        exact stop rule.
 //    Since T only decreases along the ray, applying a whole partial is exact
 //    unless the stop falls inside it, which is exactly when T T_A < eps_stop.
 //  * Per segment: trilinear interpolation of the raw corner densities at K
 //    midpoints, exponential-linear activation, tau = l/K sum sigma,
 //    alpha = 1 - exp(-tau), C += T alpha c, D += T alpha (t0+t1)/2,
 //    T *= 1 - alpha, stop once T < eps_stop.
-//  * The backward runs the same three phases (identical arithmetic, so the same
+//  * The backward runs the same phases (identical arithmetic, so the same
 //    stops).  With w_k = T_k alpha_k it uses
 //    dC/dtau_k = T_{k+1} c_k - sum_{j>k} w_j c_j, the suffix sum being
 //    C_final - (prefix through k), so it needs no division by (1 - alpha) and
 //    no reverse traversal.  Phase 2 records, for every actor interval reached,
 //    the prefix state at its entry; phase 3 then replays every reached actor
-//    interval with gradients from that state.  Gradients of records visited in
-//    lockstep are reduced across the warp before the atomics.
-//  * A ray with more actor intervals than slots (4, or 8 where 5 or more boxes
-//    cover the tile) handles those beyond with a per-lane walk of the actor's
-//    sub-list (correct, but divergent).
+//    interval with gradients from that state.
 #include "dv_composite.cuh"
 
 namespace dv {

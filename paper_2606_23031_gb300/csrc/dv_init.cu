@@ -40,10 +40,11 @@ __device__ __forceinline__ uint64_t pack_grid(uint64_t x, uint64_t y, uint64_t z
     return (z << 42) | (y << 21) | x;
 }
 
-// corner points as sort keys of 3 (max_level + 1) bits (a coordinate is at most 2^max_level): the same order as
-// the packed points, in fewer radix passes (5 instead of 8 at level 12)
-__global__ void k_corner_emit(const uint64_t* __restrict__ keys, int64_t n, int max_level, uint64_t* __restrict__ ck,
-                              uint32_t* __restrict__ cv) {
+// corner points as sort keys of 3 b bits, b = max_level + 1 (a coordinate of a leaf inside the root is at most
+// 2^max_level): the same order as the packed points, in fewer radix passes (5 instead of 8 at level 12).  b = 21, the
+// packed point itself, where some leaf lies outside the root.
+__global__ void k_corner_emit(const uint64_t* __restrict__ keys, int64_t n, int max_level, int b,
+                              uint64_t* __restrict__ ck, uint32_t* __restrict__ cv) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n * 8) return;
     const int64_t v = t >> 3;
@@ -54,7 +55,6 @@ __global__ void k_corner_emit(const uint64_t* __restrict__ keys, int64_t n, int 
     const uint64_t i = ((k & kIMask) + (c & 1)) << sh;
     const uint64_t j = (((k >> 19) & kIMask) + ((c >> 1) & 1)) << sh;
     const uint64_t kk = (((k >> 38) & kIMask) + ((c >> 2) & 1)) << sh;
-    const int b = max_level + 1;
     ck[t] = (kk << (2 * b)) | (j << b) | i;
     cv[t] = (uint32_t)t;
 }
@@ -68,13 +68,12 @@ __global__ void k_corner_flag(const uint64_t* __restrict__ sk, int64_t m, uint32
 // pos = exclusive scan of first: sorted entry t belongs to distinct point pos[t] + first[t] - 1
 __global__ void k_corner_assign(const uint64_t* __restrict__ sk, const uint32_t* __restrict__ sv,
                                 const uint32_t* __restrict__ first, const uint32_t* __restrict__ pos, int64_t m,
-                                int max_level, uint64_t* __restrict__ grid_out, uint32_t* __restrict__ index_out) {
+                                int b, uint64_t* __restrict__ grid_out, uint32_t* __restrict__ index_out) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= m) return;
     const uint32_t id = pos[t] + first[t] - 1u;
     index_out[sv[t]] = id;
     if (first[t]) {
-        const int b = max_level + 1;
         const uint64_t k = sk[t], m1 = (1ull << b) - 1;
         grid_out[id] = pack_grid(k & m1, (k >> b) & m1, k >> (2 * b));
     }
@@ -498,13 +497,19 @@ __global__ void k_corner_scatter(const uint32_t* __restrict__ index, int64_t n8,
     if (g != 0.0f) atomicAdd(d_corner + index[t], g);
 }
 
-// levels of the keys (bit mask), to validate against max_level
+// levels of the keys (bit mask), to validate against max_level, and whether some key's index is outside its level's grid
 __global__ void __launch_bounds__(256) k_levels(const uint64_t* __restrict__ keys, int64_t n, uint32_t* __restrict__ levels) {
-    uint32_t lev = 0;
-    for (int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x; t < n; t += (int64_t)gridDim.x * 256)
-        lev |= 1u << ((keys[t] >> 57) & 31);
+    uint32_t lev = 0, outside = 0;
+    for (int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x; t < n; t += (int64_t)gridDim.x * 256) {
+        const uint64_t k = keys[t];
+        const int l = (int)((k >> 57) & 31);
+        lev |= 1u << l;
+        outside |= (((k & kIMask) | ((k >> 19) & kIMask) | ((k >> 38) & kIMask)) >> l) != 0 ? 1u : 0u;
+    }
     lev = __reduce_or_sync(0xffffffffu, lev);
+    outside = __reduce_or_sync(0xffffffffu, outside);
     if ((threadIdx.x & 31) == 0 && (lev & ~*(volatile uint32_t*)levels)) atomicOr(levels, lev);
+    if ((threadIdx.x & 31) == 0 && outside) levels[1] = 1u;
 }
 
 // A leaf is kept if its box top reaches z_min and some camera sees it (see the header).  A camera's verdict comes
@@ -665,26 +670,27 @@ cudaError_t corner_scatter(const uint32_t* index, int64_t n, const float* d_dens
     return cudaGetLastError();
 }
 
-cudaError_t key_levels(const uint64_t* keys, int64_t n, uint32_t* levels_host, Arena& ar, cudaStream_t s) {
-    *levels_host = 0;
+cudaError_t key_levels(const uint64_t* keys, int64_t n, uint32_t levels_host[2], Arena& ar, cudaStream_t s) {
+    levels_host[0] = levels_host[1] = 0;
     if (n <= 0) return cudaSuccess;
-    uint32_t* d = ar.alloc<uint32_t>(1);
+    uint32_t* d = ar.alloc<uint32_t>(2);
     if (!d) return ar.err;
-    cudaError_t e = cudaMemsetAsync(d, 0, sizeof(uint32_t), s);
+    cudaError_t e = cudaMemsetAsync(d, 0, 2 * sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
     k_levels<<<std::min<unsigned>(nb(n), 2u * (unsigned)sm_count()), 256, 0, s>>>(keys, n, d);
     count_launches(1);
-    e = cudaMemcpyAsync(levels_host, d, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+    e = cudaMemcpyAsync(levels_host, d, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     return e;
 }
 
-cudaError_t shared_corners(const uint64_t* keys, int64_t n, int max_level, uint64_t* grid_out, uint32_t* index_out,
-                           int64_t* n_corners, Arena& ar, cudaStream_t s, bool* sort_timeout) {
+cudaError_t shared_corners(const uint64_t* keys, int64_t n, int max_level, bool outside, uint64_t* grid_out,
+                           uint32_t* index_out, int64_t* n_corners, Arena& ar, cudaStream_t s, bool* sort_timeout) {
     *n_corners = 0;
     *sort_timeout = false;
     if (n <= 0) return cudaSuccess;
     const int64_t m = n * 8;
+    const int b = outside ? 21 : max_level + 1;  // bits of a coordinate
     uint64_t* k0 = ar.alloc<uint64_t>(m);
     uint64_t* k1 = ar.alloc<uint64_t>(m);
     uint32_t* v0 = ar.alloc<uint32_t>(m);
@@ -695,17 +701,17 @@ cudaError_t shared_corners(const uint64_t* keys, int64_t n, int max_level, uint6
     if (ar.err != cudaSuccess) return ar.err;
     cudaError_t e = cudaMemsetAsync(total + 1, 0, sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
-    k_corner_emit<<<nb(m), 256, 0, s>>>(keys, n, max_level, k0, v0);
+    k_corner_emit<<<nb(m), 256, 0, s>>>(keys, n, max_level, b, k0, v0);
     count_launches(1);
     uint64_t* kk = k0;
     uint32_t* vv = v0;
-    e = radix_sort_u64(kk, vv, k1, v1, m, 3 * (max_level + 1), ar, s, total + 1);
+    e = radix_sort_u64(kk, vv, k1, v1, m, 3 * b, ar, s, total + 1);
     if (e != cudaSuccess) return e;
     k_corner_flag<<<nb(m), 256, 0, s>>>(kk, m, first);
     count_launches(1);
     e = scan_u32_to_u32(first, pos, m, total, ar, s);
     if (e != cudaSuccess) return e;
-    k_corner_assign<<<nb(m), 256, 0, s>>>(kk, vv, first, pos, m, max_level, grid_out, index_out);
+    k_corner_assign<<<nb(m), 256, 0, s>>>(kk, vv, first, pos, m, b, grid_out, index_out);
     count_launches(1);
     uint32_t h[2] = {0, 0};
     e = cudaMemcpyAsync(h, total, sizeof(h), cudaMemcpyDeviceToHost, s);

@@ -267,8 +267,9 @@ cudaError_t feat_fuse(int64_t n_pix, const int64_t* off, const uint32_t* vox, co
 
 // LiDAR-guided initialisation (see dv_init.cu); the calls that return a size synchronise the stream.
 // shared_corners sorts: it sets *sort_timeout (host) when the sort's bounded wait ran out.
-cudaError_t key_levels(const uint64_t* keys, int64_t n, uint32_t* levels_host, Arena& ar, cudaStream_t s);
-cudaError_t shared_corners(const uint64_t* keys, int64_t n, int max_level, uint64_t* grid_out, uint32_t* index_out,
+// levels_host: the keys' levels as a bit mask, and 1 where some key's index is outside its level's grid
+cudaError_t key_levels(const uint64_t* keys, int64_t n, uint32_t levels_host[2], Arena& ar, cudaStream_t s);
+cudaError_t shared_corners(const uint64_t* keys, int64_t n, int max_level, bool outside, uint64_t* grid_out, uint32_t* index_out,
                            int64_t* n_corners, Arena& ar, cudaStream_t s, bool* sort_timeout);
 cudaError_t soft_prior(const uint64_t* grid, int64_t n_corners, const double* center, double root_size, int max_level,
                        const float* cloud, int64_t m, float s_min, float v_close, float v_far, float* dens, Arena& ar,
