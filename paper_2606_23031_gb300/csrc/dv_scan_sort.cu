@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(OS_THREADS) k_os_pass(const K* __restrict__ ke
 constexpr int OL_ITEMS = 16;
 constexpr int OL_TILE = OS_THREADS * OL_ITEMS;
 
-// per-warp digit counts of a tile's keys; with `place`, each key's rank among its warp's keys of the digit
+// per-warp digit counts of a tile's keys, and each key's rank among its warp's keys of the digit
 template <typename K>
 __device__ __forceinline__ void rank_warp(const K* key, int64_t first, int64_t n, int shift, uint32_t mask,
                                           uint32_t* mine, uint32_t* place) {
@@ -344,11 +344,12 @@ __device__ __forceinline__ void rank_warp(const K* key, int64_t first, int64_t n
         __syncwarp();
         if (ok && (peers & lt) == 0u) mine[d] = before + __popc(peers);
         __syncwarp();
-        if (place) place[i] = before + __popc(peers & lt);
+        place[i] = before + __popc(peers & lt);
     }
 }
 
-// hist[digit][tile]
+// hist[digit][tile].  Shared atomics that return nothing: equal digits of a warp add up at once (with the scatter's
+// matches instead 31 us a pass of 6M keys, so 20 us; 32M-leaf 4K render 6.52 -> 6.29 ms)
 template <typename K>
 __global__ void __launch_bounds__(OS_THREADS) k_ol_count(const K* __restrict__ keys, int64_t n, int shift, uint32_t mask,
                                                          uint32_t* __restrict__ hist) {
@@ -363,7 +364,9 @@ __global__ void __launch_bounds__(OS_THREADS) k_ol_count(const K* __restrict__ k
 #pragma unroll
     for (int i = 0; i < OL_ITEMS; ++i) key[i] = first + 32 * i < n ? keys[first + 32 * i] : K(0);
     __syncthreads();
-    rank_warp<K>(key, first, n, shift, mask, cnt[warp], nullptr);
+#pragma unroll
+    for (int i = 0; i < OL_ITEMS; ++i)
+        if (first + 32 * i < n) atomicAdd(&cnt[warp][(uint32_t)(key[i] >> shift) & mask], 1u);
     __syncthreads();
     uint32_t c = 0;
 #pragma unroll
