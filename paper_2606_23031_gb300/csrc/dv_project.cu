@@ -114,17 +114,17 @@ __device__ __forceinline__ uint32_t side_path(uint32_t idx, int level, int64_t X
     return (1u << top) | (((cell >> top) & 1u ? ~idx : idx) & low);
 }
 
-// Whether voxel gv of `view` may be visible.  Most voxels lie outside the frustum by far: the bounding sphere
+// Whether a leaf of octree o may be visible in `view`.  Most voxels lie outside the frustum by far: the bounding sphere
 // against the near and far planes and the four sides, each side 1.5 pixels outside the image, decides those with a
 // tenth of the arithmetic of the corners.  It leaves out nothing that the corners (project_voxel) would keep: the
 // radius covers the rounding of both (4e-6 of the coordinates' size), and where the sphere comes so close to the
 // camera plane that its projection exceeds 2e5 pixels (the corner test's own margin then grows past a pixel) the
 // corners decide.
-__device__ __forceinline__ bool maybe_visible(const BatchParams& bp, int view, int64_t gv, uint32_t* __restrict__ flags) {
-    const int o = gv < bp.vox_offset[1] ? 0 : find_octree(bp, gv);
+__device__ __forceinline__ bool maybe_visible(const BatchParams& bp, int view, int o, uint64_t key,
+                                              uint32_t* __restrict__ flags) {
     const ViewParams& fp = bp.views[view];
     const OctParams& P = bp.octs[view * bp.n_oct + o];
-    const Leaf L = decode_leaf(P, P.key[gv - bp.vox_offset[o]]);
+    const Leaf L = decode_leaf(P, key);
     if (L.level > P.max_level || L.i >> L.level || L.j >> L.level || L.k >> L.level) {
         atomicOr(flags, DV_FLAG_BAD_LEVEL);
         __threadfence();  // visible to the block that reports the flags
@@ -223,21 +223,24 @@ __device__ __forceinline__ uint32_t project_voxel(const BatchParams& bp, int vie
 
 constexpr int MAX_KEY_PASSES = 8;  // 8-bit digits of a 64-bit key
 
-// A block takes `rounds` times 256 voxels of one view.  Its threads test them all (maybe_visible), the voxels left
-// gather in a queue in shared memory, and the block projects those, 256 at a time: left in place they would take
-// the corner arithmetic and the depth key to nearly every warp, at an eighth of its lanes (8M-leaf frame, six
-// cameras: 1,166 -> 672 us; the 500k-leaf frame's step is as long either way).  Per 256 the block reserves one run of the sort input for the visible ones
+// A block takes ROUNDS times 256 voxels of one view.  Its threads load the keys of all rounds at once and test them
+// (maybe_visible), the voxels left gather in a queue in shared memory, and the block projects those, 256 at a time:
+// left in place they would take the corner arithmetic and the depth key to nearly every warp, at an eighth of its
+// lanes.  What bounds it is the chain of dependent steps of a block (key, test, reservation, finish ticket), so six
+// blocks an SM at 40 registers (some spilled) beat four at 63.  8M-leaf frame, six cameras: voxels in place 1,166
+// us, queue 672, keys at once 630, six blocks 546 (8 rounds 514, but no shorter step).  Below 100,000 (view, voxel)s,
+// where 4 rounds leave SMs without a block, ROUNDS = 1; the 500k-leaf frame's step is as long either way.
+// Per 256 projected the block reserves one run of the sort input for the visible ones
 // (scal[0] counts them, scal[1] their pairs); it adds the digits of their keys to key_hist
 // [key_passes][256], and the block that finishes last copies scal[0..2] into host_out[0..2] (the
 // device's wait-error word folded into the flags) and then `seq` into host_out[3], so the host learns
 // the sizes from this kernel alone, as soon as they are final.  scal[3] counts finished blocks.
 // Block 0 also clears the call's five work words, and the grid the tile ranges.  Grid: (blocks of one view's
 // voxels, views).
-constexpr int PROJ_ROUNDS = 4;
-
-__global__ void __launch_bounds__(256) k_project(const __grid_constant__ BatchParams bp, uint64_t* __restrict__ rect,
+template <int ROUNDS>
+__global__ void __launch_bounds__(256, 6) k_project(const __grid_constant__ BatchParams bp, uint64_t* __restrict__ rect,
                                                  uint64_t* __restrict__ out_key, uint32_t* __restrict__ out_g,
-                                                 uint32_t* __restrict__ key_hist, int key_passes, int rounds,
+                                                 uint32_t* __restrict__ key_hist, int key_passes,
                                                  uint2* __restrict__ range, unsigned long long* __restrict__ scal,
                                                  volatile uint64_t* host_out, uint64_t seq,
                                                  uint32_t* __restrict__ spin_err, unsigned long long* __restrict__ work) {
@@ -248,19 +251,31 @@ __global__ void __launch_bounds__(256) k_project(const __grid_constant__ BatchPa
     for (int64_t t = (int64_t)block * 256 + threadIdx.x; t < bp.n_tiles; t += (int64_t)n_block * 256)
         range[t] = make_uint2(0u, 0u);
     __shared__ uint32_t h[MAX_KEY_PASSES][256];
-    __shared__ uint16_t s_queue[PROJ_ROUNDS * 256];  // voxels of the block left to project
+    __shared__ uint16_t s_queue[ROUNDS * 256];  // voxels of the block left to project
     __shared__ uint32_t s_wv[8];
     __shared__ unsigned long long s_wp[8];
     __shared__ unsigned long long s_base;
     __shared__ uint32_t s_nq;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int view = blockIdx.y;
-    const int64_t gv0 = (int64_t)blockIdx.x * 256 * rounds;  // the block's first voxel of the view
+    const int64_t gv0 = (int64_t)blockIdx.x * 256 * ROUNDS;  // the block's first voxel of the view
     if (tid == 0) s_nq = 0;
-    __syncthreads();
-    for (int r = 0; r < rounds; ++r) {
+    // the keys of all rounds in flight together
+    uint64_t vk[ROUNDS];
+    int vo[ROUNDS];
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) {
         const int64_t gv = gv0 + r * 256 + tid;
-        const bool in = gv < bp.n_vox && maybe_visible(bp, view, gv, reinterpret_cast<uint32_t*>(scal + 2));
+        vo[r] = -1;
+        if (gv < bp.n_vox) {
+            vo[r] = gv < bp.vox_offset[1] ? 0 : find_octree(bp, gv);
+            vk[r] = __ldg(bp.octs[vo[r]].key + (gv - bp.vox_offset[vo[r]]));
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) {
+        const bool in = vo[r] >= 0 && maybe_visible(bp, view, vo[r], vk[r], reinterpret_cast<uint32_t*>(scal + 2));
         const unsigned bal = __ballot_sync(0xffffffffu, in);
         uint32_t at = 0;
         if (lane == 0 && bal) at = atomicAdd(&s_nq, (uint32_t)__popc(bal));
@@ -760,9 +775,10 @@ cudaError_t launch_project(const BatchParams& bp, uint64_t* rect, uint64_t* out_
     if (passes > MAX_KEY_PASSES) return cudaErrorInvalidValue;
     // with no voxel at all, empty blocks still clear the work words and report the (zero) sizes
     // fewer blocks than one or two per SM would leave the chip idle below this
-    const int rounds = bp.n_vox * bp.n_view >= 100000 ? PROJ_ROUNDS : 1;
-    launch_pdl(k_project, dim3(bp.n_vox > 0 ? nblk(bp.n_vox, 256 * rounds) : 1u, (unsigned)bp.n_view), dim3(256), s, bp,
-               rect, out_key, out_g, key_hist, passes, rounds, tile_range, scal, (volatile uint64_t*)host_out, seq,
+    const bool queue = bp.n_vox * bp.n_view >= 100000;
+    launch_pdl(queue ? k_project<4> : k_project<1>,
+               dim3(bp.n_vox > 0 ? nblk(bp.n_vox, queue ? 1024 : 256) : 1u, (unsigned)bp.n_view), dim3(256), s, bp,
+               rect, out_key, out_g, key_hist, passes, tile_range, scal, (volatile uint64_t*)host_out, seq,
                spin_err, work);
     count_launches(1);
     return cudaGetLastError();
