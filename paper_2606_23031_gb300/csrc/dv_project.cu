@@ -69,7 +69,7 @@ __device__ __forceinline__ Leaf decode_leaf(const OctParams& P, uint64_t key) {
     L.i = (uint32_t)(key & M19);
     L.j = (uint32_t)((key >> 19) & M19);
     L.k = (uint32_t)((key >> 38) & M19);
-    L.s = ldexpf(P.root_size, -L.level);
+    L.s = P.root_size * __int_as_float((127 - L.level) << 23);  // times 2^-level (at most 31)
     L.mn[0] = fmaf((float)L.i, L.s, P.root_min[0]);
     L.mn[1] = fmaf((float)L.j, L.s, P.root_min[1]);
     L.mn[2] = fmaf((float)L.k, L.s, P.root_min[2]);
@@ -114,29 +114,20 @@ __device__ __forceinline__ uint32_t side_path(uint32_t idx, int level, int64_t X
     return (1u << top) | (((cell >> top) & 1u ? ~idx : idx) & low);
 }
 
-// Whether a leaf of octree o may be visible in `view`.  Most voxels lie outside the frustum by far: the bounding sphere
-// against the near and far planes and the four sides, each side 1.5 pixels outside the image, decides those with a
-// tenth of the arithmetic of the corners.  It leaves out nothing that the corners (project_voxel) would keep: the
-// radius covers the rounding of both (4e-6 of the coordinates' size), and where the sphere comes so close to the
-// camera plane that its projection exceeds 2e5 pixels (the corner test's own margin then grows past a pixel) the
-// corners decide.
-__device__ __forceinline__ bool maybe_visible(const BatchParams& bp, int view, int o, uint64_t key,
-                                              uint32_t* __restrict__ flags) {
-    const ViewParams& fp = bp.views[view];
-    const OctParams& P = bp.octs[view * bp.n_oct + o];
-    const Leaf L = decode_leaf(P, key);
-    if (L.level > P.max_level || L.i >> L.level || L.j >> L.level || L.k >> L.level) {
-        atomicOr(flags, DV_FLAG_BAD_LEVEL);
-        __threadfence();  // visible to the block that reports the flags
-        return false;
-    }
-    const float h = 0.5f * L.s;
-    const float x0 = L.mn[0] + h, y0 = L.mn[1] + h, z0 = L.mn[2] + h;
+// Whether anything inside the sphere of radius r around (x0, y0, z0) in octree P's frame may be visible in a view.
+// Most voxels lie outside the frustum by far: a bounding sphere against the near and far planes and the four sides,
+// each side 1.5 pixels outside the image, decides those with a tenth of the arithmetic of the corners.  It
+// leaves out nothing that the corners (project_voxel) would keep: the radius covers the rounding of both (4e-6 of
+// the coordinates' size, `ext` that of the extent around the centre), and where the sphere comes so close to
+// the camera plane that its projection exceeds 2e5 pixels (the corner test's own margin then grows past a pixel)
+// the corners decide.
+__device__ __forceinline__ bool sphere_in_view(const ViewParams& fp, const OctParams& P, float x0, float y0, float z0,
+                                               float r, float ext) {
     float c[3];
 #pragma unroll
-    for (int r = 0; r < 3; ++r) c[r] = fmaf(P.M[r * 3 + 0], x0, fmaf(P.M[r * 3 + 1], y0, fmaf(P.M[r * 3 + 2], z0, P.m[r])));
-    const float size = fabsf(x0) + fabsf(y0) + fabsf(z0) + fabsf(P.m[0]) + fabsf(P.m[1]) + fabsf(P.m[2]);
-    const float rad = fmaf(0.8661f, L.s, 4e-6f * size);
+    for (int k = 0; k < 3; ++k) c[k] = fmaf(P.M[k * 3 + 0], x0, fmaf(P.M[k * 3 + 1], y0, fmaf(P.M[k * 3 + 2], z0, P.m[k])));
+    const float size = fabsf(x0) + fabsf(y0) + fabsf(z0) + fabsf(P.m[0]) + fabsf(P.m[1]) + fabsf(P.m[2]) + ext;
+    const float rad = fmaf(4e-6f, size, r);
     const float zn = c[2] - rad;
     if (c[2] + rad < fp.z_clip || zn > fp.far_) return false;
     if (zn > fp.z_clip && fmaxf(fp.fx * (fabsf(c[0]) + rad), fp.fy * (fabsf(c[1]) + rad)) < 2e5f * zn) {
@@ -146,6 +137,22 @@ __device__ __forceinline__ bool maybe_visible(const BatchParams& bp, int view, i
             return false;
     }
     return true;
+}
+
+// a leaf's level and indices are within its octree's; else the call's flag is set
+__device__ __forceinline__ bool leaf_ok(const OctParams& P, const Leaf& L, uint32_t* __restrict__ flags) {
+    if (L.level > P.max_level || L.i >> L.level || L.j >> L.level || L.k >> L.level) {
+        atomicOr(flags, DV_FLAG_BAD_LEVEL);
+        __threadfence();  // visible to the block that reports the flags
+        return false;
+    }
+    return true;
+}
+
+// whether a leaf may be visible in a view (P: its octree there)
+__device__ __forceinline__ bool leaf_in_view(const ViewParams& fp, const OctParams& P, const Leaf& L) {
+    const float h = 0.5f * L.s;
+    return sphere_in_view(fp, P, L.mn[0] + h, L.mn[1] + h, L.mn[2] + h, 0.8661f * L.s, 0.0f);
 }
 
 // Projection of voxel gv of `view`: returns its tile count (0: not visible) and, when visible, its
@@ -223,22 +230,26 @@ __device__ __forceinline__ uint32_t project_voxel(const BatchParams& bp, int vie
 
 constexpr int MAX_KEY_PASSES = 8;  // 8-bit digits of a 64-bit key
 
-// A block takes ROUNDS times 256 voxels of one view.  Its threads load the keys of all rounds at once and test them
-// (maybe_visible), the voxels left gather in a queue in shared memory, and the block projects those, 256 at a time:
+// A block takes ROUNDS times 256 voxels in one view, or in up to VIEWS.  Its threads load the keys of all rounds at
+// once and test them (leaf_in_view), the voxels left gather in a queue in shared memory, and the block projects those, 256 at a time:
 // left in place they would take the corner arithmetic and the depth key to nearly every warp, at an eighth of its
 // lanes.  What bounds it is the chain of dependent steps of a block (key, test, reservation, finish ticket), so six
-// blocks an SM at 40 registers (some spilled) beat four at 63.  8M-leaf frame, six cameras: voxels in place 1,166
+// blocks an SM at 40 registers (some spilled) beat four at 63 where there are more than four for each (a frame of
+// 560k voxels has fewer: 21.9 against 24.0 us).  8M-leaf frame, six cameras: voxels in place 1,166
 // us, queue 672, keys at once 630, six blocks 546 (8 rounds 514, but no shorter step).  Below 100,000 (view, voxel)s,
 // where 4 rounds leave SMs without a block, ROUNDS = 1; the 500k-leaf frame's step is as long either way.
+// With three views or more a warp first tests the box around its 32 leaves, one view a lane, and the leaves only
+// against the views left (neighbours in the array mostly are in space): 555 -> 390 us there, the step 7.11 -> 6.95 ms.
+// With two views that one more test costs what it saves (32M leaves, two 4K cameras: 6.26 against 6.31 ms).
 // Per 256 projected the block reserves one run of the sort input for the visible ones
 // (scal[0] counts them, scal[1] their pairs); it adds the digits of their keys to key_hist
 // [key_passes][256], and the block that finishes last copies scal[0..2] into host_out[0..2] (the
 // device's wait-error word folded into the flags) and then `seq` into host_out[3], so the host learns
 // the sizes from this kernel alone, as soon as they are final.  scal[3] counts finished blocks.
 // Block 0 also clears the call's five work words, and the grid the tile ranges.  Grid: (blocks of one view's
-// voxels, views).
-template <int ROUNDS>
-__global__ void __launch_bounds__(256, 6) k_project(const __grid_constant__ BatchParams bp, uint64_t* __restrict__ rect,
+// voxels, groups of VIEWS views).
+template <int ROUNDS, int VIEWS, int CTAS>
+__global__ void __launch_bounds__(256, CTAS) k_project(const __grid_constant__ BatchParams bp, uint64_t* __restrict__ rect,
                                                  uint64_t* __restrict__ out_key, uint32_t* __restrict__ out_g,
                                                  uint32_t* __restrict__ key_hist, int key_passes,
                                                  uint2* __restrict__ range, unsigned long long* __restrict__ scal,
@@ -251,14 +262,15 @@ __global__ void __launch_bounds__(256, 6) k_project(const __grid_constant__ Batc
     for (int64_t t = (int64_t)block * 256 + threadIdx.x; t < bp.n_tiles; t += (int64_t)n_block * 256)
         range[t] = make_uint2(0u, 0u);
     __shared__ uint32_t h[MAX_KEY_PASSES][256];
-    __shared__ uint16_t s_queue[ROUNDS * 256];  // voxels of the block left to project
+    __shared__ uint16_t s_queue[ROUNDS * 256 * VIEWS];  // view of the group, round and thread of the voxels left to project
     __shared__ uint32_t s_wv[8];
     __shared__ unsigned long long s_wp[8];
     __shared__ unsigned long long s_base;
     __shared__ uint32_t s_nq;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int view = blockIdx.y;
-    const int64_t gv0 = (int64_t)blockIdx.x * 256 * ROUNDS;  // the block's first voxel of the view
+    const int view0 = blockIdx.y * VIEWS, n_view = min(VIEWS, bp.n_view - view0);
+    const int64_t gv0 = (int64_t)blockIdx.x * 256 * ROUNDS;  // the block's first voxel of a view
+    uint32_t* flags = reinterpret_cast<uint32_t*>(scal + 2);
     if (tid == 0) s_nq = 0;
     // the keys of all rounds in flight together
     uint64_t vk[ROUNDS];
@@ -273,14 +285,54 @@ __global__ void __launch_bounds__(256, 6) k_project(const __grid_constant__ Batc
         }
     }
     __syncthreads();
-#pragma unroll
-    for (int r = 0; r < ROUNDS; ++r) {
-        const bool in = vo[r] >= 0 && maybe_visible(bp, view, vo[r], vk[r], reinterpret_cast<uint32_t*>(scal + 2));
+    auto push = [&](bool in, int e) {
         const unsigned bal = __ballot_sync(0xffffffffu, in);
         uint32_t at = 0;
         if (lane == 0 && bal) at = atomicAdd(&s_nq, (uint32_t)__popc(bal));
         at = __shfl_sync(0xffffffffu, at, 0);
-        if (in) s_queue[at + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(r * 256 + tid);
+        if (in) s_queue[at + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)e;
+    };
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) {
+        const int o = vo[r];
+        bool ok = o >= 0;
+        Leaf L;
+        if (ok) {
+            const OctParams& P = bp.octs[view0 * bp.n_oct + o];
+            L = decode_leaf(P, vk[r]);
+            ok = leaf_ok(P, L, flags);
+        }
+        const int e = r * 256 + tid;
+        if constexpr (VIEWS == 1) {
+            push(ok && leaf_in_view(bp.views[view0], bp.octs[view0 * bp.n_oct + o], L), e);
+        } else {
+            unsigned todo = (1u << n_view) - 1u;  // views that may see some of the warp's leaves
+            const unsigned any = __ballot_sync(0xffffffffu, ok);
+            if (!any) continue;
+            const int o0 = __shfl_sync(0xffffffffu, o, __ffs(any) - 1);
+            if (__all_sync(0xffffffffu, !ok || o == o0)) {
+                // the box around them, in cells of the octree's finest level; lane v tests it against view v
+                const OctParams& P = bp.octs[(view0 + min(lane, n_view - 1)) * bp.n_oct + o0];
+                const int sh = ok ? P.max_level - L.level : 0;
+                const uint32_t one = 1u << sh;
+                const uint32_t x = ok ? L.i << sh : 0u, y = ok ? L.j << sh : 0u, z = ok ? L.k << sh : 0u;
+                auto lowest = [&](uint32_t i) { return __reduce_min_sync(0xffffffffu, ok ? i : 0xffffffffu); };
+                auto end = [&](uint32_t i) { return __reduce_max_sync(0xffffffffu, ok ? i + one : 0u); };
+                const uint32_t lx = lowest(x), ly = lowest(y), lz = lowest(z), hx = end(x), hy = end(y), hz = end(z);
+                const float u = P.root_size * __int_as_float((127 - P.max_level) << 23), h = 0.5f * u;
+                const float ex = h * (float)(hx - lx), ey = h * (float)(hy - ly), ez = h * (float)(hz - lz);
+                const bool in = lane < n_view &&
+                    sphere_in_view(bp.views[view0 + min(lane, n_view - 1)], P, fmaf((float)(lx + hx), h, P.root_min[0]),
+                                   fmaf((float)(ly + hy), h, P.root_min[1]), fmaf((float)(lz + hz), h, P.root_min[2]),
+                                   1.0001f * sqrtf(fmaf(ex, ex, fmaf(ey, ey, ez * ez))), ex + ey + ez);
+                todo = __ballot_sync(0xffffffffu, in);
+            }
+            for (; todo; todo &= todo - 1) {
+                const int v = __ffs((int)todo) - 1;
+                const bool in = ok && leaf_in_view(bp.views[view0 + v], bp.octs[(view0 + v) * bp.n_oct + o], L);
+                push(in, v * (ROUNDS * 256) + e);
+            }
+        }
     }
     __syncthreads();
     const uint32_t nq = s_nq;
@@ -290,8 +342,11 @@ __global__ void __launch_bounds__(256, 6) k_project(const __grid_constant__ Batc
             uint64_t rc = 0, key = 0;
             uint32_t c = 0;
             int64_t gv = 0;
+            int view = view0;
             if (q0 + tid < nq) {
-                gv = gv0 + s_queue[q0 + tid];
+                const uint32_t e = s_queue[q0 + tid];
+                view = view0 + (int)(e / (ROUNDS * 256));
+                gv = gv0 + e % (ROUNDS * 256);
                 c = project_voxel(bp, view, gv, rc, key);
             }
             const unsigned bal = __ballot_sync(0xffffffffu, c != 0);
@@ -775,9 +830,12 @@ cudaError_t launch_project(const BatchParams& bp, uint64_t* rect, uint64_t* out_
     if (passes > MAX_KEY_PASSES) return cudaErrorInvalidValue;
     // with no voxel at all, empty blocks still clear the work words and report the (zero) sizes
     // fewer blocks than one or two per SM would leave the chip idle below this
-    const bool queue = bp.n_vox * bp.n_view >= 100000;
-    launch_pdl(queue ? k_project<4> : k_project<1>,
-               dim3(bp.n_vox > 0 ? nblk(bp.n_vox, queue ? 1024 : 256) : 1u, (unsigned)bp.n_view), dim3(256), s, bp,
+    const bool queue = bp.n_vox * bp.n_view >= 100000, multi = queue && bp.n_view >= 3;
+    const dim3 grid(bp.n_vox > 0 ? nblk(bp.n_vox, queue ? 1024 : 256) : 1u,
+                    (unsigned)(multi ? (bp.n_view + 7) / 8 : bp.n_view));
+    const bool one_wave = (int64_t)grid.x * grid.y <= 4 * sm_count();
+    launch_pdl(multi ? k_project<4, 8, 6> : !queue ? k_project<1, 1, 4> : one_wave ? k_project<4, 1, 4> : k_project<4, 1, 6>,
+               grid, dim3(256), s, bp,
                rect, out_key, out_g, key_hist, passes, tile_range, scal, (volatile uint64_t*)host_out, seq,
                spin_err, work);
     count_launches(1);

@@ -132,6 +132,28 @@ def test_projection_queue(dv, n):
     check_forward(im(rgb, 3), im(depth), im(alpha), o[0], o[1], o[2], f"{n} voxels")
 
 
+# three and nine views (a group of eight and a remainder), in which a warp tests the box around its leaves first, on
+# leaves in order, out of order and with warps that hold leaves of two octrees: the images of each view alone, which
+# is below the queue, bit for bit
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_view,shuffle", [(3, False), (3, True), (9, False)])
+def test_projection_of_several_views(dv, n_view, shuffle):
+    rng = np.random.default_rng(n_view)
+    key = _grid(6, 0.0, rng, 40003)
+    octs = [_octree(key[rng.permutation(key.size)] if shuffle else key, 0.5, rng, 8.0)]
+    octs += [_octree(_grid(3, 0.0, rng, 77), 2.0, rng, 1.0, synth.ACTOR, (0.4, 0.45, 0.3)) for _ in range(2)]
+    poses = [synth.Pose()] + [synth.Pose(synth.random_rotation(rng), rng.uniform(-2, 2, 3)) for _ in range(2)]
+    cams = [synth.pinhole(35, 19, 50.0, synth.Pose(synth.random_rotation(rng), rng.uniform(-3, 3, 3)), 0.05, 4.0)
+            for _ in range(n_view)]
+    ds = device_scene(synth.Scene(octs, poses))
+    assert sum(o.n for o in octs) < 100000 <= n_view * sum(o.n for o in octs)
+    both = gpu_render(ds, poses, cams)[:3]
+    for c, cam in enumerate(cams):
+        for a, b in zip(both, gpu_render(ds, poses, [cam])[:3]):
+            n = cam.W * cam.H
+            np.testing.assert_array_equal(a[c * n:(c + 1) * n].cpu().numpy(), b.cpu().numpy())
+
+
 def _keys_t(keys):
     import torch
     return torch.as_tensor(np.asarray(keys, np.uint64).view(np.int64), device="cuda")
