@@ -155,13 +155,15 @@ struct WarpRing {
 //   s_iv[k][0/1][px] = the interval [a, b), s_id[k][px] its actor (position in the tile's list)
 //   s_st[k][..][px]  = phase 1: the actor's partial; phase 2 overwrites it with the state at the
 //                      interval's entry when it is replayed.  Rows:
-//     ST_T, ST_N = transmittance and segment count (phase 2: 0 not reached, 1 partial applied, 2 replay);
+//     ST_T, ST_N = transmittance and segment count (NO_PARTIAL: left out; phase 2: 0 not reached, 1 partial
+//     applied, 2 replay);
 //     ST_R = residual sum (backward); ST_B, ST_E = first slot and end of the interval's segments (export);
 //     else ST_C.. = C0, C1, C2, D, ST_P = transmittance before the partial's last segment, with normals
 //     N0, N1, N2 from ST_V
 // A CTA of a spread tile has 32 pixels in its 128 columns, so there slot k sits in row k % NTA, columns
 // 32 (k / NTA) and on: four times the slots (rays along the road cross many boxes).
 constexpr int ST_T = 0, ST_N = 1, ST_R = 2, ST_B = 2, ST_E = 3, ST_C = 2, ST_P = 6, ST_V = 7;
+constexpr float NO_PARTIAL = -1.0f;
 
 // BWD: replay with gradients.  WEX: replay that writes every composited segment's (voxel,
 // weight) into the pixel's slots of the weights export (no outputs, no gradients).
@@ -597,8 +599,8 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
     // Transmittance never rises along a ray, so if the partials of the lane's earlier intervals
     // already multiply to less than eps_stop the ray stops before this one, and its partial is
     // not needed (phase 2 multiplies the same factors in the same order, and the background's on
-    // top, so it cannot get past them).  Another warp's partial counts once it is written; before
-    // that its factor is 1.
+    // top, so with T <= 1 it cannot get past them; enter_actor has the other rays).  Another warp's
+    // partial counts once it is written; before that its factor is 1.
     for (int i = wi; i < n_ta; i += nw) {
         const int q = s_near[i];
         const int k = valid ? slot_of(q) : -1;
@@ -607,6 +609,7 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
             float T = 1.0f;
             for (int x = 0; x < k; ++x) T *= *(volatile float*)&st(x, ST_T);
             act = !(T < bp.eps_stop);
+            if (!act) st(k, ST_N) = NO_PARTIAL;
         }
         if (!__any_sync(0xffffffffu, act)) continue;
         Pix<NRM> pt;
@@ -661,7 +664,16 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
         if (valid) advance();
         // enters actor interval `it`: apply its partial, or stop inside it, or walk it per lane
         auto enter_actor = [&](const ActInt& it) {
-            if (it.q >= cap) {
+            // The partial holds for a ray that enters with T <= 1: it may have been left out, or have stopped,
+            // because the ray would have stopped by then.  A ray that gets here all the same (T above 1 behind
+            // negative densities under the identity activation, or eps_stop above 1 and no segment yet) walks
+            // the interval with the exact stop rule.
+            bool walk = it.q >= cap;
+            if (!walk) {
+                const float t = st(it.q, ST_T);
+                walk = st(it.q, ST_N) == NO_PARTIAL || (t < bp.eps_stop && !(ps.T * t < bp.eps_stop));
+            }
+            if (walk) {
                 // the out-of-line walk takes copies: an object whose address reaches a call stays in
                 // local memory everywhere, so the hot-path state (ps, bw, dc, nxt, ex) never does
                 Pix<NRM> pl = ps;

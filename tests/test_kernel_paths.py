@@ -94,6 +94,43 @@ def test_actor_tiles(dv, n, level, crowded):
     assert np.abs(total - alpha.cpu().numpy().ravel()).max() <= 1e-5
 
 
+# rays that reach an actor whose partial composite was left out or stopped early, both of which assume T <= 1:
+# behind negative densities under the identity activation (T of some 5 in front of the actors).  Values follow T, so
+# the bounds are relative to the largest
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,level", [(3, 5), (7, 4), (12, 1)])
+@pytest.mark.parametrize("eps,identity", [(0.3, True)])
+def test_actor_partials_behind_transmittance_above_one(dv, n, level, eps, identity):
+    import torch
+    sc, cam, _ = _row_of_actors(n, level)
+    if identity:
+        sc.octrees[0].dens *= np.float32(-40.0)
+        for o in sc.octrees[1:]:
+            o.dens *= np.float32(9.0 * n)
+    act = oracle.ACT_IDENTITY if identity else oracle.ACT_EXPLIN
+    P = cam.W * cam.H
+    rng = np.random.default_rng(n)
+    g = [np.float64(np.float32(x)) for x in (rng.normal(size=(P, 3)), 0.1 * rng.normal(size=P), rng.normal(size=P))]
+    ds = device_scene(sc)
+    rgb, depth, alpha, st = dv.dv_render(ds, sc.poses, [cam], dv.make_opts(1, eps, act), save_state=True)
+    W = dv.dv_state_weights(st)
+    t = lambda a: torch.as_tensor(np.ascontiguousarray(a, np.float32), device="cuda")
+    d_dens = [torch.zeros_like(o.dens) for o in ds]
+    d_sh = [torch.zeros_like(o.sh) for o in ds]
+    dv.dv_render_backward(st, t(g[0]), t(g[1]), t(g[2]), d_dens, d_sh)
+    torch.cuda.synchronize()
+    st.free()
+    o = oracle.render(sc.octrees, sc.poses, cam, oracle.Opts(1, eps, act))
+    for x, ref, tol in ((rgb, o[0], 1e-4), (depth, o[1], 1e-3), (alpha, o[2], 1e-4)):
+        assert np.abs(x.cpu().numpy().reshape(ref.shape) - ref).max() <= tol * np.abs(ref).max()
+    off, w = W.offsets.cpu().numpy(), W.weight.cpu().numpy().astype(np.float64)
+    total = np.add.reduceat(np.append(w, 0.0), np.minimum(off[:-1], w.size)) * (np.diff(off) > 0)
+    assert np.abs(total - alpha.cpu().numpy().ravel()).max() <= 1e-4 * max(1.0, np.abs(o[2]).max())
+    od, os_ = oracle.backward(sc.octrees, sc.poses, cam, g[0], g[1], g[2], oracle.Opts(1, eps, act))
+    check_grads([x.cpu().numpy() for x in d_dens], od, f"{n} actors d_dens")
+    check_grads([x.cpu().numpy() for x in d_sh], os_, f"{n} actors d_sh")
+
+
 # voxels of about 20, 5 and 0.6 pixels
 @pytest.mark.gpu
 @pytest.mark.parametrize("level,normals", [(1, False), (1, True), (3, True), (6, False), (6, True)])
