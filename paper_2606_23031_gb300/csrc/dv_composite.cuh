@@ -388,7 +388,7 @@ __device__ __forceinline__ void bwd_single_step(Pix<NRM>& ps, const Bwd<NRM>& bw
         acc[NRM ? 12 : 0] = bw.gN1 * w;
         acc[NRM ? 13 : 0] = bw.gN2 * w;
     }
-    if (ps.T < bp.eps_stop) ps.stop();
+    if (hit && ps.T < bp.eps_stop) ps.stop();  // (a miss stops nothing, also where eps_stop is above 1)
 }
 
 // Sum of acc[0..NV-1] over the warp, transposed.  Each butterfly level (lane distance 16, 8, 4, 2,

@@ -95,11 +95,11 @@ def test_actor_tiles(dv, n, level, crowded):
 
 
 # rays that reach an actor whose partial composite was left out or stopped early, both of which assume T <= 1:
-# behind negative densities under the identity activation (T of some 5 in front of the actors).  Values follow T, so
-# the bounds are relative to the largest
+# behind negative densities under the identity activation (T of some 5 in front of the actors), and with eps_stop
+# above 1 (a ray then ends with its first segment).  Values follow T, so the bounds are relative to the largest
 @pytest.mark.gpu
 @pytest.mark.parametrize("n,level", [(3, 5), (7, 4), (12, 1)])
-@pytest.mark.parametrize("eps,identity", [(0.3, True)])
+@pytest.mark.parametrize("eps,identity", [(0.3, True), (2.0, False)])
 def test_actor_partials_behind_transmittance_above_one(dv, n, level, eps, identity):
     import torch
     sc, cam, _ = _row_of_actors(n, level)
