@@ -916,6 +916,15 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
             walk_actor(pt, s_act[q], act ? iv(k, 0) : 0.0f, std::integral_constant<bool, BWD>(),
                        std::integral_constant<bool, WEX>());
             ps.tests += pt.tests;
+            if constexpr (WEX) {
+                // the replay's T can differ in the last bits from the entry's T times the partial's, on which the
+                // forward counted the segments; slots of segments that it does not get to have weight 0
+                if (act)
+                    for (; ex.n < ex.lim; ++ex.n) {
+                        ex.vid[ex.base + ex.n] = 0u;
+                        ex.w[ex.base + ex.n] = 0.0f;
+                    }
+            }
             if (!REPLAY && act) {
                 ps.C0 = pt.C0;
                 ps.C1 = pt.C1;

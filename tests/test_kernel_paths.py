@@ -131,6 +131,38 @@ def test_actor_partials_behind_transmittance_above_one(dv, n, level, eps, identi
     check_grads([x.cpu().numpy() for x in d_sh], os_, f"{n} actors d_sh")
 
 
+# every exported slot is written, also where the transmittance behind an actor is within rounding of eps_stop: an
+# interval's replay from its entry may then stop before segments that the forward, applying its partial, counted.
+# The actor is a dense slab and a long tail of segments without weight; eps_stop goes through the floats around a
+# pixel's final transmittance
+@pytest.mark.gpu
+def test_export_writes_every_slot(dv):
+    import torch
+    rng = np.random.default_rng(4)
+    key = _grid(2, 0.0, rng, 64)
+    bg = _octree(key[oi._unpack(key)[1] < 2], 0.05, rng, 4.0)  # nothing behind the actor's slab
+    actor = _octree(_grid(4, 0.0, rng, 4096), 1.0, rng, 0.8, synth.ACTOR, (0.4, 0.4, 0.4))
+    actor.dens[oi._unpack(actor.key)[1] >= 6] = -60.0
+    sc = synth.Scene([bg, actor], [synth.Pose(), synth.Pose()])
+    cam = synth.pinhole(16, 8, 6.0, synth.look_at((-6.0, 0.0, 0.0), (0.0, 0.0, 0.0)), 0.1, 60.0)
+    ds = device_scene(sc)
+    T = 1.0 - dv.dv_render(ds, sc.poses, [cam], dv.make_opts(1, 0.0))[2].cpu().numpy().astype(np.float64)
+    assert T.min() > 0.25 and T.max() < 0.5
+    for p in range(0, cam.W * cam.H, 2):
+        for j in range(-4, 5):
+            eps = float(np.float32(T[p] + j * 2.0 ** -25))
+            alpha, st = dv.dv_render(ds, sc.poses, [cam], dv.make_opts(1, eps), save_state=True)[2:]
+            W = dv.dv_state_weights(st)
+            W.voxel.fill_(0x7fffffff)
+            W.weight.fill_(float("nan"))
+            dv.dv_state_weights(st, out=W)
+            st.free()
+            assert int(W.voxel.max()) < bg.n + actor.n and int(W.voxel.min()) >= 0
+            pix = torch.repeat_interleave(torch.arange(cam.W * cam.H, device="cuda"), W.offsets.diff())
+            total = torch.zeros(cam.W * cam.H, device="cuda").index_add_(0, pix, W.weight)
+            assert float((total - alpha).abs().max()) <= 1e-5
+
+
 # voxels of about 20, 5 and 0.6 pixels
 @pytest.mark.gpu
 @pytest.mark.parametrize("level,normals", [(1, False), (1, True), (3, True), (6, False), (6, True)])
