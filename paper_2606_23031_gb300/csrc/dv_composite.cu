@@ -469,7 +469,7 @@ void composite_launch(CompositeArgs A, const Fork* fk, cudaStream_t s) {
 
 template <bool BWD, bool NRM, bool WEX>
 void composite_k(const CompositeArgs& A, const Fork* fk, cudaStream_t s) {
-    if (A.bp.K == 1)
+    if (one_sample(A.bp, BWD))
         composite_launch<BWD, 1, NRM, WEX>(A, fk, s);
     else
         composite_launch<BWD, 0, NRM, WEX>(A, fk, s);

@@ -344,7 +344,8 @@ __device__ __forceinline__ void add_segment(Pix<NRM>& ps, const Bwd<NRM>& bw, co
 // (a plain tile, or one actor interval): [u0, u1] is the lane's segment, the empty segment [0, 0] for a
 // lane that misses or has finished (zero optical depth, weight and gradient, state unchanged).  The
 // record's gradient values (8 densities, 3 colour, + 3 normal) are written into acc, not added, so the
-// caller clears nothing and the warp runs it without branches once any lane hits.
+// caller clears nothing and the warp runs it without branches once any lane hits.  (The stop rule is tested for
+// the misses too, which eps_stop above 1 would stop: one_sample has those.)
 template <bool NRM>
 __device__ __forceinline__ void bwd_single_step(Pix<NRM>& ps, const Bwd<NRM>& bw, const BatchParams& bp, float4 g,
                                                 float4 da, float4 dd, float4 col, float4 nv, const float* d, float u0,
@@ -388,7 +389,7 @@ __device__ __forceinline__ void bwd_single_step(Pix<NRM>& ps, const Bwd<NRM>& bw
         acc[NRM ? 12 : 0] = bw.gN1 * w;
         acc[NRM ? 13 : 0] = bw.gN2 * w;
     }
-    if (hit && ps.T < bp.eps_stop) ps.stop();  // (a miss stops nothing, also where eps_stop is above 1)
+    if (ps.T < bp.eps_stop) ps.stop();
 }
 
 // Sum of acc[0..NV-1] over the warp, transposed.  Each butterfly level (lane distance 16, 8, 4, 2,
@@ -606,6 +607,11 @@ __device__ __forceinline__ void add_work(unsigned long long* work, uint32_t test
 }
 
 }  // namespace
+
+// Whether a pass takes the variants for one sample per segment.  The backward's do not test for a hit before the stop
+// rule, which a ray at T = 1 meets without one where eps_stop is above 1; the general ones do.  (The test in the
+// step itself: backward of the 1080p frame some 20 us longer.)
+inline bool one_sample(const BatchParams& bp, bool bwd) { return bp.K == 1 && !(bwd && bp.eps_stop > 1.0f); }
 
 // The actor tiles' part of a compositing pass (dv_composite_act.cu): the n_tiles tiles of A.tile_order,
 // the pass being the forward, the backward (bwd) or the weights export (wex).  `large`: tiles that 5 or

@@ -950,7 +950,7 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
 template <bool BWD, bool NRM, bool WEX>
 void launch_variant(const CompositeArgs& A, unsigned grid, bool large, cudaStream_t s) {
     const dim3 g(grid), b(CT_THREADS);
-    if (A.bp.K == 1) {
+    if (one_sample(A.bp, BWD)) {
         if (large)
             launch_pdl(k_composite_act<BWD, 1, NRM, WEX, NTA_LARGE>, g, b, s, A);
         else
