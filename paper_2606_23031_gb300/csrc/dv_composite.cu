@@ -48,15 +48,18 @@ namespace {
 // 215, any: 2,540 / 253).
 constexpr int LANE_PIX = 14;
 // Resident CTAs per SM: the forward without normals fits 56 registers (9 CTAs: 1,481 -> 1,455 us on the 8M-leaf
-// frame); the others need 64.
-constexpr int plain_ctas(bool fwd) { return fwd ? 9 : 8; }
+// frame); the others need 64, the backward with normals and several samples 72 (two 1883x1229 views of 168k leaves,
+// K = 2: step 1,433 -> 1,393 us).
+constexpr int plain_ctas(bool bwd, int ks, bool nrm, bool wex) {
+    return !bwd && ks == 1 && !nrm && !wex ? 9 : bwd && ks == 0 && nrm ? 7 : 8;
+}
 
 // Tiles that no actor box covers (most of a frame): every ray is background only, so the tile's list
 // is the background's.
 // BWD: replay with gradients.  WEX: replay that writes every composited segment's (voxel, weight) into
 // the pixel's slots of the weights export (no outputs, no gradients).
 template <bool BWD, int KS, bool NRM, bool WEX>
-__global__ void __launch_bounds__(CT_THREADS, plain_ctas(!BWD && KS == 1 && !NRM && !WEX))
+__global__ void __launch_bounds__(CT_THREADS, plain_ctas(BWD, KS, NRM, WEX))
     k_composite(const __grid_constant__ CompositeArgs A) {
     pdl_wait();
     pdl_launch_dependents();

@@ -15,6 +15,13 @@
 //  * A tile with SPREAD_MIN or more pairs gets a CTA for each 8x4 block, whose four warps take different
 //    actors (a partial and a replay need nothing but the interval and its entry state); other tiles get a
 //    CTA per half, a warp per block.
+//  * Warps that run apart fetch their instructions apart, and a kernel of this size does not fit the caches near
+//    the schedulers: with the walk and the visit inlined wherever they are used, waits for instructions were
+//    5.3 cycles an issue on tiles whose voxels cover many pixels (57k leaves, 8 actors, 2442x1704, K = 2: 595 us
+//    against 437 for lockstep visits from a CTA-wide ring).  So the forward has one copy of the visit, and with
+//    several samples one of the walk for phases 1 and 3 (that render 1,210 -> 1,084 us; 1,120 with two walks, which
+//    are the faster with one sample: 480x270 view 0.52 -> 0.48 ms).  The backward is slower with its copies folded
+//    (collectives inside the lanes' own loops: 957x541 with normals and K = 4 0.62 -> 0.82 ms) and keeps them.
 //  * Measured (GB300, whole renders), lockstep visits from a CTA-wide ring -> this: the 480x270 street
 //    view with 20 actors 4.1 -> 0.65 ms, the 32M-leaf render of two 4K cameras 15.4 -> 9.0 ms, a 957x541
 //    training step with normals and K = 4 2.2 -> 0.65 ms.
@@ -133,12 +140,15 @@ __device__ __noinline__ void walk_actor_lane(Pix<NRM>& ps, const Bwd<NRM>& bw, c
 }
 
 
-#ifndef DV_FWD_MIN_BLOCKS
-#define DV_FWD_MIN_BLOCKS 5  // resident CTAs per SM the forward is compiled for
-#endif
-#ifndef DV_BWD_MIN_BLOCKS
-#define DV_BWD_MIN_BLOCKS 4
-#endif
+// Resident CTAs per SM a variant is compiled for: 4, at 128 registers, so that CTAs of the two variants, which run side
+// by side, still fit an SM together (the forward's shared memory: 45 KB with 4 slots, 64 KB with 8, with normals 55
+// and 80 KB of 227 KB; 5 at 96 registers spill up to 172 bytes: 480x270 view 0.50 -> 0.48 ms, two 4K cameras
+// 6.40 -> 6.20 ms; 3 for 8 slots, at 168 registers, 0.52 ms for the view); 3 for the backward with several
+// samples, which spills at 128 (957x541 with normals and K = 4 0.62 -> 0.58 ms; with one sample 3 are slower).
+template <bool BWD, int KS>
+constexpr int act_ctas() {
+    return BWD && KS == 0 ? 3 : 4;
+}
 
 // A warp's staging buffers
 template <bool NRM>
@@ -168,7 +178,7 @@ constexpr float NO_PARTIAL = -1.0f;
 // BWD: replay with gradients.  WEX: replay that writes every composited segment's (voxel,
 // weight) into the pixel's slots of the weights export (no outputs, no gradients).
 template <bool BWD, int KS, bool NRM, bool WEX, int NTA>
-__global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS : DV_FWD_MIN_BLOCKS)
+__global__ void __launch_bounds__(CT_THREADS, act_ctas<BWD, KS>())
     k_composite_act(const __grid_constant__ CompositeArgs A) {
     pdl_wait();
     pdl_launch_dependents();
@@ -595,52 +605,8 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
         });
     };
 
-    // ---- phase 1: partial composite of the actor intervals ----
-    // Transmittance never rises along a ray, so if the partials of the lane's earlier intervals
-    // already multiply to less than eps_stop the ray stops before this one, and its partial is
-    // not needed (phase 2 multiplies the same factors in the same order, and the background's on
-    // top, so with T <= 1 it cannot get past them; enter_actor has the other rays).  Another warp's
-    // partial counts once it is written; before that its factor is 1.
-    for (int i = wi; i < n_ta; i += nw) {
-        const int q = s_near[i];
-        const int k = valid ? slot_of(q) : -1;
-        bool act = k >= 0;
-        if (act) {
-            float T = 1.0f;
-            for (int x = 0; x < k; ++x) T *= *(volatile float*)&st(x, ST_T);
-            act = !(T < bp.eps_stop);
-            if (!act) st(k, ST_N) = NO_PARTIAL;
-        }
-        if (!__any_sync(0xffffffffu, act)) continue;
-        Pix<NRM> pt;
-        init_pix<NRM>(pt, act ? iv(k, 1) : -1.0f);
-        // a lane whose own transmittance already falls below eps_stop will stop inside this
-        // actor whatever T it enters with (T <= 1), so its partial may stop there too
-        walk_actor(pt, s_act[q], act ? iv(k, 0) : 0.0f, std::false_type(), std::false_type());
-        ps.tests += pt.tests;
-        if (act) {
-            st(k, ST_N) = __int_as_float((int)pt.n);
-            if constexpr (RFORM) {
-                st(k, ST_R) = pt.R;
-            } else if constexpr (!WEX) {
-                st(k, ST_C) = pt.C0;
-                st(k, ST_C + 1) = pt.C1;
-                st(k, ST_C + 2) = pt.C2;
-                st(k, ST_C + 3) = pt.D;
-                st(k, ST_P) = pt.Tp;
-                if constexpr (NRM) {
-                    st(k, ST_V) = pt.N0;
-                    st(k, ST_V + 1) = pt.N1;
-                    st(k, ST_V + 2) = pt.N2;
-                }
-            }
-            *(volatile float*)&st(k, ST_T) = pt.T;
-        }
-    }
-    if (spread) __syncthreads();
-
     // ---- phase 2: background walk, applying actor partials in order ----
-    if (owner) {
+    auto background = [&]() {
         float tau_cur = t_near;
         ActInt nxt;
         nxt.o = -1;
@@ -818,8 +784,10 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
                         float a0, b0, a1, b1;
                         const bool in0 = clip(g0, a0, b0), in1 = clip(g1, a1, b1) && two;
                         if (nxt.o >= 0 && ((in0 && nxt.a < b0) || (in1 && nxt.a < b1))) {
-                            visit(bf, j0, nullptr);
-                            if (two && !ps.done()) visit(bf, j1, nullptr);
+                            // (a loop: one copy of the visit)
+#pragma unroll 1
+                            for (uint32_t x = 0; x < (two ? 2u : 1u) && !ps.done(); ++x)
+                                visit(bf, x ? j1 : j0, nullptr);
                         } else {
                             a0 = fmaxf(a0, tau_cur);
                             a1 = fmaxf(a1, tau_cur);
@@ -879,22 +847,45 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
             advance();
         }
         __syncwarp();
-    }
-    if (REPLAY && spread) __syncthreads();
+    };
 
+    // ---- phase 1: partial composite of the actor intervals ----
+    // Transmittance never rises along a ray, so if the partials of the lane's earlier intervals
+    // already multiply to less than eps_stop the ray stops before this one, and its partial is
+    // not needed (phase 2 multiplies the same factors in the same order, and the background's on
+    // top, so with T <= 1 it cannot get past them; enter_actor has the other rays).  Another warp's
+    // partial counts once it is written; before that its factor is 1.
     // ---- phase 3: actor intervals replayed from their entry state ----
     //   forward: only those where the ray stops before the partial's end (by the pixels' own warp);
     //   backward and export: every one reached, shared by the CTA's warps
-    if (REPLAY || owner) {
-        for (int i = REPLAY ? wi : 0; i < n_ta; i += REPLAY ? nw : 1) {
+    // (one loop for both, and so one copy of the walk, in the forward with several samples: see the top of the file)
+#pragma unroll (REPLAY || KS == 1 ? 2 : 1)
+    for (int phase = 1; phase <= 3; phase += 2) {
+        const bool partial = phase == 1;
+        if (!partial) {
+            if (spread) __syncthreads();
+            if (owner) background();
+            if (REPLAY && spread) __syncthreads();
+            if (!REPLAY && !owner) break;
+        }
+        const bool shared = partial || REPLAY;
+        for (int i = shared ? wi : 0; i < n_ta; i += shared ? nw : 1) {
             const int q = s_near[i];
             const int k = valid ? slot_of(q) : -1;
-            const int status = k >= 0 ? (int)st(k, ST_N) : 0;
-            const bool act = REPLAY ? status >= 1 : status == 2;
+            bool act = k >= 0;
+            if (act && partial) {
+                float T = 1.0f;
+                for (int x = 0; x < k; ++x) T *= *(volatile float*)&st(x, ST_T);
+                act = !(T < bp.eps_stop);
+                if (!act) st(k, ST_N) = NO_PARTIAL;
+            } else if (act) {
+                const int status = (int)st(k, ST_N);
+                act = REPLAY ? status >= 1 : status == 2;
+            }
             if (!__any_sync(0xffffffffu, act)) continue;
             Pix<NRM> pt;
             init_pix<NRM>(pt, act ? iv(k, 1) : -1.0f);
-            if (act) {
+            if (act && !partial) {
                 pt.T = st(k, ST_T);
                 if constexpr (RFORM) {
                     pt.R = st(k, ST_R);
@@ -913,19 +904,40 @@ __global__ void __launch_bounds__(CT_THREADS, (BWD || WEX) ? DV_BWD_MIN_BLOCKS :
                     }
                 }
             }
-            walk_actor(pt, s_act[q], act ? iv(k, 0) : 0.0f, std::integral_constant<bool, BWD>(),
-                       std::integral_constant<bool, WEX>());
+            // a lane whose own transmittance already falls below eps_stop will stop inside this actor whatever T
+            // it enters with (T <= 1), so its partial may stop there too
+            const float a = act ? iv(k, 0) : 0.0f;
+            if (!REPLAY || partial)
+                walk_actor(pt, s_act[q], a, std::false_type(), std::false_type());
+            else
+                walk_actor(pt, s_act[q], a, std::integral_constant<bool, BWD>(), std::integral_constant<bool, WEX>());
             ps.tests += pt.tests;
-            if constexpr (WEX) {
+            if (!act) continue;
+            if (partial) {
+                st(k, ST_N) = __int_as_float((int)pt.n);
+                if constexpr (RFORM) {
+                    st(k, ST_R) = pt.R;
+                } else if constexpr (!WEX) {
+                    st(k, ST_C) = pt.C0;
+                    st(k, ST_C + 1) = pt.C1;
+                    st(k, ST_C + 2) = pt.C2;
+                    st(k, ST_C + 3) = pt.D;
+                    st(k, ST_P) = pt.Tp;
+                    if constexpr (NRM) {
+                        st(k, ST_V) = pt.N0;
+                        st(k, ST_V + 1) = pt.N1;
+                        st(k, ST_V + 2) = pt.N2;
+                    }
+                }
+                *(volatile float*)&st(k, ST_T) = pt.T;
+            } else if constexpr (WEX) {
                 // the replay's T can differ in the last bits from the entry's T times the partial's, on which the
                 // forward counted the segments; slots of segments that it does not get to have weight 0
-                if (act)
-                    for (; ex.n < ex.lim; ++ex.n) {
-                        ex.vid[ex.base + ex.n] = 0u;
-                        ex.w[ex.base + ex.n] = 0.0f;
-                    }
-            }
-            if (!REPLAY && act) {
+                for (; ex.n < ex.lim; ++ex.n) {
+                    ex.vid[ex.base + ex.n] = 0u;
+                    ex.w[ex.base + ex.n] = 0.0f;
+                }
+            } else if constexpr (!REPLAY) {
                 ps.C0 = pt.C0;
                 ps.C1 = pt.C1;
                 ps.C2 = pt.C2;
