@@ -236,9 +236,9 @@ constexpr int MAX_KEY_PASSES = 8;  // 8-bit digits of a 64-bit key
 // lanes.  What bounds it is the chain of dependent steps of a block (key, test, reservation, finish ticket), so six
 // blocks an SM at 40 registers (some spilled) beat four at 63 where there are more than four for each (a frame of
 // 560k voxels has fewer: 21.9 against 24.0 us).  8M-leaf frame, six cameras: voxels in place 1,166
-// us, queue 672, keys at once 630, six blocks 546 (8 rounds 514, but no shorter step).  Below 100,000 (view, voxel)s,
-// where 4 rounds leave SMs without a block, ROUNDS = 1; the 500k-leaf frame's step is as long either way.
-// With three views or more a warp first tests the box around its 32 leaves, one view a lane, and the leaves only
+// us, queue 672, keys at once 630, six blocks 546 (8 rounds 514, but no shorter step).  ROUNDS = 1 leaves the queue little
+// to gather and is for few voxels (launch_project has the lines).
+// In a group of views a warp first tests the box around its 32 leaves, one view a lane, and the leaves only
 // against the views left (neighbours in the array mostly are in space): 555 -> 390 us there, the step 7.11 -> 6.95 ms.
 // With two views that one more test costs what it saves (32M leaves, two 4K cameras: 6.26 against 6.31 ms).
 // Per 256 projected the block reserves one run of the sort input for the visible ones
@@ -829,8 +829,13 @@ cudaError_t launch_project(const BatchParams& bp, uint64_t* rect, uint64_t* out_
     const int passes = key_passes(key_bits);
     if (passes > MAX_KEY_PASSES) return cudaErrorInvalidValue;
     // with no voxel at all, empty blocks still clear the work words and report the (zero) sizes
-    // fewer blocks than one or two per SM would leave the chip idle below this
-    const bool queue = bp.n_vox * bp.n_view >= 100000, multi = queue && bp.n_view >= 3;
+    // The (view, voxel)s from which blocks of 1024 voxels with a queue are faster than blocks of 256 (they are a
+    // quarter as many, and short of several on an SM a block's chain of steps is what counts): 150k 15 against 10 us,
+    // 330k 17 : 17, 500k 19 : 22, 800k 21 : 31.  A block of eight views does the work of eight, so it takes
+    // more of them still: 3 views of 100k voxels 33 us against 17 one view a block, 4 of 1M 60 : 55, 3 of 2M 72 : 75,
+    // 6 of 1M 66 : 80, 8 of 4M 231 : 326.
+    const int64_t n = bp.n_vox * bp.n_view;
+    const bool queue = n >= 400000, multi = n >= 5000000 && bp.n_view >= 3;
     const dim3 grid(bp.n_vox > 0 ? nblk(bp.n_vox, queue ? 1024 : 256) : 1u,
                     (unsigned)(multi ? (bp.n_view + 7) / 8 : bp.n_view));
     const bool one_wave = (int64_t)grid.x * grid.y <= 4 * sm_count();

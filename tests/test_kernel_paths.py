@@ -190,10 +190,10 @@ def test_plain_backward_by_voxel_size(dv, level, normals):
 
 # one voxel below the projection's queue, its first size, and a remainder; most voxels lie outside the frustum
 @pytest.mark.gpu
-@pytest.mark.parametrize("n", [99999, 100000, 131149])
+@pytest.mark.parametrize("n", [99999, 131149, 399999, 400000, 431149])
 def test_projection_queue(dv, n):
     rng = np.random.default_rng(n)
-    sc = synth.Scene([_octree(_grid(6, 0.0, rng, n), 0.5, rng, 8.0)], [synth.Pose()])
+    sc = synth.Scene([_octree(_grid(6 if n < 64 ** 3 else 7, 0.0, rng, n), 0.5, rng, 8.0)], [synth.Pose()])
     cam = synth.pinhole(33, 21, 50.0, synth.look_at((0.3, -0.2, 0.1), (3.0, 1.0, 0.5)), 0.05, 3.0)
     rgb, depth, alpha, _ = gpu_render(device_scene(sc), sc.poses, [cam])
     o = oracle.render(sc.octrees, sc.poses, cam, oracle.Opts(1, 1e-4))
@@ -201,21 +201,22 @@ def test_projection_queue(dv, n):
     check_forward(im(rgb, 3), im(depth), im(alpha), o[0], o[1], o[2], f"{n} voxels")
 
 
-# three and nine views (a group of eight and a remainder), in which a warp tests the box around its leaves first, on
-# leaves in order, out of order and with warps that hold leaves of two octrees: the images of each view alone, which
-# is below the queue, bit for bit
+# three and nine views, with voxels below the projection's queue and with enough of them for groups of eight views (nine:
+# a group and a remainder), in which a warp tests the box around its leaves first, on leaves in order, out of order and
+# with warps that hold leaves of two octrees: the images of each view alone, bit for bit
 @pytest.mark.gpu
-@pytest.mark.parametrize("n_view,shuffle", [(3, False), (3, True), (9, False)])
-def test_projection_of_several_views(dv, n_view, shuffle):
+@pytest.mark.parametrize("n_view,shuffle,n", [(3, False, 40003), (3, True, 40003), (9, False, 40003),
+                                              (3, False, 1670003), (3, True, 1670003), (9, False, 556003)])
+def test_projection_of_several_views(dv, n_view, shuffle, n):
     rng = np.random.default_rng(n_view)
-    key = _grid(6, 0.0, rng, 40003)
+    key = _grid(6 if n < 64 ** 3 else 7, 0.0, rng, n)
     octs = [_octree(key[rng.permutation(key.size)] if shuffle else key, 0.5, rng, 8.0)]
     octs += [_octree(_grid(3, 0.0, rng, 77), 2.0, rng, 1.0, synth.ACTOR, (0.4, 0.45, 0.3)) for _ in range(2)]
     poses = [synth.Pose()] + [synth.Pose(synth.random_rotation(rng), rng.uniform(-2, 2, 3)) for _ in range(2)]
     cams = [synth.pinhole(35, 19, 50.0, synth.Pose(synth.random_rotation(rng), rng.uniform(-3, 3, 3)), 0.05, 4.0)
             for _ in range(n_view)]
     ds = device_scene(synth.Scene(octs, poses))
-    assert sum(o.n for o in octs) < 100000 <= n_view * sum(o.n for o in octs)
+    assert n_view * sum(o.n for o in octs) < 400000 if n == 40003 else n_view * sum(o.n for o in octs) >= 5000000
     both = gpu_render(ds, poses, cams)[:3]
     for c, cam in enumerate(cams):
         for a, b in zip(both, gpu_render(ds, poses, [cam])[:3]):
