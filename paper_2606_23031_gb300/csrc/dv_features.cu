@@ -315,35 +315,33 @@ __global__ void __launch_bounds__(FL_THREADS, 3) k_fuse_local(int64_t n_pix, con
             if (VEC && e0 == S.off[0]) fl_cp_async_wait_all();  // the feature slice has landed
             __syncthreads();
             // a half-warp per row with slots, a lane per 4-channel quad: no sums to bring together
-            const uint32_t n_occ = S.n_occ;
-            for (uint32_t oi = 2 * warp + half; oi < n_occ; oi += FL_THREADS / 16) {
+            const uint32_t ov = S.start[FL_ROWS], ov_end = S.start[FL_TE];  // the overflow row, the last
+            const uint32_t n_rows = S.n_occ - (ov_end > ov ? 1u : 0u);
+            for (uint32_t oi = 2 * warp + half; oi < n_rows; oi += FL_THREADS / 16) {
                 const uint32_t r = S.occ[oi];
                 const uint32_t s0 = S.start[r], s1 = S.start[r + 1];
-                if (r < FL_ROWS) {
-                    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-                    float ws = 0.0f;
+                float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+                float ws = 0.0f;
 #pragma unroll 4
-                    for (uint32_t i = s0; i < s1; ++i) {
-                        const uint2 x = S.slot[i];
-                        const float wv = __uint_as_float(x.x);
-                        ft_fma(a, wv, S.f[x.y & 0xffffu][q]);
-                        ws += wv;
-                    }
-                    const uint32_t v = S.key[r];
-                    fl_flush4<VEC>(acc, v, C, c0 + 4 * q, a);
-                    if (q == 0 && wsum && c0 == 0 && ws != 0.0f) atomicAdd(wsum + v, ws);
-                } else {
-                    // overflow row: every slot added on its own
-                    for (uint32_t i = s0; i < s1; ++i) {
-                        const uint2 x = S.slot[i];
-                        const float wv = __uint_as_float(x.x);
-                        const uint32_t v = __ldg(vox + e0 + (x.y >> 16));
-                        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-                        ft_fma(a, wv, S.f[x.y & 0xffffu][q]);
-                        fl_flush4<VEC>(acc, v, C, c0 + 4 * q, a);
-                        if (q == 0 && wsum && c0 == 0 && wv != 0.0f) atomicAdd(wsum + v, wv);
-                    }
+                for (uint32_t i = s0; i < s1; ++i) {
+                    const uint2 x = S.slot[i];
+                    const float wv = __uint_as_float(x.x);
+                    ft_fma(a, wv, S.f[x.y & 0xffffu][q]);
+                    ws += wv;
                 }
+                const uint32_t v = S.key[r];
+                fl_flush4<VEC>(acc, v, C, c0 + 4 * q, a);
+                if (q == 0 && wsum && c0 == 0 && ws != 0.0f) atomicAdd(wsum + v, ws);
+            }
+            // the overflow row: every slot added on its own, the block's half-warps taking them in turn
+            for (uint32_t i = ov + 2 * warp + half; i < ov_end; i += FL_THREADS / 16) {
+                const uint2 x = S.slot[i];
+                const float wv = __uint_as_float(x.x);
+                const uint32_t v = __ldg(vox + e0 + (x.y >> 16));
+                float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+                ft_fma(a, wv, S.f[x.y & 0xffffu][q]);
+                fl_flush4<VEC>(acc, v, C, c0 + 4 * q, a);
+                if (q == 0 && wsum && c0 == 0 && wv != 0.0f) atomicAdd(wsum + v, wv);
             }
             __syncthreads();
             for (int i = tid; i < FL_ROWS; i += FL_THREADS) S.key[i] = FL_EMPTY;
