@@ -610,6 +610,15 @@ def dv_launch_count(reset: bool = False) -> int:
 # autograd
 # ---------------------------------------------------------------------------
 
+def _zeroed(shapes, device):
+    """Zeroed float32 tensors, each with storage of its own, cleared together (a ``torch.zeros`` for each is a launch and
+    some 20 us of host time for each)."""
+    import torch
+    ts = [torch.empty(s, device=device, dtype=torch.float32) for s in shapes]
+    torch._foreach_zero_(ts)
+    return ts
+
+
 def _autograd_fn():
     import torch
 
@@ -636,15 +645,7 @@ def _autograd_fn():
             n = ctx_.n
             st = ctx_.state
             dev = next(g.device for g in (g_rgb, g_depth, g_alpha, g_normal) if g is not None)
-            shapes = [s[0] for s in ctx_.shapes] + [s[1] for s in ctx_.shapes]
-            if n == 1:
-                grads = [T.zeros(s, device=dev, dtype=T.float32) for s in shapes]
-            else:
-                # one zeroed buffer for all gradients, each starting on a 16-byte boundary: a tensor of its own for each
-                # is a launch and some 20 us of host time for each (with one octree the views cost as much)
-                sizes = [(s.numel() + 3) // 4 * 4 for s in shapes]
-                flat = T.zeros(sum(sizes), device=dev, dtype=T.float32)
-                grads = [b[:s.numel()].view(s) for b, s in zip(flat.split(sizes), shapes)]
+            grads = _zeroed([s[0] for s in ctx_.shapes] + [s[1] for s in ctx_.shapes], dev)
             d_dens, d_sh = grads[:n], grads[n:]
             c = lambda t: None if t is None else t.contiguous()
             dv_render_backward(st, c(g_rgb), c(g_depth), c(g_alpha), d_dens, d_sh,

@@ -362,6 +362,20 @@ def test_sky_shared_cells(dv, He, We):
         assert (np.abs(a.cpu().numpy() - b) <= lim).all()
 
 
+@pytest.mark.gpu
+def test_gradients_have_storage_of_their_own(dv):
+    # dropping one octree's gradient frees it, saving one writes it alone
+    rng = np.random.default_rng(2)
+    octs = [_octree(_grid(2, 0.5, rng), 1.0, rng, 2.0)]
+    octs += [_octree(_grid(2, 0.5, rng), 1.0, rng, 0.5, synth.ACTOR, (0.25, 0.25, 0.25)) for _ in range(2)]
+    ds = device_scene(synth.Scene(octs, [synth.Pose()] * 3))
+    ts = [t.requires_grad_() for o in ds for t in (o.dens, o.sh)]
+    out = dv.render(ds, [synth.Pose()] * 3, [orbit(9, 7, 40.0, 20.0)])
+    sum(x.sum() for x in out).backward()
+    assert len({t.grad.untyped_storage().data_ptr() for t in ts}) == len(ts)
+    assert all(t.grad.untyped_storage().nbytes() == 4 * t.numel() for t in ts)
+
+
 def _side_path(idx, level, X, Lk):
     """The projection's closed form of one axis of the depth-order path (32-bit arithmetic)."""
     mask = (1 << level) - 1
