@@ -353,7 +353,7 @@ __device__ __noinline__ bool box_within(double root_size, int l, int x, int y, i
 // levels' cell sizes are the root's times powers of two, so the quotients are too).  They and the distances come
 // from the point's integer and fractional parts in finest-level units (the fractions in FP32); an index whose
 // fraction is within 1e-5 of a step, and a distance within 2e-5 of the threshold (or any, for thresholds below
-// 0.05 units), is taken from FP64.
+// 0.05 units or from 1e9 units), is taken from FP64.
 __global__ void __launch_bounds__(256) k_subdiv_flags(const float4* __restrict__ pts, int64_t m, Frame f,
                                                       double root_size, double fine, double inv_fine,
                                                       const uint32_t* __restrict__ levels_p, double thr,
@@ -366,6 +366,7 @@ __global__ void __launch_bounds__(256) k_subdiv_flags(const float4* __restrict__
     const float pc[3] = {pt.x, pt.y, pt.z};
     const double thr_d = fmin(thr * inv_fine, 1e9), thr_i = floor(thr_d);
     const float thr_u = (float)thr_d, thr_f = (float)(thr_d - thr_i);
+    const bool huge = thr_d == 1e9;  // not the threshold any more: every index and distance from FP64
     double p[3];
     int flo[3], fhi[3], pi[3];
     float pf[3];
@@ -380,7 +381,7 @@ __global__ void __launch_bounds__(256) k_subdiv_flags(const float4* __restrict__
         auto index = [&](float fr, int64_t base, double x) {
             const float fl = floorf(fr), r = fr - fl;
             int64_t i = base + (int)fl;
-            if (r < 1e-5f || r > 1.0f - 1e-5f) {
+            if (huge || r < 1e-5f || r > 1.0f - 1e-5f) {
                 const double e = floor(x / fine);
                 i = (int64_t)fmin(fmax(e, -1.0), (double)(1 << SD_FINE));
             }

@@ -324,6 +324,18 @@ def test_subdivide_thresholds(dv, center, root, thr):
     np.testing.assert_array_equal(out.cpu().numpy().view(np.uint64), ref)
 
 
+# a threshold of more than 1e9 cells of the finest level, and a point nearly as far away: every leaf is within it
+@pytest.mark.gpu
+def test_subdivide_threshold_of_many_roots(dv):
+    import torch
+    keys = np.concatenate([_grid(l, 2.0, np.random.default_rng(l)) for l in (1, 2, 3)])
+    center, root, thr = (0.0, 0.0, 0.0), 1.1, 5000.0
+    cloud = torch.tensor([[-4196.0, 0.0, 0.0]], device="cuda")
+    out = dv.dv_subdivide_round(_keys_t(keys), 3, center, root, cloud, thr)
+    assert _reached(keys, center, root, cloud.cpu().numpy(), thr).all()
+    assert out.numel() == 8 * keys.size
+
+
 @pytest.mark.gpu
 def test_visibility_many_cameras(dv):
     # cameras all around, inside and outside the root, with narrow and wide views; a ragged last block
