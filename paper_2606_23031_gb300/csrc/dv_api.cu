@@ -1282,7 +1282,7 @@ dv_status dv_features_fuse(dv_ctx* ctx, int64_t n_pix, const int64_t* offsets, c
 // ---- LiDAR-guided initialisation (Sec. 3.3) ----
 
 static dv_status init_begin(dv_ctx* ctx, const uint64_t* keys, int64_t n, int32_t max_level, dv::Arena& ar,
-                            cudaStream_t s, bool* outside = nullptr) {
+                            cudaStream_t s, bool* outside = nullptr, uint32_t* levels = nullptr) {
     if (!ctx) return DV_ERR_INVALID_ARG;
     ctx->err.clear();
     if (n < 0 || (n > 0 && !keys)) return fail(ctx, DV_ERR_INVALID_ARG, "bad key array");
@@ -1293,6 +1293,7 @@ static dv_status init_begin(dv_ctx* ctx, const uint64_t* keys, int64_t n, int32_
     if (e != cudaSuccess) return cuda_fail(ctx, e, "key levels");
     if (lv[0] >> (max_level + 1)) return fail(ctx, DV_ERR_INVALID_ARG, "a leaf level above max_level");
     if (outside) *outside = lv[1] != 0;
+    if (levels) *levels = lv[0];
     return DV_OK;
 }
 
@@ -1357,10 +1358,11 @@ dv_status dv_subdivide_round(dv_ctx* ctx, const uint64_t* keys, int64_t n, int32
     dv::Arena ar;
     ar.pool = ctx->pool;
     ar.stream = s;
-    dv_status st = init_begin(ctx, keys, n, max_level, ar, s);
+    uint32_t levels = 0;
+    dv_status st = init_begin(ctx, keys, n, max_level, ar, s, nullptr, &levels);
     cudaError_t e = cudaSuccess;
     if (st == DV_OK)
-        e = dv::subdivide_round(keys, n, center, root_size, max_level, cloud, n_points, threshold, out, n_out, ar, s);
+        e = dv::subdivide_round(keys, n, levels, center, root_size, max_level, cloud, n_points, threshold, out, n_out, ar, s);
     ar.release();
     if (st != DV_OK) return st;
     if (e != cudaSuccess) return cuda_fail(ctx, e, "subdivision");

@@ -10,7 +10,8 @@
 //    v_far, so beyond that radius the corner takes v_far.
 //  * Subdivision: every LiDAR point visits, for each level, the leaf cells whose box lies within
 //    the threshold of it (exact point-box distance) and looks each up in a hash table of the leaf keys;
-//    found leaves are flagged.  The output keeps the unflagged leaves in input order, then the
+//    found leaves are flagged.  At levels where the cells in reach of a point are many (a threshold of several
+//    leaves), every leaf looks for a point in reach of it instead, in a grid of the points.  The output keeps the unflagged leaves in input order, then the
 //    children of the flagged ones, child 0 of every flagged leaf first, then child 1, ...
 //
 // What bounds these kernels.  Their results are defined in FP64, and this GPU issues FP64 at 1/64 of the
@@ -154,8 +155,13 @@ int ht_bits(int64_t n) {
 
 // ---- point grid of the soft prior: cell -> [start, start + cnt) of the points ordered by cell ----
 
-// EXACT: the cell of the FP64 quotient (the prior's cells); else some cell near it (points only have to be
-// brought together)
+// some cell near the coordinate's FP64 quotient, a monotone function of it: kept in range as a number before it is
+// converted (a point may be anything)
+__device__ __forceinline__ int near_cell(float x, double root_min, double inv_h) {
+    return (int)fminf(fmaxf((x - (float)root_min) * (float)inv_h, -1e6f), 1e6f);
+}
+
+// EXACT: the cell of the FP64 quotient (the prior's cells); else near_cell
 template <bool EXACT>
 __global__ void __launch_bounds__(256) k_cell_count(const float* __restrict__ cloud, int64_t m, Frame f, double h,
                                                     double inv_h, uint64_t* __restrict__ table, int bits,
@@ -168,8 +174,8 @@ __global__ void __launch_bounds__(256) k_cell_count(const float* __restrict__ cl
     for (int a = 0; a < 3; ++a) {
         if constexpr (EXACT)
             c[a] = (int64_t)floor_div((double)cloud[t * 3 + a] - f.root_min[a], h, inv_h);
-        else  // kept in range as a number before it is converted (a point may be anything)
-            c[a] = (int64_t)(int)fminf(fmaxf((cloud[t * 3 + a] - (float)f.root_min[a]) * (float)inv_h, -1e6f), 1e6f);
+        else
+            c[a] = near_cell(cloud[t * 3 + a], f.root_min[a], inv_h);
     }
     const uint32_t s = ht_enter(table, bits, cell_key(c[0], c[1], c[2]), fail);
     slot[t] = s;
@@ -308,14 +314,12 @@ constexpr int SD_SIDE = 1 << SD_COARSE;
 // enters every leaf key (the lowest index of equal keys counts) and the levels below each coarse cell
 __global__ void __launch_bounds__(256) k_leaf_enter(const uint64_t* __restrict__ keys, int64_t n,
                                                     uint64_t* __restrict__ table, uint32_t* __restrict__ idx, int bits,
-                                                    uint32_t* __restrict__ coarse, uint32_t* __restrict__ levels,
-                                                    uint32_t* __restrict__ fail) {
+                                                    uint32_t* __restrict__ coarse, uint32_t* __restrict__ fail) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    uint32_t lev = 0;
     if (t < n) {
         const uint64_t k = keys[t];
         const int l = (int)((k >> 57) & 31);
-        lev = 1u << l;
+        const uint32_t lev = 1u << l;
         if (k != HT_EMPTY) atomicMin(idx + ht_enter(table, bits, k, fail), (uint32_t)t);
         if (l >= SD_COARSE) {
             const int sh = l - SD_COARSE;
@@ -327,8 +331,6 @@ __global__ void __launch_bounds__(256) k_leaf_enter(const uint64_t* __restrict__
             }
         }
     }
-    lev = __reduce_or_sync(0xffffffffu, lev);
-    if ((threadIdx.x & 31) == 0 && (lev & ~*(volatile uint32_t*)levels)) atomicOr(levels, lev);
 }
 
 // Whether a point (from the root's corner) lies within thr of the box of cell (x, y, z) of level l.  Out of
@@ -356,7 +358,7 @@ __device__ __noinline__ bool box_within(double root_size, int l, int x, int y, i
 // 0.05 units or from 1e9 units), is taken from FP64.
 __global__ void __launch_bounds__(256) k_subdiv_flags(const float4* __restrict__ pts, int64_t m, Frame f,
                                                       double root_size, double fine, double inv_fine,
-                                                      const uint32_t* __restrict__ levels_p, double thr,
+                                                      uint32_t look_at, double thr,
                                                       const uint64_t* __restrict__ table,
                                                       const uint32_t* __restrict__ idx, int bits,
                                                       const uint32_t* __restrict__ coarse, uint8_t* __restrict__ split) {
@@ -390,7 +392,7 @@ __global__ void __launch_bounds__(256) k_subdiv_flags(const float4* __restrict__
         flo[a] = index(pf[a] - thr_f, (int64_t)pi[a] - (int64_t)thr_i, p[a] - thr);
         fhi[a] = index(pf[a] + thr_f, (int64_t)pi[a] + (int64_t)thr_i, p[a] + thr);
     }
-    uint32_t levels = live ? *levels_p : 0u;
+    uint32_t levels = live ? look_at : 0u;  // the levels looked at from the points
     {
         // only levels that some coarse cell around the point holds
         int c0[3], c1[3], n = 1;
@@ -454,6 +456,103 @@ __global__ void __launch_bounds__(256) k_subdiv_flags(const float4* __restrict__
             }
         }
     }
+}
+
+constexpr int64_t FAR_CELLS = 4096;  // cells of the point grid a leaf looks into at most, else at all points
+
+// One warp per leaf of the levels in `far`: flags the leaf if a point is within thr of its box.  The points lie in a
+// grid of cells of half the threshold, so those in reach of a leaf (a third of the threshold or smaller, see
+// subdivide_round) are in at most 7^3 cells: every lane probes one, the leaf's own first, and the warp tests the
+// points of the cells found until one is in reach.  (k_subdiv_flags looks at (2 thr / leaf + 2)^3 cells for a point.)
+// A point's cell is a monotone function of its coordinates, so the cells of the reach's two ends bound those of the
+// points in it; where they are too many (coordinates that FP32 hardly resolves at the threshold, thresholds beyond
+// the root), all points are tested.  Decided in FP32 from the leaf's centre split into two floats, within 2e-5
+// of the threshold in FP64 by k_subdiv_flags' rule.
+__global__ void __launch_bounds__(256) k_subdiv_far(const uint64_t* __restrict__ keys, int64_t n, uint32_t far, Frame f,
+                                                    double root_size, double thr, const uint64_t* __restrict__ table,
+                                                    const uint32_t* __restrict__ idx, int bits,
+                                                    const uint64_t* __restrict__ cells, int cell_bits,
+                                                    const uint32_t* __restrict__ cnt, const uint32_t* __restrict__ start,
+                                                    const float4* __restrict__ pts, int64_t m, double inv_h,
+                                                    uint8_t* __restrict__ split) {
+    const int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (t >= n) return;
+    const uint64_t k = keys[t];
+    const int l = (int)((k >> 57) & 31);
+    if (!((far >> l) & 1u)) return;
+    const int x = (int)(k & kIMask), y = (int)((k >> 19) & kIMask), z = (int)((k >> 38) & kIMask);
+    // a key that is no cell of the grid is in no point's reach; of equal keys the lowest index counts
+    if (k >> 62 || (x | y | z) >> l) return;
+    const uint32_t e = ht_find(table, bits, k, true);
+    if (e == ~0u || (int64_t)idx[e] != t) return;
+    const double s = ldexp(root_size, -l);
+    const int at[3] = {x, y, z};
+    float qh[3], ql[3];
+    int c0[3], w[3];
+    int64_t n_cell = 1;
+    float big = 0.0f;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const double b0 = f.root_min[a] + (double)at[a] * s, q = b0 + 0.5 * s;
+        qh[a] = (float)q;
+        ql[a] = (float)(q - (double)qh[a]);
+        big = fmaxf(big, fabsf(qh[a]));
+        // the cells k_cell_count gives to the ends of the reach
+        const float lo = __double2float_rd(b0 - thr * (1.0 + 1e-9)), hi = __double2float_ru(b0 + s + thr * (1.0 + 1e-9));
+        c0[a] = near_cell(lo, f.root_min[a], inv_h);
+        w[a] = near_cell(hi, f.root_min[a], inv_h) - c0[a] + 1;
+        n_cell *= min(max(w[a], 1), 1 << 20);
+    }
+    const float thr_u = (float)thr, half = (float)(0.5 * s);
+    const bool fp32 = thr_u > 1e-15f && thr_u < 1e15f && thr_u > 1e-8f * big;
+    const float t2_lo = thr_u * thr_u * (1.0f - 2e-5f), t2_hi = thr_u * thr_u * (1.0f + 2e-5f);
+    auto reached = [&](float4 pt) {
+        if (fp32) {
+            auto gap = [&](float p, int a) {
+                const float g = fabsf((p - qh[a]) - ql[a]) - half;
+                return g <= 0.0f ? 0.0f : g;  // (not a number stays that)
+            };
+            const float gx = gap(pt.x, 0), gy = gap(pt.y, 1), gz = gap(pt.z, 2);
+            const float d2 = fmaf(gx, gx, fmaf(gy, gy, gz * gz));
+            if (!(d2 <= t2_hi)) return false;
+            if (d2 < t2_lo) return true;
+        }
+        const float pc[3] = {pt.x, pt.y, pt.z};
+        double p[3];
+        bool in = true;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            p[a] = (double)pc[a] - f.root_min[a];
+            const double i0 = floor((p[a] - thr) / s), i1 = floor((p[a] + thr) / s);
+            in = in && fmax(i0, -1.0) <= (double)at[a] && fmax(i1, -1.0) >= (double)at[a];
+        }
+        return in && box_within(root_size, l, x, y, z, p[0], p[1], p[2], thr);
+    };
+    // the points [e0, e0 + m0), the lanes in turn; true if one is in reach
+    auto any_reached = [&](int64_t e0, int64_t m0) {
+        for (int64_t j = 0; j < m0; j += 32)
+            if (__any_sync(0xffffffffu, j + lane < m0 && reached(__ldg(pts + e0 + j + lane)))) return true;
+        return false;
+    };
+    bool hit = false;
+    if (n_cell > FAR_CELLS) {
+        hit = any_reached(0, m);
+    } else {
+        const int nc = (int)n_cell;
+        for (int b = 0; b < nc && !hit; b += 32) {
+            const int c = (b + lane + nc / 2) % nc;
+            const uint64_t key = cell_key(c0[0] + c % w[0], c0[1] + c / w[0] % w[1], c0[2] + c / (w[0] * w[1]));
+            const uint32_t slot = ht_find(cells, cell_bits, key, b + lane < nc);
+            const uint32_t e0 = slot != ~0u ? start[slot] : 0u, m0 = slot != ~0u ? cnt[slot] : 0u;
+            for (unsigned found = __ballot_sync(0xffffffffu, m0 != 0u); found && !hit; found &= found - 1) {
+                const int src = __ffs((int)found) - 1;
+                const int64_t from = __shfl_sync(0xffffffffu, e0, src), many = __shfl_sync(0xffffffffu, m0, src);
+                hit = any_reached(from, min(many, m - from));
+            }
+        }
+    }
+    if (hit && lane == 0) split[t] = 1;
 }
 
 __global__ void k_subdiv_write(const uint64_t* __restrict__ keys, int64_t n, const uint8_t* __restrict__ split,
@@ -769,9 +868,17 @@ cudaError_t soft_prior(const uint64_t* grid, int64_t n_corners, const double* ce
     return cudaErrorUnknown;  // no table of eight times the capacity has room within HT_PROBES of every key's home
 }
 
-cudaError_t subdivide_round(const uint64_t* keys, int64_t n, const double* center, double root_size, int max_level,
-                            const float* cloud, int64_t m, float thr, uint64_t* out, int64_t* n_out, Arena& ar,
-                            cudaStream_t s) {
+// Levels at which a leaf looks for points: those where the cells in reach of a point may be more than FAR_FROM, and more
+// than this share of the leaves.  Without them a threshold of some leaves' size runs for minutes ((2 thr / leaf + 2)^3
+// cells a point and level, all in lockstep).  Both sides, all levels one way, in ms at thresholds of 3, 6, 12 and
+// 16 of the finest leaves (512 to 39,304 cells): 30k leaves and 81k points 1.0, 4.7, 38, 87 from the points and 0.6, 0.3,
+// 0.4, 0.3 from the leaves; 500k and 1.35M 4.4, 23, 163, 373 and 29, 17, 1.9, 1.8; 1M and 2.7M 8.1, 44, 321, 728
+// and 314, 194, 4.6, 3.9 (points in many cells around a leaf and none in its reach cost the most).
+constexpr double FAR_FROM = 512.0, FAR_SHARE = 1.0 / 100.0;
+
+cudaError_t subdivide_round(const uint64_t* keys, int64_t n, uint32_t levels, const double* center, double root_size,
+                            int max_level, const float* cloud, int64_t m, float thr, uint64_t* out, int64_t* n_out,
+                            Arena& ar, cudaStream_t s) {
     *n_out = n;
     if (n <= 0) return cudaSuccess;
     const Frame f = make_frame(center, root_size, max_level);
@@ -782,52 +889,59 @@ cudaError_t subdivide_round(const uint64_t* keys, int64_t n, const double* cente
     uint32_t* no = ar.alloc<uint32_t>(n);
     uint32_t* pos_s = ar.alloc<uint32_t>(n);
     uint32_t* pos_k = ar.alloc<uint32_t>(n);
-    uint32_t* tot = ar.alloc<uint32_t>(4);  // split, kept; levels present, a key without a slot
+    uint32_t* tot = ar.alloc<uint32_t>(3);  // split, kept, a key without a slot
     if (ar.err != cudaSuccess) return ar.err;
-    cudaError_t e = cudaSuccess;
-    uint32_t hd[4] = {0, 0, 0, 0};
-    float4* pts = nullptr;
-    if (m > 0) {
-        // the points ordered by cells of 16 thresholds (flags kernel with the points as they come 1,300 us, cells of
-        // 1, 4, 16, 64 thresholds 1,284, 924, 730, 714 us, and 75 to 110 us for the order).  A point that finds no slot
-        // counts in its last slot: the order is all that matters
-        const int bits = std::min(ht_bits(m), 32);
-        const size_t cap = (size_t)1 << bits;
-        uint64_t* table = ar.alloc<uint64_t>(cap);
-        uint32_t* cnt = ar.alloc<uint32_t>(cap + 2);
-        uint32_t* start = ar.alloc<uint32_t>(cap);
-        uint32_t* slot = ar.alloc<uint32_t>(m);
-        uint32_t* rank = ar.alloc<uint32_t>(m);
-        pts = ar.alloc<float4>(m);
-        if (ar.err != cudaSuccess) return ar.err;
-        e = cudaMemsetAsync(table, 0xff, cap * sizeof(uint64_t), s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(cnt, 0, (cap + 2) * sizeof(uint32_t), s);
-        if (e != cudaSuccess) return e;
-        const double h = std::max(16.0 * (double)thr, ldexp(root_size, -SD_FINE));
-        k_cell_count<false><<<nb(m), 256, 0, s>>>(cloud, m, f, h, 1.0 / h, table, bits, cnt, slot, rank, cnt + cap + 1);
-        k_cell_alloc<<<(unsigned)(cap / 256), 256, 0, s>>>(cnt, (int64_t)cap, start, cnt + cap);
-        k_cell_scatter<<<nb(m), 256, 0, s>>>(cloud, m, slot, rank, start, pts);
-        count_launches(3);
+    uint32_t far = 0;
+    for (int l = 0; l <= max_level; ++l) {
+        const double side = std::min(2.0 * (double)thr / ldexp(root_size, -l) + 2.0, ldexp(1.0, l));
+        if (side * side * side > std::max(FAR_FROM, FAR_SHARE * (double)n)) far |= levels & (1u << l);
     }
+    uint32_t hd[3] = {0, 0, 0};
     for (int more = 0; more < HT_TRIES; ++more) {
-        if (e == cudaSuccess) e = cudaMemsetAsync(split, 0, n, s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(tot, 0, 4 * sizeof(uint32_t), s);
+        cudaError_t e = cudaMemsetAsync(split, 0, n, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(tot, 0, 3 * sizeof(uint32_t), s);
         if (e != cudaSuccess) return e;
         if (m > 0) {
-            const int bits = ht_bits(n) + more;
-            const size_t cap = (size_t)1 << bits;
+            // The points ordered by cells of 16 thresholds (flags kernel with the points as they come 1,300 us, cells of
+            // 1, 4, 16, 64 thresholds 1,284, 924, 730, 714 us, and 75 to 110 us for the order): a point that finds no
+            // slot counts in its last slot, the order is all that matters.  Where leaves look for points, cells of half
+            // a threshold, in which every point has its slot.
+            const int pbits = std::min(ht_bits(m) + (far ? more : 0), 32), bits = ht_bits(n) + more;
+            const size_t pcap = (size_t)1 << pbits, cap = (size_t)1 << bits;
+            uint64_t* cells = ar.alloc<uint64_t>(pcap);
+            uint32_t* cnt = ar.alloc<uint32_t>(pcap + 2);
+            uint32_t* start = ar.alloc<uint32_t>(pcap);
+            uint32_t* slot = ar.alloc<uint32_t>(m);
+            uint32_t* rank = ar.alloc<uint32_t>(m);
+            float4* pts = ar.alloc<float4>(m);
             uint64_t* table = ar.alloc<uint64_t>(cap);
             uint32_t* idx = ar.alloc<uint32_t>(cap);
             if (ar.err != cudaSuccess) return ar.err;
-            e = cudaMemsetAsync(table, 0xff, cap * sizeof(uint64_t), s);
+            e = cudaMemsetAsync(cells, 0xff, pcap * sizeof(uint64_t), s);
+            if (e == cudaSuccess) e = cudaMemsetAsync(cnt, 0, (pcap + 2) * sizeof(uint32_t), s);
+            if (e == cudaSuccess) e = cudaMemsetAsync(table, 0xff, cap * sizeof(uint64_t), s);
             if (e == cudaSuccess) e = cudaMemsetAsync(idx, 0xff, cap * sizeof(uint32_t), s);
             if (e == cudaSuccess) e = cudaMemsetAsync(coarse, 0, COARSE * sizeof(uint32_t), s);
             if (e != cudaSuccess) return e;
-            k_leaf_enter<<<nb(n), 256, 0, s>>>(keys, n, table, idx, bits, coarse, tot + 2, tot + 3);
-            k_subdiv_flags<<<nb(m), 256, 0, s>>>(pts, m, f, root_size, ldexp(root_size, -SD_FINE),
-                                                 (double)(1 << SD_FINE) / root_size, tot + 2, thr, table, idx, bits, coarse,
-                                                 split);
-            count_launches(2);
+            const double h = far ? 0.5 * std::min((double)thr, 4.0 * root_size)
+                                 : std::max(16.0 * (double)thr, ldexp(root_size, -SD_FINE));
+            k_cell_count<false><<<nb(m), 256, 0, s>>>(cloud, m, f, h, 1.0 / h, cells, pbits, cnt, slot, rank,
+                                                      far ? tot + 2 : cnt + pcap + 1);
+            k_cell_alloc<<<(unsigned)(pcap / 256), 256, 0, s>>>(cnt, (int64_t)pcap, start, cnt + pcap);
+            k_cell_scatter<<<nb(m), 256, 0, s>>>(cloud, m, slot, rank, start, pts);
+            k_leaf_enter<<<nb(n), 256, 0, s>>>(keys, n, table, idx, bits, coarse, tot + 2);
+            count_launches(4);
+            if (levels & ~far) {
+                k_subdiv_flags<<<nb(m), 256, 0, s>>>(pts, m, f, root_size, ldexp(root_size, -SD_FINE),
+                                                     (double)(1 << SD_FINE) / root_size, levels & ~far, thr, table, idx,
+                                                     bits, coarse, split);
+                count_launches(1);
+            }
+            if (far) {
+                k_subdiv_far<<<(unsigned)((n + 7) / 8), 256, 0, s>>>(keys, n, far, f, root_size, thr, table, idx, bits, cells,
+                                                                     pbits, cnt, start, pts, m, 1.0 / h, split);
+                count_launches(1);
+            }
         }
         k_not<<<nb(n), 256, 0, s>>>(split, n, yes, no);
         count_launches(1);
@@ -836,9 +950,9 @@ cudaError_t subdivide_round(const uint64_t* keys, int64_t n, const double* cente
         if (e == cudaSuccess) e = cudaMemcpyAsync(hd, tot, sizeof(hd), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return e;
-        if (!hd[3]) break;
+        if (!hd[2]) break;
     }
-    if (hd[3]) return cudaErrorUnknown;  // see soft_prior
+    if (hd[2]) return cudaErrorUnknown;  // see soft_prior
     const int64_t n_split = hd[0], n_keep = hd[1];
     k_subdiv_write<<<nb(n), 256, 0, s>>>(keys, n, split, pos_k, pos_s, n_keep, n_split, out);
     count_launches(1);

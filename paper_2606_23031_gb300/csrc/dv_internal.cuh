@@ -274,9 +274,10 @@ cudaError_t shared_corners(const uint64_t* keys, int64_t n, int max_level, bool 
 cudaError_t soft_prior(const uint64_t* grid, int64_t n_corners, const double* center, double root_size, int max_level,
                        const float* cloud, int64_t m, float s_min, float v_close, float v_far, float* dens, Arena& ar,
                        cudaStream_t s);
-cudaError_t subdivide_round(const uint64_t* keys, int64_t n, const double* center, double root_size, int max_level,
-                            const float* cloud, int64_t m, float thr, uint64_t* out, int64_t* n_out, Arena& ar,
-                            cudaStream_t s);
+// levels: those of the keys, as a bit mask
+cudaError_t subdivide_round(const uint64_t* keys, int64_t n, uint32_t levels, const double* center, double root_size,
+                            int max_level, const float* cloud, int64_t m, float thr, uint64_t* out, int64_t* n_out,
+                            Arena& ar, cudaStream_t s);
 // uniform leaf grid of an actor (Sec. 3.3, assets): keys of the 8^level leaves (i fastest) and every
 // corner density set to v_init
 cudaError_t asset_grid(int level, float v_init, uint64_t* keys, float* dens, cudaStream_t s);

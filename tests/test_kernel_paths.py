@@ -336,6 +336,46 @@ def test_subdivide_threshold_of_many_roots(dv):
     assert out.numel() == 8 * keys.size
 
 
+# thresholds of several leaves, at which leaves look for points (beside coarse leaves that points look for): a cluster in
+# a corner whose reach ends inside the set, exact ties, equal keys (the first counts), a leaf outside the grid, points
+# that are not numbers; far from the origin; more of the points' cells than are looked into; and cells of which a point
+# has 7e13 in reach
+@pytest.mark.gpu
+@pytest.mark.parametrize("center,root,thr,levels", [((0.0, 0.0, 0.0), 2.0, 0.5, (1, 3, 5, 6)),
+                                                    ((4000.5, -2500.25, 80.0), 3.7, 0.61, (2, 6)),
+                                                    ((0.0, 0.0, 0.0), 2.0, 300.0, (1, 4, 7)),
+                                                    ((1.0, 2.0, 3.0), 10.0, 3.0, (2, 9, 16))])
+def test_subdivide_reach_of_many_leaves(dv, center, root, thr, levels):
+    import torch
+    rng = np.random.default_rng(9)
+    parts = []
+    for l in levels:
+        m = 1 << l
+        c = rng.integers(0, m, (min(600, m ** 3), 3))
+        parts.append(np.unique(synth.pack_keys(np.full(len(c), l), *c.T)))
+    keys = np.concatenate(parts)
+    keys = keys[rng.permutation(keys.size)]
+    L = levels[-1]
+    keys = np.concatenate([keys, synth.pack_keys([L, L], [1 << L, 3], [0, 5], [1, 2 << L]), keys[:40]])
+    corner = np.asarray(center) - 0.4 * root
+    cloud = corner + rng.uniform(-0.15, 0.1, (60, 3)) * root
+    if root == 2.0:
+        cloud = np.concatenate([cloud, corner.round(1) + rng.integers(-3, 4, (20, 3)) / 16.0])
+    cloud = np.float32(np.concatenate([cloud, cloud[:5]]))
+    thr = float(np.float32(thr))
+    bad = np.float32([[np.nan, 0, 0], [np.inf, 0, 0], [1e30, -1e30, 0]])
+    out = dv.dv_subdivide_round(_keys_t(keys), L, center, root, torch.as_tensor(np.concatenate([bad, cloud]), device="cuda"), thr)
+    lev, *ijk = oi._unpack(keys)
+    first = np.zeros(keys.size, bool)
+    first[np.unique(keys, return_index=True)[1]] = True
+    hit = _reached(keys, center, root, cloud, thr) & first & (np.stack(ijk, 1) < (1 << lev)[:, None]).all(1)
+    assert hit.any() and ((~hit & first).sum() > 50 or thr > root)
+    lev, i, j, k = (x[hit] for x in oi._unpack(keys))
+    ref = np.concatenate([keys[~hit]] + [oi._pack(lev + 1, 2 * i + (c & 1), 2 * j + (c >> 1 & 1), 2 * k + (c >> 2))
+                                         for c in range(8)])
+    np.testing.assert_array_equal(out.cpu().numpy().view(np.uint64), ref)
+
+
 @pytest.mark.gpu
 def test_visibility_many_cameras(dv):
     # cameras all around, inside and outside the root, with narrow and wide views; a ragged last block
