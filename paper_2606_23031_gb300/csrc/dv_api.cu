@@ -1335,11 +1335,12 @@ dv_status dv_soft_prior(dv_ctx* ctx, const uint64_t* grid, int64_t n_corners, co
     dv::Arena ar;
     ar.pool = ctx->pool;
     ar.stream = s;
+    bool no_room = false;
     cudaError_t e = dv::soft_prior(grid, n_corners, center, root_size, max_level, cloud, n_points, s_min, v_close, v_far,
-                                   dens, ar, s);
-    if (e == cudaSuccess && n_points > 0) e = cudaStreamSynchronize(s);
+                                   dens, ar, s, &no_room);
     ar.release();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "soft prior");
+    if (no_room) return fail(ctx, DV_ERR_CAPACITY, "the point cells found no room in a hash table; output invalid");
     return DV_OK;
 }
 
@@ -1359,13 +1360,16 @@ dv_status dv_subdivide_round(dv_ctx* ctx, const uint64_t* keys, int64_t n, int32
     ar.pool = ctx->pool;
     ar.stream = s;
     uint32_t levels = 0;
+    bool no_room = false;
     dv_status st = init_begin(ctx, keys, n, max_level, ar, s, nullptr, &levels);
     cudaError_t e = cudaSuccess;
     if (st == DV_OK)
-        e = dv::subdivide_round(keys, n, levels, center, root_size, max_level, cloud, n_points, threshold, out, n_out, ar, s);
+        e = dv::subdivide_round(keys, n, levels, center, root_size, max_level, cloud, n_points, threshold, out, n_out, ar,
+                                s, &no_room);
     ar.release();
     if (st != DV_OK) return st;
     if (e != cudaSuccess) return cuda_fail(ctx, e, "subdivision");
+    if (no_room) return fail(ctx, DV_ERR_CAPACITY, "the leaf keys found no room in a hash table; nothing was written");
     return DV_OK;
 }
 

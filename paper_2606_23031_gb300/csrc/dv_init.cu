@@ -103,13 +103,16 @@ __device__ __forceinline__ double floor_div(double x, double unit, double inv) {
 
 // ---- open-addressing tables of 64-bit keys (power-of-two capacity, at most half full) ----
 // A key is entered within HT_PROBES slots of its home, or the call's flag is set and the host takes a
-// larger table, so every probe loop has a fixed bound.  Searches are made by whole warps in step (a lane's
+// larger table and, with another salt, other homes, so every probe loop has a fixed bound.  Searches are made by whole warps in step (a lane's
 // own loop would run its lanes one after another).
 constexpr uint64_t HT_EMPTY = ~0ull;  // never a cell key (63 bits) nor a key looked up (62 bits)
 constexpr int HT_PROBES = 64;
 constexpr int HT_TRIES = 4;  // tables of 1, 2, 4, 8 times the capacity
+// of a try; 0 for the first.  (Any odd multiplier: the keys differ from the salted ones by bits all over the word.)
+constexpr uint64_t ht_salt(int more) { return (uint64_t)more * 0xd6e8feb86659fd93ull; }
 
-__device__ __forceinline__ uint32_t ht_first(uint64_t key, int bits) {
+__device__ __forceinline__ uint32_t ht_first(uint64_t key, int bits, uint64_t salt) {
+    key ^= salt;
     key ^= key >> 32;
     key *= 0x9e3779b97f4a7c15ull;  // 2^64 / golden ratio, odd
     key ^= key >> 29;
@@ -118,9 +121,9 @@ __device__ __forceinline__ uint32_t ht_first(uint64_t key, int bits) {
 }
 
 // the key's slot, entering it where it is new
-__device__ __forceinline__ uint32_t ht_enter(uint64_t* table, int bits, uint64_t key, uint32_t* fail) {
+__device__ __forceinline__ uint32_t ht_enter(uint64_t* table, int bits, uint64_t salt, uint64_t key, uint32_t* fail) {
     const uint32_t mask = (uint32_t)((1ull << bits) - 1);
-    uint32_t h = ht_first(key, bits);
+    uint32_t h = ht_first(key, bits, salt);
     for (int i = 0; i < HT_PROBES; ++i) {
         const unsigned long long old = atomicCAS(reinterpret_cast<unsigned long long*>(table + h), HT_EMPTY, key);
         if (old == HT_EMPTY || old == key) return h;
@@ -131,9 +134,10 @@ __device__ __forceinline__ uint32_t ht_enter(uint64_t* table, int bits, uint64_t
 }
 
 // the slots of the warp's keys, ~0u where a key is absent or its lane not active (all 32 lanes call)
-__device__ __forceinline__ uint32_t ht_find(const uint64_t* __restrict__ table, int bits, uint64_t key, bool active) {
+__device__ __forceinline__ uint32_t ht_find(const uint64_t* __restrict__ table, int bits, uint64_t salt, uint64_t key,
+                                            bool active) {
     const uint32_t mask = (uint32_t)((1ull << bits) - 1);
-    uint32_t h = ht_first(key, bits), found = ~0u;
+    uint32_t h = ht_first(key, bits, salt), found = ~0u;
     for (int i = 0; i < HT_PROBES; ++i) {
         if (!__any_sync(0xffffffffu, active)) break;
         if (active) {
@@ -164,7 +168,7 @@ __device__ __forceinline__ int near_cell(float x, double root_min, double inv_h)
 // EXACT: the cell of the FP64 quotient (the prior's cells); else near_cell
 template <bool EXACT>
 __global__ void __launch_bounds__(256) k_cell_count(const float* __restrict__ cloud, int64_t m, Frame f, double h,
-                                                    double inv_h, uint64_t* __restrict__ table, int bits,
+                                                    double inv_h, uint64_t* __restrict__ table, int bits, uint64_t salt,
                                                     uint32_t* __restrict__ cnt, uint32_t* __restrict__ slot,
                                                     uint32_t* __restrict__ rank, uint32_t* __restrict__ fail) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -177,7 +181,7 @@ __global__ void __launch_bounds__(256) k_cell_count(const float* __restrict__ cl
         else
             c[a] = near_cell(cloud[t * 3 + a], f.root_min[a], inv_h);
     }
-    const uint32_t s = ht_enter(table, bits, cell_key(c[0], c[1], c[2]), fail);
+    const uint32_t s = ht_enter(table, bits, salt, cell_key(c[0], c[1], c[2]), fail);
     slot[t] = s;
     rank[t] = atomicAdd(cnt + s, 1u);
 }
@@ -225,7 +229,7 @@ __global__ void __launch_bounds__(256) k_cell_scatter(const float* __restrict__ 
 // second point comes within 2e-5 of it, all such points' are.
 __global__ void __launch_bounds__(256) k_soft_prior(const uint64_t* __restrict__ grid, int64_t n_corners, Frame f,
                                                     double h, double inv_h, const uint64_t* __restrict__ table,
-                                                    int bits, const uint32_t* __restrict__ cnt,
+                                                    int bits, uint64_t salt, const uint32_t* __restrict__ cnt,
                                                     const uint32_t* __restrict__ start, int64_t m,
                                                     const float4* __restrict__ pts, float s, float v_close,
                                                     float v_far, float* __restrict__ dens) {
@@ -265,7 +269,7 @@ __global__ void __launch_bounds__(256) k_soft_prior(const uint64_t* __restrict__
                 const int dx = r % 3 - 1, dy = (r / 3) % 3 - 1, dz = r / 9 - 1;
                 const float gx = gap(0, dx), gy = gap(1, dy), gz = gap(2, dz);
                 const bool look = live && !(fmaf(gx, gx, fmaf(gy, gy, gz * gz)) * 0.99999f > bound());
-                const uint32_t slot = ht_find(table, bits, cell_key(c[0] + dx, c[1] + dy, c[2] + dz), look);
+                const uint32_t slot = ht_find(table, bits, salt, cell_key(c[0] + dx, c[1] + dy, c[2] + dz), look);
                 if (slot != ~0u) {
                     const uint32_t e0 = start[slot], n = min(cnt[slot], (uint32_t)m - e0);
                     for (uint32_t i = 0; i < n; ++i) {
@@ -314,13 +318,14 @@ constexpr int SD_SIDE = 1 << SD_COARSE;
 // enters every leaf key (the lowest index of equal keys counts) and the levels below each coarse cell
 __global__ void __launch_bounds__(256) k_leaf_enter(const uint64_t* __restrict__ keys, int64_t n,
                                                     uint64_t* __restrict__ table, uint32_t* __restrict__ idx, int bits,
-                                                    uint32_t* __restrict__ coarse, uint32_t* __restrict__ fail) {
+                                                    uint64_t salt, uint32_t* __restrict__ coarse,
+                                                    uint32_t* __restrict__ fail) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t < n) {
         const uint64_t k = keys[t];
         const int l = (int)((k >> 57) & 31);
         const uint32_t lev = 1u << l;
-        if (k != HT_EMPTY) atomicMin(idx + ht_enter(table, bits, k, fail), (uint32_t)t);
+        if (k != HT_EMPTY) atomicMin(idx + ht_enter(table, bits, salt, k, fail), (uint32_t)t);
         if (l >= SD_COARSE) {
             const int sh = l - SD_COARSE;
             const uint32_t x = (uint32_t)((k & kIMask) >> sh), y = (uint32_t)(((k >> 19) & kIMask) >> sh),
@@ -360,7 +365,7 @@ __global__ void __launch_bounds__(256) k_subdiv_flags(const float4* __restrict__
                                                       double root_size, double fine, double inv_fine,
                                                       uint32_t look_at, double thr,
                                                       const uint64_t* __restrict__ table,
-                                                      const uint32_t* __restrict__ idx, int bits,
+                                                      const uint32_t* __restrict__ idx, int bits, uint64_t salt,
                                                       const uint32_t* __restrict__ coarse, uint8_t* __restrict__ split) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool live = t < m;
@@ -444,7 +449,7 @@ __global__ void __launch_bounds__(256) k_subdiv_flags(const float4* __restrict__
             }
             __syncwarp();
             const uint64_t key = ((uint64_t)l << 57) | ((uint64_t)z << 38) | ((uint64_t)y << 19) | (uint64_t)x;
-            const uint32_t e = ht_find(table, bits, key, look);
+            const uint32_t e = ht_find(table, bits, salt, key, look);
             if (e != ~0u) split[idx[e]] = 1;
             // the next cell, x fastest
             if (++x == lo[0] + n[0]) {
@@ -471,7 +476,7 @@ constexpr int64_t FAR_CELLS = 4096;  // cells of the point grid a leaf looks int
 __global__ void __launch_bounds__(256) k_subdiv_far(const uint64_t* __restrict__ keys, int64_t n, uint32_t far, Frame f,
                                                     double root_size, double thr, const uint64_t* __restrict__ table,
                                                     const uint32_t* __restrict__ idx, int bits,
-                                                    const uint64_t* __restrict__ cells, int cell_bits,
+                                                    const uint64_t* __restrict__ cells, int cell_bits, uint64_t salt,
                                                     const uint32_t* __restrict__ cnt, const uint32_t* __restrict__ start,
                                                     const float4* __restrict__ pts, int64_t m, double inv_h,
                                                     uint8_t* __restrict__ split) {
@@ -484,7 +489,7 @@ __global__ void __launch_bounds__(256) k_subdiv_far(const uint64_t* __restrict__
     const int x = (int)(k & kIMask), y = (int)((k >> 19) & kIMask), z = (int)((k >> 38) & kIMask);
     // a key that is no cell of the grid is in no point's reach; of equal keys the lowest index counts
     if (k >> 62 || (x | y | z) >> l) return;
-    const uint32_t e = ht_find(table, bits, k, true);
+    const uint32_t e = ht_find(table, bits, salt, k, true);
     if (e == ~0u || (int64_t)idx[e] != t) return;
     const double s = ldexp(root_size, -l);
     const int at[3] = {x, y, z};
@@ -543,7 +548,7 @@ __global__ void __launch_bounds__(256) k_subdiv_far(const uint64_t* __restrict__
         for (int b = 0; b < nc && !hit; b += 32) {
             const int c = (b + lane + nc / 2) % nc;
             const uint64_t key = cell_key(c0[0] + c % w[0], c0[1] + c / w[0] % w[1], c0[2] + c / (w[0] * w[1]));
-            const uint32_t slot = ht_find(cells, cell_bits, key, b + lane < nc);
+            const uint32_t slot = ht_find(cells, cell_bits, salt, key, b + lane < nc);
             const uint32_t e0 = slot != ~0u ? start[slot] : 0u, m0 = slot != ~0u ? cnt[slot] : 0u;
             for (unsigned found = __ballot_sync(0xffffffffu, m0 != 0u); found && !hit; found &= found - 1) {
                 const int src = __ffs((int)found) - 1;
@@ -830,12 +835,13 @@ static Frame make_frame(const double* center, double root_size, int max_level) {
 
 cudaError_t soft_prior(const uint64_t* grid, int64_t n_corners, const double* center, double root_size, int max_level,
                        const float* cloud, int64_t m, float s_min, float v_close, float v_far, float* dens, Arena& ar,
-                       cudaStream_t s) {
+                       cudaStream_t s, bool* no_room) {
+    *no_room = false;
     if (n_corners <= 0) return cudaSuccess;
     const Frame f = make_frame(center, root_size, max_level);
     const double h = 3.0 * (double)s_min, inv_h = 1.0 / h;
     if (m <= 0) {
-        k_soft_prior<<<nb(n_corners), 256, 0, s>>>(grid, n_corners, f, h, inv_h, nullptr, 0, nullptr, nullptr, 0, nullptr,
+        k_soft_prior<<<nb(n_corners), 256, 0, s>>>(grid, n_corners, f, h, inv_h, nullptr, 0, 0, nullptr, nullptr, 0, nullptr,
                                                    s_min, v_close, v_far, dens);
         count_launches(1);
         return cudaGetLastError();
@@ -843,8 +849,11 @@ cudaError_t soft_prior(const uint64_t* grid, int64_t n_corners, const double* ce
     uint32_t* slot = ar.alloc<uint32_t>(m);
     uint32_t* rank = ar.alloc<uint32_t>(m);
     float4* pts = ar.alloc<float4>(m);
+    const int held = ar.n;
     for (int more = 0; more < HT_TRIES; ++more) {
+        ar.release(held);  // a table that was too small
         const int bits = std::min(ht_bits(m) + more, 32);
+        const uint64_t salt = ht_salt(more);
         const size_t cap = (size_t)1 << bits;
         uint64_t* table = ar.alloc<uint64_t>(cap);
         uint32_t* cnt = ar.alloc<uint32_t>(cap + 2);  // then: points placed so far, a key without a slot
@@ -853,10 +862,10 @@ cudaError_t soft_prior(const uint64_t* grid, int64_t n_corners, const double* ce
         cudaError_t e = cudaMemsetAsync(table, 0xff, cap * sizeof(uint64_t), s);
         if (e == cudaSuccess) e = cudaMemsetAsync(cnt, 0, (cap + 2) * sizeof(uint32_t), s);
         if (e != cudaSuccess) return e;
-        k_cell_count<true><<<nb(m), 256, 0, s>>>(cloud, m, f, h, inv_h, table, bits, cnt, slot, rank, cnt + cap + 1);
+        k_cell_count<true><<<nb(m), 256, 0, s>>>(cloud, m, f, h, inv_h, table, bits, salt, cnt, slot, rank, cnt + cap + 1);
         k_cell_alloc<<<(unsigned)(cap / 256), 256, 0, s>>>(cnt, (int64_t)cap, start, cnt + cap);
         k_cell_scatter<<<nb(m), 256, 0, s>>>(cloud, m, slot, rank, start, pts);
-        k_soft_prior<<<nb(n_corners), 256, 0, s>>>(grid, n_corners, f, h, inv_h, table, bits, cnt, start, m, pts, s_min,
+        k_soft_prior<<<nb(n_corners), 256, 0, s>>>(grid, n_corners, f, h, inv_h, table, bits, salt, cnt, start, m, pts, s_min,
                                                    v_close, v_far, dens);
         count_launches(4);
         uint32_t failed = 0;
@@ -865,7 +874,8 @@ cudaError_t soft_prior(const uint64_t* grid, int64_t n_corners, const double* ce
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess || !failed) return e;
     }
-    return cudaErrorUnknown;  // no table of eight times the capacity has room within HT_PROBES of every key's home
+    *no_room = true;  // no table up to eight times the capacity has room within HT_PROBES of every key's home
+    return cudaSuccess;
 }
 
 // Levels at which a leaf looks for points: those where the cells in reach of a point may be more than FAR_FROM, and more
@@ -878,8 +888,9 @@ constexpr double FAR_FROM = 512.0, FAR_SHARE = 1.0 / 100.0;
 
 cudaError_t subdivide_round(const uint64_t* keys, int64_t n, uint32_t levels, const double* center, double root_size,
                             int max_level, const float* cloud, int64_t m, float thr, uint64_t* out, int64_t* n_out,
-                            Arena& ar, cudaStream_t s) {
+                            Arena& ar, cudaStream_t s, bool* no_room) {
     *n_out = n;
+    *no_room = false;
     if (n <= 0) return cudaSuccess;
     const Frame f = make_frame(center, root_size, max_level);
     constexpr int COARSE = SD_SIDE * SD_SIDE * SD_SIDE;
@@ -897,7 +908,10 @@ cudaError_t subdivide_round(const uint64_t* keys, int64_t n, uint32_t levels, co
         if (side * side * side > std::max(FAR_FROM, FAR_SHARE * (double)n)) far |= levels & (1u << l);
     }
     uint32_t hd[3] = {0, 0, 0};
+    const int held = ar.n;
     for (int more = 0; more < HT_TRIES; ++more) {
+        ar.release(held);  // a table that was too small
+        const uint64_t salt = ht_salt(more);
         cudaError_t e = cudaMemsetAsync(split, 0, n, s);
         if (e == cudaSuccess) e = cudaMemsetAsync(tot, 0, 3 * sizeof(uint32_t), s);
         if (e != cudaSuccess) return e;
@@ -925,21 +939,21 @@ cudaError_t subdivide_round(const uint64_t* keys, int64_t n, uint32_t levels, co
             if (e != cudaSuccess) return e;
             const double h = far ? 0.5 * std::min((double)thr, 4.0 * root_size)
                                  : std::max(16.0 * (double)thr, ldexp(root_size, -SD_FINE));
-            k_cell_count<false><<<nb(m), 256, 0, s>>>(cloud, m, f, h, 1.0 / h, cells, pbits, cnt, slot, rank,
+            k_cell_count<false><<<nb(m), 256, 0, s>>>(cloud, m, f, h, 1.0 / h, cells, pbits, salt, cnt, slot, rank,
                                                       far ? tot + 2 : cnt + pcap + 1);
             k_cell_alloc<<<(unsigned)(pcap / 256), 256, 0, s>>>(cnt, (int64_t)pcap, start, cnt + pcap);
             k_cell_scatter<<<nb(m), 256, 0, s>>>(cloud, m, slot, rank, start, pts);
-            k_leaf_enter<<<nb(n), 256, 0, s>>>(keys, n, table, idx, bits, coarse, tot + 2);
+            k_leaf_enter<<<nb(n), 256, 0, s>>>(keys, n, table, idx, bits, salt, coarse, tot + 2);
             count_launches(4);
             if (levels & ~far) {
                 k_subdiv_flags<<<nb(m), 256, 0, s>>>(pts, m, f, root_size, ldexp(root_size, -SD_FINE),
                                                      (double)(1 << SD_FINE) / root_size, levels & ~far, thr, table, idx,
-                                                     bits, coarse, split);
+                                                     bits, salt, coarse, split);
                 count_launches(1);
             }
             if (far) {
                 k_subdiv_far<<<(unsigned)((n + 7) / 8), 256, 0, s>>>(keys, n, far, f, root_size, thr, table, idx, bits, cells,
-                                                                     pbits, cnt, start, pts, m, 1.0 / h, split);
+                                                                     pbits, salt, cnt, start, pts, m, 1.0 / h, split);
                 count_launches(1);
             }
         }
@@ -952,7 +966,11 @@ cudaError_t subdivide_round(const uint64_t* keys, int64_t n, uint32_t levels, co
         if (e != cudaSuccess) return e;
         if (!hd[2]) break;
     }
-    if (hd[2]) return cudaErrorUnknown;  // see soft_prior
+    if (hd[2]) {  // see soft_prior
+        *no_room = true;
+        *n_out = 0;
+        return cudaSuccess;
+    }
     const int64_t n_split = hd[0], n_keep = hd[1];
     k_subdiv_write<<<nb(n), 256, 0, s>>>(keys, n, split, pos_k, pos_s, n_keep, n_split, out);
     count_launches(1);

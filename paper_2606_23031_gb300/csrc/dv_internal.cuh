@@ -149,9 +149,10 @@ struct Arena {
         ptrs[n++] = p;
         return (T*)p;
     }
-    void release() {
-        for (int i = 0; i < n; ++i) cudaFreeAsync(ptrs[i], stream);
-        n = 0;
+    // frees the blocks from the keep-th on
+    void release(int keep = 0) {
+        for (int i = keep; i < n; ++i) cudaFreeAsync(ptrs[i], stream);
+        n = n < keep ? n : keep;
     }
 };
 
@@ -273,11 +274,12 @@ cudaError_t shared_corners(const uint64_t* keys, int64_t n, int max_level, bool 
                            int64_t* n_corners, Arena& ar, cudaStream_t s, bool* sort_timeout);
 cudaError_t soft_prior(const uint64_t* grid, int64_t n_corners, const double* center, double root_size, int max_level,
                        const float* cloud, int64_t m, float s_min, float v_close, float v_far, float* dens, Arena& ar,
-                       cudaStream_t s);
-// levels: those of the keys, as a bit mask
+                       cudaStream_t s, bool* no_room);
+// levels: those of the keys, as a bit mask.  *no_room (here and in soft_prior; host): no hash table tried had room for
+// every key, the result is invalid
 cudaError_t subdivide_round(const uint64_t* keys, int64_t n, uint32_t levels, const double* center, double root_size,
                             int max_level, const float* cloud, int64_t m, float thr, uint64_t* out, int64_t* n_out,
-                            Arena& ar, cudaStream_t s);
+                            Arena& ar, cudaStream_t s, bool* no_room);
 // uniform leaf grid of an actor (Sec. 3.3, assets): keys of the 8^level leaves (i fastest) and every
 // corner density set to v_init
 cudaError_t asset_grid(int level, float v_init, uint64_t* keys, float* dens, cudaStream_t s);

@@ -376,6 +376,49 @@ def test_subdivide_reach_of_many_leaves(dv, center, root, thr, levels):
     np.testing.assert_array_equal(out.cpu().numpy().view(np.uint64), ref)
 
 
+def _crowded(candidates):
+    """100 keys whose homes in the hash tables of 2^10 to 2^13 slots (unsalted) are the same slot each."""
+    with np.errstate(over="ignore"):
+        h = candidates ^ (candidates >> np.uint64(32))
+        h = h * np.uint64(0x9e3779b97f4a7c15)
+        h = (h ^ (h >> np.uint64(29))) * np.uint64(0x9e3779b97f4a7c15)
+    home = (h >> np.uint64(51)).astype(np.int64)
+    return candidates[home == np.bincount(home).argmax()][:100]
+
+
+# keys that find no slot within the probes of their home in any unsalted table: leaf keys of the subdivision, cells of
+# the prior's points
+@pytest.mark.gpu
+def test_crowded_hash_tables(dv):
+    import torch
+    rng = np.random.default_rng(12)
+    L, center, root = 12, (0.0, 0.0, 0.0), 4096.0
+    c = rng.integers(0, 1 << L, (1 << 20, 3))
+    keys = _crowded(np.unique(synth.pack_keys(np.full(len(c), L), *c.T)))
+    _, *ijk = oi._unpack(keys)
+    centres = np.stack(ijk, 1) + 0.5 - 2048.0
+    assert len(keys) == 100
+    cloud = torch.as_tensor(np.float32(centres[::2]), device="cuda")
+    out = dv.dv_subdivide_round(_keys_t(keys), L, center, root, cloud, 0.25)
+    hit = _reached(keys, center, root, centres[::2], 0.25)
+    assert hit[::2].all()
+    np.testing.assert_array_equal(out[:(~hit).sum()].cpu().numpy().view(np.uint64), keys[~hit])
+    assert out.numel() == (~hit).sum() + 8 * hit.sum()
+    # cells of the points at s_min = 1 / 3: the finest cells, offset by 2^20
+    cell = np.unique(np.concatenate([(z + (1 << 20) << 42) | (y + (1 << 20) << 21) | (x + (1 << 20))
+                                     for x, y, z in [rng.integers(0, 1 << L, (3, 1 << 20))]]).astype(np.uint64))
+    cell = _crowded(cell).astype(np.int64)
+    assert len(cell) == 100
+    at = np.stack([cell & 0x1fffff, (cell >> 21) & 0x1fffff, cell >> 42], 1) - (1 << 20)
+    s = float(np.float32(1.0 / 3.0))
+    pts = np.float32(at + 0.5 - 2048.0)
+    grid, _ = dv.dv_shared_corners(_keys_t(synth.pack_keys(np.full(100, L), *at.T)), L)
+    dens = dv.dv_soft_prior(grid, center, root, L, torch.as_tensor(pts, device="cuda"), s).cpu().numpy()
+    p, _ = oi.shared_corners(synth.pack_keys(np.full(100, L), *at.T), L)
+    ref = oi.soft_prior(oi.nearest_distance(oi.grid_to_world(p, center, root, L), np.float64(pts)), s)
+    np.testing.assert_allclose(dens, ref, rtol=0, atol=1e-5)
+
+
 @pytest.mark.gpu
 def test_visibility_many_cameras(dv):
     # cameras all around, inside and outside the root, with narrow and wide views; a ragged last block
