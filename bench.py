@@ -209,9 +209,11 @@ def stage_models(stats, work, n_vox_total, n_pix, K, sh_bytes_per_vox, key_bits)
 # unchanged.
 STAGE_KERNELS = {
     "project": (("k_project",), ("dv_project.cu", "dv_internal.cuh")),
-    "sort_vox": (("k_os_pass<unsigned long",), ("dv_scan_sort.cu", "dv_internal.cuh")),
+    "sort_vox": (("k_os_pass<unsigned long", "k_ol_count<unsigned long", "k_ol_scatter<unsigned long"),
+                 ("dv_scan_sort.cu", "dv_internal.cuh")),
     "records": (("k_records_emit",), ("dv_project.cu", "dv_internal.cuh")),
-    "sort_pairs": (("k_os_pass<unsigned int",), ("dv_scan_sort.cu", "dv_internal.cuh")),
+    "sort_pairs": (("k_os_pass<unsigned int", "k_ol_count<unsigned int", "k_ol_scatter<unsigned int"),
+                   ("dv_scan_sort.cu", "dv_internal.cuh")),
     "ranges": (("k_pair_mask", "k_tile_count", "k_tile_scatter"), ("dv_project.cu", "dv_internal.cuh")),
     "composite_fwd": (("k_composite<0", "k_composite_act<0"),
                       ("dv_composite.cu", "dv_composite_act.cu", "dv_composite.cuh", "dv_internal.cuh", "dv_project.cu")),
@@ -985,6 +987,9 @@ def build_traffic(csv_path, out_path=TRAFFIC):
         for sname, (kernels, _) in STAGE_KERNELS.items():
             if any(kn in e["name"] for kn in kernels):
                 st = sname
+        # a large sort scans its digit counts between counting and scattering
+        if "k_scan_" in e["name"] and stage_of and stage_of[-1] in ("sort_vox", "sort_pairs"):
+            st = stage_of[-1]
         stage_of.append(st)
     # the profiled pass renders the frame twice (plain, then with normals): the stages of the plain
     # frame are its first occurrence of each stage until the first composite_bwd and sh_bwd

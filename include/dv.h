@@ -337,7 +337,8 @@ dv_status dv_shared_corners(dv_ctx* ctx, const uint64_t* keys, int64_t n, int32_
  * the corner to the nearest point of cloud[n_points][3] (device, world frame;
  * the paper's values are v_close = -2, v_far = -10).  Points farther than
  * 3 s_min are not searched: they would change the prior by at most
- * 8 exp(-18) ~ 1e-7, below float resolution at v_far.
+ * 8 exp(-18) ~ 1e-7, below float resolution at v_far.  DV_ERR_CAPACITY (dens
+ * invalid) if the points' cells found no room in a hash table.
  */
 dv_status dv_soft_prior(dv_ctx* ctx, const uint64_t* grid, int64_t n_corners, const double* center, double root_size,
                         int32_t max_level, const float* cloud, int64_t n_points, float s_min, float v_close,
@@ -346,10 +347,13 @@ dv_status dv_soft_prior(dv_ctx* ctx, const uint64_t* grid, int64_t n_corners, co
 /*
  * One round of proximity subdivision (Sec. 3.3, step 2): every leaf whose box
  * lies within `threshold` (Euclidean point-to-box distance) of a point of cloud
- * is replaced by its eight children.  out (device, capacity 8n) receives the
- * kept leaves in input order, then child 0 of every split leaf (in input
- * order), then child 1, ..., child 7; *n_out (host) its length.  Children must
- * stay within level 18 (max_level < 18).
+ * is replaced by its eight children.  (At exactly the threshold, a leaf of size s
+ * counts where its index along each axis is one of floor((p - threshold) / s) to
+ * floor((p + threshold) / s): with its lower face there, not with its upper one.)
+ * out (device, capacity 8n) receives the kept leaves in input order, then child 0
+ * of every split leaf (in input order), then child 1, ..., child 7; *n_out (host)
+ * its length.  Children must stay within level 18 (max_level < 18).  DV_ERR_CAPACITY (nothing written) if the
+ * leaf keys found no room in a hash table.
  */
 dv_status dv_subdivide_round(dv_ctx* ctx, const uint64_t* keys, int64_t n, int32_t max_level, const double* center,
                              double root_size, const float* cloud, int64_t n_points, float threshold, uint64_t* out,

@@ -59,6 +59,25 @@ def test_traffic_grouping_and_units(tmp_path):
     assert k["launches"] == 2 and k["bytes"] == 11_500_000.0 and k["us"] == 109.0
 
 
+def test_traffic_of_large_sorts(tmp_path):
+    # counted sorts: the scans between a pass's counts and its scatter are the sort's, others are not
+    launches = [("k_project(x)", "1.0", "0", "10")]
+    for key in ("unsigned long", "unsigned int"):
+        launches += [(f"void k_ol_count<{key}>(x)", "1.0", "0", "1"), ("void k_scan_reduce<unsigned int, unsigned int>(x)", "0.5", "0", "2"),
+                     ("void k_scan_top<unsigned int>(x)", "0.5", "0", "3"), ("void k_scan_down<unsigned int, unsigned int>(x)", "0.5", "0", "4"),
+                     (f"void k_ol_scatter<{key}>(x)", "2.0", "0", "5")]
+        launches.append(("k_records_emit(x)", "1.0", "0", "1"))
+    launches += [("void k_scan_top<unsigned long>(x)", "9.0", "0", "9"), ("void k_sh_bwd<0>(x)", "2.0", "0", "15")]
+    src = tmp_path / "launches.csv"
+    src.write_text(_csv(launches))
+    out = tmp_path / "traffic.json"
+    assert bench.build_traffic(str(src), str(out)) == 0
+    st = json.loads(out.read_text())["stages"]
+    for name in ("sort_vox", "sort_pairs"):
+        assert st[name]["bytes_per_launch"] == 4_500_000 and st[name]["us_ncu"] == 15.0
+    assert st["records"]["bytes_per_launch"] == 2_000_000
+
+
 def test_stage_models_hand_checked():
     stats = {"n_visible": 10, "n_pairs": 40, "n_tiles": 300}
     work = {"tests": 1000, "box_tests": 50, "segments": 400}

@@ -57,10 +57,12 @@ def _row_of_actors(n, level):
     return synth.Scene(octs, poses), cam, count.max()
 
 
-# 1 to 4 and 5 or more boxes on a tile; up to 8, 9 to 32 and more than 32 intervals on a ray; few and many pairs
+# 1 to 4 and 5 or more boxes on a tile; up to 8, 9 to 32 and more than 32 intervals on a ray; few and many pairs; the
+# code for one sample and for several
 @pytest.mark.gpu
+@pytest.mark.parametrize("K", [2, 1])
 @pytest.mark.parametrize("n,level,crowded", [(3, 5, True), (7, 4, True), (14, 4, True), (36, 4, True), (12, 1, False)])
-def test_actor_tiles(dv, n, level, crowded):
+def test_actor_tiles(dv, n, level, crowded, K):
     import torch
     sc, cam, most = _row_of_actors(n, level)
     assert most >= 1023 if crowded else most < 300
@@ -69,7 +71,7 @@ def test_actor_tiles(dv, n, level, crowded):
     g = [np.float64(np.float32(x)) for x in (rng.normal(size=(P, 3)), 0.1 * rng.normal(size=P), rng.normal(size=P),
                                              rng.normal(size=(P, 3)))]
     ds = device_scene(sc)
-    opts = dv.make_opts(2, 1e-4)
+    opts = dv.make_opts(K, 1e-4)
     rgb, depth, alpha, nrm, st = dv.dv_render(ds, sc.poses, [cam], opts, save_state=True, normals=True)
     t = lambda a: torch.as_tensor(np.ascontiguousarray(a, np.float32), device="cuda")
     d_dens = [torch.zeros_like(o.dens) for o in ds]
@@ -77,11 +79,11 @@ def test_actor_tiles(dv, n, level, crowded):
     dv.dv_render_backward(st, t(g[0]), t(g[1]), t(g[2]), d_dens, d_sh, d_normal=t(g[3]))
     torch.cuda.synchronize()
     st.free()
-    o = oracle.render(sc.octrees, sc.poses, cam, oracle.Opts(2, 1e-4), normals=True)
+    o = oracle.render(sc.octrees, sc.poses, cam, oracle.Opts(K, 1e-4), normals=True)
     im = lambda x, c=None: split_images(x.cpu().numpy(), [cam], c)[0]
     check_forward(im(rgb, 3), im(depth), im(alpha), o[0], o[1], o[2], f"{n} actors")
     assert np.abs(im(nrm, 3) - o[4]).max() <= N_ATOL
-    od, os_ = oracle.backward(sc.octrees, sc.poses, cam, g[0], g[1], g[2], oracle.Opts(2, 1e-4), g_normal=g[3])
+    od, os_ = oracle.backward(sc.octrees, sc.poses, cam, g[0], g[1], g[2], oracle.Opts(K, 1e-4), g_normal=g[3])
     check_grads([x.cpu().numpy() for x in d_dens], od, f"{n} actors d_dens")
     check_grads([x.cpu().numpy() for x in d_sh], os_, f"{n} actors d_sh")
     # the exported weights of a pixel add up to its alpha
@@ -486,6 +488,31 @@ def _side_path(idx, level, X, Lk):
     return (1 << top) | ((~idx if (cell >> top) & 1 else idx) & ((1 << top) - 1))
 
 
+# the device's depth order, through images that depend on it: leaves of four levels, cameras on the planes of nodes of
+# several levels, on a face and a corner of the root, inside leaves and outside the root on either side of each axis
+@pytest.mark.gpu
+@pytest.mark.parametrize("eye", [(0.0, 0.0, 0.0), (0.25, -0.5, 0.125), (0.5, 0.0625, -0.75), (0.11, -0.23, 0.37),
+                                 (-1.0, 0.3, 0.0), (1.0, 1.0, -1.0), (1.75, -1.5, 1.25), (-2.0, 0.25, 0.5)])
+def test_depth_order(dv, eye):
+    rng = np.random.default_rng(21)
+    i, j, k = np.unravel_index(np.arange(8), (2, 2, 2))
+    keys = []
+    for level in (1, 2, 3, 4):  # most of a level's cells are split further
+        split = rng.uniform(size=i.size) < (0.0 if level == 4 else 0.8)
+        keys.append(synth.pack_keys(np.full((~split).sum(), level), i[~split], j[~split], k[~split]))
+        c = np.arange(8)
+        i, j, k = ((2 * x[split][:, None] + (c >> n & 1)).ravel() for n, x in ((0, i), (1, j), (2, k)))
+    key = np.concatenate(keys)
+    sc = synth.Scene([_octree(key[rng.permutation(key.size)], 1.0, rng, 2.0, degree=0)], [synth.Pose()])
+    for at in ((0.05, 0.1, -0.2), (0.9, -0.7, 0.3)):
+        cam = synth.pinhole(31, 23, 70.0, synth.look_at(eye, at), 0.02, 20.0)
+        rgb, depth, alpha, _ = gpu_render(device_scene(sc), sc.poses, [cam], eps=0.0)
+        o = oracle.render(sc.octrees, sc.poses, cam, oracle.Opts(1, 0.0))
+        im = lambda x, c=None: split_images(x.cpu().numpy(), [cam], c)[0]
+        check_forward(im(rgb, 3), im(depth), im(alpha), o[0], o[1], o[2], f"eye {eye}")
+
+
+# (the formula alone, in Python; test_depth_order has the kernel)
 @pytest.mark.parametrize("Lk", [0, 1, 4])
 def test_depth_path_closed_form(Lk):
     # node by node: at each node on the way to the leaf, the bit is flipped where the camera lies on the positive
