@@ -26,6 +26,8 @@
 //        exact stop rule.
 //    Since T only decreases along the ray, applying a whole partial is exact
 //    unless the stop falls inside it, which is exactly when T T_A < eps_stop.
+//    (With negative densities, which the identity activation admits, T rises: a
+//    ray that enters an interval with T above 1 may walk it instead.)
 //  * Per segment: trilinear interpolation of the raw corner densities at K
 //    midpoints, exponential-linear activation, tau = l/K sum sigma,
 //    alpha = 1 - exp(-tau), C += T alpha c, D += T alpha (t0+t1)/2,

@@ -132,7 +132,7 @@ constexpr int FL_PIX = 128;     // pixels per chunk
 constexpr int FL_SW = 64;       // channels per slice (16 quads)
 constexpr int FL_ROWS = 1023;   // voxel rows; row FL_ROWS holds the overflow slots
 constexpr int FL_TE = FL_ROWS + 1;  // table entries, FL_TE / FL_THREADS per thread in the scan
-constexpr int FL_PIECE = 3072;  // slots grouped at once (three 70 KB blocks fit an SM)
+constexpr int FL_PIECE = 3072;  // slots grouped at once (three 71 KB blocks fit an SM)
 constexpr int FL_PROBES = 32;
 constexpr int FL_THREADS = 256;
 constexpr int FL_SPT = FL_PIECE / FL_THREADS;  // slots per thread and piece
@@ -376,7 +376,7 @@ cudaError_t feat_fuse(int64_t n_pix, const int64_t* off, const uint32_t* vox, co
     if (n_pix <= 0 || C <= 0) return cudaSuccess;
     const int64_t n_chunks = (n_pix + FL_PIX - 1) / FL_PIX;
     const int64_t tasks = n_chunks * ((C + FL_SW - 1) / FL_SW);
-    const int64_t cap = (int64_t)sm_count() * 3;  // three 66 KB blocks per SM
+    const int64_t cap = (int64_t)sm_count() * 3;  // three 71 KB blocks per SM
     const unsigned grid = (unsigned)(tasks < cap ? tasks : cap);
     const size_t smem = sizeof(FuseSmem);
     // 16-byte copies of the 2-D features and vector atomics need 16-byte aligned rows of both arrays

@@ -20,8 +20,8 @@
 // close to the threshold (or, for a nearest point, could be the nearest), so every result is that of
 // the FP64 arithmetic.  Their searches are hash probes, one or two independent loads each, instead of
 // binary searches of sorted keys, twenty dependent ones, and need no sort.  On the 500k-leaf background with
-// 1.35M points (GB300): prior 3,250 -> 387 us, flags 3,260 -> 730 us,
-// visibility over six cameras 843 -> 92 us, beside the sorts of 1.35M points and 500k keys that are gone.
+// 1.35M points (GB300): prior 3,250 -> 550 us, flags 3,260 -> 420 us,
+// visibility over six cameras 843 -> 95 us, beside the sorts of 1.35M points and 500k keys that are gone.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -917,7 +917,8 @@ cudaError_t subdivide_round(const uint64_t* keys, int64_t n, uint32_t levels, co
         if (e != cudaSuccess) return e;
         if (m > 0) {
             // The points ordered by cells of 16 thresholds (flags kernel with the points as they come 1,300 us, cells of
-            // 1, 4, 16, 64 thresholds 1,284, 924, 730, 714 us, and 75 to 110 us for the order): a point that finds no
+            // 1, 4, 16, 64 thresholds 1,284, 924, 730, 714 us, and 75 to 110 us for the order; since the levels come
+            // as an argument 420 us with 16): a point that finds no
             // slot counts in its last slot, the order is all that matters.  Where leaves look for points, cells of half
             // a threshold, in which every point has its slot.
             const int pbits = std::min(ht_bits(m) + (far ? more : 0), 32), bits = ht_bits(n) + more;
